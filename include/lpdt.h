@@ -197,7 +197,10 @@ lpdt_status lpdt_quantize_static(const float *x, int32_t nodes, int64_t n_per_no
  *            shortcut (the block-output gradient joins the gradient of the block's first convolution),
  *            fused into the contraction's epilogue; dAacc is not affected.
  * ws       : lpdt_qconv_workspace_size(desc, which) bytes, which = 0 fwd,
- *            1 bwd_data, 2 bwd_weight.
+ *            1 bwd_data, 2 bwd_weight.  Part of it holds padded copies of operands
+ *            whose channel count is no multiple of 16; a workspace without room for
+ *            them (fwd: none at all) is accepted and the product, the same to the
+ *            bit, runs on the CUDA cores.
  * Errors: INVALID_ARG, UNSUPPORTED (shape outside every kernel's range),
  *         WORKSPACE, CUDA; TIMEOUT is reported through dev_status.
  */

@@ -1,9 +1,10 @@
 // Front end of the quantized contractions: argument validation, workspace
 // accounting and the choice between the tensor-core engine and the CUDA-core
-// kernels.  Layers whose input channel count is not a multiple of 16 (the RGB
-// first layer) reach the tensor-core engine through zero-padded copies of the
-// activations and weights held in the workspace: zero channels add nothing to an
-// integer sum, so the result is unchanged.
+// kernels.  Operands whose channel count is not a multiple of 16 (the RGB first
+// layer, a classifier's class scores) have rows that TMA cannot address; the engine
+// reads copies of them in the workspace whose rows are padded with zeros to the next
+// multiple: zero channels add nothing to an integer sum, so the result is unchanged.
+// Results keep the caller's channel count.
 #include <stdlib.h>
 #include "common.cuh"
 #include "qconv_internal.cuh"
@@ -12,20 +13,38 @@ using namespace lpdt;
 
 namespace lpdt {
 
-// dst[row][0..Cp) = src[row][0..C) followed by zeros.  One thread per 16-byte piece of a
-// destination row (Cp is a multiple of 16), written with a single 16-byte store.
-__global__ void pad_channels_kernel(const int8_t *__restrict__ src, int8_t *__restrict__ dst, int64_t rows,
-                                    int C, int Cp) {
+// dst[row][0..Cp) = src[row][0..C) followed by zeros, Cp the next multiple of 16.  One thread per 16-byte piece of a
+// destination row, assembled from the aligned 4-byte words that hold it (rows start at any byte) and written with a
+// single 16-byte store.  blockIdx.y selects one of up to two tensors: both operands of a product in one launch.
+struct PadJob { const int8_t *src; int8_t *dst; int64_t rows; int C; };
+__global__ void pad_channels_kernel(const PadJob j0, const PadJob j1) {
     pdl_enter();
-    const int pieces = Cp / 16;
-    const int64_t total = rows * pieces;
+    const PadJob j = blockIdx.y ? j1 : j0;
+    const int C = j.C, pieces = (C + 15) / 16, Cp = pieces * 16;
+    const int64_t total = j.rows * pieces, bytes = j.rows * C;
+    const bool words = ((uintptr_t)j.src & 3) == 0;
     for (int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; o < total; o += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t row = o / pieces;
-        const int c0 = (int)(o % pieces) * 16;
-        union { int8_t b[16]; uint4 v; } u;
+        const int64_t row = total <= 0x7fffffff ? (int64_t)((uint32_t)o / (uint32_t)pieces) : o / pieces;
+        const int c0 = (int)(o - row * pieces) * 16, n = C - c0 < 16 ? C - c0 : 16;
+        const int64_t off = row * C + c0;
+        union { int8_t b[16]; uint32_t w[4]; uint4 v; } u;
+        if (words && ((off + n + 3) & ~(int64_t)3) <= bytes) {      // the last word lies inside the tensor
+            const uint32_t *p = reinterpret_cast<const uint32_t *>(j.src + (off & ~(int64_t)3));
+            const int sh = (int)(off & 3), need = (sh + n + 3) / 4;
+            uint32_t w[5];
 #pragma unroll
-        for (int k = 0; k < 16; ++k) u.b[k] = (c0 + k < C) ? src[row * C + c0 + k] : (int8_t)0;
-        *reinterpret_cast<uint4 *>(dst + row * Cp + c0) = u.v;
+            for (int k = 0; k < 5; ++k) w[k] = k < need ? __ldg(p + k) : 0u;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const uint32_t x = __funnelshift_r(w[k], w[k + 1], 8 * sh);
+                const int left = n - 4 * k;                          // bytes of this word that exist
+                u.w[k] = left >= 4 ? x : left <= 0 ? 0u : x & ((1u << (8 * left)) - 1u);
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < 16; ++k) u.b[k] = k < n ? j.src[off + k] : (int8_t)0;
+        }
+        *reinterpret_cast<uint4 *>(j.dst + row * Cp + c0) = u.v;
     }
 }
 
@@ -45,7 +64,6 @@ static bool tc_enabled() {
     }
     return !disabled;
 }
-static bool use_tc(const lpdt_conv_desc &d) { return tc_enabled() && tc::tc_supported(d); }
 // LPDT_DISABLE_HALO=1 keeps 16-channel layers on the general tensor-core kernel.
 static bool use_halo(const lpdt_conv_desc &d, int mode) {
     static int disabled = -1;
@@ -55,23 +73,21 @@ static bool use_halo(const lpdt_conv_desc &d, int mode) {
     }
     return !disabled && tc::halo_supported(d, mode);
 }
+static int pad16(int c) { return (c + 15) / 16 * 16; }
+static tc::Pitches pitches(const lpdt_conv_desc &d) { return {pad16(d.Cin), pad16(d.Cout), pad16(d.Cin)}; }
+
+// Operands in rows of pad16(channels) bytes.
 static lpdt_status run_pix(const lpdt_conv_desc &d, int mode, const int8_t *A, const float *s1, const int8_t *Wq,
                            const float *s2, const float *bias, int64_t bias_stride, float *Y, int32_t *Yacc,
-                           int32_t *dev_status, cudaStream_t st, bool uns = false, const float *addend = nullptr) {
-    if (use_halo(d, mode)) {
-        lpdt_status r = tc::tc_pix_halo(d, mode, A, s1, Wq, s2, bias, bias_stride, Y, Yacc, dev_status, st, uns, addend);
+                           int32_t *dev_status, cudaStream_t st, bool uns, const float *addend,
+                           const tc::AffineArgs *aff) {
+    lpdt_conv_desc dh = d;                   // the halo kernel pads the summed side only: its results are whole rows
+    if (mode == 0) dh.Cin = pad16(d.Cin);
+    if (!aff && use_halo(dh, mode)) {
+        lpdt_status r = tc::tc_pix_halo(dh, mode, A, s1, Wq, s2, bias, bias_stride, Y, Yacc, dev_status, st, uns, addend);
         if (r != LPDT_ERR_UNSUPPORTED) return r;
     }
-    return tc::tc_pix(d, mode, A, s1, Wq, s2, bias, bias_stride, Y, Yacc, dev_status, st, uns, addend);
-}
-
-static int pad16(int c) { return (c + 15) / 16 * 16; }
-// Input channels padded to a multiple of 16 make the shape eligible.
-static bool use_tc_padded(const lpdt_conv_desc &d, lpdt_conv_desc *dp) {
-    if (!tc_enabled() || d.Cin % 16 == 0) return false;
-    *dp = d;
-    dp->Cin = pad16(d.Cin);
-    return tc::tc_supported(*dp);
+    return tc::tc_pix(d, mode, A, s1, Wq, s2, bias, bias_stride, Y, Yacc, dev_status, st, uns, addend, aff, pitches(d));
 }
 
 static lpdt_status check_desc(const lpdt_conv_desc *d) {
@@ -82,49 +98,92 @@ static lpdt_status check_desc(const lpdt_conv_desc *d) {
     return LPDT_OK;
 }
 
-struct PadPlan { size_t a_bytes, w_bytes, acc_bytes; };
+// Zero-padded copies of the operands whose channel count is no multiple of 16 (0 bytes for the others).
+struct PadPlan { size_t in, err, w; };
 static PadPlan pad_plan(const lpdt_conv_desc &d) {
-    const size_t Cp = pad16(d.Cin);
-    PadPlan p;
-    p.a_bytes = align_up((size_t)d.nodes * d.B * d.H * d.W * Cp, 256);
-    p.w_bytes = align_up((size_t)d.nodes * d.Cout * d.R * d.S * Cp, 256);
-    p.acc_bytes = align_up((size_t)d.nodes * d.Cout * d.R * d.S * Cp * sizeof(int32_t), 256);
+    const int Ho = conv_out(d.H, d.pad, d.R, d.stride), Wo = conv_out(d.W, d.pad, d.S, d.stride);
+    PadPlan p = {0, 0, 0};
+    if (d.Cin % 16) {
+        p.in = align_up((size_t)d.nodes * d.B * d.H * d.W * pad16(d.Cin), 256);
+        p.w = align_up((size_t)d.nodes * d.Cout * d.R * d.S * pad16(d.Cin), 256);
+    }
+    if (d.Cout % 16) p.err = align_up((size_t)d.nodes * d.B * Ho * Wo * pad16(d.Cout), 256);
     return p;
 }
+static PadJob pad_job(const int8_t *src, void *dst, int64_t rows, int C) { return {src, (int8_t *)dst, rows, C}; }
+// One launch for up to two tensors (rows = 0: none).
+static lpdt_status pad_launch(PadJob a, PadJob b, cudaStream_t st) {
+    if (a.rows == 0) { a = b; b.rows = 0; }
+    if (a.rows == 0) return LPDT_OK;
+    const int64_t na = a.rows * (pad16(a.C) / 16), nb = b.rows ? b.rows * (pad16(b.C) / 16) : 0;
+    launch_k(pad_channels_kernel, dim3(grid_for(na > nb ? na : nb), b.rows ? 2 : 1), 256, 0, st, a, b);
+    LPDT_LAUNCH_CHECK();
+    return LPDT_OK;
+}
 
-extern "C" size_t lpdt_qconv_workspace_size(const lpdt_conv_desc *d, int32_t which) {
+// The least workspace a call is accepted with: [transposed weights] of the CUDA-core backward-data kernel,
+// [int32 sums | padded input] of backward-weight.  With less than lpdt_qconv_workspace_size, which adds the padded
+// copies that the tensor-core engine reads, a shape that needs them runs on the CUDA cores.
+static size_t least_workspace(const lpdt_conv_desc *d, int32_t which) {
     if (!d || d->nodes <= 0 || check_desc(d) != LPDT_OK) return 256;
     const size_t wn = (size_t)d->nodes * d->Cout * d->R * d->S * d->Cin;
+    const PadPlan p = pad_plan(*d);
     size_t need = 256;
-    if (which == 1) need = align_up(wn, 256);                       // transposed weights
-    if (which == 2) need = align_up(wn * sizeof(int32_t), 256);     // int32 partial sums
-    if (d->Cin % 16) {
-        const PadPlan p = pad_plan(*d);
-        if (which == 0 && p.a_bytes + p.w_bytes > need) need = p.a_bytes + p.w_bytes;
-        if (which == 2) need += p.a_bytes;                              // + zero-padded copy of the input
-    }
+    if (which == 0 && p.in + p.w > need) need = p.in + p.w;
+    if (which == 1) need = align_up(wn, 256);
+    if (which == 2) need = align_up(wn * sizeof(int32_t), 256) + p.in;
+    return need;
+}
+extern "C" size_t lpdt_qconv_workspace_size(const lpdt_conv_desc *d, int32_t which) {
+    size_t need = least_workspace(d, which);
+    if (!d || d->nodes <= 0 || check_desc(d) != LPDT_OK) return need;
+    const PadPlan p = pad_plan(*d);
+    if (which == 1 && p.err + p.w > need) need = p.err + p.w;
+    if (which == 2) need += p.err;
     return need;
 }
 
-// Forward contraction on raw codes (signed, or unsigned when `uns`): kernel choice only.
+// Whether the tensor-core engine may take the shape with a workspace of ws_bytes.  Only shapes that need padded
+// copies look at the workspace.
+static bool use_tc(const lpdt_conv_desc &d, int which, const void *ws, size_t ws_bytes) {
+    if (!tc_enabled() || !tc::tc_supported(d)) return false;
+    const bool pads = which == 0 ? d.Cin % 16 : (d.Cin % 16 || d.Cout % 16);
+    return !pads || (ws && aligned(ws, 256) && ws_bytes >= lpdt_qconv_workspace_size(&d, which));
+}
+// Products that finish sooner on the CUDA cores although the tensor cores could take them: few results, each a dot
+// product of a few dozen steps (a classifier's scores and their adjoint).  The tensor-core kernel's fixed cost (barriers,
+// TMEM, first boxes) is about 6 us; measured 40 x 32 x 64 -> 10 forward 2.8 against 6.0 us and its adjoint 4.9
+// against 5.6, 8 x 32 x 512 -> 10 forward 9.9 against 6.7.  Only shapes that need padding; the others fill the tiles.
+static bool tiny_dot(const lpdt_conv_desc &d, int64_t results, int K, bool vec4) {
+    return (d.Cin % 16 || d.Cout % 16) && results <= (int64_t)kNumSMs * 2048 && (vec4 ? K / 4 : K) <= 64;
+}
+// An operand of `C` channels the engine can read: its padded copy, or itself at a 16-byte boundary.
+static bool readable(const void *p, int C) { return C % 16 != 0 || aligned(p, 16); }
+
+// Forward contraction on raw codes (signed, or unsigned when `uns`): kernel choice only.  With `aff` the zero-point
+// terms are applied in the epilogue, or UNSUPPORTED is returned.
 static lpdt_status fwd_impl(const lpdt_conv_desc *d, const int8_t *A, const float *sA, const int8_t *Wq,
                             const float *sW, const float *bias, int64_t bias_node_stride, float *Y, int32_t *Yacc,
-                            void *ws, size_t ws_bytes, int32_t *dev_status, cudaStream_t st, bool uns) {
+                            void *ws, size_t ws_bytes, int32_t *dev_status, cudaStream_t st, bool uns,
+                            const tc::AffineArgs *aff = nullptr) {
     const bool out_ok = (!Y || aligned(Y, 16)) && (!Yacc || aligned(Yacc, 16));
-    if (use_tc(*d) && aligned(A, 16) && aligned(Wq, 16) && out_ok)
-        return run_pix(*d, 0, A, sA, Wq, sW, bias, bias_node_stride, Y, Yacc, dev_status, st, uns);
-    lpdt_conv_desc dp;
-    if (use_tc_padded(*d, &dp) && out_ok && ws && aligned(ws, 256) &&
-        ws_bytes >= lpdt_qconv_workspace_size(d, 0)) {
-        const PadPlan pp = pad_plan(*d);
-        int8_t *Ap = (int8_t *)ws, *Wp = Ap + pp.a_bytes;
-        const int64_t arows = (int64_t)d->nodes * d->B * d->H * d->W, wrows = (int64_t)d->nodes * d->Cout * d->R * d->S;
-        launch_k(pad_channels_kernel, grid_for(arows * dp.Cin / 16), 256, 0, st, A, Ap, arows, d->Cin, dp.Cin);
-        LPDT_LAUNCH_CHECK();
-        launch_k(pad_channels_kernel, grid_for(wrows * dp.Cin / 16), 256, 0, st, Wq, Wp, wrows, d->Cin, dp.Cin);
-        LPDT_LAUNCH_CHECK();
-        return run_pix(dp, 0, Ap, sA, Wp, sW, bias, bias_node_stride, Y, Yacc, dev_status, st, uns);
+    const int64_t results = (int64_t)d->nodes * d->B * conv_out(d->H, d->pad, d->R, d->stride) *
+                            conv_out(d->W, d->pad, d->S, d->stride) * d->Cout;
+    const bool vec4 = d->Cin % 4 == 0 && aligned(A, 4) && aligned(Wq, 4);
+    if ((aff || !tiny_dot(*d, results, d->R * d->S * d->Cin, vec4)) && use_tc(*d, 0, ws, ws_bytes) && readable(A, d->Cin) && readable(Wq, d->Cin) && out_ok) {
+        const bool pad = d->Cin % 16 != 0;
+        const int8_t *Ae = A, *We = Wq;
+        if (pad) {
+            const PadPlan pp = pad_plan(*d);
+            Ae = (int8_t *)ws; We = Ae + pp.in;
+            lpdt_status s = pad_launch(pad_job(A, ws, (int64_t)d->nodes * d->B * d->H * d->W, d->Cin),
+                                       pad_job(Wq, (char *)ws + pp.in, (int64_t)d->nodes * d->Cout * d->R * d->S, d->Cin), st);
+            if (s != LPDT_OK) return s;
+        }
+        lpdt_status r = run_pix(*d, 0, Ae, sA, We, sW, bias, bias_node_stride, Y, Yacc, dev_status, st, uns, nullptr, aff);
+        if (r != LPDT_ERR_UNSUPPORTED || (!pad && d->Cout % 16 == 0)) return r;
     }
+    if (aff) return LPDT_ERR_UNSUPPORTED;
     return generic_fwd(*d, A, sA, Wq, sW, bias, bias_node_stride, Y, Yacc, st, uns);
 }
 
@@ -294,14 +353,18 @@ static size_t affine_raw_bytes(const lpdt_conv_desc *d) {
 static size_t affine_asum_bytes(const lpdt_conv_desc *d) {
     return align_up((size_t)d->nodes * d->B * d->H * d->W * sizeof(int32_t), 256);
 }
+// The prefix table may be read up to 31 entries past its end by the tensor-core epilogue: at least 256 bytes of
+// workspace (the contraction's own) follow it.
 static size_t affine_prefix_bytes(const lpdt_conv_desc *d) {     // prefix table + per-tap channel sums
     return align_up((size_t)d->nodes * d->Cout * (d->R + 1) * (d->S + 1) * sizeof(int32_t), 256) +
            align_up((size_t)d->nodes * d->Cout * d->R * d->S * sizeof(int32_t), 256);
 }
 
+static size_t affine_fwd_own(const lpdt_conv_desc *d) { return affine_raw_bytes(d) + affine_asum_bytes(d) + affine_prefix_bytes(d); }
+
 extern "C" size_t lpdt_qconv_fwd_affine_workspace_size(const lpdt_conv_desc *d) {
     if (!d || d->nodes <= 0 || check_desc(d) != LPDT_OK) return 256;
-    return affine_raw_bytes(d) + affine_asum_bytes(d) + affine_prefix_bytes(d) + lpdt_qconv_workspace_size(d, 0);
+    return affine_fwd_own(d) + lpdt_qconv_workspace_size(d, 0);
 }
 
 extern "C" lpdt_status lpdt_qconv_fwd_affine(const lpdt_conv_desc *d, const uint8_t *A, const float *sA,
@@ -315,7 +378,7 @@ extern "C" lpdt_status lpdt_qconv_fwd_affine(const lpdt_conv_desc *d, const uint
     LPDT_CHECK_ARG(A && Wq && zA && zW && (Y || Yacc));
     LPDT_CHECK_ARG(!Y || (sA && sW));
     LPDT_CHECK_ARG(!bias || bias_node_stride >= d->Cout || d->nodes == 1);
-    if (!ws || !aligned(ws, 256) || ws_bytes < lpdt_qconv_fwd_affine_workspace_size(d)) return LPDT_ERR_WORKSPACE;
+    if (!ws || !aligned(ws, 256) || ws_bytes < affine_fwd_own(d) + least_workspace(d, 0)) return LPDT_ERR_WORKSPACE;
     cudaStream_t st = as_stream(stream);
     const int Ho = conv_out(d->H, d->pad, d->R, d->stride), Wo = conv_out(d->W, d->pad, d->S, d->stride);
     int32_t *raw = (int32_t *)ws;
@@ -335,15 +398,15 @@ extern "C" lpdt_status lpdt_qconv_fwd_affine(const lpdt_conv_desc *d, const uint
     // memory, no second pass over the result).  LPDT_AFFINE_SEPARATE=1 keeps the separate correction pass.
     static int separate = -1;
     if (separate < 0) { const char *e = getenv("LPDT_AFFINE_SEPARATE"); separate = (e && e[0] == '1') ? 1 : 0; }
-    if (!separate && use_tc(*d) && d->Cout % 4 == 0 && aligned(A, 16) && aligned(Wq, 16) && (!Y || aligned(Y, 16)) &&
-        (!Yacc || aligned(Yacc, 16))) {
+    const size_t inner_bytes = ws_bytes - (size_t)((char *)inner - (char *)ws);
+    if (!separate && d->Cout % 4 == 0) {
         const tc::AffineArgs aff = {asum, P, zA, zW};
-        lpdt_status r = tc::tc_pix(*d, 0, reinterpret_cast<const int8_t *>(A), sA, reinterpret_cast<const int8_t *>(Wq), sW,
-                                   bias, bias_node_stride, Y, Yacc, dev_status, st, true, nullptr, &aff);
+        lpdt_status r = fwd_impl(d, reinterpret_cast<const int8_t *>(A), sA, reinterpret_cast<const int8_t *>(Wq), sW,
+                                 bias, bias_node_stride, Y, Yacc, inner, inner_bytes, dev_status, st, true, &aff);
         if (r != LPDT_ERR_UNSUPPORTED) return r;
     }
     s = fwd_impl(d, reinterpret_cast<const int8_t *>(A), nullptr, reinterpret_cast<const int8_t *>(Wq), nullptr, nullptr,
-                 0, nullptr, raw, inner, lpdt_qconv_workspace_size(d, 0), dev_status, st, true);
+                 0, nullptr, raw, inner, inner_bytes, dev_status, st, true);
     if (s != LPDT_OK) return s;
     const bool v4 = d->Cout % 4 == 0 && (!Y || aligned(Y, 16)) && (!Yacc || aligned(Yacc, 16));
     const int64_t work = (int64_t)d->nodes * d->B * Ho * Wo * (d->Cout / (v4 ? 4 : 1));
@@ -360,9 +423,21 @@ extern "C" lpdt_status lpdt_qconv_fwd_affine(const lpdt_conv_desc *d, const uint
 // Backward-data contraction on raw codes (signed, or unsigned when `uns`): kernel choice only.
 static lpdt_status bwd_data_impl(const lpdt_conv_desc *d, const int8_t *E, const float *sE, const int8_t *Wq,
                                  const float *sW, float *dA, int32_t *dAacc, const float *addend, void *ws,
-                                 int32_t *dev_status, cudaStream_t st, bool uns) {
-    if (use_tc(*d) && aligned(E, 16) && aligned(Wq, 16) && (!dA || aligned(dA, 16)) && (!dAacc || aligned(dAacc, 16)))
-        return run_pix(*d, 1, E, sE, Wq, sW, nullptr, 0, dA, dAacc, dev_status, st, uns, addend);
+                                 size_t ws_bytes, int32_t *dev_status, cudaStream_t st, bool uns) {
+    const int64_t results = (int64_t)d->nodes * d->B * d->H * d->W * d->Cin;
+    const bool vec4 = d->Cout % 4 == 0 && aligned(E, 4);
+    if (!tiny_dot(*d, results, d->R * d->S * d->Cout, vec4) && use_tc(*d, 1, ws, ws_bytes) && readable(E, d->Cout) && readable(Wq, d->Cin) && (!dA || aligned(dA, 16)) &&
+        (!dAacc || aligned(dAacc, 16))) {
+        const int Ho = conv_out(d->H, d->pad, d->R, d->stride), Wo = conv_out(d->W, d->pad, d->S, d->stride);
+        const PadPlan pp = pad_plan(*d);
+        void *Ep = ws, *Wp = (char *)ws + pp.err;
+        lpdt_status s = pad_launch(pad_job(E, Ep, pp.err ? (int64_t)d->nodes * d->B * Ho * Wo : 0, d->Cout),
+                                   pad_job(Wq, Wp, pp.w ? (int64_t)d->nodes * d->Cout * d->R * d->S : 0, d->Cin), st);
+        if (s != LPDT_OK) return s;
+        lpdt_status r = run_pix(*d, 1, pp.err ? (int8_t *)Ep : E, sE, pp.w ? (int8_t *)Wp : Wq, sW, nullptr, 0, dA, dAacc,
+                                dev_status, st, uns, addend, nullptr);
+        if (r != LPDT_ERR_UNSUPPORTED || (!pp.err && !pp.w)) return r;
+    }
     return generic_bwd_data(*d, E, sE, Wq, sW, dA, dAacc, addend, ws, st, uns);
 }
 
@@ -376,27 +451,26 @@ extern "C" lpdt_status lpdt_qconv_bwd_data(const lpdt_conv_desc *d, const int8_t
     LPDT_CHECK_ARG(E && Wq && (dA || dAacc));
     LPDT_CHECK_ARG(!dA || (sE && sW));
     LPDT_CHECK_ARG(!addend || (dA && addend != dA && aligned(addend, 16)));
-    if (!ws || ws_bytes < lpdt_qconv_workspace_size(d, 1)) return LPDT_ERR_WORKSPACE;
-    return bwd_data_impl(d, E, sE, Wq, sW, dA, dAacc, addend, ws, dev_status, as_stream(stream), false);
+    if (!ws || ws_bytes < least_workspace(d, 1)) return LPDT_ERR_WORKSPACE;
+    return bwd_data_impl(d, E, sE, Wq, sW, dA, dAacc, addend, ws, ws_bytes, dev_status, as_stream(stream), false);
 }
 
 // Backward-weight contraction on raw codes.  Workspace: [int32 sums (used unless the caller gave dWacc) |
-// zero-padded input copy].
+// padded input | padded layer gradient].
 static lpdt_status bwd_weight_impl(const lpdt_conv_desc *d, const int8_t *E, const float *sE, const int8_t *A,
                                    const float *sA, float *dW, int64_t dw_node_stride, int32_t *dWacc, void *ws,
-                                   int32_t *dev_status, cudaStream_t st, bool uns) {
+                                   size_t ws_bytes, int32_t *dev_status, cudaStream_t st, bool uns) {
     const size_t acc_bytes = align_up((size_t)d->nodes * d->Cout * d->R * d->S * d->Cin * sizeof(int32_t), 256);
     int32_t *acc_ws = (int32_t *)ws;
-    lpdt_conv_desc dp;
-    if (use_tc(*d) && d->B > 0 && aligned(E, 16) && aligned(A, 16)) {
-        lpdt_status r = tc::tc_wgrad(*d, d->Cin, E, sE, A, sA, dWacc, acc_ws, dW, dw_node_stride, dev_status, st, uns);
-        if (r != LPDT_ERR_UNSUPPORTED) return r;
-    } else if (use_tc_padded(*d, &dp) && d->B > 0 && aligned(E, 16)) {
-        int8_t *Ap = (int8_t *)((char *)ws + acc_bytes);
-        const int64_t arows = (int64_t)d->nodes * d->B * d->H * d->W;
-        launch_k(pad_channels_kernel, grid_for(arows * dp.Cin / 16), 256, 0, st, A, Ap, arows, d->Cin, dp.Cin);
-        LPDT_LAUNCH_CHECK();
-        lpdt_status r = tc::tc_wgrad(dp, d->Cin, E, sE, Ap, sA, dWacc, acc_ws, dW, dw_node_stride, dev_status, st, uns);
+    if (use_tc(*d, 2, ws, ws_bytes) && d->B > 0 && readable(E, d->Cout) && readable(A, d->Cin)) {
+        const int Ho = conv_out(d->H, d->pad, d->R, d->stride), Wo = conv_out(d->W, d->pad, d->S, d->stride);
+        const PadPlan pp = pad_plan(*d);
+        void *Ap = (char *)ws + acc_bytes, *Ep = (char *)Ap + pp.in;
+        lpdt_status s = pad_launch(pad_job(A, Ap, pp.in ? (int64_t)d->nodes * d->B * d->H * d->W : 0, d->Cin),
+                                   pad_job(E, Ep, pp.err ? (int64_t)d->nodes * d->B * Ho * Wo : 0, d->Cout), st);
+        if (s != LPDT_OK) return s;
+        lpdt_status r = tc::tc_wgrad(*d, pp.err ? (int8_t *)Ep : E, sE, pp.in ? (int8_t *)Ap : A, sA, dWacc, acc_ws, dW,
+                                     dw_node_stride, dev_status, st, uns, pitches(*d));
         if (r != LPDT_ERR_UNSUPPORTED) return r;
     }
     return generic_bwd_weight(*d, E, sE, A, sA, dW, dw_node_stride, dWacc, acc_ws, st, uns);
@@ -412,8 +486,8 @@ extern "C" lpdt_status lpdt_qconv_bwd_weight(const lpdt_conv_desc *d, const int8
     LPDT_CHECK_ARG((d->B == 0 || (E && A)) && (dW || dWacc));      // an empty batch has no operands to point at
     LPDT_CHECK_ARG(!dW || (sE && sA));
     LPDT_CHECK_ARG(!dW || dw_node_stride >= (int64_t)d->Cout * d->R * d->S * d->Cin || d->nodes == 1);
-    if (!ws || ws_bytes < lpdt_qconv_workspace_size(d, 2) || !aligned(ws, 256)) return LPDT_ERR_WORKSPACE;
-    return bwd_weight_impl(d, E, sE, A, sA, dW, dw_node_stride, dWacc, ws, dev_status, as_stream(stream), false);
+    if (!ws || ws_bytes < least_workspace(d, 2) || !aligned(ws, 256)) return LPDT_ERR_WORKSPACE;
+    return bwd_weight_impl(d, E, sE, A, sA, dW, dw_node_stride, dWacc, ws, ws_bytes, dev_status, as_stream(stream), false);
 }
 
 // ---- backward products on affine (zero-point) operands -----------------------------------------
@@ -571,9 +645,13 @@ static size_t affine_wsum_bytes(const lpdt_conv_desc *d) {
     return align_up((size_t)d->nodes * d->R * d->S * d->Cin * sizeof(int32_t), 256);
 }
 
+static size_t affine_bwd_data_own(const lpdt_conv_desc *d) {
+    return affine_bwd_data_raw_bytes(d) + affine_esum_bytes(d) + affine_wsum_bytes(d);
+}
+
 extern "C" size_t lpdt_qconv_bwd_data_affine_workspace_size(const lpdt_conv_desc *d) {
     if (!d || d->nodes <= 0 || check_desc(d) != LPDT_OK) return 256;
-    return affine_bwd_data_raw_bytes(d) + affine_esum_bytes(d) + affine_wsum_bytes(d) + lpdt_qconv_workspace_size(d, 1);
+    return affine_bwd_data_own(d) + lpdt_qconv_workspace_size(d, 1);
 }
 
 extern "C" lpdt_status lpdt_qconv_bwd_data_affine(const lpdt_conv_desc *d, const uint8_t *E, const float *sE,
@@ -585,7 +663,7 @@ extern "C" lpdt_status lpdt_qconv_bwd_data_affine(const lpdt_conv_desc *d, const
     if (d->nodes == 0 || d->B == 0) return LPDT_OK;
     LPDT_CHECK_ARG(E && Wq && zE && zW && (dA || dAacc));
     LPDT_CHECK_ARG(!dA || (sE && sW));
-    if (!ws || !aligned(ws, 256) || ws_bytes < lpdt_qconv_bwd_data_affine_workspace_size(d)) return LPDT_ERR_WORKSPACE;
+    if (!ws || !aligned(ws, 256) || ws_bytes < affine_bwd_data_own(d) + least_workspace(d, 1)) return LPDT_ERR_WORKSPACE;
     cudaStream_t st = as_stream(stream);
     const int Ho = conv_out(d->H, d->pad, d->R, d->stride), Wo = conv_out(d->W, d->pad, d->S, d->stride);
     int32_t *raw = (int32_t *)ws;
@@ -593,7 +671,7 @@ extern "C" lpdt_status lpdt_qconv_bwd_data_affine(const lpdt_conv_desc *d, const
     int32_t *wsum = (int32_t *)((char *)esum + affine_esum_bytes(d));
     void *inner = (char *)wsum + affine_wsum_bytes(d);
     s = bwd_data_impl(d, reinterpret_cast<const int8_t *>(E), nullptr, reinterpret_cast<const int8_t *>(Wq), nullptr,
-                      nullptr, raw, nullptr, inner, dev_status, st, true);
+                      nullptr, raw, nullptr, inner, ws_bytes - (size_t)((char *)inner - (char *)ws), dev_status, st, true);
     if (s != LPDT_OK) return s;
     s = row_sum_launch(E, (int64_t)d->nodes * d->B * Ho * Wo, d->Cout, esum, st);
     if (s != LPDT_OK) return s;
@@ -623,10 +701,14 @@ static size_t affine_tab_bytes(const lpdt_conv_desc *d, int C) {
     return align_up((size_t)d->nodes * d->R * d->S * C * sizeof(int32_t), 256);
 }
 
+static size_t affine_bwd_weight_own(const lpdt_conv_desc *d) {
+    return affine_wg_raw_bytes(d) + affine_colE_bytes(d) + affine_colA_bytes(d) + affine_tab_bytes(d, d->Cout) +
+           affine_tab_bytes(d, d->Cin);
+}
+
 extern "C" size_t lpdt_qconv_bwd_weight_affine_workspace_size(const lpdt_conv_desc *d) {
     if (!d || d->nodes <= 0 || check_desc(d) != LPDT_OK) return 256;
-    return affine_wg_raw_bytes(d) + affine_colE_bytes(d) + affine_colA_bytes(d) + affine_tab_bytes(d, d->Cout) +
-           affine_tab_bytes(d, d->Cin) + lpdt_qconv_workspace_size(d, 2);
+    return affine_bwd_weight_own(d) + lpdt_qconv_workspace_size(d, 2);
 }
 
 extern "C" lpdt_status lpdt_qconv_bwd_weight_affine(const lpdt_conv_desc *d, const uint8_t *E, const float *sE,
@@ -641,7 +723,7 @@ extern "C" lpdt_status lpdt_qconv_bwd_weight_affine(const lpdt_conv_desc *d, con
     LPDT_CHECK_ARG(!dW || (sE && sA));
     LPDT_CHECK_ARG(!dW || dw_node_stride >= (int64_t)d->Cout * d->R * d->S * d->Cin || d->nodes == 1);
     if (d->nodes > 65535) return LPDT_ERR_UNSUPPORTED;
-    if (!ws || !aligned(ws, 256) || ws_bytes < lpdt_qconv_bwd_weight_affine_workspace_size(d)) return LPDT_ERR_WORKSPACE;
+    if (!ws || !aligned(ws, 256) || ws_bytes < affine_bwd_weight_own(d) + least_workspace(d, 2)) return LPDT_ERR_WORKSPACE;
     cudaStream_t st = as_stream(stream);
     const int Ho = conv_out(d->H, d->pad, d->R, d->stride), Wo = conv_out(d->W, d->pad, d->S, d->stride);
     int32_t *raw = (int32_t *)ws;
@@ -651,7 +733,7 @@ extern "C" lpdt_status lpdt_qconv_bwd_weight_affine(const lpdt_conv_desc *d, con
     int32_t *tabA = (int32_t *)((char *)tabE + affine_tab_bytes(d, d->Cout));
     void *inner = (char *)tabA + affine_tab_bytes(d, d->Cin);
     s = bwd_weight_impl(d, reinterpret_cast<const int8_t *>(E), nullptr, reinterpret_cast<const int8_t *>(A), nullptr,
-                        nullptr, 0, raw, inner, dev_status, st, true);
+                        nullptr, 0, raw, inner, ws_bytes - (size_t)((char *)inner - (char *)ws), dev_status, st, true);
     if (s != LPDT_OK) return s;
     launch_k(batch_sum_u8_kernel, grid_for((int64_t)d->nodes * Ho * Wo * d->Cout), 256, 0, st, E, d->nodes, d->B,
              (int64_t)Ho * Wo * d->Cout, colE);

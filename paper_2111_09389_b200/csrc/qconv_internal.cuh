@@ -21,8 +21,10 @@ lpdt_status dequant_acc_launch(const int32_t *acc, int nodes, int64_t per_node, 
                                const float *s2, float *out, int64_t out_stride, cudaStream_t st);
 
 namespace tc {
-// Tensor-core engine (tcgen05 kind::i8): stride-1 convolutions and GEMMs whose
-// channel counts are multiples of 16.  mode 0 = forward, 1 = backward-data.
+// Tensor-core engine (tcgen05 kind::i8): convolutions of stride 1 and 2 and GEMMs.
+// mode 0 = forward, 1 = backward-data.
+// Bytes between the channel rows of the operands in memory (multiples of 16, at least the channel count).
+struct Pitches { int in, err, w; };      // activations (Cin), layer gradients (Cout), weights (Cin)
 bool tc_supported(const lpdt_conv_desc &d);
 // Zero-point correction applied in the forward epilogue (unsigned operands): per-pixel channel sums of the
 // input [nodes][B][H][W], prefix table of the weights' channel sums over the filter taps
@@ -30,16 +32,16 @@ bool tc_supported(const lpdt_conv_desc &d);
 struct AffineArgs { const int32_t *asum, *wpre, *zA, *zW; };
 lpdt_status tc_pix(const lpdt_conv_desc &d, int mode, const int8_t *A, const float *s1, const int8_t *Wq,
                    const float *s2, const float *bias, int64_t bias_stride, float *Y, int32_t *Yacc,
-                   int32_t *dev_status, cudaStream_t st, bool uns = false, const float *addend = nullptr,
-                   const AffineArgs *aff = nullptr);
+                   int32_t *dev_status, cudaStream_t st, bool uns, const float *addend,
+                   const AffineArgs *aff, Pitches pt);
 // Halo-tile kernel for 16-channel operands at stride 1 (one TMA request per tile).
 bool halo_supported(const lpdt_conv_desc &d, int mode);
 lpdt_status tc_pix_halo(const lpdt_conv_desc &d, int mode, const int8_t *A, const float *s1, const int8_t *Wq,
                         const float *s2, const float *bias, int64_t bias_stride, float *Y, int32_t *Yacc,
                         int32_t *dev_status, cudaStream_t st, bool uns = false, const float *addend = nullptr);
-lpdt_status tc_wgrad(const lpdt_conv_desc &d, int cin_real, const int8_t *E, const float *sE, const int8_t *A,
+lpdt_status tc_wgrad(const lpdt_conv_desc &d, const int8_t *E, const float *sE, const int8_t *A,
                      const float *sA, int32_t *acc_user, int32_t *acc_ws, float *dW, int64_t dw_stride,
-                     int32_t *dev_status, cudaStream_t st, bool uns = false);
+                     int32_t *dev_status, cudaStream_t st, bool uns, Pitches pt);
 }  // namespace tc
 
 }  // namespace lpdt

@@ -26,6 +26,7 @@
 // kernel's fp32 result leaves through shared memory and bulk tensor stores where
 // its layout allows.  Every wait is bounded (tc_common.cuh).
 #include <stdlib.h>
+#include <type_traits>
 #include "qconv_internal.cuh"
 #include "tc_common.cuh"
 
@@ -38,7 +39,23 @@ constexpr int kMaxTaps = 64;
 
 // Row format of an operand tile: RB bytes per row and the UMMA layout code.
 __host__ __device__ inline uint32_t layout_code(int RB) { return RB == 128 ? 2u : RB == 64 ? 4u : RB == 32 ? 6u : 0u; }
-static int row_bytes_for(int C) { return C % 128 == 0 ? 128 : C % 64 == 0 ? 64 : C % 32 == 0 ? 32 : 16; }
+// Row bytes of an operand's boxes for C channels.  The last box of a pixel may reach past the channels: TMA fills it
+// with zeros, which add nothing to a sum, so C need not be a multiple of the row.  Wide rows move more bytes per TMA
+// row and per MMA; `w` holds the relative cost of a padded byte for rows of 128, 64, 32 and 16 bytes.
+static int row_bytes_for(int C, const int (&w)[4]) {
+    if (C % 128 == 0) return 128;
+    int best = 16, cost = 0;
+    for (int i = 0; i < 4; ++i) {
+        const int rb = 128 >> i, c = (C + rb - 1) / rb * rb * w[i];
+        if (cost == 0 || c < cost) { cost = c; best = rb; }
+    }
+    return best;
+}
+// Pixel kernel: 4096 x 1008 x 1008 forward takes 11.6 us with eight boxes of 128 bytes and 29.7 us with 63 of 16.
+constexpr int kPixRowCost[4] = {20, 22, 28, 50};
+// Backward-weight: the rows become M lanes and N columns, where padding costs nearly as much as narrow rows
+// (144 -> 144 3x3: rows of 32 bytes 36 us, 64 bytes 41.5 us, 16 bytes 40 us; 272 -> 272: 64 bytes 105 us, 32 bytes 127 us).
+constexpr int kWgRowCost[4] = {20, 22, 25, 28};
 static CUtensorMapSwizzle swizzle_for(int RB) {
     return RB == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : RB == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
          : RB == 32 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_NONE;
@@ -63,6 +80,7 @@ struct PixParams {
     int ncls, cls_ph[4], cls_pw[4], cls_iters[4];
     TapTable tt[4];
     int Nc, Kc;               // N channels, K channels per tap
+    int cpt;                  // operand-A boxes per tap (the last may be part zeros)
     int RBa, RBn;             // row bytes of operand A (K side) and, backward-data, of the N side
     int merged;               // operand A fetched through the merged (channel, width) map
     int raster;               // 1: CTAs take tiles round-robin in a blocked M x N order (long-K tiles, L2 reuse)
@@ -75,6 +93,8 @@ struct PixParams {
     int32_t *dev_status;
     // fp32 result through shared memory and bulk tensor stores: every epilogue warp stages its 32 pixels x 32
     // channels (128-byte rows, 128-byte swizzle) and stores them as one box {32 channels, bw, bh, bb pixels}
+    // (the box is clipped at the last channel).  The ROW instantiation stages the raw sums in the same buffers and
+    // writes them row by row with plain stores.
     int tma_out, out_off;     // out_off: byte offset of the staging area in shared memory (1024-byte aligned)
     int bw, bh;               // the warp's sub-box of the pixel tile: bw x bh x 32/(bw*bh) pixels
     // Forward product on affine (zero-point) operands, corrected in the epilogue (null asum: plain product):
@@ -111,7 +131,9 @@ __device__ __forceinline__ AffinePixel affine_pixel(const PixParams &p, int node
     a.interior = r_lo == 0 && s_lo == 0;          // the three other corners are zero
     return a;
 }
-// acc[k] += fixed - za * rw[channel c0 + k], k < NV (NV a multiple of 4, c0 a multiple of 4)
+// acc[k] += fixed - za * rw[channel c0 + k], k < NV (NV a multiple of 4, c0 a multiple of 4).  An N tile that reaches
+// past the last channel reads up to 31 entries past a table row: the caller keeps them inside its workspace, and the
+// results of those columns are never written.
 template <int NV>
 __device__ __forceinline__ void affine_apply(const PixParams &p, const AffinePixel &a, int node, int c0, uint32_t (&v)[NV]) {
     const int32_t *t = p.wpre + (long long)node * (p.aR + 1) * (p.aS + 1) * p.Nc + c0;
@@ -178,7 +200,9 @@ __device__ __forceinline__ TileCoord decode_raster(const PixParams &p, int tile)
 
 // MINB = 2: the register budget of two resident CTAs per SM, for layers whose K loop is a few stages long: a
 // CTA's fill and drain (first operand boxes, the last tile's epilogue) then overlap its neighbour's main loop.
-template <int MINB>
+// ROW: results whose channel count is no multiple of 4 (no 16-byte rows, so neither bulk stores nor vector stores):
+// the epilogue warps write 32 consecutive channels of one pixel per store instruction.
+template <int MINB, bool ROW>
 __global__ void __launch_bounds__(kPixThreads, MINB)
 conv_pix_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapW,
                 const __grid_constant__ CUtensorMap mapY, const PixParams p) {
@@ -209,7 +233,7 @@ conv_pix_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
     tc_fence_after();
     pdl_enter();          // nothing above touches global memory
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, ctl->tmem_base, 0);
-    const int cpt = p.Kc / p.RBa;          // A boxes per tap
+    const int cpt = p.cpt;
 
     if (warp == 0) {
         {
@@ -340,6 +364,49 @@ conv_pix_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
             const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + acc * p.BN;
             AffinePixel aff = {};
             if (p.asum && valid) aff = affine_pixel(p, c.node, b, h, w);
+            if (ROW) {
+                // 32 channels at a time: raw sums -> this warp's staging buffer (128-byte rows, 16-byte pieces
+                // XOR-swizzled by the row), then 32 consecutive elements of the result rows a store: 128 contiguous
+                // bytes of one pixel, or (fewer than 32 channels) the channels of several pixels.
+                const uint32_t sw = (uint32_t)(lane & 7);
+                const uint32_t vmask = __ballot_sync(0xffffffffu, valid);
+                for (int cc = half * 32; cc < p.BN && n0 + cc < p.Nc; cc += 64) {
+                    uint32_t v[32];
+                    tmem_ld_32x32(t_row + cc, v);
+                    tmem_ld_wait();
+                    int4 *grow = reinterpret_cast<int4 *>(buf + lane * 128);
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        grow[(uint32_t)k ^ sw] = make_int4((int)v[4 * k], (int)v[4 * k + 1], (int)v[4 * k + 2], (int)v[4 * k + 3]);
+                    __syncwarp();
+                    // element e = r * nc + k of the 32 pixels x nc channels, 32 elements a step
+                    const int nc = p.Nc - n0 - cc < 32 ? p.Nc - n0 - cc : 32;
+                    const uint32_t inv = (65536u + nc - 1) / nc;       // e / nc = (e * inv) >> 16 for e < 1024, nc <= 32
+                    auto write = [&](auto plain) {
+#pragma unroll 8
+                        for (int it = 0; it < nc; ++it) {
+                            const uint32_t e = it * 32 + lane, r = (e * inv) >> 16, k = e - r * nc;
+                            const long long o = __shfl_sync(0xffffffffu, pix, (int)r) * p.Nc + n0 + cc + k;
+                            const int a = *reinterpret_cast<const int *>(buf + r * 128 + (((k >> 2) ^ (r & 7)) << 4) + (k & 3) * 4);
+                            if (!((vmask >> r) & 1u)) continue;
+                            if (decltype(plain)::value) { p.Y[o] = __fmul_rn(__int2float_rn(a), sc); continue; }
+                            if (p.Yacc) p.Yacc[o] = a;
+                            if (p.Y) {
+                                float f = __fmul_rn(__int2float_rn(a), sc);
+                                if (p.bias) f = __fadd_rn(f, p.bias[(long long)c.node * p.bias_stride + n0 + cc + k]);
+                                if (p.addend) f = __fadd_rn(f, p.addend[o]);
+                                p.Y[o] = f;
+                            }
+                        }
+                    };
+                    if (p.Yacc || p.bias || p.addend) write(std::false_type()); else write(std::true_type());
+                    __syncwarp();
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&ctl->tmem_empty[acc]));
+                continue;
+            }
             if (p.tma_out) {
                 // 32 channels at a time: accumulators -> fp32 -> this warp's staging buffer (one 128-byte row per
                 // lane, 16-byte pieces XOR-swizzled by the row so that the lanes spread over all banks, which is
@@ -349,7 +416,8 @@ conv_pix_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
                 const uint32_t sw = (uint32_t)(lane & 7);
                 uint32_t v[32];
                 int cc = half * 32;
-                bool have = cc < p.BN;
+                const int bn = p.Nc - n0 < p.BN ? p.Nc - n0 : p.BN;          // channels of this tile
+                bool have = cc < bn;
                 if (have) tmem_ld_32x32(t_row + cc, v);
                 while (have) {
                     tmem_ld_wait();
@@ -358,17 +426,18 @@ conv_pix_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
 #pragma unroll
                     for (int k = 0; k < 32; ++k) f[k] = __fmul_rn(__int2float_rn((int)v[k]), sc);
                     const int ncc = cc + 64;
-                    const bool more = ncc < p.BN;
+                    const bool more = ncc < bn;
                     if (more) tmem_ld_32x32(t_row + ncc, v);
                     if (p.bias) {
 #pragma unroll
                         for (int k = 0; k < 32; ++k)
-                            f[k] = __fadd_rn(f[k], p.bias[(long long)c.node * p.bias_stride + n0 + cc + k]);
+                            if (cc + k < bn) f[k] = __fadd_rn(f[k], p.bias[(long long)c.node * p.bias_stride + n0 + cc + k]);
                     }
                     if (p.addend && valid) {
                         const float4 *ad = reinterpret_cast<const float4 *>(p.addend + pix * p.Nc + n0 + cc);
 #pragma unroll
                         for (int k = 0; k < 8; ++k) {
+                            if (cc + 4 * k >= bn) continue;
                             const float4 a4 = ad[k];
                             f[4 * k] = __fadd_rn(f[4 * k], a4.x); f[4 * k + 1] = __fadd_rn(f[4 * k + 1], a4.y);
                             f[4 * k + 2] = __fadd_rn(f[4 * k + 2], a4.z); f[4 * k + 3] = __fadd_rn(f[4 * k + 3], a4.w);
@@ -394,38 +463,40 @@ conv_pix_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
                 if (lane == 0) mbar_arrive(smem_u32(&ctl->tmem_empty[acc]));
                 continue;
             }
-            for (int cc = half * 16; cc < p.BN; cc += 32) {
+            for (int cc = half * 16; cc < p.BN && n0 + cc < p.Nc; cc += 32) {
                 uint32_t v[16];
                 tmem_ld_32x16(t_row + cc, v);
                 tmem_ld_wait();
                 if (valid) {
                     const long long o = pix * p.Nc + n0 + cc;
+                    const int quads = (p.Nc - n0 - cc) / 4;          // the tile may reach past the last channel
                     if (p.asum) affine_apply<16>(p, aff, c.node, n0 + cc, v);
                     if (p.Yacc) {
                         int4 *dst = reinterpret_cast<int4 *>(p.Yacc + o);
 #pragma unroll
                         for (int k = 0; k < 4; ++k)
-                            dst[k] = make_int4((int)v[4 * k], (int)v[4 * k + 1], (int)v[4 * k + 2], (int)v[4 * k + 3]);
+                            if (k < quads) dst[k] = make_int4((int)v[4 * k], (int)v[4 * k + 1], (int)v[4 * k + 2], (int)v[4 * k + 3]);
                     }
                     if (p.Y) {
                         float f[16];
 #pragma unroll
                         for (int k = 0; k < 16; ++k) {
                             f[k] = __fmul_rn(__int2float_rn((int)v[k]), sc);
-                            if (p.bias) f[k] = __fadd_rn(f[k], p.bias[(long long)c.node * p.bias_stride + n0 + cc + k]);
+                            if (p.bias && k < 4 * quads)
+                                f[k] = __fadd_rn(f[k], p.bias[(long long)c.node * p.bias_stride + n0 + cc + k]);
                         }
-                        if (p.addend) {
-                            const float4 *ad = reinterpret_cast<const float4 *>(p.addend + o);
+                        float4 *dst = reinterpret_cast<float4 *>(p.Y + o);
+                        const float4 *ad = reinterpret_cast<const float4 *>(p.addend + o);
 #pragma unroll
-                            for (int k = 0; k < 4; ++k) {
+                        for (int k = 0; k < 4; ++k) {
+                            if (k >= quads) break;
+                            if (p.addend) {
                                 const float4 a4 = ad[k];
                                 f[4 * k] = __fadd_rn(f[4 * k], a4.x); f[4 * k + 1] = __fadd_rn(f[4 * k + 1], a4.y);
                                 f[4 * k + 2] = __fadd_rn(f[4 * k + 2], a4.z); f[4 * k + 3] = __fadd_rn(f[4 * k + 3], a4.w);
                             }
+                            dst[k] = make_float4(f[4 * k], f[4 * k + 1], f[4 * k + 2], f[4 * k + 3]);
                         }
-                        float4 *dst = reinterpret_cast<float4 *>(p.Y + o);
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) dst[k] = make_float4(f[4 * k], f[4 * k + 1], f[4 * k + 2], f[4 * k + 3]);
                     }
                 }
             }
@@ -449,7 +520,7 @@ struct WgParams {
     int halo, PW, PH, halo_bytes;                 // 16-channel halo mode: one input box per pixel tile (see below)
     int mgroups, ngroups, mtiles, BNc, total_units;
     int stages, tmem_cols;
-    int cin_real;                                 // channels of the caller's weight layout (< Cin when the input was zero-padded)
+    int cpt;                                      // input boxes per tap (the last may be part zeros)
     int32_t *acc_out;                             // int32 sums [nodes][Cout][taps][cin_real] (nullable if 1 split)
     float *dW; long long dw_stride;               // fp32 result, written here only if 1 split (nullable)
     const float *s1, *s2;                         // per-node scales of the two operands
@@ -477,7 +548,7 @@ conv_wgrad_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
     const int stage_bytes = x_region + 128 * p.BNc;
     const int kb0 = blockIdx.x * p.kb_per_split;
     int kb1 = kb0 + p.kb_per_split; if (kb1 > p.kblocks) kb1 = p.kblocks;
-    const int cpt = p.Cin / p.RBx;
+    const int cpt = p.cpt;
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < p.stages; ++i) { mbar_init(smem_u32(&ctl->full[i]), 1); mbar_init(smem_u32(&ctl->empty[i]), 1); }
@@ -572,7 +643,7 @@ conv_wgrad_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
         if (mbar_wait(smem_u32(&ctl->tmem_full[0]), 0, &ctl->abort_flag, p.dev_status)) {
             tc_fence_after();
             const float sc = (p.dW && p.splits == 1) ? __fmul_rn(p.s1[node], p.s2[node]) : 0.f;
-            const long long cstride = (long long)p.taps * p.cin_real;
+            const long long cstride = (long long)p.taps * p.Cin;
             for (int t = 0; t < p.mtiles; ++t) {
                 int tap, ci; bool valid;
                 if (p.halo) {                                       // lane = (s, ci) of filter row t
@@ -583,16 +654,25 @@ conv_wgrad_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
                     valid = (i < nX) && (mu < p.total_units);
                     tap = mu / cpt; ci = (mu % cpt) * p.RBx + row % p.RBx;
                 }
-                valid = valid && (ci < p.cin_real);
+                valid = valid && (ci < p.Cin);
                 const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + t * p.BNc;
-                for (int c = 0; c < p.BNc; c += 16) {
+                for (int c = 0; c < p.BNc && n0 + c < p.Cout; c += 16) {
                     uint32_t v[16];
                     tmem_ld_32x16(t_row + c, v);
                     tmem_ld_wait();
                     if (!valid) continue;
-                    const long long o = ((long long)(n0 + c) * p.taps + tap) * p.cin_real + ci;
+                    const long long o = ((long long)(n0 + c) * p.taps + tap) * p.Cin + ci;
                     int32_t *acc = p.acc_out + (long long)node * p.Cout * cstride + o;
-                    if (p.splits > 1) {
+                    const int nk = p.Cout - n0 - c;
+                    if (nk < 16) {                               // the N group reaches past the last channel
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) {
+                            if (k >= nk) continue;
+                            if (p.splits > 1) { if ((int)v[k] != 0) atomicAdd(acc + k * cstride, (int)v[k]); continue; }
+                            if (p.acc_out) acc[k * cstride] = (int)v[k];
+                            if (p.dW) p.dW[(long long)node * p.dw_stride + o + k * cstride] = __fmul_rn(__int2float_rn((int)v[k]), sc);
+                        }
+                    } else if (p.splits > 1) {
 #pragma unroll
                         for (int k = 0; k < 16; ++k)
                             if ((int)v[k] != 0) atomicAdd(acc + k * cstride, (int)v[k]);
@@ -637,10 +717,12 @@ static void pick_tile(int H, int W, int max_tw, int *TB, int *TH, int *TW) {
 // Activation map: box = {RB channel bytes, TW, TH, TB pixels, 1 node}.  With estride 2 the
 // box samples every second pixel (the traversal stride of the tensor map), which is how
 // a stride-2 convolution reads its input.
-static bool act_map(CUtensorMap *m, const int8_t *base, int nodes, int B, int H, int W, int C, int RB,
+// `pitch` bytes (a multiple of 16) lie between the channel rows of two pixels.
+static bool act_map(CUtensorMap *m, const int8_t *base, int nodes, int B, int H, int W, int C, int pitch, int RB,
                     int TB, int TH, int TW, int estride = 1) {
     uint64_t dims[5] = {(uint64_t)C, (uint64_t)W, (uint64_t)H, (uint64_t)B, (uint64_t)nodes};
-    uint64_t strides[4] = {(uint64_t)C, (uint64_t)W * C, (uint64_t)H * W * C, (uint64_t)B * H * W * C};
+    const uint64_t P = (uint64_t)pitch;
+    uint64_t strides[4] = {P, W * P, H * W * P, B * H * (W * P)};
     uint32_t box[5] = {(uint32_t)RB, (uint32_t)(TW * estride), (uint32_t)(TH * estride), (uint32_t)TB, 1};
     uint32_t es[5] = {1, (uint32_t)estride, (uint32_t)estride, 1, 1};
     return make_map_u8(m, base, 5, dims, strides, box, swizzle_for(RB), es);
@@ -654,10 +736,10 @@ static bool act_map_merged(CUtensorMap *m, const int8_t *base, int nodes, int B,
     return make_map_u8(m, base, 4, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_NONE);
 }
 
-static bool weight_map(CUtensorMap *m, const int8_t *base, int nodes, int Cout, int taps, int Cin, int box_inner,
-                       int box_rows) {
+static bool weight_map(CUtensorMap *m, const int8_t *base, int nodes, int Cout, int taps, int Cin, int pitch,
+                       int box_inner, int box_rows) {
     uint64_t dims[3] = {(uint64_t)Cin, (uint64_t)taps, (uint64_t)nodes * Cout};
-    uint64_t strides[2] = {(uint64_t)Cin, (uint64_t)taps * Cin};
+    uint64_t strides[2] = {(uint64_t)pitch, (uint64_t)taps * pitch};
     uint32_t box[3] = {(uint32_t)box_inner, 1, (uint32_t)box_rows};
     return make_map_u8(m, base, 3, dims, strides, box, swizzle_for(box_inner));
 }
@@ -674,7 +756,6 @@ static bool pix_two_enabled() {
 
 bool tc_supported(const lpdt_conv_desc &d) {
     if (d.stride != 1 && d.stride != 2) return false;
-    if (d.Cin % 16 || d.Cout % 16) return false;
     if (d.R * d.S > kMaxTaps || d.R > 100 || d.S > 100 || d.pad > 100) return false;
     if (!encode_tiled_fn()) return false;
     return true;
@@ -687,14 +768,28 @@ static bool pix_tma_out_enabled() {
     return off == 0;
 }
 
-static int largest_div(int C, int cap, int unit) {      // largest multiple of unit dividing C, <= cap
-    for (int v = cap - cap % unit; v >= unit; v -= unit) if (C % v == 0) return v;
-    return unit;
+// Width of an N tile for N channels, a multiple of `unit` up to 256.  A tile's time goes with 128 + bn, the operand
+// rows that its MMAs read from shared memory per step (they bound narrow tiles), and every SM takes
+// ceil(mtiles * ntiles / 148) of them (mtiles = 0: many tiles, only their sum counts).  Ties go to the fewer padded
+// channels.  4096 x 1040 x 1040 forward: 5 x 32 tiles of 224 are two waves (16.0 us), 9 x 32 of 128 as well but
+// shorter ones (13.5 us).
+static int pick_bn(int N, int unit, long long mtiles) {
+    if (N <= unit) return unit;
+    const unsigned mt = mtiles * N <= 0x7fffffff ? (unsigned)mtiles : 0u;
+    int best = unit;
+    unsigned cost = 0, waste = 0;
+    for (int bn = (N >= 64 && unit < 64) ? 64 : unit; bn <= 256 && bn < N + unit; bn += unit) {
+        const unsigned nt = (unsigned)(N + bn - 1) / (unsigned)bn, w = nt * bn;
+        const unsigned c = (mt ? (mt * nt + kNumSMs - 1) / kNumSMs : nt) * (128 + bn);
+        if (cost == 0 || c < cost || (c == cost && w < waste)) { cost = c; waste = w; best = bn; }
+    }
+    return best;
 }
 
 lpdt_status tc_pix(const lpdt_conv_desc &d, int mode, const int8_t *A, const float *s1, const int8_t *Wq,
                    const float *s2, const float *bias, int64_t bias_stride, float *Y, int32_t *Yacc,
-                   int32_t *dev_status, cudaStream_t st, bool uns, const float *addend, const AffineArgs *aff) {
+                   int32_t *dev_status, cudaStream_t st, bool uns, const float *addend, const AffineArgs *aff,
+                   Pitches pt) {
     const int Ho = conv_out(d.H, d.pad, d.R, d.stride), Wo = conv_out(d.W, d.pad, d.S, d.stride);
     PixParams p = {};
     p.addend = addend;
@@ -738,23 +833,25 @@ lpdt_status tc_pix(const lpdt_conv_desc &d, int mode, const int8_t *A, const flo
             }
         }
     }
-    p.RBa = row_bytes_for(p.Kc);
-    p.RBn = row_bytes_for(p.Nc);
+    p.RBa = row_bytes_for(p.Kc, kPixRowCost);
+    p.RBn = row_bytes_for(p.Nc, kPixRowCost);
     const int estride = mode == 0 ? d.stride : 1;
-    p.merged = (p.Kc == 16 && estride == 1) ? 1 : 0;
+    const int pitchA = mode == 0 ? pt.in : pt.err;
+    p.merged = (pitchA == 16 && estride == 1) ? 1 : 0;
+    if (p.merged) p.RBa = 16;
     pick_tile(p.Hm, p.Wm, p.merged ? 16 : 128, &p.TB, &p.TH, &p.TW);
     if (p.TW * estride > 256 || p.TH * estride > 256) return LPDT_ERR_UNSUPPORTED;
     p.tilesB = (int)ceil_div(d.B, p.TB); p.tilesH = (int)ceil_div(p.Hm, p.TH); p.tilesW = (int)ceil_div(p.Wm, p.TW);
-    p.BN = largest_div(p.Nc, 256, mode == 0 ? 16 : p.RBn);
-    {   // few tiles (small maps, small batches, small GEMMs): narrower N tiles while the doubled count still fits
-        // one wave of SMs.  Measured: 32 -> 64 -> 128 tiles gains 10-80 %; past one wave the narrower tile's
-        // extra shared-memory traffic per MMA loses 10-25 %.
-        const long long mtiles = (long long)p.nodes * p.tilesB * p.tilesH * p.tilesW * p.ncls;
-        const int unit = mode == 0 ? 16 : p.RBn;
-        while (p.BN >= 128 && p.BN % 2 == 0 && (p.BN / 2) % unit == 0 && 2 * mtiles * (p.Nc / p.BN) <= kNumSMs) p.BN /= 2;
-    }
-    p.tilesN = p.Nc / p.BN;
-    const int cpt = p.Kc / p.RBa;
+    // how the result leaves (see PixParams): rows of a multiple of 16 bytes through bulk stores (fp32 only, one class),
+    // other multiples of 4 channels by vector stores, the rest row by row
+    const bool row = p.Nc % 4 != 0;
+    p.tma_out = (!row && Y && !Yacc && aligned(Y, 16) && p.ncls == 1 && p.out_mul == 1 && p.Nc > 16 &&
+                 pix_tma_out_enabled()) ? 1 : 0;
+    int unit = (row || p.tma_out) ? 32 : 16;
+    if (mode == 1 && p.RBn > unit) unit = p.RBn;
+    p.BN = pick_bn(p.Nc, unit, (long long)p.nodes * p.tilesB * p.tilesH * p.tilesW * p.ncls);
+    p.tilesN = (int)ceil_div(p.Nc, p.BN);
+    const int cpt = p.cpt = (int)ceil_div(p.Kc, p.RBa);
     const int unit_bytes = 128 * p.RBa + p.BN * p.RBa;
     // K units per stage: stage <= 48 KB, at most 16 units, an even count for 16-byte rows (one MMA
     // consumes two of them); the least padded work over the classes wins, ties go to the larger stage
@@ -777,14 +874,11 @@ lpdt_status tc_pix(const lpdt_conv_desc &d, int mode, const int8_t *A, const flo
     // long K loops (GEMM-like): blocked round-robin tile order; short ones: contiguous ranges
     p.raster = (p.ncls == 1 && p.cls_iters[0] >= 8) ? 1 : 0;
     const int stage_bytes = U * unit_bytes;
-    // fp32 result through shared memory and bulk tensor stores (not with raw accumulators, not for the strided
-    // pixel classes of a stride-2 backward-data pass): 8 warps x 4 KB of staging after the ring
-    p.tma_out = (Y && !Yacc && aligned(Y, 16) && p.ncls == 1 && p.out_mul == 1 && p.BN % 32 == 0 &&
-                 pix_tma_out_enabled()) ? 1 : 0;
     p.bw = p.TW < 32 ? p.TW : 32;
     p.bh = p.TH < 32 / p.bw ? p.TH : 32 / p.bw;
-    const int out_bytes = p.tma_out ? 32 * 1024 + 1024 : 0;        // 8 warps x 4 KB + slack to reach a 1024-byte boundary
-    p.stages = ((p.tma_out ? 227 * 1024 - out_bytes : kSmemBudget) - 1024) / stage_bytes;
+    const bool staged = p.tma_out || row;
+    const int out_bytes = staged ? 32 * 1024 + 1024 : 0;        // 8 warps x 4 KB + slack to reach a 1024-byte boundary
+    p.stages = ((staged ? 227 * 1024 - out_bytes : kSmemBudget) - 1024) / stage_bytes;
     if (p.stages > 8) p.stages = 8;
     if (p.stages < 2) return LPDT_ERR_UNSUPPORTED;
     p.tmem_cols = pow2_at_least(2 * p.BN);
@@ -809,14 +903,16 @@ lpdt_status tc_pix(const lpdt_conv_desc &d, int mode, const int8_t *A, const flo
     // (bwd-data: image Ho x Wo, Cout, dense)
     const int Ha = mode == 0 ? d.H : Ho, Wa = mode == 0 ? d.W : Wo;
     if (p.merged) { if (!act_map_merged(&mA, A, d.nodes, d.B, Ha, Wa, p.TB, p.TH, p.TW)) return LPDT_ERR_CUDA; }
-    else if (!act_map(&mA, A, d.nodes, d.B, Ha, Wa, p.Kc, p.RBa, p.TB, p.TH, p.TW, estride)) return LPDT_ERR_CUDA;
-    if (mode == 0) { if (!weight_map(&mW, Wq, d.nodes, d.Cout, d.R * d.S, d.Cin, p.RBa, p.BN)) return LPDT_ERR_CUDA; }
-    else if (!weight_map(&mW, Wq, d.nodes, d.Cout, d.R * d.S, d.Cin, p.RBn, p.RBa)) return LPDT_ERR_CUDA;
+    else if (!act_map(&mA, A, d.nodes, d.B, Ha, Wa, p.Kc, pitchA, p.RBa, p.TB, p.TH, p.TW, estride)) return LPDT_ERR_CUDA;
+    if (mode == 0) { if (!weight_map(&mW, Wq, d.nodes, d.Cout, d.R * d.S, d.Cin, pt.w, p.RBa, p.BN)) return LPDT_ERR_CUDA; }
+    else if (!weight_map(&mW, Wq, d.nodes, d.Cout, d.R * d.S, d.Cin, pt.w, p.RBn, p.RBa)) return LPDT_ERR_CUDA;
     size_t smem = 1024 + (size_t)p.stages * stage_bytes;
     CUtensorMap mY = CUtensorMap{};
-    if (p.tma_out) {
+    if (staged) {
         p.out_off = (int)align_up(smem, 1024);
         smem = (size_t)p.out_off + 32 * 1024;
+    }
+    if (p.tma_out) {
         uint64_t dims[5] = {(uint64_t)p.Nc, (uint64_t)p.Wout, (uint64_t)p.Hout, (uint64_t)d.B, (uint64_t)d.nodes};
         uint64_t strides[4] = {(uint64_t)p.Nc * 4, (uint64_t)p.Wout * p.Nc * 4, (uint64_t)p.Hout * p.Wout * p.Nc * 4,
                                (uint64_t)d.B * p.Hout * p.Wout * p.Nc * 4};
@@ -826,35 +922,39 @@ lpdt_status tc_pix(const lpdt_conv_desc &d, int mode, const int8_t *A, const flo
     }
     if (smem < (two ? kMinSmemTwo : kMinSmem)) smem = two ? kMinSmemTwo : kMinSmem;
     if (smem > (two ? (size_t)113 * 1024 : (size_t)227 * 1024)) return LPDT_ERR_UNSUPPORTED;
-    static PerDeviceOnce attr;
+    using Fn = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const PixParams);
+    static const Fn fns[2][2] = {{conv_pix_kernel<1, false>, conv_pix_kernel<1, true>},
+                                 {conv_pix_kernel<2, false>, conv_pix_kernel<2, true>}};
+    // set when an instantiation is first used: the attribute loads its code
+    static PerDeviceOnce attr[2][2];
     int dev;
-    if (attr.pending(&dev)) {
-        LPDT_CUDA(cudaFuncSetAttribute(conv_pix_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-        LPDT_CUDA(cudaFuncSetAttribute(conv_pix_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 113 * 1024));
-        attr.mark(dev);
+    if (attr[two ? 1 : 0][row ? 1 : 0].pending(&dev)) {
+        LPDT_CUDA(cudaFuncSetAttribute(fns[two ? 1 : 0][row ? 1 : 0], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (two ? 113 : 227) * 1024));
+        attr[two ? 1 : 0][row ? 1 : 0].mark(dev);
     }
     const int slots = two ? 2 * kNumSMs : kNumSMs;
     const int grid = (int)(tiles < slots ? tiles : slots);
     g_last_kernel = "lpdt::tc::conv_pix_kernel";
-    if (two) launch_k(conv_pix_kernel<2>, grid, kPixThreads, smem, st, mA, mW, mY, p);
-    else launch_k(conv_pix_kernel<1>, grid, kPixThreads, smem, st, mA, mW, mY, p);
+    launch_k(fns[two ? 1 : 0][row ? 1 : 0], grid, kPixThreads, smem, st, mA, mW, mY, p);
     LPDT_LAUNCH_CHECK();
     return LPDT_OK;
 }
 
-// acc_user: the caller's raw-sum array or null; acc_ws: scratch of the same shape [nodes][Cout][taps][cin_real]
-// (the caller's weight layout); dW: fp32 result or null.  With one split the kernel writes both outputs
+// acc_user: the caller's raw-sum array or null; acc_ws: scratch of the same shape [nodes][Cout][taps][Cin]; dW: fp32 result or null.  With one split the kernel writes both outputs
 // itself; with several it accumulates into zeroed int32 storage and a conversion launch follows.
-lpdt_status tc_wgrad(const lpdt_conv_desc &d, int cin_real, const int8_t *E, const float *sE, const int8_t *A,
+lpdt_status tc_wgrad(const lpdt_conv_desc &d, const int8_t *E, const float *sE, const int8_t *A,
                      const float *sA, int32_t *acc_user, int32_t *acc_ws, float *dW, int64_t dw_stride,
-                     int32_t *dev_status, cudaStream_t st, bool uns) {
+                     int32_t *dev_status, cudaStream_t st, bool uns, Pitches pt) {
     const int Ho = conv_out(d.H, d.pad, d.R, d.stride), Wo = conv_out(d.W, d.pad, d.S, d.stride);
     WgParams p = {};
     p.nodes = d.nodes; p.B = d.B; p.Ho = Ho; p.Wo = Wo; p.Cin = d.Cin; p.Cout = d.Cout;
     p.R = d.R; p.S = d.S; p.pad = d.pad; p.taps = d.R * d.S; p.stride = d.stride;
-    p.RBx = row_bytes_for(d.Cin); p.RBe = row_bytes_for(d.Cout);
-    p.merged = (d.Cin == 16 && d.stride == 1) ? 1 : 0;
-    p.BNc = largest_div(d.Cout, 256, p.RBe);
+    p.RBx = row_bytes_for(d.Cin, kWgRowCost); p.RBe = row_bytes_for(d.Cout, kWgRowCost);
+    p.merged = (pt.in == 16 && d.stride == 1) ? 1 : 0;
+    if (p.merged) p.RBx = 16;
+    p.cpt = (int)ceil_div(d.Cin, p.RBx);
+    p.BNc = pick_bn(d.Cout, p.RBe, 0);
     p.halo = (p.merged && d.S <= 8 && d.R * p.BNc <= 512 && d.R <= 16) ? 1 : 0;
     if (p.halo) { p.TW = 8; p.TH = 16; p.TB = 1; p.PW = 8 + d.S - 1; p.PH = 16 + d.R - 1; p.halo_bytes = (int)align_up((size_t)p.PW * p.PH * 16 + 256, 1024); }
     else pick_tile(Ho, Wo, p.merged ? 16 : 128, &p.TB, &p.TH, &p.TW);
@@ -862,16 +962,16 @@ lpdt_status tc_wgrad(const lpdt_conv_desc &d, int cin_real, const int8_t *E, con
     p.tilesB = (int)ceil_div(d.B, p.TB); p.tilesH = (int)ceil_div(Ho, p.TH); p.tilesW = (int)ceil_div(Wo, p.TW);
     p.kblocks = p.tilesB * p.tilesH * p.tilesW;
     const int G = 128 / p.RBx;
-    p.total_units = p.taps * (d.Cin / p.RBx);
+    p.total_units = p.taps * p.cpt;
     const int all_tiles = (int)ceil_div(p.total_units, G);
     // Short pixel loops (GEMM-like shapes with few rows): rather narrower N groups, so that the output tiles alone
     // give the SMs work, than a split of a loop of a few blocks whose partial sums meet in atomics.
     // (Measured on the GEMM sweep: up to 64 output tiles this is 2.3-3.4 times faster; from 128 tiles on the split
     // wins.)
-    const bool short_k = !p.halo && p.kblocks <= 16 && (long long)d.nodes * all_tiles * (d.Cout / p.BNc) <= 64;
+    const bool short_k = !p.halo && p.kblocks <= 16 && (long long)d.nodes * all_tiles * ceil_div(d.Cout, p.BNc) <= 64;
     if (short_k)
-        while (p.BNc >= 2 * p.RBe && p.BNc >= 256 && (long long)d.nodes * all_tiles * (d.Cout / p.BNc) < kNumSMs) p.BNc /= 2;
-    p.ngroups = d.Cout / p.BNc;
+        while (p.BNc >= 2 * p.RBe && p.BNc >= 256 && (long long)d.nodes * all_tiles * ceil_div(d.Cout, p.BNc) < kNumSMs) p.BNc /= 2;
+    p.ngroups = (int)ceil_div(d.Cout, p.BNc);
     int mt = 512 / p.BNc;                                        // accumulators that fit in TMEM
     const int mt_smem = (96 * 1024 - 128 * p.BNc) / 16384;       // stage <= 96 KB -> at least two stages
     if (mt > mt_smem) mt = mt_smem;
@@ -903,7 +1003,7 @@ lpdt_status tc_wgrad(const lpdt_conv_desc &d, int cin_real, const int8_t *E, con
     if (splits < 1) splits = 1;
     p.kb_per_split = (int)ceil_div(p.kblocks, splits);
     p.splits = (int)ceil_div(p.kblocks, p.kb_per_split);
-    p.cin_real = cin_real; p.dW = dW; p.dw_stride = dw_stride; p.s1 = sE; p.s2 = sA;
+    p.dW = dW; p.dw_stride = dw_stride; p.s1 = sE; p.s2 = sA;
     p.acc_out = p.splits == 1 ? acc_user : (acc_user ? acc_user : acc_ws);
     p.dev_status = dev_status; p.uns = uns ? 1 : 0;
     CUtensorMap mX, mE;
@@ -913,8 +1013,8 @@ lpdt_status tc_wgrad(const lpdt_conv_desc &d, int cin_real, const int8_t *E, con
         uint32_t box[4] = {(uint32_t)p.PW * 16, (uint32_t)p.PH, 1, 1};
         if (!make_map_u8(&mX, A, 4, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_NONE)) return LPDT_ERR_CUDA;
     } else if (p.merged) { if (!act_map_merged(&mX, A, d.nodes, d.B, d.H, d.W, p.TB, p.TH, p.TW)) return LPDT_ERR_CUDA; }
-    else if (!act_map(&mX, A, d.nodes, d.B, d.H, d.W, d.Cin, p.RBx, p.TB, p.TH, p.TW, d.stride)) return LPDT_ERR_CUDA;
-    if (!act_map(&mE, E, d.nodes, d.B, Ho, Wo, d.Cout, p.RBe, p.TB, p.TH, p.TW)) return LPDT_ERR_CUDA;
+    else if (!act_map(&mX, A, d.nodes, d.B, d.H, d.W, d.Cin, pt.in, p.RBx, p.TB, p.TH, p.TW, d.stride)) return LPDT_ERR_CUDA;
+    if (!act_map(&mE, E, d.nodes, d.B, Ho, Wo, d.Cout, pt.err, p.RBe, p.TB, p.TH, p.TW)) return LPDT_ERR_CUDA;
     size_t smem = 1024 + (size_t)p.stages * stage_bytes;
     if (smem < (size_t)(228 * 1024) / (per_sm + 1)) smem = (size_t)(228 * 1024) / (per_sm + 1);
     if (smem > 227 * 1024) return LPDT_ERR_UNSUPPORTED;
@@ -925,7 +1025,7 @@ lpdt_status tc_wgrad(const lpdt_conv_desc &d, int cin_real, const int8_t *E, con
         attr.mark(dev);
     }
     if (d.nodes > 65535 || p.mgroups * p.ngroups > 65535) return LPDT_ERR_UNSUPPORTED;
-    const int64_t per_node = (int64_t)d.Cout * p.taps * cin_real;
+    const int64_t per_node = (int64_t)d.Cout * p.taps * d.Cin;
     if (p.splits > 1) {
         if (!p.acc_out) return LPDT_ERR_WORKSPACE;
         LPDT_CUDA(cudaMemsetAsync(p.acc_out, 0, (size_t)d.nodes * per_node * sizeof(int32_t), st));

@@ -229,6 +229,50 @@ def test_qconv_bwd_affine(case):
     assert not dW[:, wn:].any()
 
 
+# channel counts that no 16-byte row holds, or that end inside a box of the tensor-core kernels
+RAGGED_CASES = [
+    (2, 130, 1, 1, 200, 270, 1, 1, 1, 0),    # linear: 200 = 128 + 72 inputs, results in rows of 270 (no 16-byte rows)
+    (1, 300, 1, 1, 1001, 17, 1, 1, 1, 0),    # odd on both sides, three row tiles
+    (1, 5, 9, 11, 7, 21, 3, 3, 1, 1),
+    (2, 3, 13, 10, 33, 50, 3, 3, 2, 1),      # strided, both ragged
+    (2, 2, 16, 16, 3, 24, 3, 3, 2, 1),       # strided first layer: 24 results in a tile of 32
+    (1, 2, 8, 8, 130, 36, 3, 3, 1, 1),
+    (1, 2, 6, 6, 16, 15, 3, 3, 1, 1),        # whole input rows, one result short of a row
+    (1, 3, 5, 5, 20, 16, 5, 5, 1, 2),
+    (1, 2, 12, 12, 144, 80, 3, 3, 1, 1),     # multiples of 16 whose last box is part zeros
+    (2, 3, 7, 7, 272, 400, 1, 1, 1, 0),      # several N tiles, the last one part empty
+    (1, 2, 9, 9, 48, 336, 3, 3, 2, 1),
+    (3, 1, 4, 4, 1, 1, 3, 3, 1, 1),          # a single channel
+]
+
+
+@pytest.mark.parametrize("case", RAGGED_CASES)
+def test_qconv_ragged_channels(case):
+    test_qconv_all_three(case)
+    test_qconv_fwd_affine(case)
+    test_qconv_bwd_affine(case)
+
+
+@pytest.mark.parametrize("case", [RAGGED_CASES[0], RAGGED_CASES[3]])
+def test_qconv_ragged_channels_without_room_for_copies(case):
+    # the least workspace (no room for padded operand copies) and none at all where none is required: same sums
+    nodes, B, H, W, Cin, Cout, R, S, stride, pad = case
+    A, Wq, E, _, _ = _conv_inputs(case)
+    desc = api.conv_desc(*case)
+    wn = nodes * Cout * R * S * Cin
+    up = lambda n: (n + 255) // 256 * 256
+    Yacc = torch.empty(E.shape, dtype=torch.int32, device="cuda")
+    api.lpdt_qconv_fwd(desc, dev(A), None, dev(Wq), None, Yacc=Yacc)
+    assert np.array_equal(Yacc.cpu().numpy(), oracle.qconv_fwd(A, Wq, stride, pad)[0])
+    dAacc = torch.empty(A.shape, dtype=torch.int32, device="cuda")
+    api.lpdt_qconv_bwd_data(desc, dev(E), None, dev(Wq), None, dAacc=dAacc, ws=ws_bytes(up(wn)))
+    assert np.array_equal(dAacc.cpu().numpy(), oracle.qconv_bwd_data(E, Wq, H, W, stride, pad)[0])
+    dWacc = torch.empty(Wq.shape, dtype=torch.int32, device="cuda")
+    least = up(4 * wn) + up(nodes * B * H * W * ((Cin + 15) // 16 * 16))
+    api.lpdt_qconv_bwd_weight(desc, dev(E), None, dev(A), None, dWacc=dWacc, ws=ws_bytes(least))
+    assert np.array_equal(dWacc.cpu().numpy(), oracle.qconv_bwd_weight(E, A, R, S, stride, pad)[0])
+
+
 def test_qconv_fwd_affine_matches_quantizer_output():
     # end to end with lpdt_quantize's affine mode: real 0 maps to the zero point, so a zero-padded real
     # convolution of the dequantized tensors equals scale * acc
