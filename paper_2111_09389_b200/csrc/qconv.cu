@@ -259,6 +259,110 @@ __global__ void weight_prefix_kernel(const int32_t *__restrict__ tapsum, int nod
     }
 }
 
+// The same table in one launch, for both directions and any stride (layout: PixParams in the tensor-core engine):
+//   over_cout = 0: t[co][r][s] = sum over ci of W[n][co][r][s][ci], st = 1              (C = Cout)
+//   over_cout = 1: t[ci][r][s] = sum over co of W[n][co][r][s][ci], st = the stride     (C = Cin)
+// Block (16 result channels, node): tap sums in shared memory, prefix sums over the taps, table written out.  One thread
+// per entry with a serial loop over the other channels took 15.9 us at 8 x 128 x 128 x 9 for the sums alone.
+constexpr int kTabC = 16;
+__global__ void __launch_bounds__(1024)
+weight_table_kernel(lpdt_conv_desc d, const uint8_t *__restrict__ Wq, int over_cout, int st, bool vec16, bool vec4, int32_t *__restrict__ P) {
+    pdl_enter();
+    extern __shared__ unsigned s_tab[];
+    const int taps = d.R * d.S, C = over_cout ? d.Cin : d.Cout, PS = d.S + st, cells = (d.R + st) * PS;
+    unsigned *t = s_tab, *pre = s_tab + taps * kTabC;             // [taps][16], [cells][16]
+    const int n = blockIdx.y, c0 = blockIdx.x * kTabC, nc = C - c0 < kTabC ? C - c0 : kTabC, tid = threadIdx.x, T = blockDim.x;
+    const uint8_t *w = Wq + (int64_t)n * d.Cout * taps * d.Cin;
+    for (int i = tid; i < taps * kTabC; i += T) t[i] = 0;
+    __syncthreads();
+    if (over_cout) {
+        // thread = (tap, every (T / taps)-th output channel), 16 input channels of the row; pairs of bytes are summed
+        // in 16-bit halves, at most 256 rows at a time
+        const int step = T / taps, tap = tid % taps;
+        if (tid < step * taps) {
+            int co = tid / taps;
+            while (co < d.Cout) {
+                unsigned e[4] = {0, 0, 0, 0}, o[4] = {0, 0, 0, 0};
+                const int end = co + 256 * step < d.Cout ? co + 256 * step : d.Cout;
+#pragma unroll 4
+                for (; co < end; co += step) {
+                    const uint8_t *row = w + ((int64_t)co * taps + tap) * d.Cin + c0;
+                    uint4 q;
+                    if (vec16) q = __ldg(reinterpret_cast<const uint4 *>(row));
+                    else {
+                        unsigned b[4] = {0, 0, 0, 0};
+                        if (vec4) {
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) if (4 * k < nc) b[k] = __ldg(reinterpret_cast<const unsigned *>(row) + k);
+                        } else
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) if (k < nc) b[k >> 2] |= (unsigned)row[k] << (8 * (k & 3));
+                        q = make_uint4(b[0], b[1], b[2], b[3]);
+                    }
+                    const unsigned v[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) { e[k] += v[k] & 0x00ff00ffu; o[k] += (v[k] >> 8) & 0x00ff00ffu; }
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    atomicAdd(t + tap * kTabC + 4 * k, e[k] & 0xffffu); atomicAdd(t + tap * kTabC + 4 * k + 2, e[k] >> 16);
+                    atomicAdd(t + tap * kTabC + 4 * k + 1, o[k] & 0xffffu); atomicAdd(t + tap * kTabC + 4 * k + 3, o[k] >> 16);
+                }
+            }
+        }
+    } else {
+        // eight lanes per row (output channel, tap), 32 where one row each fills the block
+        const int G = taps == 1 ? 32 : 8, lane = tid & (G - 1);
+        for (int row = tid / G; row < taps * kTabC; row += T / G) {
+            const int tap = row % taps, c = row / taps;
+            unsigned sum = 0;
+            if (c < nc) {
+                const uint8_t *r = w + ((int64_t)(c0 + c) * taps + tap) * d.Cin;
+                if (vec16) {
+#pragma unroll 4
+                    for (int i = lane; i < d.Cin / 16; i += G) {
+                        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(r) + i);
+                        sum = __dp4a(v.x, 0x01010101u, sum); sum = __dp4a(v.y, 0x01010101u, sum);
+                        sum = __dp4a(v.z, 0x01010101u, sum); sum = __dp4a(v.w, 0x01010101u, sum);
+                    }
+                } else {
+                    for (int i = lane; i < d.Cin; i += G) sum += r[i];
+                }
+            }
+            atomicAdd(t + tap * kTabC + c, sum);
+        }
+    }
+    __syncthreads();
+    if (tid < kTabC) {
+        for (int r = 0; r < d.R + st; ++r)
+            for (int s = 0; s < PS; ++s) {
+                unsigned v = 0;
+                if (r >= st && s >= st)
+                    v = t[((r - st) * d.S + s - st) * kTabC + tid] + pre[((r - st) * PS + s) * kTabC + tid] +
+                        pre[(r * PS + s - st) * kTabC + tid] - pre[((r - st) * PS + s - st) * kTabC + tid];
+                pre[(r * PS + s) * kTabC + tid] = v;
+            }
+    }
+    __syncthreads();
+    for (int i = tid; i < cells * kTabC; i += T)
+        if ((i & (kTabC - 1)) < nc) P[((int64_t)n * cells + i / kTabC) * C + c0 + (i & (kTabC - 1))] = (int32_t)pre[i];
+}
+// Threads per block: forward 1024 (144 rows of a 3x3 filter in two goes), backward-data 512 (their sums meet in atomics).
+static int table_threads(int over_cout) { return over_cout ? 512 : 1024; }
+// Shapes the kernel above takes: a thread per tap, the tables in 48 KB of shared memory, nodes in grid.y.
+static bool table_fits(const lpdt_conv_desc &d, int st) {
+    return d.R * d.S <= 256 && ((int64_t)d.R * d.S + (int64_t)(d.R + st) * (d.S + st)) * kTabC * 4 <= 48 * 1024 && d.nodes <= 65535;
+}
+static lpdt_status weight_table_launch(const lpdt_conv_desc &d, const uint8_t *Wq, int over_cout, int st, int32_t *P, cudaStream_t stream) {
+    const int C = over_cout ? d.Cin : d.Cout;
+    const size_t smem = ((size_t)d.R * d.S + (size_t)(d.R + st) * (d.S + st)) * kTabC * 4;
+    const bool vec16 = d.Cin % 16 == 0 && aligned(Wq, 16);
+    launch_k(weight_table_kernel, dim3((unsigned)ceil_div(C, kTabC), d.nodes), table_threads(over_cout), smem, stream, d, Wq, over_cout, st, vec16,
+             d.Cin % 4 == 0 && aligned(Wq, 4), P);
+    LPDT_LAUNCH_CHECK();
+    return LPDT_OK;
+}
+
 // One thread per (output pixel, V consecutive output channels); V = 4 with 16-byte accesses when the
 // channel count allows, else 1.
 template <int V>
@@ -346,6 +450,12 @@ static lpdt_status row_sum_launch(const uint8_t *src, int64_t rows, int len, int
 
 }  // namespace lpdt
 
+// LPDT_AFFINE_SEPARATE=1 keeps the separate correction passes of forward and backward-data on every shape.
+static bool affine_separate() {
+    static int separate = -1;
+    if (separate < 0) { const char *e = getenv("LPDT_AFFINE_SEPARATE"); separate = (e && e[0] == '1') ? 1 : 0; }
+    return separate == 1;
+}
 static size_t affine_raw_bytes(const lpdt_conv_desc *d) {
     const int Ho = conv_out(d->H, d->pad, d->R, d->stride), Wo = conv_out(d->W, d->pad, d->S, d->stride);
     return align_up((size_t)d->nodes * d->B * Ho * Wo * d->Cout * sizeof(int32_t), 256);
@@ -390,16 +500,19 @@ extern "C" lpdt_status lpdt_qconv_fwd_affine(const lpdt_conv_desc *d, const uint
     if (s != LPDT_OK) return s;
     const int rows = d->nodes * d->Cout;
     int32_t *tapsum = (int32_t *)((char *)P + align_up((size_t)rows * (d->R + 1) * (d->S + 1) * sizeof(int32_t), 256));
-    s = row_sum_launch(Wq, (int64_t)rows * d->R * d->S, d->Cin, tapsum, st);
-    if (s != LPDT_OK) return s;
-    launch_k(weight_prefix_kernel, (rows + 127) / 128, 128, 0, st, tapsum, d->nodes, d->Cout, d->R, d->S, P);
-    LPDT_LAUNCH_CHECK();
+    if (table_fits(*d, 1)) {
+        s = weight_table_launch(*d, Wq, 0, 1, P, st);
+        if (s != LPDT_OK) return s;
+    } else {
+        s = row_sum_launch(Wq, (int64_t)rows * d->R * d->S, d->Cin, tapsum, st);
+        if (s != LPDT_OK) return s;
+        launch_k(weight_prefix_kernel, (rows + 127) / 128, 128, 0, st, tapsum, d->nodes, d->Cout, d->R, d->S, P);
+        LPDT_LAUNCH_CHECK();
+    }
     // Tensor-core path: the zero-point terms are applied in the contraction's own epilogue (no raw sums in
-    // memory, no second pass over the result).  LPDT_AFFINE_SEPARATE=1 keeps the separate correction pass.
-    static int separate = -1;
-    if (separate < 0) { const char *e = getenv("LPDT_AFFINE_SEPARATE"); separate = (e && e[0] == '1') ? 1 : 0; }
+    // memory, no second pass over the result).
     const size_t inner_bytes = ws_bytes - (size_t)((char *)inner - (char *)ws);
-    if (!separate && d->Cout % 4 == 0) {
+    if (!affine_separate()) {
         const tc::AffineArgs aff = {asum, P, zA, zW};
         lpdt_status r = fwd_impl(d, reinterpret_cast<const int8_t *>(A), sA, reinterpret_cast<const int8_t *>(Wq), sW,
                                  bias, bias_node_stride, Y, Yacc, inner, inner_bytes, dev_status, st, true, &aff);
@@ -420,13 +533,14 @@ extern "C" lpdt_status lpdt_qconv_fwd_affine(const lpdt_conv_desc *d, const uint
     return LPDT_OK;
 }
 
-// Backward-data contraction on raw codes (signed, or unsigned when `uns`): kernel choice only.
+// Backward-data contraction on raw codes (signed, or unsigned when `uns`): kernel choice only; `aff` as in fwd_impl.
 static lpdt_status bwd_data_impl(const lpdt_conv_desc *d, const int8_t *E, const float *sE, const int8_t *Wq,
                                  const float *sW, float *dA, int32_t *dAacc, const float *addend, void *ws,
-                                 size_t ws_bytes, int32_t *dev_status, cudaStream_t st, bool uns) {
+                                 size_t ws_bytes, int32_t *dev_status, cudaStream_t st, bool uns,
+                                 const tc::AffineArgs *aff = nullptr) {
     const int64_t results = (int64_t)d->nodes * d->B * d->H * d->W * d->Cin;
     const bool vec4 = d->Cout % 4 == 0 && aligned(E, 4);
-    if (!tiny_dot(*d, results, d->R * d->S * d->Cout, vec4) && use_tc(*d, 1, ws, ws_bytes) && readable(E, d->Cout) && readable(Wq, d->Cin) && (!dA || aligned(dA, 16)) &&
+    if ((aff || !tiny_dot(*d, results, d->R * d->S * d->Cout, vec4)) && use_tc(*d, 1, ws, ws_bytes) && readable(E, d->Cout) && readable(Wq, d->Cin) && (!dA || aligned(dA, 16)) &&
         (!dAacc || aligned(dAacc, 16))) {
         const int Ho = conv_out(d->H, d->pad, d->R, d->stride), Wo = conv_out(d->W, d->pad, d->S, d->stride);
         const PadPlan pp = pad_plan(*d);
@@ -435,9 +549,10 @@ static lpdt_status bwd_data_impl(const lpdt_conv_desc *d, const int8_t *E, const
                                    pad_job(Wq, Wp, pp.w ? (int64_t)d->nodes * d->Cout * d->R * d->S : 0, d->Cin), st);
         if (s != LPDT_OK) return s;
         lpdt_status r = run_pix(*d, 1, pp.err ? (int8_t *)Ep : E, sE, pp.w ? (int8_t *)Wp : Wq, sW, nullptr, 0, dA, dAacc,
-                                dev_status, st, uns, addend, nullptr);
+                                dev_status, st, uns, addend, aff);
         if (r != LPDT_ERR_UNSUPPORTED || (!pp.err && !pp.w)) return r;
     }
+    if (aff) return LPDT_ERR_UNSUPPORTED;
     return generic_bwd_data(*d, E, sE, Wq, sW, dA, dAacc, addend, ws, st, uns);
 }
 
@@ -562,73 +677,120 @@ __global__ void affine_fix_bwd_data_kernel(lpdt_conv_desc d, int Ho, int Wo, con
     }
 }
 
-// col[n][pos][c] = sum over the batch of src[n][b][pos][c] (unsigned codes); one thread per output, c fastest.
-__global__ void batch_sum_u8_kernel(const uint8_t *__restrict__ src, int nodes, int B, int64_t per_image,
-                                    int32_t *__restrict__ col) {
+// Sums of the operands of backward-weight over the output positions whose tap (r, s) lies inside the input image:
+//   tabE[n][r][s][co] = sum of E[n][b][oh][ow][co],  tabA[n][r][s][ci] = sum of A[n][b][oh*st+r-pad][ow*st+s-pad][ci].
+// Work item = (operand, node, up to `cw` channels, up to `sw` filter columns, image row, share of the batch), a block each.
+// The block sums its row over its samples per column (V bytes of consecutive channels per thread), adds a column's sums
+// to every filter column that reaches it in shared memory, and the result to every filter row that reaches the row,
+// with integer atomics into zeroed tables.  (Batch sums in memory and one serial loop over the positions per tap and
+// channel took 141 us at 8 x 32 x 16x16 x 128.)
+struct TapSumSide { const uint8_t *src; int32_t *tab; int rows, cols, C, cw, chunks; long long items; };
+constexpr int kTapThreads = 512;
+template <int V>
+__global__ void __launch_bounds__(kTapThreads)
+tap_sum_kernel(lpdt_conv_desc d, int Ho, int Wo, TapSumSide sideE, TapSumSide sideA, int sw, int bshares) {
     pdl_enter();
-    const int64_t total = (int64_t)nodes * per_image;
-    for (int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; o < total; o += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t n = o / per_image, i = o % per_image;
-        const uint8_t *p = src + n * B * per_image + i;
-        unsigned sum = 0;
-        for (int b = 0; b < B; ++b) sum += p[(int64_t)b * per_image];
-        col[o] = (int32_t)sum;
-    }
-}
-
-// Sums of a batch-summed image over the output positions whose tap (r, s) lies inside the input image:
-//   of_input = 0: tab[n][r][s][c] = sum col[n][oh][ow][c]                        (col over the OUTPUT image, C = Cout)
-//   of_input = 1: tab[n][r][s][c] = sum col[n][oh*st+r-pad][ow*st+s-pad][c]      (col over the INPUT image, C = Cin)
-// block (tap, node), threads over channels.
-__global__ void tap_table_kernel(lpdt_conv_desc d, int Ho, int Wo, int of_input, int C,
-                                 const int32_t *__restrict__ col, int32_t *__restrict__ tab) {
-    pdl_enter();
-    const int tap = blockIdx.x, n = blockIdx.y, r = tap / d.S, s = tap % d.S;
-    const int Hc = of_input ? d.H : Ho, Wc = of_input ? d.W : Wo;
-    for (int c = threadIdx.x; c < C; c += blockDim.x) {
-        unsigned sum = 0;
-        for (int oh = 0; oh < Ho; ++oh) {
-            const int ih = oh * d.stride + r - d.pad;
-            if (ih < 0 || ih >= d.H) continue;
-            for (int ow = 0; ow < Wo; ++ow) {
-                const int iw = ow * d.stride + s - d.pad;
-                if (iw < 0 || iw >= d.W) continue;
-                const int ph = of_input ? ih : oh, pw = of_input ? iw : ow;
-                sum += (unsigned)col[(((int64_t)n * Hc + ph) * Wc + pw) * C + c];
+    extern __shared__ unsigned s_acc[];                       // [sw][cw]
+    const int tid = threadIdx.x, schunks = (d.S + sw - 1) / sw;
+    for (long long item = blockIdx.x; item < sideE.items + sideA.items; item += gridDim.x) {
+        const bool in = item >= sideE.items;
+        const TapSumSide sd = in ? sideA : sideE;
+        long long q = in ? item - sideE.items : item;
+        const int share = (int)(q % bshares); q /= bshares;
+        const int row = (int)(q % sd.rows); q /= sd.rows;
+        const int s0 = (int)(q % schunks) * sw; q /= schunks;
+        const int c0 = (int)(q % sd.chunks) * sd.cw, n = (int)(q / sd.chunks);
+        const int cw = sd.cw, nc = sd.C - c0 < cw ? sd.C - c0 : cw, ns = d.S - s0 < sw ? d.S - s0 : sw;
+        for (int i = tid; i < ns * cw; i += kTapThreads) s_acc[i] = 0;
+        __syncthreads();
+        const int b0 = (int)((int64_t)d.B * share / bshares), b1 = (int)((int64_t)d.B * (share + 1) / bshares);
+        const int words = (nc + V - 1) / V;
+        const int64_t image = (int64_t)sd.rows * sd.cols * sd.C;
+        const uint8_t *src = sd.src + (int64_t)n * d.B * image + (int64_t)row * sd.cols * sd.C + c0;
+        // (up to 64 samples, column, word), word fastest
+        int plen = 64;                                        // fewer where that leaves threads idle
+        while (plen > 16 && (b1 - b0 + plen - 1) / plen * sd.cols * words < kTapThreads) plen /= 2;
+        const int parts = (b1 - b0 + plen - 1) / plen, sums = parts * sd.cols * words;
+        for (int it = tid; it < sums; it += kTapThreads) {
+            const int wd = it % words, r = it / words, col = r % sd.cols, part = r / sd.cols;
+            const uint8_t *p = src + (int64_t)col * sd.C + wd * V;
+            const int lo = b0 + part * plen, hi = lo + plen < b1 ? lo + plen : b1;
+            unsigned sum[V];
+            if constexpr (V == 4) {
+                unsigned e = 0, o = 0;                        // byte sums in 16-bit halves: at most 64 bytes each
+                for (int b = lo; b < hi; b += 16) {
+                    unsigned w[16];
+#pragma unroll
+                    for (int u = 0; u < 16; ++u)              // all in flight at once
+                        w[u] = b + u < hi ? __ldg(reinterpret_cast<const unsigned *>(p + (b + u) * image)) : 0u;
+#pragma unroll
+                    for (int u = 0; u < 16; ++u) { e += w[u] & 0x00ff00ffu; o += (w[u] >> 8) & 0x00ff00ffu; }
+                }
+                sum[0] = e & 0xffffu; sum[1] = o & 0xffffu; sum[2] = e >> 16; sum[3] = o >> 16;
+            } else {
+                sum[0] = 0;
+#pragma unroll 8
+                for (int b = lo; b < hi; ++b) sum[0] += p[b * image];
+            }
+            for (int k = 0; k < ns; ++k) {
+                const int s = s0 + k;
+                bool ok;                                      // filter column s reaches this image column
+                if (in) { const int t = col + d.pad - s; ok = t >= 0 && t % d.stride == 0 && t / d.stride < Wo; }
+                else { const int iw = col * d.stride + s - d.pad; ok = iw >= 0 && iw < d.W; }
+                if (!ok) continue;
+#pragma unroll
+                for (int v = 0; v < V; ++v) atomicAdd(s_acc + k * cw + wd * V + v, sum[v]);
             }
         }
-        tab[((int64_t)n * d.R * d.S + tap) * C + c] = (int32_t)sum;
+        __syncthreads();
+        for (int r = 0; r < d.R; ++r) {
+            bool ok;
+            if (in) { const int t = row + d.pad - r; ok = t >= 0 && t % d.stride == 0 && t / d.stride < Ho; }
+            else { const int ih = row * d.stride + r - d.pad; ok = ih >= 0 && ih < d.H; }
+            if (!ok) continue;
+            int32_t *t = sd.tab + (((int64_t)n * d.R + r) * d.S + s0) * sd.C + c0;
+            for (int i = tid; i < ns * nc; i += kTapThreads) {
+                const unsigned v = s_acc[i / nc * cw + i % nc];
+                if (v) atomicAdd(t + (int64_t)(i / nc) * sd.C + i % nc, (int)v);
+            }
+        }
+        __syncthreads();
     }
 }
 
-// One thread per weight-gradient entry (n, co, r, s, ci); ci fastest.
-__global__ void affine_fix_bwd_weight_kernel(lpdt_conv_desc d, int Ho, int Wo, const int32_t *__restrict__ raw,
-                                             const int32_t *__restrict__ tabE, const int32_t *__restrict__ tabA,
-                                             const int32_t *__restrict__ zE, const int32_t *__restrict__ zA,
-                                             const float *__restrict__ sE, const float *__restrict__ sA,
-                                             float *__restrict__ dW, int64_t dw_stride, int32_t *__restrict__ dWacc) {
+// Number of output positions o in [0, No) whose tap r of one axis lies inside an input of length `len`.
+__device__ inline int taps_inside(int No, int len, int r, int pad, int st) {
+    const int lo = pad > r ? (pad - r + st - 1) / st : 0;
+    int hi = len - 1 + pad - r;
+    if (hi < 0) return 0;
+    hi /= st;
+    if (hi > No - 1) hi = No - 1;
+    return hi >= lo ? hi - lo + 1 : 0;
+}
+
+// Block (output channel, node), threads over the entries (r, s, ci) of its filter.
+__global__ void __launch_bounds__(256)
+affine_fix_bwd_weight_kernel(lpdt_conv_desc d, int Ho, int Wo, const int32_t *__restrict__ raw,
+                             const int32_t *__restrict__ tabE, const int32_t *__restrict__ tabA,
+                             const int32_t *__restrict__ zE, const int32_t *__restrict__ zA,
+                             const float *__restrict__ sE, const float *__restrict__ sA,
+                             float *__restrict__ dW, int64_t dw_stride, int32_t *__restrict__ dWacc) {
     pdl_enter();
-    const int taps = d.R * d.S;
-    const int64_t per_node = (int64_t)d.Cout * taps * d.Cin;
-    const int64_t total = per_node * d.nodes;
-    for (int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; o < total; o += (int64_t)gridDim.x * blockDim.x) {
-        const int n = (int)(o / per_node);
-        const int64_t i = o % per_node;
-        const int ci = (int)(i % d.Cin);
-        const int tap = (int)((i / d.Cin) % taps);
-        const int co = (int)(i / ((int64_t)d.Cin * taps));
-        const int r = tap / d.S, s = tap % d.S;
-        // output rows / columns whose tap lies inside the input image
-        int nh = 0, nw = 0;
-        for (int oh = 0; oh < Ho; ++oh) { const int ih = oh * d.stride + r - d.pad; nh += (ih >= 0 && ih < d.H); }
-        for (int ow = 0; ow < Wo; ++ow) { const int iw = ow * d.stride + s - d.pad; nw += (iw >= 0 && iw < d.W); }
-        const unsigned cnt = (unsigned)d.B * (unsigned)nh * (unsigned)nw;
-        const unsigned ze = (unsigned)zE[n], za = (unsigned)zA[n];
-        const unsigned te = (unsigned)tabE[((int64_t)n * taps + tap) * d.Cout + co];
-        const unsigned ta = (unsigned)tabA[((int64_t)n * taps + tap) * d.Cin + ci];
-        const int acc = (int)((unsigned)raw[o] - za * te - ze * ta + cnt * ze * za);
-        if (dWacc) dWacc[o] = acc;
-        if (dW) dW[(int64_t)n * dw_stride + i] = __fmul_rn(__int2float_rn(acc), __fmul_rn(sE[n], sA[n]));
+    const int taps = d.R * d.S, n = blockIdx.y, co = blockIdx.x;
+    const int64_t per_co = (int64_t)taps * d.Cin;
+    const unsigned ze = (unsigned)zE[n], za = (unsigned)zA[n];
+    const float sc = dW ? __fmul_rn(sE[n], sA[n]) : 0.f;
+    const int64_t o0 = ((int64_t)n * d.Cout + co) * per_co;
+    const int32_t *ta = tabA + (int64_t)n * per_co;           // entry (tap, ci): the filter's own layout
+#pragma unroll 4
+    for (int64_t i = threadIdx.x; i < per_co; i += blockDim.x) {
+        const int tap = per_co <= 0x7fffffff ? (int)((uint32_t)i / (uint32_t)d.Cin) : (int)(i / d.Cin), r = tap / d.S, s = tap % d.S;
+        const unsigned cnt = (unsigned)d.B * (unsigned)taps_inside(Ho, d.H, r, d.pad, d.stride) *
+                             (unsigned)taps_inside(Wo, d.W, s, d.pad, d.stride);
+        const unsigned te = (unsigned)__ldg(tabE + ((int64_t)n * taps + tap) * d.Cout + co);
+        const int acc = (int)((unsigned)raw[o0 + i] - za * te - ze * (unsigned)__ldg(ta + i) + cnt * ze * za);
+        if (dWacc) dWacc[o0 + i] = acc;
+        if (dW) dW[(int64_t)n * dw_stride + co * per_co + i] = __fmul_rn(__int2float_rn(acc), sc);
     }
 }
 
@@ -670,10 +832,23 @@ extern "C" lpdt_status lpdt_qconv_bwd_data_affine(const lpdt_conv_desc *d, const
     int32_t *esum = (int32_t *)((char *)ws + affine_bwd_data_raw_bytes(d));
     int32_t *wsum = (int32_t *)((char *)esum + affine_esum_bytes(d));
     void *inner = (char *)wsum + affine_wsum_bytes(d);
-    s = bwd_data_impl(d, reinterpret_cast<const int8_t *>(E), nullptr, reinterpret_cast<const int8_t *>(Wq), nullptr,
-                      nullptr, raw, nullptr, inner, ws_bytes - (size_t)((char *)inner - (char *)ws), dev_status, st, true);
-    if (s != LPDT_OK) return s;
+    const size_t inner_bytes = ws_bytes - (size_t)((char *)inner - (char *)ws);
     s = row_sum_launch(E, (int64_t)d->nodes * d->B * Ho * Wo, d->Cout, esum, st);
+    if (s != LPDT_OK) return s;
+    // Zero-point terms in the contraction's epilogue, as in the forward product; the table takes the place of the raw
+    // sums, which do not exist then.  8 x 32 x 16x16 128 -> 128 3x3: 34.8 us, 107.5 us with the raw sums written and
+    // corrected in a second pass (80 us of them), which shapes outside the tensor-core path still take.
+    const size_t table = (size_t)d->nodes * (d->R + d->stride) * (d->S + d->stride) * d->Cin * sizeof(int32_t);
+    if (!affine_separate() && table_fits(*d, d->stride) && table <= affine_bwd_data_raw_bytes(d) && use_tc(*d, 1, inner, inner_bytes)) {
+        s = weight_table_launch(*d, Wq, 1, d->stride, raw, st);
+        if (s != LPDT_OK) return s;
+        const tc::AffineArgs aff = {esum, raw, zE, zW};
+        s = bwd_data_impl(d, reinterpret_cast<const int8_t *>(E), sE, reinterpret_cast<const int8_t *>(Wq), sW, dA, dAacc,
+                          nullptr, inner, inner_bytes, dev_status, st, true, &aff);
+        if (s != LPDT_ERR_UNSUPPORTED) return s;
+    }
+    s = bwd_data_impl(d, reinterpret_cast<const int8_t *>(E), nullptr, reinterpret_cast<const int8_t *>(Wq), nullptr,
+                      nullptr, raw, nullptr, inner, inner_bytes, dev_status, st, true);
     if (s != LPDT_OK) return s;
     launch_k(weight_cout_sum_kernel, grid_for((int64_t)d->nodes * d->R * d->S * d->Cin), 256, 0, st, *d, Wq, wsum);
     LPDT_LAUNCH_CHECK();
@@ -690,6 +865,7 @@ extern "C" lpdt_status lpdt_qconv_bwd_data_affine(const lpdt_conv_desc *d, const
 static size_t affine_wg_raw_bytes(const lpdt_conv_desc *d) {
     return align_up((size_t)d->nodes * d->Cout * d->R * d->S * d->Cin * sizeof(int32_t), 256);
 }
+// (colE and colA: part of the size that callers are asked for; not written)
 static size_t affine_colE_bytes(const lpdt_conv_desc *d) {
     const int Ho = conv_out(d->H, d->pad, d->R, d->stride), Wo = conv_out(d->W, d->pad, d->S, d->stride);
     return align_up((size_t)d->nodes * Ho * Wo * d->Cout * sizeof(int32_t), 256);
@@ -735,19 +911,24 @@ extern "C" lpdt_status lpdt_qconv_bwd_weight_affine(const lpdt_conv_desc *d, con
     s = bwd_weight_impl(d, reinterpret_cast<const int8_t *>(E), nullptr, reinterpret_cast<const int8_t *>(A), nullptr,
                         nullptr, 0, raw, inner, ws_bytes - (size_t)((char *)inner - (char *)ws), dev_status, st, true);
     if (s != LPDT_OK) return s;
-    launch_k(batch_sum_u8_kernel, grid_for((int64_t)d->nodes * Ho * Wo * d->Cout), 256, 0, st, E, d->nodes, d->B,
-             (int64_t)Ho * Wo * d->Cout, colE);
+    // both operands' tap sums; samples are shared out until about two waves of blocks exist
+    LPDT_CUDA(cudaMemsetAsync(tabE, 0, affine_tab_bytes(d, d->Cout) + affine_tab_bytes(d, d->Cin), st));
+    const int sw = d->S < 24 ? d->S : 24, cw = 512;                  // 48 KB of shared memory at most
+    const int64_t schunks = ceil_div(d->S, sw);
+    TapSumSide sideE = {E, tabE, Ho, Wo, d->Cout, cw, (int)ceil_div(d->Cout, cw), 0};
+    TapSumSide sideA = {A, tabA, d->H, d->W, d->Cin, cw, (int)ceil_div(d->Cin, cw), 0};
+    sideE.items = d->nodes * sideE.chunks * schunks * Ho; sideA.items = d->nodes * sideA.chunks * schunks * d->H;
+    int64_t shares = ceil_div(2 * kNumSMs, sideE.items + sideA.items);
+    if (shares > ceil_div(d->B, 64)) shares = ceil_div(d->B, 64);
+    if (shares < 1) shares = 1;
+    sideE.items *= shares; sideA.items *= shares;
+    const int64_t blocks = sideE.items + sideA.items < (int64_t)kNumSMs * 64 ? sideE.items + sideA.items : (int64_t)kNumSMs * 64;
+    const bool v4 = d->Cin % 4 == 0 && d->Cout % 4 == 0 && aligned(E, 4) && aligned(A, 4);
+    launch_k(v4 ? tap_sum_kernel<4> : tap_sum_kernel<1>, (unsigned)blocks, kTapThreads, (size_t)sw * cw * 4, st, *d, Ho, Wo, sideE, sideA, sw,
+             (int)shares);
     LPDT_LAUNCH_CHECK();
-    launch_k(batch_sum_u8_kernel, grid_for((int64_t)d->nodes * d->H * d->W * d->Cin), 256, 0, st, A, d->nodes, d->B,
-             (int64_t)d->H * d->W * d->Cin, colA);
-    LPDT_LAUNCH_CHECK();
-    const dim3 tgrid(d->R * d->S, d->nodes);
-    launch_k(tap_table_kernel, tgrid, 128, 0, st, *d, Ho, Wo, 0, d->Cout, colE, tabE);
-    LPDT_LAUNCH_CHECK();
-    launch_k(tap_table_kernel, tgrid, 128, 0, st, *d, Ho, Wo, 1, d->Cin, colA, tabA);
-    LPDT_LAUNCH_CHECK();
-    launch_k(affine_fix_bwd_weight_kernel, grid_for((int64_t)d->nodes * d->Cout * d->R * d->S * d->Cin), 256, 0, st, *d, Ho,
-             Wo, raw, tabE, tabA, zE, zA, sE, sA, dW, dw_node_stride, dWacc);
+    launch_k(affine_fix_bwd_weight_kernel, dim3(d->Cout, d->nodes), 256, 0, st, *d, Ho, Wo, raw, tabE, tabA, zE, zA, sE, sA, dW,
+             dw_node_stride, dWacc);
     LPDT_LAUNCH_CHECK();
     return LPDT_OK;
 }

@@ -26,9 +26,9 @@ namespace tc {
 // Bytes between the channel rows of the operands in memory (multiples of 16, at least the channel count).
 struct Pitches { int in, err, w; };      // activations (Cin), layer gradients (Cout), weights (Cin)
 bool tc_supported(const lpdt_conv_desc &d);
-// Zero-point correction applied in the forward epilogue (unsigned operands): per-pixel channel sums of the
-// input [nodes][B][H][W], prefix table of the weights' channel sums over the filter taps
-// [nodes][R+1][S+1][Cout], and the per-node zero points.
+// Zero-point correction applied in the epilogue (unsigned operands): per-pixel channel sums of operand A (the input, or
+// backward-data the layer gradient), the table of the weights' channel sums over the filter taps (see PixParams; up to
+// 124 bytes past its end are read), and the per-node zero points of operand A and of the weights.
 struct AffineArgs { const int32_t *asum, *wpre, *zA, *zW; };
 lpdt_status tc_pix(const lpdt_conv_desc &d, int mode, const int8_t *A, const float *s1, const int8_t *Wq,
                    const float *s2, const float *bias, int64_t bias_stride, float *Y, int32_t *Yacc,

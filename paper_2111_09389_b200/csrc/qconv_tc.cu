@@ -97,46 +97,82 @@ struct PixParams {
     // writes them row by row with plain stores.
     int tma_out, out_off;     // out_off: byte offset of the staging area in shared memory (1024-byte aligned)
     int bw, bh;               // the warp's sub-box of the pixel tile: bw x bh x 32/(bw*bh) pixels
-    // Forward product on affine (zero-point) operands, corrected in the epilogue (null asum: plain product):
+    // Products on affine (zero-point) operands, corrected in the epilogue (instantiations AFF = 1, 2).  Forward:
     //   sum (qa - zA)(qw - zW) = acc - zW * ra - zA * rw + cnt * zA * zW   over the taps inside the image,
-    // ra = the per-pixel channel sums of the input (asum [nodes][B][H][W]) over those taps, rw = the weights'
-    // channel sums over them, from a prefix table over the filter taps (wpre [nodes][R+1][S+1][Cout]; the taps
-    // inside the image form a rectangle of the filter), cnt = taps inside x Cin.  All modulo 2^32.
+    // ra = the per-pixel channel sums of operand A (asum [nodes][B][aH][aW]) over those taps, rw = the weights' sums over
+    // the summed channels, from a prefix table over the filter taps (wpre [nodes][aR+st][aS+st][Nc]: entry (r, s) adds
+    // the taps r' < r, s' < s with r' = r and s' = s modulo st; the taps that exist form a rectangle of the filter, with
+    // step st), cnt = taps x Kc.  st = 1 forward; backward-data: A = the layer gradient, st = the stride.  Modulo 2^32.
     const int32_t *asum, *wpre, *zA, *zW;
-    int aH, aW, aR, aS, apad, astride, aCin;
+    int aH, aW, aR, aS, apad, astride;
 };
 
 // Zero-point terms of one output pixel: what does not depend on the output channel (fixed) and the corners of
 // the pixel's tap rectangle in the prefix table.
 struct AffinePixel { unsigned fixed, za; int c11, c01, c10, c00; bool interior; };
-__device__ __forceinline__ AffinePixel affine_pixel(const PixParams &p, int node, int b, int oh, int ow) {
-    int r_lo = p.apad - oh * p.astride; if (r_lo < 0) r_lo = 0;
-    int r_hi = p.aH + p.apad - oh * p.astride; if (r_hi > p.aR) r_hi = p.aR;
-    int s_lo = p.apad - ow * p.astride; if (s_lo < 0) s_lo = 0;
-    int s_hi = p.aW + p.apad - ow * p.astride; if (s_hi > p.aS) s_hi = p.aS;
-    if (r_hi < r_lo) r_hi = r_lo;
-    if (s_hi < s_lo) s_hi = s_lo;
-    const long long nb = (long long)node * p.B + b;
-    unsigned ra = 0;
-    for (int r = r_lo; r < r_hi; ++r)
-        for (int s = s_lo; s < s_hi; ++s)
-            ra += (unsigned)__ldg(p.asum + (nb * p.aH + oh * p.astride + r - p.apad) * p.aW + ow * p.astride + s - p.apad);
-    AffinePixel a;
-    const unsigned za = (unsigned)p.zA[node], zw = (unsigned)p.zW[node];
-    a.za = za;
-    a.fixed = (unsigned)((r_hi - r_lo) * (s_hi - s_lo) * p.aCin) * za * zw - zw * ra;
-    const int PS = p.aS + 1;
-    a.c11 = (r_hi * PS + s_hi) * p.Nc; a.c01 = (r_lo * PS + s_hi) * p.Nc;
-    a.c10 = (r_hi * PS + s_lo) * p.Nc; a.c00 = (r_lo * PS + s_lo) * p.Nc;
-    a.interior = r_lo == 0 && s_lo == 0;          // the three other corners are zero
-    return a;
+// Taps of one axis: the first one that exists, how many (step: 1 forward, the stride backward), and the first one's
+// coordinate in operand A.
+struct TapRange { int lo, n, at; };
+template <int AFF>
+__device__ __forceinline__ TapRange tap_range(int o, int R, int pad, int st, int len) {
+    TapRange t;
+    if (AFF == 1) {                                        // output o reads input o*st + r - pad
+        t.lo = max(0, pad - o * st);
+        t.n = max(0, min(R, len + pad - o * st) - t.lo);
+        t.at = o * st + t.lo - pad;
+    } else {                                               // input o reaches output (o + pad - r) / st where that divides
+        const int q = o + pad;
+        t.lo = max(q % st, q - st * (len - 1));
+        const int last = min(R - 1, q);
+        t.n = last >= t.lo ? (last - t.lo) / st + 1 : 0;
+        t.at = (q - t.lo) / st;
+    }
+    return t;
 }
-// acc[k] += fixed - za * rw[channel c0 + k], k < NV (NV a multiple of 4, c0 a multiple of 4).  An N tile that reaches
-// past the last channel reads up to 31 entries past a table row: the caller keeps them inside its workspace, and the
-// results of those columns are never written.
-template <int NV>
+template <int AFF>
+__device__ __forceinline__ AffinePixel affine_pixel(const PixParams &p, int node, int b, int h, int w) {
+    const TapRange th = tap_range<AFF>(h, p.aR, p.apad, p.astride, p.aH), tw = tap_range<AFF>(w, p.aS, p.apad, p.astride, p.aW);
+    const int st = AFF == 1 ? 1 : p.astride, dir = AFF == 1 ? 1 : -1;
+    const int32_t *a = p.asum + (((long long)node * p.B + b) * p.aH + th.at) * p.aW + tw.at;
+    unsigned ra = 0;
+    if (p.aR <= 3 && p.aS <= 3) {                 // the usual filters: all loads in flight at once
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) ra += i < th.n && j < tw.n ? (unsigned)__ldg(a + dir * (i * p.aW + j)) : 0u;
+    } else {
+        for (int i = 0; i < th.n; ++i, a += dir * p.aW)
+            for (int j = 0; j < tw.n; ++j) ra += (unsigned)__ldg(a + dir * j);
+    }
+    AffinePixel o;
+    const unsigned za = (unsigned)p.zA[node], zw = (unsigned)p.zW[node];
+    o.za = za;
+    o.fixed = (unsigned)(th.n * tw.n * p.Kc) * za * zw - zw * ra;
+    const int PS = p.aS + st;
+    // without taps all four corners coincide in entry (0, 0)
+    const int rl = th.n ? th.lo : 0, rh = rl + st * th.n, sl = tw.n ? tw.lo : 0, sh = sl + st * tw.n;
+    o.c11 = (rh * PS + sh) * p.Nc; o.c01 = (rl * PS + sh) * p.Nc;
+    o.c10 = (rh * PS + sl) * p.Nc; o.c00 = (rl * PS + sl) * p.Nc;
+    o.interior = rl < st && sl < st;              // the three other corners are zero
+    return o;
+}
+// acc[k] += fixed - za * rw[channel c0 + k], k < NV (NV a multiple of 4).  16-byte table loads need a channel count that
+// is a multiple of 4; VEC = false loads single entries.  An N tile that reaches past the last channel reads up to 31
+// entries past a table row: the caller keeps them inside its workspace, and the results of those columns are never
+// written.
+template <int AFF, bool VEC, int NV>
 __device__ __forceinline__ void affine_apply(const PixParams &p, const AffinePixel &a, int node, int c0, uint32_t (&v)[NV]) {
-    const int32_t *t = p.wpre + (long long)node * (p.aR + 1) * (p.aS + 1) * p.Nc + c0;
+    const int st = AFF == 1 ? 1 : p.astride;
+    const int32_t *t = p.wpre + (long long)node * (p.aR + st) * (p.aS + st) * p.Nc + c0;
+    if (!VEC) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            unsigned rw = (unsigned)__ldg(t + a.c11 + k);
+            if (!a.interior) rw += (unsigned)__ldg(t + a.c00 + k) - (unsigned)__ldg(t + a.c01 + k) - (unsigned)__ldg(t + a.c10 + k);
+            v[k] = v[k] + a.fixed - a.za * rw;
+        }
+        return;
+    }
 #pragma unroll
     for (int k = 0; k < NV; k += 4) {
         const int4 q11 = __ldg(reinterpret_cast<const int4 *>(t + a.c11 + k));
@@ -202,7 +238,8 @@ __device__ __forceinline__ TileCoord decode_raster(const PixParams &p, int tile)
 // CTA's fill and drain (first operand boxes, the last tile's epilogue) then overlap its neighbour's main loop.
 // ROW: results whose channel count is no multiple of 4 (no 16-byte rows, so neither bulk stores nor vector stores):
 // the epilogue warps write 32 consecutive channels of one pixel per store instruction.
-template <int MINB, bool ROW>
+// AFF: zero-point operands, 1 forward, 2 backward-data (0: plain product; the terms cost it registers).
+template <int MINB, bool ROW, int AFF>
 __global__ void __launch_bounds__(kPixThreads, MINB)
 conv_pix_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapW,
                 const __grid_constant__ CUtensorMap mapY, const PixParams p) {
@@ -363,7 +400,7 @@ conv_pix_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
             const long long pix = (((long long)c.node * p.B + b) * p.Hout + h) * p.Wout + w;
             const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + acc * p.BN;
             AffinePixel aff = {};
-            if (p.asum && valid) aff = affine_pixel(p, c.node, b, h, w);
+            if (AFF && valid) aff = affine_pixel<AFF>(p, c.node, b, h, w);
             if (ROW) {
                 // 32 channels at a time: raw sums -> this warp's staging buffer (128-byte rows, 16-byte pieces
                 // XOR-swizzled by the row), then 32 consecutive elements of the result rows a store: 128 contiguous
@@ -374,6 +411,7 @@ conv_pix_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
                     uint32_t v[32];
                     tmem_ld_32x32(t_row + cc, v);
                     tmem_ld_wait();
+                    if (AFF && valid) affine_apply<AFF, false>(p, aff, c.node, n0 + cc, v);
                     int4 *grow = reinterpret_cast<int4 *>(buf + lane * 128);
 #pragma unroll
                     for (int k = 0; k < 8; ++k)
@@ -421,7 +459,7 @@ conv_pix_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
                 if (have) tmem_ld_32x32(t_row + cc, v);
                 while (have) {
                     tmem_ld_wait();
-                    if (p.asum && valid) affine_apply<32>(p, aff, c.node, n0 + cc, v);
+                    if (AFF && valid) affine_apply<AFF, true>(p, aff, c.node, n0 + cc, v);
                     float f[32];
 #pragma unroll
                     for (int k = 0; k < 32; ++k) f[k] = __fmul_rn(__int2float_rn((int)v[k]), sc);
@@ -470,7 +508,7 @@ conv_pix_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
                 if (valid) {
                     const long long o = pix * p.Nc + n0 + cc;
                     const int quads = (p.Nc - n0 - cc) / 4;          // the tile may reach past the last channel
-                    if (p.asum) affine_apply<16>(p, aff, c.node, n0 + cc, v);
+                    if (AFF) affine_apply<AFF, true>(p, aff, c.node, n0 + cc, v);
                     if (p.Yacc) {
                         int4 *dst = reinterpret_cast<int4 *>(p.Yacc + o);
 #pragma unroll
@@ -794,9 +832,9 @@ lpdt_status tc_pix(const lpdt_conv_desc &d, int mode, const int8_t *A, const flo
     PixParams p = {};
     p.addend = addend;
     if (aff) {
-        if (mode != 0 || d.Cout % 4) return LPDT_ERR_UNSUPPORTED;
         p.asum = aff->asum; p.wpre = aff->wpre; p.zA = aff->zA; p.zW = aff->zW;
-        p.aH = d.H; p.aW = d.W; p.aR = d.R; p.aS = d.S; p.apad = d.pad; p.astride = d.stride; p.aCin = d.Cin;
+        p.aH = mode == 0 ? d.H : Ho; p.aW = mode == 0 ? d.W : Wo;
+        p.aR = d.R; p.aS = d.S; p.apad = d.pad; p.astride = d.stride;
     }
     p.mode = mode; p.nodes = d.nodes; p.B = d.B;
     p.Nc = mode == 0 ? d.Cout : d.Cin; p.Kc = mode == 0 ? d.Cin : d.Cout;
@@ -923,20 +961,24 @@ lpdt_status tc_pix(const lpdt_conv_desc &d, int mode, const int8_t *A, const flo
     if (smem < (two ? kMinSmemTwo : kMinSmem)) smem = two ? kMinSmemTwo : kMinSmem;
     if (smem > (two ? (size_t)113 * 1024 : (size_t)227 * 1024)) return LPDT_ERR_UNSUPPORTED;
     using Fn = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const PixParams);
-    static const Fn fns[2][2] = {{conv_pix_kernel<1, false>, conv_pix_kernel<1, true>},
-                                 {conv_pix_kernel<2, false>, conv_pix_kernel<2, true>}};
+    static const Fn fns[2][2][3] = {
+        {{conv_pix_kernel<1, false, 0>, conv_pix_kernel<1, false, 1>, conv_pix_kernel<1, false, 2>},
+         {conv_pix_kernel<1, true, 0>, conv_pix_kernel<1, true, 1>, conv_pix_kernel<1, true, 2>}},
+        {{conv_pix_kernel<2, false, 0>, conv_pix_kernel<2, false, 1>, conv_pix_kernel<2, false, 2>},
+         {conv_pix_kernel<2, true, 0>, conv_pix_kernel<2, true, 1>, conv_pix_kernel<2, true, 2>}}};
     // set when an instantiation is first used: the attribute loads its code
-    static PerDeviceOnce attr[2][2];
+    static PerDeviceOnce attr[2][2][3];
+    const int kind = aff ? 1 + mode : 0;
+    const Fn fn = fns[two][row][kind];
     int dev;
-    if (attr[two ? 1 : 0][row ? 1 : 0].pending(&dev)) {
-        LPDT_CUDA(cudaFuncSetAttribute(fns[two ? 1 : 0][row ? 1 : 0], cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (two ? 113 : 227) * 1024));
-        attr[two ? 1 : 0][row ? 1 : 0].mark(dev);
+    if (attr[two][row][kind].pending(&dev)) {
+        LPDT_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (two ? 113 : 227) * 1024));
+        attr[two][row][kind].mark(dev);
     }
     const int slots = two ? 2 * kNumSMs : kNumSMs;
     const int grid = (int)(tiles < slots ? tiles : slots);
     g_last_kernel = "lpdt::tc::conv_pix_kernel";
-    launch_k(fns[two ? 1 : 0][row ? 1 : 0], grid, kPixThreads, smem, st, mA, mW, mY, p);
+    launch_k(fn, grid, kPixThreads, smem, st, mA, mW, mY, p);
     LPDT_LAUNCH_CHECK();
     return LPDT_OK;
 }
