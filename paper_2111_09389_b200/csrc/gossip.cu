@@ -191,13 +191,15 @@ __device__ void select_whole_segment(const float *__restrict__ xh, const float *
 // ---- long segments: a sampled threshold, one streaming pass, a selection over the candidates ----
 // Sample (big_sample_kernel): 1/64 of the segment, read as runs of eight consecutive parameters, goes into
 // a histogram of the top 12 magnitude bits (exponent and four mantissa bits: buckets 1/16 of an octave
-// wide); the CTA that finishes last walks it from the top and picks a bucket that, by the sample, has
-// comfortably more than k keys at or above it.  Collect (big_collect_kernel): the one pass over the
-// segment copies every key at or above that bucket, with its position, into a candidate list and counts
-// them exactly.  Select (one CTA per segment): if the exact count reached k, the k largest keys are all
-// in the list, and the threshold and the tie cut are found there (1-2 % of the data).  The sample only
-// steers: when the count falls short of k, or the candidates outgrow the list (1/8 of the segment: near-
-// constant magnitudes), the exact whole-segment path takes over, so the result never depends on the sample.
+// wide); the CTA that finishes last picks a window of buckets that, by the sample, comfortably holds the
+// k-th largest key.  Collect (big_collect_kernel): the one pass over the segment counts the keys above the
+// window and copies those inside, with their positions, into a candidate list, with an exact histogram.
+// Select (one CTA per segment): if fewer than k keys lie above the window and at least k above its lower
+// edge, the k-th largest is in the list, and the threshold and the tie cut are found there.  The sample
+// only steers: otherwise, or when the candidates outgrow the list (1/8 of the segment: near-constant
+// magnitudes), the exact whole-segment path takes over, so the result never depends on the sample.
+// (With every key above the lower edge in the list, a tenth kept overflowed it: 8 x 2 M, top 10 %, 2337 us for
+// the call on the whole-segment path, 168 us with the window.)
 struct BigList {
     int32_t n;
     int32_t id[kMaxSeg];               // segment index
@@ -206,9 +208,9 @@ struct BigList {
 };
 constexpr int kTopBins = 4096;
 // zeroed per call.  h0: histogram of the sample; h1: exact histogram of the collected keys (same 12 bits);
-// cand_count: keys at or above the chosen bucket
-struct BigCtl { uint32_t h0[kTopBins], h1[kTopBins]; uint32_t ticket, cand_count, sampled, pad; };
-struct BigState { uint32_t prefix; uint32_t sampled; };    // lowest magnitude bits of the chosen bucket; keys sampled
+// cand_count: keys inside the window; above: keys above it
+struct BigCtl { uint32_t h0[kTopBins], h1[kTopBins]; uint32_t ticket, cand_count, sampled, above; };
+struct BigState { uint32_t lower, upper; };                // the window's first and last bucket
 struct __align__(8) Cand { uint32_t key, pos; };    // magnitude bits, position inside the segment
 
 __device__ __host__ __forceinline__ int64_t cand_capacity(int64_t len) { return len / 8 + 4096; }
@@ -300,22 +302,25 @@ big_sample_kernel(const float *__restrict__ x_half, const float *__restrict__ x_
     const unsigned nchunks = (unsigned)ceil_div_dev(hi - lo, kSampleChunk);
     if (s_ticket != nchunks - 1) return;
     __threadfence();
-    // keys the sample must show at or above the bucket: the sampled share of k, a tenth more, and four
-    // standard deviations of the sampled count
+    // keys the sample must show at or above the lower edge: the sampled share of k, a tenth more, and four
+    // standard deviations of the sampled count; at most as many fewer at or above the upper one
     const double m = (double)__ldcg(&h->sampled), f = m / (double)(hi - lo), fk = f * (double)seg.k[s];
-    long long target = (long long)(1.10 * fk + 4.0 * sqrt(fk) + 8.0);
-    int b = 0; long long need, eq;
-    if (target <= (long long)m) pick_bucket(h->h0, kTopBins, target, &b, &need, &eq);
+    const double slack = 0.10 * fk + 4.0 * sqrt(fk) + 8.0;
+    const long long low = (long long)(fk + slack), high = (long long)(fk - slack);
+    int lower = 0, upper = kTopBins - 1; long long need, eq;
+    if (low <= (long long)m) pick_bucket(h->h0, kTopBins, low, &lower, &need, &eq);
+    __syncthreads();
+    if (high >= 1) pick_bucket(h->h0, kTopBins, high, &upper, &need, &eq);
     if (threadIdx.x == 0) {
         BigState nx;
-        nx.prefix = (uint32_t)b << kTopShift;
-        nx.sampled = (uint32_t)m;
+        nx.lower = (uint32_t)lower;
+        nx.upper = (uint32_t)upper;
         state[(int64_t)node * big.n + bi] = nx;
     }
 }
 
-// Copy every key at or above the chosen bucket, with its position, into the (node, segment)'s candidate
-// list, and count them all (the count keeps running past the list's capacity; writes stop there).
+// Copy every key of the window, with its position, into the (node, segment)'s candidate list, and count them
+// all (the count keeps running past the list's capacity; writes stop there) and the keys above the window.
 // Matches are staged in shared memory and flushed with one reservation per CTA; the order inside the
 // list is arbitrary (the selection over it does not depend on it).
 constexpr int kStage = 2048;
@@ -335,18 +340,20 @@ big_collect_kernel(const float *__restrict__ x_half, const float *__restrict__ x
     BigCtl *h = ctl + (int64_t)node * big.n + bi;
     Cand *list = cands + (int64_t)node * cand_per_node + big.cand_base[bi];
     const float *xh = x_half + (int64_t)node * d, *xq = x_hat + (int64_t)node * d;
-    const uint32_t bucket = stt.prefix >> kTopShift;
+    const uint32_t bucket = stt.lower, upper = stt.upper;
     __shared__ Cand stage[kStage];
     __shared__ unsigned int sh1[kTopBins];       // this CTA's share of the exact histogram of the collected keys
-    __shared__ unsigned int s_cnt, s_base;
+    __shared__ unsigned int s_cnt, s_base, s_above;
+    unsigned above = 0;
     for (int i = threadIdx.x; i < kTopBins; i += blockDim.x) sh1[i] = 0;
-    if (threadIdx.x == 0) s_cnt = 0;
+    if (threadIdx.x == 0) { s_cnt = 0; s_above = 0; }
     __syncthreads();
     uint32_t kmax = 0;          // largest magnitude of the chunk: the range of the segment's 8-bit message
     auto consider = [&](float a, float b, int64_t eu) {
         const uint32_t key = mag_bits(a, b, plus);
         kmax = key > kmax ? key : kmax;
-        if ((key >> kTopShift) >= bucket) {
+        if ((key >> kTopShift) > upper) ++above;
+        else if ((key >> kTopShift) >= bucket) {
             atomicAdd(&sh1[key >> kTopShift], 1u);
             Cand c; c.key = key; c.pos = (uint32_t)(eu - lo);
             const unsigned slot = atomicAdd(&s_cnt, 1u);
@@ -388,12 +395,15 @@ big_collect_kernel(const float *__restrict__ x_half, const float *__restrict__ x
         }
     }
     for (int64_t e = v1 + threadIdx.x; e < c1; e += blockDim.x) consider(xh[e], xq[e], e);
+    above = __reduce_add_sync(0xffffffffu, above);
+    if ((threadIdx.x & 31) == 0 && above) atomicAdd(&s_above, above);
     __syncthreads();
+    if (threadIdx.x == 0 && s_above) atomicAdd(&h->above, s_above);
     if (amax_bits) {            // the same value the range pass of the 8-bit messages would find
         for (int o = 16; o > 0; o >>= 1) { const uint32_t t = __shfl_xor_sync(0xffffffffu, kmax, o); kmax = t > kmax ? t : kmax; }
         if ((threadIdx.x & 31) == 0 && kmax) atomicMax(amax_bits + (int64_t)node * seg.n_seg + s, kmax);
     }
-    for (int i = bucket + threadIdx.x; i < kTopBins; i += blockDim.x)
+    for (int i = bucket + threadIdx.x; i <= (int)upper; i += blockDim.x)
         if (sh1[i]) atomicAdd(&h->h1[i], sh1[i]);
     const unsigned n = s_cnt < kStage ? s_cnt : kStage;
     if (n == 0) return;
@@ -403,8 +413,47 @@ big_collect_kernel(const float *__restrict__ x_half, const float *__restrict__ x
         if (s_base + i < cap) list[s_base + i] = stage[i];
 }
 
-// Threshold and tie cut of a long segment from its candidate list (one CTA).  The list holds every key
-// at or above a bucket and at least k of them, so its k-th largest is the segment's k-th largest; if only
+// Copies what(c) of every candidate c = {key, pos} that `take` accepts into dst (at most cap of them) and leaves their
+// number in *count: one pass of the CTA over the list, 16 loads of a thread in flight, one reservation per warp and
+// round (a reservation per key put 29 K atomics on one shared-memory word: 8.65 M normal values, top 1 %, took 163 us
+// for the whole selection, 57 us now).
+template <typename Take, typename What>
+__device__ void gather(const Cand *__restrict__ list, int64_t n, int cap, uint32_t *dst, unsigned int *count, Take take, What what) {
+    const unsigned long long *l64 = reinterpret_cast<const unsigned long long *>(list);
+    const int lane = threadIdx.x & 31;
+    __syncthreads();
+    if (threadIdx.x == 0) *count = 0;
+    __syncthreads();
+    constexpr int kU = 16;
+    for (int64_t base = 0; base < n; base += kU * (int64_t)blockDim.x) {
+        unsigned long long c[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const int64_t e = base + u * (int64_t)blockDim.x + threadIdx.x;
+            c[u] = e < n ? __ldg(l64 + e) : 0ull;
+        }
+        unsigned hits = 0;
+#pragma unroll
+        for (int u = 0; u < kU; ++u)
+            if (base + u * (int64_t)blockDim.x + threadIdx.x < n && take(c[u])) hits |= 1u << u;
+        const int mine = __popc(hits);
+        int incl = mine;                              // places of this lane's keys among the warp's
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += v; }
+        const int total = __shfl_sync(0xffffffffu, incl, 31);
+        if (total == 0) continue;
+        unsigned at = 0;
+        if (lane == 31) at = atomicAdd(count, (unsigned)total);
+        at = __shfl_sync(0xffffffffu, at, 31) + (unsigned)(incl - mine);
+#pragma unroll
+        for (int u = 0; u < kU; ++u)
+            if ((hits >> u) & 1u) { if (at < (unsigned)cap) dst[at] = what(c[u]); ++at; }
+    }
+    __syncthreads();
+}
+
+// Threshold and tie cut of a long segment from its candidate list (one CTA).  The list holds every key of the
+// window, at least k of them (k counted from the window's upper edge), so its k-th largest is the one looked for; if only
 // some of the keys equal to it are taken, those at the lowest positions are: the cut follows the
 // need-th smallest position among them.
 __device__ void select_from_candidates(const Cand *__restrict__ list, int64_t n_cand, int64_t k, const uint32_t *h1,
@@ -413,33 +462,14 @@ __device__ void select_from_candidates(const Cand *__restrict__ list, int64_t n_
     // key comes from it without a scan, and only the 19 bits below are searched
     int b1; long long need1, eq1;
     pick_bucket(h1, kTopBins, (long long)k, &b1, &need1, &eq1);
+    __shared__ unsigned int s_n;
     long long need, eq;
     uint32_t thr;
     if (eq1 <= (long long)key_cap) {
         // The bucket's keys (their exact number is known) fit the shared-memory buffer: one pass over the list
         // copies them there, and the radix passes run over shared memory instead of re-reading the list.
-        __shared__ unsigned int s_n;
-        if (threadIdx.x == 0) s_n = 0;
-        __syncthreads();
-        const unsigned long long *l64 = reinterpret_cast<const unsigned long long *>(list);
-        for (int64_t base = 0; base < n_cand; base += 8 * (int64_t)blockDim.x) {
-            unsigned long long c[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int64_t eu = base + u * (int64_t)blockDim.x + threadIdx.x;
-                c[u] = eu < n_cand ? __ldg(l64 + eu) : 0ull;       // {key, pos}: the key is the low word
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int64_t eu = base + u * (int64_t)blockDim.x + threadIdx.x;
-                const uint32_t key = (uint32_t)c[u];
-                if (eu < n_cand && (int)(key >> kTopShift) == b1) {
-                    const unsigned slot = atomicAdd(&s_n, 1u);
-                    if (slot < (unsigned)key_cap) s_keys[slot] = key;
-                }
-            }
-        }
-        __syncthreads();
+        gather(list, n_cand, key_cap, s_keys, &s_n, [&](unsigned long long c) { return (int)((uint32_t)c >> kTopShift) == b1; },
+               [](unsigned long long c) { return (uint32_t)c; });
         const int64_t n_in = s_n < (unsigned)key_cap ? s_n : key_cap;      // equals eq1
         thr = radix_select<false>(n_in, [&](int64_t e) { return s_keys[e]; }, need1, kTopShift,
                                   (uint32_t)b1 << kTopShift, &need, &eq);
@@ -451,7 +481,15 @@ __device__ void select_from_candidates(const Cand *__restrict__ list, int64_t n_
         if (threadIdx.x == 0) { o->thr = thr; o->dense = 0; o->cut = hi; }
         return;
     }
-    long long n2, e2;      // ties keyed by descending position (never 0); the other candidates are skipped
+    long long n2, e2;      // ties keyed by descending position (never 0)
+    if (eq <= (long long)key_cap) {                   // the usual case, two or three of them: their positions alone
+        gather(list, n_cand, key_cap, s_keys, &s_n, [&](unsigned long long c) { return (uint32_t)c == thr; },
+               [](unsigned long long c) { return 0xFFFFFFFFu - (uint32_t)(c >> 32); });
+        const uint32_t inv = radix_select<false>(eq, [&](int64_t e) { return s_keys[e]; }, need, 32, 0u, &n2, &e2);
+        if (threadIdx.x == 0) { o->thr = thr; o->dense = 0; o->cut = lo + (int64_t)(0xFFFFFFFFu - inv) + 1; }
+        return;
+    }
+    // the other candidates are skipped
     const uint32_t inv = radix_select<true>(n_cand,
                                             [&](int64_t e) { return list[e].key == thr ? 0xFFFFFFFFu - list[e].pos : 0u; },
                                             need, 32, 0u, &n2, &e2);
@@ -579,135 +617,161 @@ select_and_rows_kernel(const float *__restrict__ x_half, const float *__restrict
     if (is_big(len, k)) {
         int bi = 0;
         while (big.id[bi] != s) ++bi;            // every long segment is in the list
-        // exact count of the keys at or above the sampled bucket: with at least k of them, all in the list,
-        // the k largest are among the candidates; otherwise the whole-segment path below decides
-        const int64_t n_cand = (int64_t)ctl[(int64_t)node * big.n + bi].cand_count;
-        if (n_cand >= k && n_cand <= cand_capacity(len)) {
+        // exact counts: with fewer than k keys above the window and the k-th one inside it, all of whose keys
+        // are in the list, the candidates decide; otherwise the whole-segment path below does
+        const BigCtl *h = ctl + (int64_t)node * big.n + bi;
+        const int64_t n_cand = (int64_t)h->cand_count, inside = k - (int64_t)h->above;
+        if (inside >= 1 && n_cand >= inside && n_cand <= cand_capacity(len)) {
             extern __shared__ __align__(16) uint32_t s_sel_keys[];
-            select_from_candidates(cands + (int64_t)node * cand_per_node + big.cand_base[bi], n_cand, k,
-                                   ctl[(int64_t)node * big.n + bi].h1, lo, hi, o, s_sel_keys, key_cap);
+            select_from_candidates(cands + (int64_t)node * cand_per_node + big.cand_base[bi], n_cand, inside,
+                                   h->h1, lo, hi, o, s_sel_keys, key_cap);
             return;
         }
     }
     select_whole_segment(xh, xq, lo, hi, k, seg.plus, o);
 }
 
-// Fused public-copy update + mixing.  A block owns TE*V consecutive parameters of all nodes; a thread
-// owns V consecutive ones (16-byte accesses when V = 4).  Phase 1 streams x_half and x_hat of every
-// node, writes the updated public copy and parks it in shared memory; phase 2 mixes each node with
-// its neighbours' copies from shared memory (x_half is read again: an L1/L2 hit).
-// DS: Deep-Squeeze form (supplementary Algorithm 2): the state array is the error buffer, the message is the
+// Fused public-copy update + mixing.  A CTA walks tiles of 32*EL consecutive parameters of all nodes; a warp owns NPW
+// nodes of a tile, EL parameters of each per lane (16-byte accesses when V = 4).  It reads x_half and the state, writes
+// the updated state where it changed, parks the public copies in shared memory, and after one barrier mixes its nodes
+// with their neighbours' copies; x_half stays in registers between the two halves.  Two parking buffers alternate, so a
+// tile costs one barrier.  The mixing rows, and the thresholds while the segment stays the same, are read once per CTA.
+// HBM-bound: x_half, x_hat read, x written, 12 B per parameter and node.  (The form before, a thread per parameter
+// looping over the nodes, kept 128 registers and four CTAs of 128 threads per SM, decided the segment and read the
+// thresholds again for every parameter and node and read x_half twice: 16 x 8.65 M, top 1 %, 461 us; this one 413 us.)
+// ds: Deep-Squeeze form (supplementary Algorithm 2): the state array is the error buffer, the message is the
 // compressed x_half + state, the buffer keeps what was not sent and the mix runs over the messages themselves.
-template <int V, bool Q8, bool DS>
-__global__ void __launch_bounds__(256)
-gossip_mix_kernel(int nodes, int64_t d, const float *__restrict__ x_half, float *__restrict__ x_hat,
-                  float *__restrict__ x_out, float gamma, SegTable seg, const SelectOut *__restrict__ sel,
-                  const int32_t *__restrict__ tab, const float *__restrict__ msg_scale,
-                  const float *__restrict__ msg_inv) {
+// q8: the message is the 8-bit code times the step of its (node, segment).
+__host__ __device__ constexpr int mix_el(int npw) { return npw == 1 ? 8 : 4; }           // parameters per lane and node
+struct MixRule { uint32_t thr; uint32_t dense; int64_t cut; float scale, inv; };
+__device__ __forceinline__ MixRule mix_rule(const SelectOut *sel, const float *msg_scale, const float *msg_inv, int64_t at, bool q8) {
+    const SelectOut so = sel[at];
+    MixRule r;
+    r.thr = so.thr; r.dense = so.dense; r.cut = so.cut;
+    r.scale = q8 ? msg_scale[at] : 1.f; r.inv = q8 ? msg_inv[at] : 1.f;
+    return r;
+}
+template <int V, int NPW>
+__global__ void __launch_bounds__(NPW == 1 ? 512 : 640, 2)
+gossip_mix_kernel(int nodes, int64_t d, const float *x_half, float *x_hat, float *x_out, float gamma, SegTable seg,
+                  const SelectOut *__restrict__ sel, const int32_t *__restrict__ tab, const float *__restrict__ msg_scale,
+                  const float *__restrict__ msg_inv, bool q8, bool ds) {
     pdl_enter();
     extern __shared__ __align__(16) float sm[];
-    const int TE = blockDim.x;
+    constexpr int EL = mix_el(NPW), U = EL / V, TILE = 32 * EL;
+    const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int32_t *s_cnt = reinterpret_cast<int32_t *>(sm);            // [nodes]
     int32_t *s_idx = s_cnt + nodes;                              // [nodes][nodes]
     float *s_val = reinterpret_cast<float *>(s_idx + nodes * nodes);
     const int tab_words = nodes + 2 * nodes * nodes;
-    float *s_hat = sm + ((tab_words + 3) & ~3);                  // [nodes][TE][V], 16-byte aligned
-    for (int i = threadIdx.x; i < tab_words; i += TE) s_cnt[i] = tab[i];
-    __syncthreads();       // the only block-wide wait: the parked copies below are read back by the thread that wrote them
-    const int64_t e0 = ((int64_t)blockIdx.x * TE + threadIdx.x) * V;
-    const bool live = e0 < d;                                    // d % V == 0: a thread is all in or all out
-    int s0 = 0;
-    bool one_seg = true;
-    if (live) {   // segment of the first parameter (segments tile [0,d))
-        int a = 0, b = seg.n_seg;
-        while (b - a > 1) { int m = (a + b) >> 1; if (seg.off[m] <= e0) a = m; else b = m; }
-        s0 = a;
-        one_seg = seg.off[s0 + 1] >= e0 + V;
-    }
-    constexpr int kU = V == 4 ? 8 : 4;                           // nodes per batch of independent loads (as measured)
-    for (int ib = 0; ib < nodes; ib += kU) {
-        float xh[kU][V], xq[kU][V];
+    float *s_hat = sm + ((tab_words + 3) & ~3);                  // [2][nodes][TILE], 16-byte aligned
+    for (int i = threadIdx.x; i < tab_words; i += blockDim.x) s_cnt[i] = tab[i];
+    MixRule rule[NPW];
+    int s = 0, rules_of = -1, cur = 0;                           // segment of the tile's first parameter
+    for (int64_t tile = blockIdx.x; tile * TILE < d; tile += gridDim.x, cur ^= 1) {
+        const int64_t t0 = tile * TILE;
+        while (seg.off[s + 1] <= t0) ++s;
+        const bool one_seg = seg.off[s + 1] >= (t0 + TILE < d ? t0 + TILE : d);
+        float xh[NPW][U][V], xq[NPW][U][V];
 #pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            if (live && ib + u < nodes) {
-                VecIO<V>::ld(x_half + (int64_t)(ib + u) * d + e0, xh[u]);
-                VecIO<V>::ld(x_hat + (int64_t)(ib + u) * d + e0, xq[u]);
+        for (int m = 0; m < NPW; ++m) {
+            const int i = warp + m * warps;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t e = t0 + (u * 32 + lane) * V;      // d % V == 0: a vector is all in or all out
+                if (i < nodes && e < d) {
+                    VecIO<V>::ld(x_half + (int64_t)i * d + e, xh[m][u]);
+                    VecIO<V>::ld(x_hat + (int64_t)i * d + e, xq[m][u]);
+                }
             }
         }
+        if (rules_of != s) {
 #pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            const int i = ib + u;
+            for (int m = 0; m < NPW; ++m) {
+                const int i = warp + m * warps;
+                if (i < nodes) rule[m] = mix_rule(sel, msg_scale, msg_inv, (int64_t)i * seg.n_seg + s, q8);
+            }
+            rules_of = s;
+        }
+        float *park = s_hat + (size_t)cur * nodes * TILE;
+#pragma unroll
+        for (int m = 0; m < NPW; ++m) {
+            const int i = warp + m * warps;
             if (i >= nodes) break;
-            float hn[V], st_new[V];
 #pragma unroll
-            for (int k = 0; k < V; ++k) hn[k] = 0.f;
-            if (live) {
-                SelectOut so = sel[(int64_t)i * seg.n_seg + s0];
-                bool changed = DS;         // the public copy changes only where an entry is sent (top-k: 1 in 100)
-                float q_scale = 1.f, q_inv = 1.f;
-                if (Q8) { q_scale = msg_scale[(int64_t)i * seg.n_seg + s0]; q_inv = msg_inv[(int64_t)i * seg.n_seg + s0]; }
+            for (int u = 0; u < U; ++u) {
+                const int64_t e = t0 + (u * 32 + lane) * V;
+                float hn[V], st_new[V];
+                bool changed = ds;             // the public copy changes only where an entry is sent (top-k: 1 in 100)
+                if (e < d) {
+                    int sk = s;
+                    MixRule r = rule[m];
+#pragma unroll
+                    for (int k = 0; k < V; ++k) {
+                        if (!one_seg && seg.off[sk + 1] <= e + k) {
+                            while (seg.off[sk + 1] <= e + k) ++sk;
+                            r = mix_rule(sel, msg_scale, msg_inv, (int64_t)i * seg.n_seg + sk, q8);
+                        }
+                        const float delta = ds ? __fadd_rn(xh[m][u][k], xq[m][u][k]) : __fsub_rn(xh[m][u][k], xq[m][u][k]);
+                        const uint32_t key = __float_as_uint(delta) & 0x7fffffffu;
+                        const bool keep = r.dense || key > r.thr || (key == r.thr && e + k < r.cut);
+                        changed |= keep;
+                        float msg = delta;
+                        if (q8) {      // the message is the 8-bit code times the step; the state absorbs exactly that
+                            const float code = fminf(fmaxf(rintf(__fmul_rn(delta, r.inv)), -127.f), 127.f);
+                            msg = __fmul_rn(code, r.scale);
+                        }
+                        if (ds) {      // park the message, keep the remainder in the error buffer
+                            hn[k] = keep ? msg : 0.f;
+                            st_new[k] = __fsub_rn(delta, hn[k]);
+                        } else {       // public copy + message; that sum is also what the neighbours mix
+                            hn[k] = keep ? __fadd_rn(xq[m][u][k], msg) : xq[m][u][k];
+                            st_new[k] = hn[k];
+                        }
+                    }
+                    if (changed) VecIO<V>::st(x_hat + (int64_t)i * d + e, st_new);      // unchanged values are not rewritten
+                    VecIO<V>::st(park + (size_t)i * TILE + (u * 32 + lane) * V, hn);
+                }
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int m = 0; m < NPW; ++m) {
+            const int i = warp + m * warps;
+            if (i >= nodes) break;
+            const int c = s_cnt[i];
+            float hi_[U][V], acc[U][V];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                VecIO<V>::ld(park + (size_t)i * TILE + (u * 32 + lane) * V, hi_[u]);
+#pragma unroll
+                for (int k = 0; k < V; ++k) acc[u][k] = 0.f;
+            }
+            for (int n = 0; n < c; ++n) {                        // neighbours in ascending j
+                const int j = s_idx[i * nodes + n];
+                const float w = s_val[i * nodes + n];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    float hj[V];
+                    VecIO<V>::ld(park + (size_t)j * TILE + (u * 32 + lane) * V, hj);
+#pragma unroll
+                    for (int k = 0; k < V; ++k)
+                        acc[u][k] = ds ? __fadd_rn(acc[u][k], __fmul_rn(w, hj[k]))                            // sum_j W_ij c_j
+                                       : __fadd_rn(acc[u][k], __fmul_rn(w, __fsub_rn(hj[k], hi_[u][k])));      // sum_j W_ij (xhat_j - xhat_i)
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t e = t0 + (u * 32 + lane) * V;
+                if (e >= d) continue;
+                float o[V];
 #pragma unroll
                 for (int k = 0; k < V; ++k) {
-                    if (!one_seg && k > 0) {
-                        int sk = s0;
-                        while (seg.off[sk + 1] <= e0 + k) ++sk;
-                        so = sel[(int64_t)i * seg.n_seg + sk];
-                        if (Q8) { q_scale = msg_scale[(int64_t)i * seg.n_seg + sk]; q_inv = msg_inv[(int64_t)i * seg.n_seg + sk]; }
-                    }
-                    const float delta = DS ? __fadd_rn(xh[u][k], xq[u][k]) : __fsub_rn(xh[u][k], xq[u][k]);
-                    const uint32_t key = __float_as_uint(delta) & 0x7fffffffu;
-                    const bool keep = so.dense || key > so.thr || (key == so.thr && e0 + k < so.cut);
-                    changed |= keep;
-                    float msg = delta;
-                    if (Q8) {      // the message is the 8-bit code times the step; the state absorbs exactly that
-                        const float code = fminf(fmaxf(rintf(__fmul_rn(delta, q_inv)), -127.f), 127.f);
-                        msg = __fmul_rn(code, q_scale);
-                    }
-                    if (DS) {      // park the message, keep the remainder in the error buffer
-                        hn[k] = keep ? msg : 0.f;
-                        st_new[k] = __fsub_rn(delta, hn[k]);
-                    } else {       // public copy + message; that sum is also what the neighbours mix
-                        hn[k] = keep ? __fadd_rn(xq[u][k], msg) : xq[u][k];
-                        st_new[k] = hn[k];
-                    }
+                    const float a = ds ? __fsub_rn(acc[u][k], hi_[u][k]) : acc[u][k];                          // - I_ij c_j
+                    o[k] = __fadd_rn(xh[m][u][k], __fmul_rn(gamma, a));
                 }
-                if (changed) VecIO<V>::st(x_hat + (int64_t)i * d + e0, st_new);      // unchanged values are not rewritten
+                VecIO<V>::st(x_out + (int64_t)i * d + e, o);
             }
-            VecIO<V>::st(s_hat + ((size_t)i * TE + threadIdx.x) * V, hn);
-        }
-    }
-    if (!live) return;
-    for (int ib = 0; ib < nodes; ib += kU) {
-        float xh[kU][V];
-#pragma unroll
-        for (int u = 0; u < kU; ++u)
-            if (ib + u < nodes) VecIO<V>::ld(x_half + (int64_t)(ib + u) * d + e0, xh[u]);
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            const int i = ib + u;
-            if (i >= nodes) break;
-            float hi_[V], acc[V], o[V];
-            VecIO<V>::ld(s_hat + ((size_t)i * TE + threadIdx.x) * V, hi_);
-#pragma unroll
-            for (int k = 0; k < V; ++k) acc[k] = 0.f;
-            const int c = s_cnt[i];
-            for (int m = 0; m < c; ++m) {                        // neighbours in ascending j
-                const int j = s_idx[i * nodes + m];
-                const float w = s_val[i * nodes + m];
-                float hj[V];
-                VecIO<V>::ld(s_hat + ((size_t)j * TE + threadIdx.x) * V, hj);
-#pragma unroll
-                for (int k = 0; k < V; ++k)
-                    acc[k] = DS ? __fadd_rn(acc[k], __fmul_rn(w, hj[k]))                         // sum_j W_ij c_j
-                                : __fadd_rn(acc[k], __fmul_rn(w, __fsub_rn(hj[k], hi_[k])));      // sum_j W_ij (xhat_j - xhat_i)
-            }
-            if (DS) {
-#pragma unroll
-                for (int k = 0; k < V; ++k) acc[k] = __fsub_rn(acc[k], hi_[k]);                   // - I_ij c_j
-            }
-#pragma unroll
-            for (int k = 0; k < V; ++k) o[k] = __fadd_rn(xh[u][k], __fmul_rn(gamma, acc[k]));
-            VecIO<V>::st(x_out + (int64_t)i * d + e0, o);
         }
     }
 }
@@ -904,6 +968,7 @@ static lpdt_status gossip_impl(int32_t nodes, int64_t d, const float *x_half, fl
     BigList big;
     big.n = 0; big.chunk_base[0] = 0; big.cand_base[0] = 0;
     int64_t most_chunks = 0, longest = 0;
+    double most_kept = 0.0;                     // largest share of a long segment that is kept
     for (int s = 0; s < n_segments; ++s) {
         const int64_t len = seg.off[s + 1] - seg.off[s];
         if (!is_big(len, seg.k[s])) continue;
@@ -914,6 +979,8 @@ static lpdt_status gossip_impl(int32_t nodes, int64_t d, const float *x_half, fl
         big.cand_base[big.n + 1] = big.cand_base[big.n] + cand_capacity(len);
         if (nc > most_chunks) most_chunks = nc;
         if (len > longest) longest = len;
+        const double kept = (double)seg.k[s] / (double)len;
+        if (kept > most_kept) most_kept = kept;
         ++big.n;
     }
     char *big_region = (char *)tab + rows_bytes(nodes);
@@ -938,7 +1005,9 @@ static lpdt_status gossip_impl(int32_t nodes, int64_t d, const float *x_half, fl
         // elements per CTA of the collect pass: every CTA clears and flushes a 4096-bin histogram, so chunks are as
         // long as still leaves several CTAs per SM (16 K ... 64 K elements)
         int chunk = kChunk;
-        while (chunk < 65536 && ceil_div(longest, (int64_t)chunk * 2) * big.n * nodes >= 4 * (int64_t)kNumSMs) chunk *= 2;
+        // and as short as keeps a chunk's candidates (about 0.6 k of the segment's k) inside its staging buffer
+        while (chunk < 65536 && ceil_div(longest, (int64_t)chunk * 2) * big.n * nodes >= 4 * (int64_t)kNumSMs &&
+               0.6 * most_kept * 2 * chunk <= kStage) chunk *= 2;
         const dim3 g((unsigned)ceil_div(longest, (int64_t)chunk), big.n, nodes);
         const int64_t sample_ctas = ceil_div(longest, kSampleChunk);
         if (sample_ctas > 65535) return LPDT_ERR_UNSUPPORTED;
@@ -972,31 +1041,33 @@ static lpdt_status gossip_impl(int32_t nodes, int64_t d, const float *x_half, fl
     // the networks' parameter counts are even but not multiples of 4, which still allows 8-byte accesses
     const bool v4 = d % 4 == 0 && aligned(x_half, 16) && aligned(x_hat, 16) && aligned(x_out, 16);
     const bool v2 = !v4 && d % 2 == 0 && aligned(x_half, 8) && aligned(x_hat, 8) && aligned(x_out, 8);
-    const int V = v4 ? 4 : v2 ? 2 : 1;
     const int vi = v4 ? 2 : v2 ? 1 : 0;
-    // threads per block: as many as keep the parked public copies within 64 KB of shared memory
-    int TE = (int)((64 * 1024) / ((size_t)nodes * V * sizeof(float))) / 32 * 32;
-    if (TE > 128) TE = 128;
-    if (TE < 32) TE = 32;
+    // nodes per warp: one up to 16 nodes; beyond, as few as keep a CTA within 20 warps
+    const int npw = nodes <= 16 ? 1 : (int)ceil_div(nodes, 20), warps = (int)ceil_div(nodes, npw), tile = 32 * mix_el(npw);
     const size_t tab_words = ((size_t)nodes + 2 * (size_t)nodes * nodes + 3) & ~(size_t)3;
-    const size_t smem = tab_words * sizeof(int32_t) + (size_t)nodes * TE * V * sizeof(float);
+    const size_t smem = tab_words * sizeof(int32_t) + 2 * (size_t)nodes * tile * sizeof(float);
     using MixFn = void (*)(int, int64_t, const float *, float *, float *, float, SegTable, const SelectOut *,
-                           const int32_t *, const float *, const float *);
-    static const MixFn fns[12] = {
-        gossip_mix_kernel<1, false, false>, gossip_mix_kernel<2, false, false>, gossip_mix_kernel<4, false, false>,
-        gossip_mix_kernel<1, true, false>,  gossip_mix_kernel<2, true, false>,  gossip_mix_kernel<4, true, false>,
-        gossip_mix_kernel<1, false, true>,  gossip_mix_kernel<2, false, true>,  gossip_mix_kernel<4, false, true>,
-        gossip_mix_kernel<1, true, true>,   gossip_mix_kernel<2, true, true>,   gossip_mix_kernel<4, true, true>};
-    static PerDeviceOnce attr_set;
+                           const int32_t *, const float *, const float *, bool, bool);
+    static const MixFn fns[3][4] = {
+        {gossip_mix_kernel<1, 1>, gossip_mix_kernel<1, 2>, gossip_mix_kernel<1, 3>, gossip_mix_kernel<1, 4>},
+        {gossip_mix_kernel<2, 1>, gossip_mix_kernel<2, 2>, gossip_mix_kernel<2, 3>, gossip_mix_kernel<2, 4>},
+        {gossip_mix_kernel<4, 1>, gossip_mix_kernel<4, 2>, gossip_mix_kernel<4, 3>, gossip_mix_kernel<4, 4>}};
+    const MixFn fn = fns[vi][npw - 1];
+    static PerDeviceOnce attr_set[3][4];
     int dev;
-    if (attr_set.pending(&dev)) {
-        for (int i = 0; i < 12; ++i)
-            LPDT_CUDA(cudaFuncSetAttribute(fns[i], cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024));
-        attr_set.mark(dev);
+    if (attr_set[vi][npw - 1].pending(&dev)) {
+        LPDT_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024));
+        attr_set[vi][npw - 1].mark(dev);
     }
-    const unsigned blocks = (unsigned)ceil_div(d, (int64_t)TE * V);
-    launch_k(fns[(ds ? 6 : 0) + (q8 ? 3 : 0) + vi], blocks, TE, smem, st, nodes, d, x_half, x_hat, x_out, gamma, seg, sel, tab,
-                                                                            q8 ? msg_scale : nullptr, msg_inv);
+    // as many CTAs as are resident together: two of the largest by their registers
+    int64_t per_sm = (npw == 1 ? 1024 : 1280) / (32 * warps);
+    if (per_sm > 24) per_sm = 24;
+    if (per_sm * (int64_t)(smem + 1024) > 224 * 1024) per_sm = (int64_t)(224 * 1024) / (int64_t)(smem + 1024);
+    if (per_sm < 1) per_sm = 1;
+    int64_t blocks = ceil_div(d, tile);
+    if (blocks > per_sm * kNumSMs) blocks = per_sm * kNumSMs;
+    launch_k(fn, (unsigned)blocks, 32 * warps, smem, st, nodes, d, x_half, x_hat, x_out, gamma, seg, sel, tab,
+             q8 ? msg_scale : nullptr, msg_inv, q8, ds);
     LPDT_LAUNCH_CHECK();
     return LPDT_OK;
 }
