@@ -563,6 +563,24 @@ lpdt_status lpdt_softmax_ce(int32_t nodes, int32_t B, int32_t K, const float *lo
 lpdt_status lpdt_colsum(int32_t nodes, int32_t B, int32_t C, const float *x,
                         float *out, int64_t out_node_stride, void *stream);
 
+/* -------------------------------------------------------------------------
+ * lpdt_run_calls - issue a recorded sequence of the calls above in one call.
+ * code    : n_words 64-bit words, item after item.  A call: lpdt_call_id of its entry
+ *           point, the index of its stream, then its arguments without the stream, a
+ *           word each (pointers and integers as values, a float as its 32 bits).
+ *           A wait: LPDT_CALL_WAIT, index of the waiting stream, index of the stream
+ *           it waits for, an event (cudaEvent_t) that the sequence may re-record.
+ * streams : n_streams stream handles that the indices refer to.
+ * failed  : (nullable) the item that was last begun; after an error, the one that failed.
+ * Every call does what it does by itself, checks included; the first error ends the
+ * sequence and is returned.  Host arrays among the arguments are read during the call.
+ * lpdt_call_id returns -1 for a name that sequences do not take.
+ */
+#define LPDT_CALL_WAIT 1000
+int32_t lpdt_call_id(const char *name);
+lpdt_status lpdt_run_calls(const uint64_t *code, int64_t n_words, void *const *streams, int32_t n_streams,
+                           int64_t *failed);
+
 #ifdef __cplusplus
 }
 #endif

@@ -80,6 +80,8 @@ SIGNATURES = {
     "lpdt_maxpool2x2_bwd": (_i32, [_i32] * 5 + [_vp] * 4),
     "lpdt_softmax_ce": (_i32, [_i32] * 3 + [_vp] * 6),
     "lpdt_colsum": (_i32, [_i32] * 3 + [_vp, _vp, _i64, _vp]),
+    "lpdt_call_id": (_i32, [C.c_char_p]),
+    "lpdt_run_calls": (_i32, [_vp, _i64, _vp, _i32, _vp]),
 }
 
 

@@ -4,15 +4,30 @@ Every function has the name of the C entry point it calls (include/lpdt.h),
 takes torch CUDA tensors as device memory, and launches on torch's current
 stream.  No arithmetic happens here.
 """
+import contextlib
 import ctypes as C
+import threading
 
 import torch
 
-from ._lib import ConvDesc, lib
+from ._lib import SIGNATURES, ConvDesc
+from ._lib import lib as _load
 
 
 # Entry points that enqueue kernels (wrapped for the optional call log and per-call timing).
 LAUNCHING = {"lpdt_quantize", "lpdt_quantize_with_range", "lpdt_quantize_static", "lpdt_quantize_batch", "lpdt_dequantize", "lpdt_qconv_fwd", "lpdt_qconv_fwd_affine", "lpdt_qconv_bwd_data_affine", "lpdt_qconv_bwd_weight_affine", "lpdt_qconv_bwd_data", "lpdt_qconv_bwd_weight", "lpdt_range_evonorm_fwd", "lpdt_range_evonorm_bwd", "lpdt_range_evonorm_fwd_q8", "lpdt_range_evonorm_bwd_q8", "lpdt_range_evonorm_bwd_params", "lpdt_range_evonorm_bwd_params_batch", "lpdt_dequantize_acc_batch", "lpdt_gossip_mix", "lpdt_gossip_mix_q8", "lpdt_deepsqueeze_mix", "lpdt_pushsum_debias", "lpdt_sgd_gossip_mix", "lpdt_evonorm_s0_fwd", "lpdt_evonorm_s0_bwd", "lpdt_range_bn_fwd", "lpdt_range_bn_bwd", "lpdt_sgd_update", "lpdt_residual_add", "lpdt_residual_add_bwd", "lpdt_avgpool", "lpdt_avgpool_bwd", "lpdt_maxpool2x2", "lpdt_maxpool2x2_bwd", "lpdt_softmax_ce", "lpdt_colsum", "lpdt_selftest_bounded_wait"}
+# A thread that records (see Calls) gets a library whose launching entry points note their arguments as they run.
+class _Recording(threading.local):
+    calls = None
+
+
+_recording = _Recording()
+
+
+def lib():
+    return _recording.calls or _load()
+
+
 # Kernel launches are counted inside the library (lpdt_launch_count); replays of a captured CUDA graph launch
 # the recorded kernels again without passing through the library, so TrainStep.replay adds them here.
 _REPLAYED = 0
@@ -78,6 +93,13 @@ def _stream():
     return torch.cuda.current_stream().cuda_stream
 
 
+def _host(a):
+    """Address of a host array for the duration of the call (a recording keeps the array for its replays)."""
+    if _recording.calls is not None:
+        _recording.calls.keep.append(a)
+    return C.addressof(a)
+
+
 def _ws(ws):
     return (_ptr(ws), 0 if ws is None else ws.numel() * ws.element_size())
 
@@ -131,7 +153,7 @@ def lpdt_message_bytes(d, seg_offsets, seg_k, value_bits=32, index_bits=32):
     ns = len(seg_k)
     so = (C.c_int64 * (ns + 1))(*[int(v) for v in seg_offsets])
     sk = (C.c_int64 * ns)(*[int(v) for v in seg_k])
-    return int(lib().lpdt_message_bytes(int(d), ns, C.addressof(so), C.addressof(sk), value_bits, index_bits))
+    return int(lib().lpdt_message_bytes(int(d), ns, _host(so), _host(sk), value_bits, index_bits))
 
 
 def lpdt_quantize_batch_workspace_size(nodes, n_tensors):
@@ -145,8 +167,8 @@ def lpdt_quantize_batch(params, nodes, row_stride, src_offsets, sizes, dst_offse
     sz = (C.c_int64 * n)(*[int(v) for v in sizes])
     do = (C.c_int64 * n)(*[int(v) for v in dst_offsets])
     p, nb = _ws(ws)
-    _check("lpdt_quantize_batch", lib().lpdt_quantize_batch(_ptr(params), nodes, row_stride, n, C.addressof(so),
-                                                            C.addressof(sz), C.addressof(do), _ptr(q), _ptr(scales),
+    _check("lpdt_quantize_batch", lib().lpdt_quantize_batch(_ptr(params), nodes, row_stride, n, _host(so),
+                                                            _host(sz), _host(do), _ptr(q), _ptr(scales),
                                                             p, nb, _stream()))
 
 
@@ -335,7 +357,7 @@ def lpdt_range_evonorm_bwd_params_batch(nodes, B, channels, workspaces, grad_off
     wp = (C.c_void_p * n)(*[_ptr(w) for w in workspaces])
     go = (C.c_int64 * n)(*[int(v) for v in grad_offsets])
     _check("lpdt_range_evonorm_bwd_params_batch", lib().lpdt_range_evonorm_bwd_params_batch(
-        nodes, B, n, C.addressof(cc), C.addressof(wp), C.addressof(go), _ptr(grads), grad_node_stride, _stream()))
+        nodes, B, n, _host(cc), _host(wp), _host(go), _ptr(grads), grad_node_stride, _stream()))
 
 
 def lpdt_dequantize_acc_batch(acc, nodes, acc_offsets, sizes, out_offsets, s1, s2, out, out_node_stride):
@@ -348,7 +370,7 @@ def lpdt_dequantize_acc_batch(acc, nodes, acc_offsets, sizes, out_offsets, s1, s
     p1 = (C.c_void_p * n)(*[_ptr(t) for t in s1])
     p2 = (C.c_void_p * n)(*[_ptr(t) for t in s2])
     _check("lpdt_dequantize_acc_batch", lib().lpdt_dequantize_acc_batch(
-        _ptr(acc), nodes, n, C.addressof(af), C.addressof(sz), C.addressof(of), C.addressof(p1), C.addressof(p2),
+        _ptr(acc), nodes, n, _host(af), _host(sz), _host(of), _host(p1), _host(p2),
         _ptr(out), out_node_stride, _stream()))
 
 
@@ -363,7 +385,7 @@ def lpdt_gossip_mix(nodes, d, x_half, x_hat, x_out, Wmix, gamma, seg_offsets, se
     sk = (C.c_int64 * ns)(*[int(v) for v in seg_k])
     p, nb = _ws(ws)
     _check("lpdt_gossip_mix", lib().lpdt_gossip_mix(nodes, d, _ptr(x_half), _ptr(x_hat), _ptr(x_out),
-                                                    _ptr(Wmix), gamma, ns, C.addressof(so), C.addressof(sk),
+                                                    _ptr(Wmix), gamma, ns, _host(so), _host(sk),
                                                     p, nb, _ptr(dev_status), _stream()))
 
 
@@ -375,7 +397,7 @@ def lpdt_gossip_mix_q8(nodes, d, x_half, x_hat, x_out, Wmix, gamma, seg_offsets,
     sk = (C.c_int64 * ns)(*[int(v) for v in seg_k])
     p, nb = _ws(ws)
     _check("lpdt_gossip_mix_q8", lib().lpdt_gossip_mix_q8(nodes, d, _ptr(x_half), _ptr(x_hat), _ptr(x_out),
-                                                          _ptr(Wmix), gamma, ns, C.addressof(so), C.addressof(sk),
+                                                          _ptr(Wmix), gamma, ns, _host(so), _host(sk),
                                                           _ptr(msg_scale), p, nb, _ptr(dev_status), _stream()))
 
 
@@ -387,7 +409,7 @@ def lpdt_deepsqueeze_mix(nodes, d, x_half, delta, x_out, Wmix, eta, seg_offsets,
     sk = (C.c_int64 * ns)(*[int(v) for v in seg_k])
     p, nb = _ws(ws)
     _check("lpdt_deepsqueeze_mix", lib().lpdt_deepsqueeze_mix(nodes, d, _ptr(x_half), _ptr(delta), _ptr(x_out),
-                                                              _ptr(Wmix), eta, ns, C.addressof(so), C.addressof(sk),
+                                                              _ptr(Wmix), eta, ns, _host(so), _host(sk),
                                                               message_bits, _ptr(msg_scale), p, nb, _ptr(dev_status),
                                                               _stream()))
 
@@ -472,3 +494,105 @@ def _with_timing(fn):
 for _n in [n for n in list(globals()) if n in LAUNCHING or n == "lpdt_fill_zero"]:
     globals()[_n] = _with_timing(globals()[_n])
 del _n
+
+
+CALL_WAIT = 1000       # LPDT_CALL_WAIT
+
+
+# ---- recorded calls ------------------------------------------------------------------------
+def wait_stream(waiting, other):
+    """waiting.wait_stream(other), noted by a recording."""
+    if _recording.calls is not None:
+        _recording.calls.items.append((None, (waiting.cuda_stream, other.cuda_stream)))
+    waiting.wait_stream(other)
+
+
+def lpdt_call_id(name):
+    """Id of an entry point in recorded sequences, or -1."""
+    return _load().lpdt_call_id(name.encode())
+
+
+def lpdt_run_calls(code, streams):
+    """code: ctypes array of 64-bit words; streams: sequence of stream handles.  Returns (status, item last begun)."""
+    handles, failed = (C.c_void_p * len(streams))(*streams), C.c_int64(0)
+    status = _load().lpdt_run_calls(C.addressof(code), len(code), C.addressof(handles), len(streams), C.addressof(failed))
+    return status, failed.value
+
+
+class Calls:
+    """The entry-point calls and stream waits that one walk of Python code makes on the current thread, issued again by
+    one native call (lpdt_run_calls).  `with calls.record():` runs the walk itself as usual.  The recording holds the
+    addresses the walk used: whoever keeps it also keeps those tensors, and records anew when any of them changes.
+
+    `scalars` names arguments that may change between replays: {name: [(entry point, argument index)]}."""
+
+    def __init__(self, scalars):
+        self.items, self.keep, self.scalars, self.code = [], [], scalars, None
+
+    def __getattr__(self, name):          # the library as seen by the recording thread
+        fn = getattr(_load(), name)
+        if name in LAUNCHING or name == "lpdt_fill_zero":
+            def call(*args):
+                status = fn(*args)
+                self.items.append((name, args))
+                return status
+            setattr(self, name, call)
+            return call
+        return fn
+
+    @contextlib.contextmanager
+    def record(self):
+        _recording.calls = self
+        try:
+            yield self
+        finally:
+            _recording.calls = None
+
+    def _encode(self):
+        """The recorded items as words; done at the first replay."""
+        words, index, self.patches = [], {}, {name: [] for name in self.scalars}
+        slot = lambda handle: index.setdefault(handle or 0, len(index))
+        self.names = []
+        for name, args in self.items:
+            self.names.append(name or "wait")
+            if name is None:
+                event = torch.cuda.Event()
+                event.record()                             # creates it
+                self.keep.append(event)
+                words += [CALL_WAIT, slot(args[0]), slot(args[1]), event.cuda_event]
+                continue
+            call = lpdt_call_id(name)
+            if call < 0:
+                return False
+            words += [call, slot(args[-1])]
+            for i, (kind, a) in enumerate(zip(SIGNATURES[name][1][:-1], args)):
+                for key, places in self.scalars.items():
+                    if (name, i) in places:
+                        self.patches[key].append((len(words), kind))
+                words.append(self._word(kind, a))
+        self.code = (C.c_uint64 * len(words))(*words)
+        self.streams = list(index)
+        self.items = None
+        return True
+
+    def _word(self, kind, a):
+        if kind is C.c_float:
+            return C.c_uint32.from_buffer(C.c_float(a)).value
+        if a is None:
+            return 0
+        if hasattr(a, "_obj"):                             # byref(descriptor)
+            self.keep.append(a._obj)
+            return C.addressof(a._obj)
+        return int(a) & 0xFFFFFFFFFFFFFFFF
+
+    def replay(self, recorded_stream, stream, **scalars):
+        """Issue the calls with `stream` in the place of the stream the recording was made on.  False if it cannot."""
+        if self.code is None and not self._encode():
+            return False
+        for name, value in scalars.items():
+            for at, kind in self.patches[name]:
+                self.code[at] = self._word(kind, value)
+        status, item = lpdt_run_calls(self.code, [stream if h == recorded_stream else h for h in self.streams])
+        if status != 0:
+            raise LpdtError(self.names[item], status)
+        return True

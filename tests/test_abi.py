@@ -36,3 +36,18 @@ def test_binding_names_match_the_abi():
         if n == "lpdt_status_string":
             continue
         assert hasattr(api, n), n
+
+
+def test_recorded_calls_are_checked():
+    """lpdt_run_calls: unknown items, items that do not fit, streams out of range and failing calls are errors."""
+    import ctypes as C
+    from paper_2111_09389_b200 import api
+    code = lambda *w: (C.c_uint64 * len(w))(*[v & 0xFFFFFFFFFFFFFFFF for v in w])
+    sgd = api.lpdt_call_id("lpdt_sgd_update")              # n, x, g, lr, out
+    assert sgd >= 0 and api.lpdt_call_id("lpdt_version") == -1 and api.lpdt_call_id("no such call") == -1
+    empty = [sgd, 0, 0, 0, 0, 0, 0]                        # no parameters: nothing to launch
+    assert api.lpdt_run_calls(code(*empty, *empty), [0]) == (0, 1)
+    assert api.lpdt_run_calls(code(*empty, sgd, 0, -1, 0, 0, 0, 0), [0]) == (1, 1)        # the second call refuses n < 0
+    for bad in ([77, 0], [-1, 0], [sgd, 1, 0, 0, 0, 0, 0], empty[:-1], [api.CALL_WAIT, 0, 0], [api.CALL_WAIT, 0, 1, 1],
+                [api.CALL_WAIT, 0, 0, 0]):
+        assert api.lpdt_run_calls(code(*bad), [0])[0] == 1, bad

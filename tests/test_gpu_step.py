@@ -4,6 +4,7 @@ import pytest
 import torch
 
 from oracle import step as ostep
+from paper_2111_09389_b200 import api
 from paper_2111_09389_b200 import workloads as wlmod
 from paper_2111_09389_b200.step import TrainStep
 
@@ -308,3 +309,50 @@ def test_step_with_requantize_inside_the_norm_layers(name, nodes, batch, kw):
     assert int(b.dev_status.item()) == 0
     for t in names:
         assert torch.equal(getattr(a, t), getattr(b, t)), t
+
+
+@pytest.mark.parametrize("name,kw", [("conv16", {}), ("conv16", dict(grad_rounding=1, message_bits=8)),
+                                     ("resnet20_topk_small", dict(node_groups=2)),
+                                     ("resnet20_topk_small", dict(quantize_wgrad=True, recompute_norm_input=True)),
+                                     ("resnet20_topk_small", dict(fuse_requantize=True, message_bits=8))])
+def test_recorded_runs_match_call_by_call(name, kw):
+    """run() issues recorded calls from its second run on: every run equals the layer walk to the bit, on another
+    stream, with another learning rate, consensus rate and seed, after a setting changed and with a replaced buffer."""
+    if name == "conv16":
+        wl = wlmod.make_workload("conv16")
+    else:
+        wl = wlmod.make_workload("resnet20_topk", nodes=4, batch=3)
+    a, b = TrainStep.from_workload(wl, **kw), TrainStep.from_workload(wl, **kw)
+
+    def both(**settings):
+        for st, step in ((a, a.run), (b, b._run)):
+            for k, v in settings.items():
+                setattr(st, k, v)
+            step()
+            st.params.copy_(st.x_out)
+        torch.cuda.synchronize()
+        for t in ("x_half", "x_hat", "x_out", "grads", "params", "out"):
+            assert torch.equal(getattr(a, t), getattr(b, t)), (t, settings)
+        assert (a.input_grad_out is None) == (b.input_grad_out is None)
+        if a.input_grad_out is not None:
+            assert torch.equal(a.input_grad_out, b.input_grad_out)
+
+    launches = []
+    for settings in ({}, {}, dict(lr=0.03, gamma=0.5, seed=9), {}):
+        before = api.lpdt_launch_count()
+        both(**settings)
+        launches.append(api.lpdt_launch_count() - before)
+    assert len(set(launches)) == 1
+    assert a._calls.code is not None                       # the last runs were replays
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        both(seed=10)
+    for st in (a, b):
+        st.x = st.x * 0.5                                  # another buffer
+        st.x_out = torch.zeros_like(st.x_out)
+    if not kw.get("node_groups"):
+        both()
+        both()
+        both(eps=1e-4)
+        both()
