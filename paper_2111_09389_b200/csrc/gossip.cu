@@ -1042,8 +1042,8 @@ static lpdt_status gossip_impl(int32_t nodes, int64_t d, const float *x_half, fl
     const bool v4 = d % 4 == 0 && aligned(x_half, 16) && aligned(x_hat, 16) && aligned(x_out, 16);
     const bool v2 = !v4 && d % 2 == 0 && aligned(x_half, 8) && aligned(x_hat, 8) && aligned(x_out, 8);
     const int vi = v4 ? 2 : v2 ? 1 : 0;
-    // nodes per warp: one up to 16 nodes; beyond, as few as keep a CTA within 20 warps
-    const int npw = nodes <= 16 ? 1 : (int)ceil_div(nodes, 20), warps = (int)ceil_div(nodes, npw), tile = 32 * mix_el(npw);
+    // nodes per warp: one up to 16 nodes (CTAs of 512 threads); beyond, as few, at least two, as keep a CTA within 20 warps
+    const int npw = nodes <= 16 ? 1 : nodes <= 40 ? 2 : (int)ceil_div(nodes, 20), warps = (int)ceil_div(nodes, npw), tile = 32 * mix_el(npw);
     const size_t tab_words = ((size_t)nodes + 2 * (size_t)nodes * nodes + 3) & ~(size_t)3;
     const size_t smem = tab_words * sizeof(int32_t) + 2 * (size_t)nodes * tile * sizeof(float);
     using MixFn = void (*)(int, int64_t, const float *, float *, float *, float, SegTable, const SelectOut *,

@@ -719,6 +719,27 @@ def test_gossip_mix(nodes, d, segs):
     close(xo2, x_ref2)
 
 
+@pytest.mark.parametrize("nodes,d,keep", [(1, 40000, 0.1), (2, 40002, 0.3), (16, 33000, 0.1), (17, 33001, 0.1), (20, 3000, 0.01),
+                                          (21, 2002, 0.1), (40, 2003, 0.5), (41, 1000, 0.1), (60, 1001, 0.1), (64, 1002, 0.01)])
+def test_gossip_node_counts_and_kept_shares(nodes, d, keep):
+    # one to four nodes per warp of the mix, parameter counts of every alignment with a part-empty last tile, two
+    # segments that meet inside a tile, kept shares whose candidates are a window of the segment; values on a coarse
+    # grid, so that ties decide the cut
+    rng = np.random.default_rng(nodes)
+    xh = (np.round(rng.standard_normal((nodes, d)) * 64) / 64).astype(np.float32)
+    xhat = (np.round(rng.standard_normal((nodes, d)) * 2) / 64).astype(np.float32)
+    W = wlmod.ring_matrix(nodes) if nodes >= 3 else np.full((nodes, nodes), 1.0 / nodes, np.float32)
+    cut = d - 77
+    so, sk = [0, cut, d], [max(1, int(cut * keep)), 7]
+    x_ref, xhat_ref, _ = oracle.gossip_mix(xh, xhat, W, 0.3, so, sk)
+    xhd, xhatd = dev(xh), dev(xhat)
+    xo = torch.empty_like(xhd)
+    ws = ws_bytes(api.lpdt_gossip_mix_workspace_size(nodes, d, 2))
+    api.lpdt_gossip_mix(nodes, d, xhd, xhatd, xo, dev(W), 0.3, so, sk, ws)
+    assert np.array_equal(xhatd.cpu().numpy(), xhat_ref)
+    close(xo, x_ref)
+
+
 def test_gossip_topk_with_massive_ties_and_alias():
     # magnitudes from a 4-value set: the tie cut decides almost every pick
     nodes, d, k = 6, 9000, 1234
