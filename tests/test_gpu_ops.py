@@ -253,6 +253,44 @@ def test_qconv_ragged_channels(case):
     test_qconv_bwd_affine(case)
 
 
+# long K loops and enough 256-channel tiles for the kernel on pairs of SMs: an odd number of pixel tiles (the last pair is
+# half empty), part-zero boxes on the summed side, a part-empty last channel tile; a convolution with a halo
+PAIR_CASES = [(12, 300, 1, 1, 1300, 1284, 1, 1, 1, 0), (2, 33, 12, 12, 128, 512, 3, 3, 1, 1)]
+
+
+@pytest.mark.parametrize("case", PAIR_CASES)
+def test_qconv_pairs_of_sms(case):
+    nodes, B, H, W, Cin, Cout, R, S, stride, pad = case
+    A, Wq, E, s1, s2 = _conv_inputs(case)
+    desc = api.conv_desc(*case)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    Y = torch.full(E.shape, float("nan"), dtype=torch.float32, device="cuda")
+    bias = np.random.default_rng(1).standard_normal((nodes, Cout)).astype(np.float32)
+    ws = ws_bytes(max(api.lpdt_qconv_workspace_size(desc, w) for w in (0, 1)))
+    api.lpdt_qconv_fwd(desc, dev(A), dev(s1), dev(Wq), dev(s2), Y=Y, bias=dev(bias), bias_node_stride=Cout, ws=ws, dev_status=status)
+    assert api.lpdt_last_kernel().endswith("conv_pair_kernel")
+    # the integer sums exactly, from float64 matrix products tap by tap; then the oracle's dequantization
+    Af, Wf, Ef = (torch.from_numpy(t).cuda().double() for t in (A, Wq, E))
+    acc = torch.zeros(E.shape, dtype=torch.float64, device="cuda")
+    dacc = torch.zeros(A.shape, dtype=torch.float64, device="cuda")
+    for n in range(nodes):
+        for r in range(R):
+            for q in range(S):
+                oh, ih = slice(max(0, pad - r), min(H, H + pad - r)), slice(max(0, r - pad), min(H, H + r - pad))
+                ow, iw = slice(max(0, pad - q), min(W, W + pad - q)), slice(max(0, q - pad), min(W, W + q - pad))
+                acc[n, :, oh, ow] += Af[n, :, ih, iw] @ Wf[n, :, r, q].t()
+                dacc[n, :, ih, iw] += Ef[n, :, oh, ow] @ Wf[n, :, r, q]
+    acc, dacc = acc.cpu().numpy().astype(np.int64).astype(np.int32), dacc.cpu().numpy().astype(np.int64).astype(np.int32)
+    assert np.array_equal(Y.cpu().numpy(), oracle.dequant_acc(acc, s1, s2, bias))
+    addend = np.random.default_rng(2).standard_normal(A.shape).astype(np.float32)
+    dA = torch.full(A.shape, float("nan"), dtype=torch.float32, device="cuda")
+    api.lpdt_qconv_bwd_data(desc, dev(E), dev(s1), dev(Wq), dev(s2), dA=dA, ws=ws, dev_status=status, addend=dev(addend))
+    if Cin >= 256:
+        assert api.lpdt_last_kernel().endswith("conv_pair_kernel")
+    assert np.array_equal(dA.cpu().numpy(), oracle.residual_add_bwd(addend, oracle.dequant_acc(dacc, s1, s2)))
+    assert int(status.item()) == 0
+
+
 @pytest.mark.parametrize("case", [RAGGED_CASES[0], RAGGED_CASES[3]])
 def test_qconv_ragged_channels_without_room_for_copies(case):
     # the least workspace (no room for padded operand copies) and none at all where none is required: same sums
