@@ -164,15 +164,14 @@ template <int AFF, bool VEC, int NV>
 __device__ __forceinline__ void affine_apply(const PixParams &p, const AffinePixel &a, int node, int c0, uint32_t (&v)[NV]) {
     const int st = AFF == 1 ? 1 : p.astride;
     const int32_t *t = p.wpre + (long long)node * (p.aR + st) * (p.aS + st) * p.Nc + c0;
-    if (!VEC) {
+    if constexpr (!VEC) {
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
             unsigned rw = (unsigned)__ldg(t + a.c11 + k);
             if (!a.interior) rw += (unsigned)__ldg(t + a.c00 + k) - (unsigned)__ldg(t + a.c01 + k) - (unsigned)__ldg(t + a.c10 + k);
             v[k] = v[k] + a.fixed - a.za * rw;
         }
-        return;
-    }
+    } else
 #pragma unroll
     for (int k = 0; k < NV; k += 4) {
         const int4 q11 = __ldg(reinterpret_cast<const int4 *>(t + a.c11 + k));

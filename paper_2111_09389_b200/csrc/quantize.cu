@@ -175,7 +175,7 @@ dequantize_kernel(const int8_t *__restrict__ q, int64_t n,
     const int z = AFFINE ? zp[node] : 0;
     const int64_t base = (int64_t)node * n;
     const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nth = (int64_t)gridDim.x * blockDim.x;
-    if (VEC) {
+    if constexpr (VEC) {
         const uint32_t *q4 = reinterpret_cast<const uint32_t *>(q + base);
         float4 *y4 = reinterpret_cast<float4 *>(y + (int64_t)node * ystride);
 #pragma unroll 4
@@ -189,9 +189,7 @@ dequantize_kernel(const int8_t *__restrict__ q, int64_t n,
             }
             y4[i] = make_float4(__fmul_rn(f[0], s), __fmul_rn(f[1], s), __fmul_rn(f[2], s), __fmul_rn(f[3], s));
         }
-        return;
-    }
-    for (int64_t i = tid; i < n; i += nth) {
+    } else for (int64_t i = tid; i < n; i += nth) {
         int code = AFFINE ? (int)(uint8_t)q[base + i] - z : (int)q[base + i];
         y[(int64_t)node * ystride + i] = __fmul_rn(__int2float_rn(code), s);
     }

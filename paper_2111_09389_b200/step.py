@@ -22,7 +22,8 @@ class TrainStep:
         if not torch.cuda.is_available():
             raise RuntimeError("TrainStep needs a CUDA device; there is no CPU path")
         self.ops, self.d, self.N, self.B = ops, d, nodes, batch
-        self._calls = None                        # the recorded step (run)
+        self._calls = self._calls_key = None      # the recorded step (run)
+        self._warm = False
         self.eps, self.lr, self.gamma = float(ren_eps), float(lr), float(gamma)
         self.seg_offsets = [0, d] if seg_offsets is None else [int(v) for v in seg_offsets]
         self.seg_k = [d] if seg_k is None else [int(v) for v in seg_k]
@@ -544,19 +545,24 @@ class TrainStep:
                 [(g.lr, g.gamma, g.seed, g.N) for g in self.groups])
 
     def run(self):
-        """One step.  The first run walks the layers call by call and records the calls; later runs on the same buffers
-        issue them from native code (identical calls, streams and order: ResNet-20 on 7 nodes 2.5 -> 1.1 ms, one layer on 4 nodes 0.23 -> 0.06 ms).  A
-        replaced buffer or changed setting records again; lr, gamma and seed may change freely."""
-        if api.RECORD is not None or api.TIMED or torch.cuda.is_current_stream_capturing():
+        """One step.  The first run walks the layers call by call, the second also records the calls, and later runs on
+        the same buffers issue them from native code (identical calls, streams and order; ResNet-20 on 7 nodes
+        2.5 -> 1.1 ms, one layer on 4 nodes 0.23 -> 0.06 ms).  After a replaced buffer or a changed setting it starts
+        over; lr, gamma and seed may change freely."""
+        if api.RECORD is not None or api.TIMED or not self._warm or torch.cuda.is_current_stream_capturing():
             self._run()
+            self._warm = True
             return
         stream = torch.cuda.current_stream()
         key = self._state_key(stream.device_index)
-        if self._calls is not None and self._calls_key == key:
+        if self._calls_key is not None and self._calls_key != key:       # seen for the first time: nothing is noted yet
+            self._calls, self._calls_key = None, key
+            self._run()
+            return
+        if self._calls is not None:
             if self._calls.replay(self._calls_stream, stream.cuda_stream, lr=self.lr, gamma=self.gamma, seed=self.seed):
                 self.out, self.input_grad_out = self._calls_out
                 return
-        self._calls = None
         calls = api.Calls(self._SCALARS)
         with calls.record():
             self._run()
