@@ -9,6 +9,8 @@ gradients staying fp32; then the SGD half-step and the CHOCO gossip mix
 (Section 3 and Algorithms 1 and 3 of the paper).  Python only orders the calls
 and owns the buffers; all arithmetic runs in the CUDA library.
 """
+import operator
+
 import torch
 
 from . import api
@@ -23,7 +25,7 @@ class TrainStep:
             raise RuntimeError("TrainStep needs a CUDA device; there is no CPU path")
         self.ops, self.d, self.N, self.B = ops, d, nodes, batch
         self._calls = self._calls_key = None      # the recorded step (run)
-        self._warm = False
+        self._warm, self._layer_buffers = False, None
         self.eps, self.lr, self.gamma = float(ren_eps), float(lr), float(gamma)
         self.seg_offsets = [0, d] if seg_offsets is None else [int(v) for v in seg_offsets]
         self.seg_k = [d] if seg_k is None else [int(v) for v in seg_k]
@@ -528,8 +530,8 @@ class TrainStep:
             api.lpdt_gossip_mix(N, d, self.x_half, self.x_hat, self.x_out, self.Wmix, self.gamma,
                                 self.seg_offsets, self.seg_k, self.ws, self.dev_status)
 
-    # what a recorded step bakes in: the addresses of the buffers a caller may replace, and every setting but those
-    # that are handed to each replay (_SCALARS)
+    # what a recorded step bakes in: the addresses of its buffers, those of the layers included, and every setting but
+    # those that are handed to each replay (_SCALARS)
     _BUFFERS = ("params", "grads", "x_half", "x_hat", "x_out", "Wmix", "x", "labels", "loss", "dev_status", "msg_scale",
                 "dy", "ranges", "ws", "ws_side", "qW_all", "sW_all", "g_acc")
     _SETTINGS = ("N", "B", "d", "eps", "grad_rounding", "quantize_wgrad", "input_grad", "message_bits",
@@ -540,7 +542,15 @@ class TrainStep:
 
     def _state_key(self, device):
         own = self.__dict__
+        if self._layer_buffers is None:           # the names of every layer's tensors (twice: always a tuple of them)
+            self._layer_buffers = []
+            for buf in [st.buf for st in (self, *self.groups)]:
+                for i, b in enumerate(buf):
+                    names = [n for n, t in b.items() if isinstance(t, torch.Tensor)]
+                    if names:
+                        self._layer_buffers.append((buf, i, operator.itemgetter(*names, names[0])))
         return (device, [None if own[n] is None else own[n].data_ptr() for n in self._BUFFERS],
+                [p for buf, i, get in self._layer_buffers for p in map(torch.Tensor.data_ptr, get(buf[i]))],
                 [own[n] for n in self._SETTINGS], tuple(self.seg_offsets), tuple(self.seg_k),
                 [(g.lr, g.gamma, g.seed, g.N) for g in self.groups])
 
