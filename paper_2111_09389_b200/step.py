@@ -554,12 +554,21 @@ class TrainStep:
                 [own[n] for n in self._SETTINGS], tuple(self.seg_offsets), tuple(self.seg_k),
                 [(g.lr, g.gamma, g.seed, g.N) for g in self.groups])
 
+    def _own_walk(self):
+        """Whether a walk over the layers executes the code below and nothing else.  A recording holds library calls only:
+        with a method of the walk overridden (in a subclass, on the class or on the object: an update with gradient
+        clipping, say) or an entry point's binding replaced, every run walks the layers."""
+        if _bindings_of(api) != _ENTRY_POINTS:
+            return False
+        return all(_methods_of(type(st)) == _METHODS and _METHOD_NAMES.isdisjoint(st.__dict__) for st in (self, *self.groups))
+
     def run(self):
         """One step.  The first run walks the layers call by call, the second also records the calls, and later runs on
         the same buffers issue them from native code (identical calls, streams and order; ResNet-20 on 7 nodes
         2.5 -> 1.1 ms, one layer on 4 nodes 0.23 -> 0.06 ms).  After a replaced buffer or a changed setting it starts
-        over; lr, gamma and seed may change freely."""
-        if api.RECORD is not None or api.TIMED or not self._warm or torch.cuda.is_current_stream_capturing():
+        over; lr, gamma and seed may change freely.  A step with code of its own (_own_walk) walks the layers every time."""
+        if (api.RECORD is not None or api.TIMED or not self._warm or torch.cuda.is_current_stream_capturing() or
+                not self._own_walk()):
             self._run()
             self._warm = True
             return
@@ -644,3 +653,10 @@ class TrainStep:
     def replay(self):
         self.graph.replay()
         api.add_replayed_launches(self.graph_launches)
+
+
+# The code that a walk over the layers executes, as it is here (TrainStep._own_walk compares).
+_METHOD_NAMES = frozenset(("_run", "_prepare", "_each_group", "forward", "_forward_layers", "backward", "_backward_layers",
+                           "_finish_gradients", "_ren_param_sums", "update", "_p", "_g"))
+_methods_of, _bindings_of = operator.attrgetter(*_METHOD_NAMES), operator.attrgetter(*sorted(api.LAUNCHING), "lpdt_fill_zero", "wait_stream")
+_METHODS, _ENTRY_POINTS = _methods_of(TrainStep), _bindings_of(api)
