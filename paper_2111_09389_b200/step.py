@@ -606,7 +606,7 @@ class TrainStep:
         again on the buffers the step left behind (every call reads and writes the same tensors)."""
         api.RECORD = log = []
         try:
-            self._run()
+            self.run()
         finally:
             api.RECORD = None
         return log
@@ -640,12 +640,12 @@ class TrainStep:
     def capture(self):
         """Record run() into a CUDA graph (one warm-up run first so that every
         one-time kernel attribute is set before capture)."""
-        self._run()
+        self.run()
         torch.cuda.synchronize()
         before = api.lpdt_launch_count()
         g = torch.cuda.CUDAGraph()
         with torch.cuda.graph(g):
-            self._run()
+            self.run()
         self.graph_launches = api.lpdt_launch_count() - before
         self.graph = g
         return g

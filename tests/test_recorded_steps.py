@@ -204,3 +204,33 @@ def test_replaced_parts_of_the_step_run_every_time(where, monkeypatch):
             rates = [c[5] for c in got if c[0] == "lpdt_sgd_update"]
             assert rates == [FLOAT_BITS(0.5)]
             assert [c[8] for c in got if c[0] == "lpdt_gossip_mix"] == [FLOAT_BITS(0.25)]
+
+
+def test_an_overridden_run_is_logged_and_captured(monkeypatch):
+    class Mine(TrainStep):
+        def run(self):
+            super().run()
+            done.append(torch.cuda.is_current_stream_capturing())
+            api.lpdt_sgd_update(self.N * self.d, self.params, self.grads, 0.5, self.x_half)
+
+    capturing = []
+
+    @contextlib.contextmanager
+    def graph(g):
+        capturing.append(g)
+        yield
+        capturing.pop()
+    monkeypatch.setattr(torch.cuda, "CUDAGraph", object)
+    monkeypatch.setattr(torch.cuda, "graph", graph)
+    monkeypatch.setattr(torch.cuda, "is_current_stream_capturing", lambda: bool(capturing))
+    done, st = [], make(cls=Mine)
+    log = st.record()
+    assert done == [False] and [r[0] for r in log][-1] == "lpdt_sgd_update"
+    for _ in range(4):
+        st.run()
+    native = Log.native
+    del done[:]
+    got = issued(st.capture)
+    assert done == [False, True]                           # the warm-up, and the captured one
+    assert [c[0] for c in got].count("lpdt_sgd_update") == 2
+    assert Log.native == native + 1                        # nothing native is captured but the warm-up's
