@@ -8,6 +8,7 @@ import contextlib
 import ctypes as C
 import threading
 
+import numpy as np
 import torch
 
 from ._lib import SIGNATURES, ConvDesc
@@ -521,10 +522,12 @@ def lpdt_run_calls(code, streams):
 
 class Calls:
     """The entry-point calls and stream waits that one walk of Python code makes on the current thread, issued again by
-    one native call (lpdt_run_calls).  `with calls.record():` runs the walk itself as usual.  The recording holds the
-    addresses the walk used: whoever keeps it also keeps those tensors, and records anew when any of them changes.
+    one native call (lpdt_run_calls).  `with calls.record():` runs the walk itself as usual.
 
-    `scalars` names arguments that may change between replays: {name: [(entry point, argument index)]}."""
+    No address outlives the walk: `bind` is told where the tensors lie that the walk read, and every recorded pointer
+    becomes a displacement from one of them; each replay is given their addresses anew, and the streams.
+
+    `scalars` names arguments that may change between replays: {name: [(entry point, argument index)]}, of one type each."""
 
     def __init__(self, scalars):
         self.items, self.keep, self.scalars, self.code = [], [], scalars, None
@@ -548,34 +551,85 @@ class Calls:
         finally:
             _recording.calls = None
 
+    def bind(self, addresses, extents, streams):
+        """addresses, extents (bytes): of every tensor the walk read, in the order in which replays pass the addresses;
+        streams: handles of every stream it used, the current one first.
+        Tensors that share memory form a cluster: a pointer into it is kept relative to the cluster's first tensor,
+        whichever of them the walk took it from, and replays require that the others lie where they lay, relative to it."""
+        self.bound, self.streams = (addresses, extents), streams
+
     def _encode(self):
-        """The recorded items as words; done at the first replay."""
-        words, index, self.patches = [], {}, {name: [] for name in self.scalars}
-        slot = lambda handle: index.setdefault(handle or 0, len(index))
-        self.names = []
+        """The recorded items as words; done at the first replay.  False if a pointer or stream is none of those bound."""
+        words, pointers, tables, names = [], [], [], []       # places of pointers; host arrays of them and their places
+        stream = {h or 0: i for i, h in reversed(list(enumerate(self.streams)))}
+        host, kinds = {C.addressof(a): a for a in self.keep}, {}
+        self.patches = {key: [] for key in self.scalars}
         for name, args in self.items:
-            self.names.append(name or "wait")
+            at = len(words)
+            names.append(name or "wait")
+            if any((h or 0) not in stream for h in (args if name is None else args[-1:])):
+                return False
             if name is None:
                 event = torch.cuda.Event()
-                event.record()                             # creates it
+                event.record()                                # creates it
                 self.keep.append(event)
-                words += [CALL_WAIT, slot(args[0]), slot(args[1]), event.cuda_event]
+                words += (CALL_WAIT, stream[args[0] or 0], stream[args[1] or 0], event.cuda_event)
                 continue
-            call = lpdt_call_id(name)
+            if name not in kinds:
+                types = SIGNATURES[name][1][:-1]
+                kinds[name] = (lpdt_call_id(name), [2 + i for i, t in enumerate(types) if t is C.c_void_p],
+                               [(2 + i, t) for i, t in enumerate(types) if t is C.c_float or t is C.POINTER(ConvDesc)],
+                               [(key, 2 + i, types[i]) for key, where in self.scalars.items() for entry, i in where if entry == name])
+            call, at_pointers, at_others, at_scalars = kinds[name]
             if call < 0:
                 return False
-            words += [call, slot(args[-1])]
-            for i, (kind, a) in enumerate(zip(SIGNATURES[name][1][:-1], args)):
-                for key, places in self.scalars.items():
-                    if (name, i) in places:
-                        self.patches[key].append((len(words), kind))
-                words.append(self._word(kind, a))
-        self.code = (C.c_uint64 * len(words))(*words)
-        self.streams = list(index)
-        self.items = None
+            words += (call, stream[args[-1] or 0])
+            words += args[:-1]
+            pointers += [at + i for i in at_pointers]
+            for i, t in at_others:
+                words[at + i] = self._word(t, words[at + i])
+            for key, i, t in at_scalars:
+                self.patches[key].append((at + i, t))
+        n = len(words)
+        given = [(i, words[i]) for i in pointers if words[i]]
+        for i in pointers:
+            words[i] = words[i] or 0
+        pointers = [i for i, a in given if a not in host]
+        for i, a in given:
+            if a in host and host[a]._type_ is C.c_void_p:    # behind the code, so that one array holds every pointer
+                tables.append((i, len(words)))
+                pointers += range(len(words), len(words) + len(host[a]))
+                words += [p or 0 for p in host[a]]
+        self._memory = np.array([w & 0xFFFFFFFFFFFFFFFF for w in words], dtype=np.uint64)
+        for i, table in tables:
+            self._memory[i] = self._memory.ctypes.data + 8 * table
+
+        # clusters of tensors by address, and the pointers' places in them
+        addresses, extents = self.bound
+        starts, ends, leads = [], [], []
+        inner, outer, shift = [], [], []
+        for a, i in sorted((a, i) for i, (a, size) in enumerate(zip(addresses, extents)) if size):
+            if ends and a < ends[-1]:
+                ends[-1] = max(ends[-1], a + extents[i])
+                inner.append(i); outer.append(leads[-1]); shift.append(a - starts[-1])
+            else:
+                starts.append(a); ends.append(a + extents[i]); leads.append(i)
+        pointers = np.array(pointers, dtype=np.int64)
+        values, starts, ends = self._memory[pointers], np.array(starts, dtype=np.uint64), np.array(ends, dtype=np.uint64)
+        cluster = np.searchsorted(starts, values, side="right") - 1
+        if (cluster < 0).any() or (values >= ends[cluster]).any():
+            return False
+        self._pointers = pointers, np.array(leads, dtype=np.int64)[cluster], values - starts[cluster]
+        self._clusters = np.array(inner, dtype=np.int64), np.array(outer, dtype=np.int64), np.array(shift, dtype=np.uint64)
+        self._aliases, self.names = [self.streams.index(h) for h in self.streams], names
+        self.code, self._address, self._given = (C.c_uint64 * n).from_buffer(self._memory), self._memory.ctypes.data, {}
+        self._handles = (C.c_void_p * len(self.streams))(), C.c_int64(0)
+        self.items = self.bound = None
         return True
 
     def _word(self, kind, a):
+        if type(a) is int and kind is not C.c_float:
+            return a & 0xFFFFFFFFFFFFFFFF
         if kind is C.c_float:
             return C.c_uint32.from_buffer(C.c_float(a)).value
         if a is None:
@@ -585,14 +639,28 @@ class Calls:
             return C.addressof(a._obj)
         return int(a) & 0xFFFFFFFFFFFFFFFF
 
-    def replay(self, recorded_stream, stream, **scalars):
-        """Issue the calls with `stream` in the place of the stream the recording was made on.  False if it cannot."""
+    def replay(self, addresses, moved, streams, **scalars):
+        """Issue the calls on the tensors that lie at `addresses` (moved: not all where the last call found them, or the
+        recording) and on `streams`.  False if they cannot be."""
         if self.code is None and not self._encode():
             return False
+        if [streams.index(h) for h in streams] != self._aliases:
+            return False
+        if moved:
+            now = np.array(addresses, dtype=np.uint64)
+            inner, outer, shift = self._clusters
+            if (now[inner] - now[outer] != shift).any():
+                return False
+            where, lead, offset = self._pointers
+            self._memory[where] = now[lead] + offset
         for name, value in scalars.items():
-            for at, kind in self.patches[name]:
-                self.code[at] = self._word(kind, value)
-        status, item = lpdt_run_calls(self.code, [stream if h == recorded_stream else h for h in self.streams])
+            if value != self._given.get(name) or type(value) is not int and (type(value) is not float or not value):
+                for at, kind in self.patches[name]:
+                    self.code[at] = self._word(kind, value)
+                self._given[name] = value
+        handles, item = self._handles
+        handles[:] = streams
+        status = _load().lpdt_run_calls(self._address, len(self.code), C.addressof(handles), len(handles), C.addressof(item))
         if status != 0:
-            raise LpdtError(self.names[item], status)
+            raise LpdtError(self.names[item.value], status)
         return True

@@ -24,8 +24,7 @@ class TrainStep:
         if not torch.cuda.is_available():
             raise RuntimeError("TrainStep needs a CUDA device; there is no CPU path")
         self.ops, self.d, self.N, self.B = ops, d, nodes, batch
-        self._calls = self._calls_key = None      # the recorded step (run)
-        self._warm, self._layer_buffers = False, None
+        self._warm, self._calls, self._reads, self._unused, self._rest = False, None, None, 0, 0      # the recorded step (run)
         self.eps, self.lr, self.gamma = float(ren_eps), float(lr), float(gamma)
         self.seg_offsets = [0, d] if seg_offsets is None else [int(v) for v in seg_offsets]
         self.seg_k = [d] if seg_k is None else [int(v) for v in seg_k]
@@ -530,63 +529,73 @@ class TrainStep:
             api.lpdt_gossip_mix(N, d, self.x_half, self.x_hat, self.x_out, self.Wmix, self.gamma,
                                 self.seg_offsets, self.seg_k, self.ws, self.dev_status)
 
-    # what a recorded step bakes in: the addresses of its buffers, those of the layers included, and every setting but
-    # those that are handed to each replay (_SCALARS)
-    _BUFFERS = ("params", "grads", "x_half", "x_hat", "x_out", "Wmix", "x", "labels", "loss", "dev_status", "msg_scale",
-                "dy", "ranges", "ws", "ws_side", "qW_all", "sW_all", "g_acc")
-    _SETTINGS = ("N", "B", "d", "eps", "grad_rounding", "quantize_wgrad", "input_grad", "message_bits",
-                 "recompute_norm_input", "fuse_requantize", "node_groups", "side")
-    _SCALARS = {"lr": [("lpdt_sgd_update", 3), ("lpdt_sgd_gossip_mix", 4)],
-                "gamma": [("lpdt_sgd_gossip_mix", 9), ("lpdt_gossip_mix", 6), ("lpdt_gossip_mix_q8", 6)],
-                "seed": [("lpdt_quantize", 6), ("lpdt_quantize_with_range", 6)]}
-
-    def _state_key(self, device):
-        own = self.__dict__
-        if self._layer_buffers is None:           # the names of every layer's tensors (twice: always a tuple of them)
-            self._layer_buffers = []
-            for buf in [st.buf for st in (self, *self.groups)]:
-                for i, b in enumerate(buf):
-                    names = [n for n, t in b.items() if isinstance(t, torch.Tensor)]
-                    if names:
-                        self._layer_buffers.append((buf, i, operator.itemgetter(*names, names[0])))
-        return (device, [None if own[n] is None else own[n].data_ptr() for n in self._BUFFERS],
-                [p for buf, i, get in self._layer_buffers for p in map(torch.Tensor.data_ptr, get(buf[i]))],
-                [own[n] for n in self._SETTINGS], tuple(self.seg_offsets), tuple(self.seg_k),
-                [(g.lr, g.gamma, g.seed, g.N) for g in self.groups])
-
     def _own_walk(self):
         """Whether a walk over the layers executes the code below and nothing else.  A recording holds library calls only:
         with a method of the walk overridden (in a subclass, on the class or on the object: an update with gradient
         clipping, say) or an entry point's binding replaced, every run walks the layers."""
-        if _bindings_of(api) != _ENTRY_POINTS:
+        if _bindings_of(_API) != _ENTRY_POINTS:
             return False
-        return all(_methods_of(type(st)) == _METHODS and _METHOD_NAMES.isdisjoint(st.__dict__) for st in (self, *self.groups))
+        for st in (self, *self.groups):
+            if _methods_of(type(st)) != _METHODS or not st.__dict__.keys().isdisjoint(_METHOD_NAMES):
+                return False
+        return True
 
     def run(self):
-        """One step.  The first run walks the layers call by call, the second also records the calls, and later runs on
-        the same buffers issue them from native code (identical calls, streams and order; ResNet-20 on 7 nodes
-        2.5 -> 1.1 ms, one layer on 4 nodes 0.23 -> 0.06 ms).  After a replaced buffer or a changed setting it starts
-        over; lr, gamma and seed may change freely.  A step with code of its own (_own_walk) walks the layers every time."""
+        """One step.  The first run walks the layers call by call, the second also notes the calls, and later runs issue
+        them from native code (identical calls, streams and order; ResNet-20 on 7 nodes 2.5 -> 1.1 ms, one layer on 4
+        nodes 0.23 -> 0.06 ms) on the buffers, with the streams and with the lr, gamma and seed of the day.  When anything
+        else changed that a walk reads (_Reads), the next run walks and a later one notes again; a step with code of its
+        own (_own_walk) walks the layers every time."""
         if (api.RECORD is not None or api.TIMED or not self._warm or torch.cuda.is_current_stream_capturing() or
                 not self._own_walk()):
             self._run()
             self._warm = True
-            return
-        stream = torch.cuda.current_stream()
-        key = self._state_key(stream.device_index)
-        if self._calls_key is not None and self._calls_key != key:       # seen for the first time: nothing is noted yet
-            self._calls, self._calls_key = None, key
+        elif self._calls is not None:
+            if not self._replay():
+                self._calls = self._reads = None
+                if self._unused > 2:              # recordings in a row that were never replayed: something keeps changing
+                    self._rest = min(1 << self._unused, 64)
+                self._run()
+        elif self._rest > 0:                      # runs until the next recording
+            self._rest -= 1
             self._run()
-            return
-        if self._calls is not None:
-            if self._calls.replay(self._calls_stream, stream.cuda_stream, lr=self.lr, gamma=self.gamma, seed=self.seed):
-                self.out, self.input_grad_out = self._calls_out
-                return
-        calls = api.Calls(self._SCALARS)
-        with calls.record():
-            self._run()
-        self._calls, self._calls_key, self._calls_stream = calls, key, stream.cuda_stream
-        self._calls_out = (self.out, self.input_grad_out)
+        else:
+            calls = api.Calls(_SCALARS)
+            with calls.record():
+                self._run()
+            self._unused += 1
+            current = torch.cuda.current_stream()
+            self._reads = _Reads(self, current)
+            if self._reads.bind(self, current, calls):
+                self._calls = calls
+            else:
+                self._rest = 64
+
+    def _streams(self, current):
+        """Handles of the streams a walk uses, the current one first."""
+        streams = [current, self.side]
+        for g in self.groups:
+            streams += (g.stream, g.side)
+        return [s.cuda_stream for s in streams]
+
+    def _replay(self):
+        reads, current = self._reads, torch.cuda.current_stream()
+        if not reads.same(self, current):
+            return False
+        try:
+            tensors = reads.tensors(self)
+            addresses = list(map(torch.Tensor.data_ptr, tensors))
+        except (AttributeError, KeyError, TypeError):         # a buffer was taken away: the walk says which it misses
+            return False
+        moved = addresses != reads.addresses
+        if moved and not reads.alike(tensors, addresses):
+            return False
+        if not self._calls.replay(addresses, moved, self._streams(current), lr=self.lr, gamma=self.gamma, seed=self.seed):
+            return False
+        reads.addresses = addresses
+        reads.leave_results(self, tensors, moved)
+        self._unused = 0
+        return True
 
     def _run(self):
         if self.groups:      # one fork for both passes: a group's backward pass follows its own forward pass
@@ -655,8 +664,125 @@ class TrainStep:
         api.add_replayed_launches(self.graph_launches)
 
 
+# Arguments of recorded calls that follow the step's attributes.
+_SCALARS = {"lr": [("lpdt_sgd_update", 3), ("lpdt_sgd_gossip_mix", 4)],
+            "gamma": [("lpdt_sgd_gossip_mix", 9), ("lpdt_gossip_mix", 6), ("lpdt_gossip_mix_q8", 6)],
+            "seed": [("lpdt_quantize", 6), ("lpdt_quantize_with_range", 6)]}
+
+
+class _Reads:
+    """What a walk over a step's layers reads, as it is when this is made: the settings, layer list and layer entries that
+    the recorded calls bake in, and where the tensors are found, whose addresses every run takes anew."""
+    BUFFERS = ("params", "grads", "x", "labels", "loss", "dy", "dev_status", "ranges", "ws", "ws_side")
+    WHOLE_STEP = ("x_half", "x_hat", "x_out", "Wmix", "msg_scale", "qW_all", "sW_all", "g_acc")      # not of a node group
+    WALK_STATE = ("x", "x_from", "addend", "fused_add", "pre_quantized", "E_ready")    # entries of a layer that the walk sets
+    # settings, and sizes that are arguments
+    SETTINGS = ("N", "B", "d", "eps", "grad_rounding", "quantize_wgrad", "input_grad", "message_bits", "recompute_norm_input",
+                "labels.__class__", "x.nbytes", "dy.nbytes", "ranges.nbytes", "ws.nbytes", "ws_side.nbytes")
+    LISTS = ("seg_offsets", "seg_k", "w_src", "w_size", "w_dst", "g_acc_off")
+    lists = operator.attrgetter(*LISTS)
+    settings, whole_settings = operator.attrgetter(*SETTINGS), operator.attrgetter(*SETTINGS, *LISTS, "ops")
+    kind = operator.attrgetter("device", "dtype", "shape")
+
+    def __init__(self, step, current):
+        self.groups = list(step.groups)
+        steps = (step, *self.groups)
+        self.device = current.device_index
+        self.layers = [list(st.buf) for st in steps]
+        names = [[n for n in self.BUFFERS + (self.WHOLE_STEP if st is step else ()) if n != "labels" or st.labels is not None]
+                 for st in steps]
+        self.getters = [operator.attrgetter(*n) for n in names]
+        # (with rounding, groups would draw with seeds of their own, and a replay is given one)
+        self.complete = all(getattr(st, n) is not None for st, ns in zip(steps, names) for n in ns) and not (
+            self.groups and any(st.grad_rounding for st in steps)) and all(g.ops is step.ops for g in self.groups) and all(
+            type(v) is list for v in self.lists(step))
+        if not self.complete:
+            return
+        self.of_layers, self.entries = [], []
+        for b in (b for layers in self.layers for b in layers):
+            own = [n for n in b if n not in self.WALK_STATE]
+            tensors = [n for n in own if isinstance(b[n], torch.Tensor)]
+            rest = [n for n in own if n not in tensors]
+            if tensors:                           # (at least two names: the getter returns a tuple)
+                self.of_layers.append((operator.itemgetter(*tensors, *tensors[:len(tensors) == 1]), b))
+            if rest:
+                self.entries.append((operator.itemgetter(*rest), b, operator.itemgetter(*rest)(b)))
+            for n in ("ws_ren", "ctl"):           # workspaces, whose size is an argument
+                if n in tensors:
+                    self.entries.append((lambda b, n=n: b[n].nbytes, b, b[n].nbytes))
+        whole, k = self.whole_settings(step), len(self.SETTINGS)
+        self.noted = (*whole[:k], *(v.copy() for v in whole[k:-1]), [dict(op) for op in step.ops])
+        self.noted_groups = [self.settings(g) for g in self.groups]
+
+    def same(self, step, current):
+        """Whether all but the tensors is as it was."""
+        try:
+            if (self.whole_settings(step) != self.noted or current.device_index != self.device or
+                    len(step.groups) != len(self.groups) or len(step.buf) != len(self.layers[0])):
+                return False
+            for st, layers in zip((step, *self.groups), self.layers):
+                if len(st.buf) != len(layers) or not all(map(operator.is_, st.buf, layers)):
+                    return False
+            for g, mine, noted in zip(step.groups, self.groups, self.noted_groups):
+                if g is not mine or g.ops is not step.ops or self.settings(g) != noted:
+                    return False
+            for get, b, noted in self.entries:
+                if get(b) != noted:
+                    return False
+            return True
+        except (AttributeError, KeyError, TypeError, ValueError, RuntimeError):      # taken away, or not to be compared
+            return False
+
+    def tensors(self, step):
+        out = []
+        for st, get in zip((step, *self.groups), self.getters):
+            out += get(st)
+        for get, b in self.of_layers:
+            out += get(b)
+        return out
+
+    def alike(self, tensors, addresses):
+        """Whether the tensors that lie elsewhere than in the last run could take the places of those of the recording."""
+        return all(self.kind(t) == kind and t.stride() == stride for t, a, old, kind, stride in
+                   zip(tensors, addresses, self.addresses, self.kinds, self.strides) if a != old)
+
+    def bind(self, step, current, calls):
+        """Ties a recording to the tensors.  False if it cannot be replayed."""
+        if not self.complete:
+            return False
+        tensors = self.tensors(step)
+        self.addresses = list(map(torch.Tensor.data_ptr, tensors))
+        self.kinds, self.strides = list(map(self.kind, tensors)), list(map(torch.Tensor.stride, tensors))
+        extents = [t.nbytes if t.is_contiguous() else 0 if t.numel() == 0 else
+                   t.element_size() * (1 + sum((n - 1) * s for n, s in zip(t.shape, t.stride()))) for t in tensors]
+        calls.bind(self.addresses, extents, step._streams(current))
+        # what the walk leaves in the step and its layers besides the buffers' contents
+        at = {id(t): i for i, t in enumerate(tensors)}
+        at[id(None)] = None
+        try:
+            self.results = [(i, n, at[id(getattr(st, n))]) for i, st in enumerate((step, *self.groups)) for n in ("out", "input_grad_out")]
+            self.state = [(b, n, at[id(b[n])]) for layers in self.layers for b in layers for n in ("x", "addend") if n in b]
+        except KeyError:
+            return False
+        return True
+
+    def leave_results(self, step, tensors, moved):
+        steps = (step, *self.groups)
+        for i, n, at in self.results:
+            setattr(steps[i], n, None if at is None else tensors[at])
+        for b, n, at in self.state if moved else ():
+            b[n] = None if at is None else tensors[at]
+
+
 # The code that a walk over the layers executes, as it is here (TrainStep._own_walk compares).
 _METHOD_NAMES = frozenset(("_run", "_prepare", "_each_group", "forward", "_forward_layers", "backward", "_backward_layers",
                            "_finish_gradients", "_ren_param_sums", "update", "_p", "_g"))
-_methods_of, _bindings_of = operator.attrgetter(*_METHOD_NAMES), operator.attrgetter(*sorted(api.LAUNCHING), "lpdt_fill_zero", "wait_stream")
-_METHODS, _ENTRY_POINTS = _methods_of(TrainStep), _bindings_of(api)
+_API = vars(api)
+_methods_of, _bindings_of = operator.attrgetter(*_METHOD_NAMES), operator.itemgetter(
+    "wait_stream", "lpdt_fill_zero", "lpdt_quantize", "lpdt_quantize_with_range", "lpdt_quantize_batch", "lpdt_dequantize",
+    "lpdt_qconv_fwd", "lpdt_qconv_bwd_data", "lpdt_qconv_bwd_weight", "lpdt_range_evonorm_fwd", "lpdt_range_evonorm_bwd",
+    "lpdt_range_evonorm_fwd_q8", "lpdt_range_evonorm_bwd_q8", "lpdt_range_evonorm_bwd_params_batch", "lpdt_dequantize_acc_batch",
+    "lpdt_gossip_mix", "lpdt_gossip_mix_q8", "lpdt_sgd_gossip_mix", "lpdt_sgd_update", "lpdt_residual_add",
+    "lpdt_residual_add_bwd", "lpdt_avgpool", "lpdt_avgpool_bwd", "lpdt_maxpool2x2", "lpdt_maxpool2x2_bwd", "lpdt_softmax_ce",
+    "lpdt_colsum")
+_METHODS, _ENTRY_POINTS = _methods_of(TrainStep), _bindings_of(_API)

@@ -360,3 +360,26 @@ def test_recorded_runs_match_call_by_call(name, kw):
             st.buf[0]["out"] = torch.full_like(st.buf[0]["out"], float("nan"))      # a layer's buffer
         both()
         assert torch.equal(a.buf[0]["out"], b.buf[0]["out"])
+
+
+@pytest.mark.parametrize("kw", [{}, dict(node_groups=2)])
+def test_recorded_runs_with_buffers_swapped_and_replaced(kw):
+    """Models that change places instead of being copied, and (without groups, whose slices keep the old ones) a new batch
+    tensor in every step; a group's workspace and batch replaced: results equal the layer walk's to the bit."""
+    wl = wlmod.make_workload("resnet20_topk", nodes=4, batch=3)
+    a, b = TrainStep.from_workload(wl, **kw), TrainStep.from_workload(wl, **kw)
+    for i in range(7):
+        for st, step in ((a, a.run), (b, b._run)):
+            if kw and i == 4:
+                g = st.groups[1]
+                g.x, g.ws, g.eps = g.x * 0.5, torch.empty_like(g.ws), 1e-4
+            step()
+            if kw:
+                st.params.copy_(st.x_out)
+            else:
+                st.params, st.x_out = st.x_out, st.params
+                st.x = st.x * 0.9
+        torch.cuda.synchronize()
+        for t in ("x_half", "x_hat", "x_out", "grads", "params", "out", "loss"):
+            assert torch.equal(getattr(a, t), getattr(b, t)), (i, t)
+    assert a._calls.code is not None or kw
