@@ -150,12 +150,15 @@ static bool use_tc(const lpdt_conv_desc &d, int which, const void *ws, size_t ws
     const bool pads = which == 0 ? d.Cin % 16 : (d.Cin % 16 || d.Cout % 16);
     return !pads || (ws && aligned(ws, 256) && ws_bytes >= lpdt_qconv_workspace_size(&d, which));
 }
-// Products that finish sooner on the CUDA cores although the tensor cores could take them: few results, each a dot
-// product of a few dozen steps (a classifier's scores and their adjoint).  The tensor-core kernel's fixed cost (barriers,
-// TMEM, first boxes) is about 6 us; measured 40 x 32 x 64 -> 10 forward 2.8 against 6.0 us and its adjoint 4.9
-// against 5.6, 8 x 32 x 512 -> 10 forward 9.9 against 6.7.  Only shapes that need padding; the others fill the tiles.
+// Products that finish sooner on the CUDA cores although the tensor cores could take them: each result a dot product of a
+// few dozen steps, and few steps in all (a classifier's scores and their adjoint, a small first layer).  The tensor-core
+// kernel's fixed cost (padded copies, barriers, TMEM, first boxes) is 6-8 us.  Measured, CUDA cores against tensor cores:
+// 40 x 32 x 64 -> 10 forward 2.8 / 6.0 us and its adjoint 4.9 / 5.6, 8 x 32 x 512 -> 10 forward 9.9 / 6.7; 3x3 from 3
+// channels 5.0 / 7.3 us at 65 K results (1.8 M steps), 9.1 / 7.6 at 131 K, 11.8 / 7.6 at 262 K.  Only shapes that need
+// padding; the others fill the tiles.
 static bool tiny_dot(const lpdt_conv_desc &d, int64_t results, int K, bool vec4) {
-    return (d.Cin % 16 || d.Cout % 16) && results <= (int64_t)kNumSMs * 2048 && (vec4 ? K / 4 : K) <= 64;
+    const int steps = vec4 ? K / 4 : K;
+    return (d.Cin % 16 || d.Cout % 16) && steps <= 64 && results * steps <= (int64_t)kNumSMs * 12288;
 }
 // An operand of `C` channels the engine can read: its padded copy, or itself at a 16-byte boundary.
 static bool readable(const void *p, int C) { return C % 16 != 0 || aligned(p, 16); }

@@ -229,20 +229,21 @@ def test_qconv_bwd_affine(case):
     assert not dW[:, wn:].any()
 
 
-# channel counts that no 16-byte row holds, or that end inside a box of the tensor-core kernels
+# channel counts that no 16-byte row holds, or that end inside a box of the tensor-core kernels.  (cc): forward products so
+# small that they run on the CUDA cores; backward-weight and the zero-point products take the tensor cores all the same
 RAGGED_CASES = [
     (2, 130, 1, 1, 200, 270, 1, 1, 1, 0),    # linear: 200 = 128 + 72 inputs, results in rows of 270 (no 16-byte rows)
     (1, 300, 1, 1, 1001, 17, 1, 1, 1, 0),    # odd on both sides, three row tiles
-    (1, 5, 9, 11, 7, 21, 3, 3, 1, 1),
+    (1, 5, 9, 11, 7, 21, 3, 3, 1, 1),        # cc
     (2, 3, 13, 10, 33, 50, 3, 3, 2, 1),      # strided, both ragged
-    (2, 2, 16, 16, 3, 24, 3, 3, 2, 1),       # strided first layer: 24 results in a tile of 32
+    (2, 2, 16, 16, 3, 24, 3, 3, 2, 1),       # strided first layer (cc)
     (1, 2, 8, 8, 130, 36, 3, 3, 1, 1),
-    (1, 2, 6, 6, 16, 15, 3, 3, 1, 1),        # whole input rows, one result short of a row
+    (1, 2, 6, 6, 16, 15, 3, 3, 1, 1),        # whole input rows, one result short of a row (cc)
     (1, 3, 5, 5, 20, 16, 5, 5, 1, 2),
     (1, 2, 12, 12, 144, 80, 3, 3, 1, 1),     # multiples of 16 whose last box is part zeros
     (2, 3, 7, 7, 272, 400, 1, 1, 1, 0),      # several N tiles, the last one part empty
     (1, 2, 9, 9, 48, 336, 3, 3, 2, 1),
-    (3, 1, 4, 4, 1, 1, 3, 3, 1, 1),          # a single channel
+    (3, 1, 4, 4, 1, 1, 3, 3, 1, 1),          # a single channel (cc)
 ]
 
 
@@ -251,6 +252,29 @@ def test_qconv_ragged_channels(case):
     test_qconv_all_three(case)
     test_qconv_fwd_affine(case)
     test_qconv_bwd_affine(case)
+
+
+# forward products on both sides of the line between CUDA cores and tensor cores, with the kernel that each takes: up to 64
+# steps a result (4 channels each where rows allow it) and 148 * 12288 steps in all
+@pytest.mark.parametrize("case,kernel", [
+    ((4, 4, 16, 16, 3, 16, 3, 3, 1, 1), "conv_fwd_generic"),        # 65 K results of 27 steps
+    ((4, 4, 16, 16, 3, 32, 3, 3, 1, 1), "conv_halo16_kernel"),      # 131 K: a first layer of 3 channels
+    ((2, 16, 16, 16, 3, 24, 3, 3, 1, 1), "conv_pix_kernel"),        # 24 results in a tile of 32
+    ((2, 130, 1, 1, 200, 270, 1, 1, 1, 0), "conv_pix_kernel"),      # results in rows of 270: no 16-byte rows
+    ((1, 60, 9, 11, 7, 21, 3, 3, 1, 1), "conv_pix_kernel"),
+    ((3, 300, 6, 6, 16, 15, 3, 3, 1, 1), "conv_pix_kernel"),        # whole input rows, one result short of a row
+    ((40, 32, 1, 1, 64, 10, 1, 1, 1, 0), "conv_fwd_generic"),       # a classifier: 13 K results of 16 steps
+    ((8, 32, 1, 1, 512, 10, 1, 1, 1, 0), "conv_pix_kernel")])       # 128 steps
+def test_qconv_forward_takes_the_sooner_cores(case, kernel):
+    nodes, B, H, W, Cin, Cout, R, S, stride, pad = case
+    A, Wq, E, s1, s2 = _conv_inputs(case)
+    desc = api.conv_desc(*case)
+    Y = torch.full(E.shape, float("nan"), dtype=torch.float32, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    api.lpdt_qconv_fwd(desc, dev(A), dev(s1), dev(Wq), dev(s2), Y=Y, ws=ws_bytes(api.lpdt_qconv_workspace_size(desc, 0)), dev_status=status)
+    assert api.lpdt_last_kernel().endswith(kernel)
+    assert np.array_equal(Y.cpu().numpy(), oracle.dequant_acc(oracle.qconv_fwd(A, Wq, stride, pad)[0], s1, s2))
+    assert int(status.item()) == 0
 
 
 # long K loops and enough 256-channel tiles for the kernel on pairs of SMs: an odd number of pixel tiles (the last pair is
