@@ -254,6 +254,23 @@ def test_qconv_ragged_channels(case):
     test_qconv_bwd_affine(case)
 
 
+@pytest.mark.parametrize("rows,cin,skew", [(300 * 1024, 3, 0), (300 * 1024 + 1, 3, 1), (100 * 1024 - 3, 33, 0), (100 * 1024 + 1, 33, 3),
+                                           (303104, 5, 0), (303103, 5, 0), (303103, 1, 2), (7, 17, 1)])
+def test_padded_copies_of_many_rows(rows, cin, skew):
+    """Operands whose rows no TMA can address, at every byte offset, on both sides of the size from which a thread copies
+    several pieces; the last row ends the allocation."""
+    rng = np.random.default_rng(rows + cin)
+    A, Wq = wlmod.random_s8(rng, (rows, cin)), wlmod.random_s8(rng, (80, cin))
+    desc = api.conv_desc(1, rows, 1, 1, cin, 80, 1, 1, 1, 0)
+    Ad = torch.empty(rows * cin + skew, dtype=torch.int8, device="cuda")[skew:].view(rows, cin)
+    Ad.copy_(dev(A))
+    Y = torch.full((rows, 80), 77, dtype=torch.int32, device="cuda")
+    ws = torch.full((api.lpdt_qconv_workspace_size(desc, 0),), 85, dtype=torch.uint8, device="cuda")
+    api.lpdt_qconv_fwd(desc, Ad, None, dev(Wq), None, Yacc=Y, ws=ws)
+    assert rows < 100 or api.lpdt_last_kernel() in ("lpdt::tc::conv_pix_kernel", "lpdt::tc::conv_halo16_kernel")
+    assert torch.equal(Y.double(), torch.from_numpy(A).cuda().double() @ torch.from_numpy(Wq).cuda().double().t())
+
+
 # forward products on both sides of the line between CUDA cores and tensor cores, with the kernel that each takes: up to 64
 # steps a result (4 channels each where rows allow it) and 148 * 12288 steps in all
 @pytest.mark.parametrize("case,kernel", [
