@@ -254,6 +254,32 @@ def test_qconv_ragged_channels(case):
     test_qconv_bwd_affine(case)
 
 
+# group widths of backward-weight: the narrowest that give every SM one tile (16, 32, 64 channels, with a part-empty last
+# group), loops of up to four blocks with wide groups of 32-byte rows, split loops; channel counts that end inside 16
+@pytest.mark.parametrize("nodes,rows,cin,cout", [(2, 815, 128, 304), (2, 2008, 32, 272), (3, 21, 32, 416), (1, 7, 16, 17), (8, 43, 64, 160),
+                                                 (2, 100, 700, 1001), (6, 20, 704, 3360), (6, 20, 704, 3345), (1, 5000, 64, 250),
+                                                 (1, 2500, 30, 10), (5, 128, 512, 512)])
+def test_backward_weight_group_widths(nodes, rows, cin, cout):
+    rng = np.random.default_rng(rows)
+    A, E = wlmod.random_s8(rng, (nodes, rows, cin)), wlmod.random_s8(rng, (nodes, rows, cout))
+    s1, s2 = rng.uniform(0.001, 0.1, (2, nodes)).astype(np.float32)
+    desc = api.conv_desc(nodes, rows, 1, 1, cin, cout, 1, 1, 1, 0)
+    ws = ws_bytes(api.lpdt_qconv_workspace_size(desc, 2))
+    acc = torch.full((nodes, cout, cin), 77, dtype=torch.int32, device="cuda")
+    dW = torch.full((nodes, cout * cin + 5), 9.0, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    api.lpdt_qconv_bwd_weight(desc, dev(E), dev(s1), dev(A), dev(s2), dW=dW, dw_node_stride=cout * cin + 5, dWacc=acc, ws=ws,
+                              dev_status=status)
+    assert api.lpdt_last_kernel().endswith("conv_wgrad_kernel") and int(status.item()) == 0
+    ref = torch.from_numpy(E).cuda().double().transpose(1, 2) @ torch.from_numpy(A).cuda().double()
+    assert torch.equal(acc.double(), ref)
+    want = oracle.dequant_acc(acc.cpu().numpy().reshape(nodes, -1), s1, s2)
+    only = torch.full_like(dW, 9.0)
+    api.lpdt_qconv_bwd_weight(desc, dev(E), dev(s1), dev(A), dev(s2), dW=only, dw_node_stride=cout * cin + 5, ws=ws)
+    for got in (dW, only):
+        assert np.array_equal(got[:, :cout * cin].cpu().numpy(), want) and bool((got[:, cout * cin:] == 9.0).all())
+
+
 @pytest.mark.parametrize("rows,cin,skew", [(300 * 1024, 3, 0), (300 * 1024 + 1, 3, 1), (100 * 1024 - 3, 33, 0), (100 * 1024 + 1, 33, 3),
                                            (303104, 5, 0), (303103, 5, 0), (303103, 1, 2), (7, 17, 1)])
 def test_padded_copies_of_many_rows(rows, cin, skew):
