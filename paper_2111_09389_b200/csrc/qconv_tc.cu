@@ -345,6 +345,7 @@ conv_pix_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
                 const int iters = p.cls_iters[cls];
                 if (++cls == p.ncls) cls = 0;
                 uint32_t accum = 0;
+                if (iters == 0 && elect_one()) mbar_arrive(smem_u32(&ctl->tmem_full[acc]));
                 for (int it = 0; it < iters; ++it, ++g) {
                     if (!mbar_wait(smem_u32(&ctl->full[st]), ph, &ctl->abort_flag, p.dev_status)) { ok = false; break; }
                     tc_fence_after();
@@ -394,6 +395,7 @@ conv_pix_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
             if (p.Y && c.node != sc_node) { sc_node = c.node; sc = __fmul_rn(p.s1[c.node], p.s2[c.node]); }
             const int acc = tcount & 1;
             const uint32_t aph = (tcount >> 1) & 1;
+            const bool no_taps = p.cls_iters[c.cls] == 0;
             if (!mbar_wait(smem_u32(&ctl->tmem_full[acc]), aph, &ctl->abort_flag, p.dev_status)) break;
             tc_fence_after();
             const long long pix = (((long long)c.node * p.B + b) * p.Hout + h) * p.Wout + w;
@@ -410,6 +412,10 @@ conv_pix_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
                     uint32_t v[32];
                     tmem_ld_32x32(t_row + cc, v);
                     tmem_ld_wait();
+                    if (no_taps) {
+#pragma unroll
+                        for (int k = 0; k < 32; ++k) v[k] = 0;
+                    }
                     if (AFF && valid) affine_apply<AFF, false>(p, aff, c.node, n0 + cc, v);
                     int4 *grow = reinterpret_cast<int4 *>(buf + lane * 128);
 #pragma unroll
@@ -504,6 +510,10 @@ conv_pix_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
                 uint32_t v[16];
                 tmem_ld_32x16(t_row + cc, v);
                 tmem_ld_wait();
+                if (no_taps) {
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) v[k] = 0;
+                }
                 if (valid) {
                     const long long o = pix * p.Nc + n0 + cc;
                     const int quads = (p.Nc - n0 - cc) / 4;          // the tile may reach past the last channel
@@ -898,6 +908,19 @@ lpdt_status tc_pix(const lpdt_conv_desc &d, int mode, const int8_t *A, const flo
     p.tma_out = (!row && Y && !Yacc && aligned(Y, 16) && p.ncls == 1 && p.out_mul == 1 && p.Nc > 16 &&
                  pix_tma_out_enabled()) ? 1 : 0;
     int unit = (row || p.tma_out) ? 32 : 16;
+    if (p.ncls > 1 && (long long)d.R * d.S * p.Kc <= 4096) {
+        // Strided backward-data with short K loops: its stores are most of the work, so padded channels count and the width
+        // of the weight rows hardly does (128 x 3 channels of 352 for 5 x 30 x 35x35 <- 160 1x1 164 us, 192 x 2 137 us;
+        // 192 x 2 of 272 for 8 x 32 x 16x16 <- 128 43.8 us, 160 x 2 39.0 us).  Relative costs of the rows as measured there.
+        const int w[4] = {100, 102, 105, 115};
+        const long long mt = (long long)p.nodes * p.tilesB * p.tilesH * p.tilesW * p.ncls;
+        long long cost = -1;
+        for (int i = 0; i < 4; ++i) {
+            const int rb = 128 >> i, bn = pick_bn(p.Nc, rb > unit ? rb : unit, mt);
+            const long long c = ceil_div(mt * ceil_div(p.Nc, bn), kNumSMs) * (128 + bn) * w[i];
+            if (cost < 0 || c < cost) { cost = c; p.RBn = rb; }
+        }
+    }
     if (mode == 1 && p.RBn > unit) unit = p.RBn;
     p.BN = pick_bn(p.Nc, unit, (long long)p.nodes * p.tilesB * p.tilesH * p.tilesW * p.ncls);
     p.tilesN = (int)ceil_div(p.Nc, p.BN);
@@ -919,7 +942,8 @@ lpdt_status tc_pix(const lpdt_conv_desc &d, int mode, const int8_t *A, const flo
     p.U = U;
     for (int c = 0; c < p.ncls; ++c) {
         p.cls_iters[c] = (int)ceil_div((long)p.tt[c].ntaps * cpt, U);
-        if (p.cls_iters[c] < 1) p.cls_iters[c] = 1;      // a class without taps still writes zeros
+        // (0 for a class without taps, three in four pixels of a 1x1 of stride 2: nothing is loaded or multiplied for it,
+        // and its pixels are written from zeros)
     }
     // long K loops (GEMM-like): blocked round-robin tile order; short ones: contiguous ranges
     p.raster = (p.ncls == 1 && p.cls_iters[0] >= 8) ? 1 : 0;

@@ -280,6 +280,28 @@ def test_backward_weight_group_widths(nodes, rows, cin, cout):
         assert np.array_equal(got[:, :cout * cin].cpu().numpy(), want) and bool((got[:, cout * cin:] == 9.0).all())
 
 
+# strided backward-data: pixels that no tap reaches (1x1 of stride 2, and a filter of two rows), results in rows of 16 bytes
+# and not, tiles of every row width, more tiles than one wave
+STRIDED_CASES = [(2, 3, 9, 9, 352, 48, 1, 1, 2, 0), (1, 2, 8, 8, 30, 16, 1, 1, 2, 0), (2, 2, 7, 11, 21, 33, 1, 1, 2, 0), (1, 40, 28, 28, 80, 32, 1, 1, 2, 0),
+                 (2, 3, 8, 8, 400, 128, 3, 3, 2, 1), (1, 2, 9, 12, 272, 96, 2, 1, 2, 0), (1, 1, 1, 1, 64, 64, 1, 1, 2, 0), (1, 2, 5, 5, 16, 20, 1, 1, 2, 2)]
+
+
+@pytest.mark.parametrize("case", STRIDED_CASES)
+def test_qconv_strided(case):
+    test_qconv_all_three(case)
+    test_qconv_fwd_affine(case)
+    test_qconv_bwd_affine(case)
+    nodes, B, H, W, Cin, Cout, R, S, stride, pad = case
+    A, Wq, E, s1, s2 = _conv_inputs(case)
+    desc = api.conv_desc(*case)
+    addend = np.random.default_rng(3).standard_normal(A.shape).astype(np.float32)
+    dA = torch.full(A.shape, float("nan"), dtype=torch.float32, device="cuda")
+    ws = ws_bytes(api.lpdt_qconv_workspace_size(desc, 1))
+    api.lpdt_qconv_bwd_data(desc, dev(E), dev(s1), dev(Wq), dev(s2), dA=dA, ws=ws, addend=dev(addend))
+    ref = oracle.residual_add_bwd(addend, oracle.dequant_acc(oracle.qconv_bwd_data(E, Wq, H, W, stride, pad)[0], s1, s2))
+    assert np.array_equal(dA.cpu().numpy(), ref)
+
+
 @pytest.mark.parametrize("rows,cin,skew", [(300 * 1024, 3, 0), (300 * 1024 + 1, 3, 1), (100 * 1024 - 3, 33, 0), (100 * 1024 + 1, 33, 3),
                                            (303104, 5, 0), (303103, 5, 0), (303103, 1, 2), (7, 17, 1)])
 def test_padded_copies_of_many_rows(rows, cin, skew):
