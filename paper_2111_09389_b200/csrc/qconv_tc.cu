@@ -759,19 +759,19 @@ conv_wgrad_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
 // ---------------------------------------------------------------------------------------------- host
 static int pow2_at_least(int v) { int p = 32; while (p < v) p <<= 1; return p; }
 
-// Pixel tile {TB, TH, TW} with TB*TH*TW = 128 covering a W x H image with least waste.
-static void pick_tile(int H, int W, int max_tw, int *TB, int *TH, int *TW) {
-    int bw = 1; long best = -1;
-    for (int t = 1; t <= max_tw; t <<= 1) {
-        long cover = (long)ceil_div(W, t) * t;
-        if (best < 0 || cover <= best) { best = cover; bw = t; }
-    }
-    int bh = 1; best = -1;
-    for (int t = 1; t <= 128 / bw; t <<= 1) {
-        long cover = (long)ceil_div(H, t) * t;
-        if (best < 0 || cover <= best) { best = cover; bh = t; }
-    }
-    *TW = bw; *TH = bh; *TB = 128 / (bw * bh);
+// Pixel tile {TB, TH, TW} with TB*TH*TW = 128 that covers B images of W x H with the fewest padded pixels; among those the
+// fewest padded columns, the widest, the fewest padded rows, the highest.  (Axis by axis, an odd width took single columns
+// of up to 128 images: 5 images of 27x27 filled 5 of 128 rows; 9 nodes, 192 -> 64 3x3 forward 253 us, 21 now.)
+static void pick_tile(int B, int H, int W, int max_tw, int *TB, int *TH, int *TW) {
+    long long best = -1, best_w = 0, best_h = 0;
+    for (int tw = max_tw < 128 ? max_tw : 128; tw >= 1; tw >>= 1)
+        for (int th = 128 / tw; th >= 1; th >>= 1) {
+            const int tb = 128 / (tw * th);
+            const long long cw = ceil_div(W, tw) * tw, ch = ceil_div(H, th) * th, cover = ceil_div(B, tb) * tb * ch * cw;
+            if (best < 0 || cover < best || (cover == best && (cw < best_w || (tw == *TW && ch < best_h)))) {
+                best = cover; best_w = cw; best_h = ch; *TB = tb; *TH = th; *TW = tw;
+            }
+        }
 }
 
 // Activation map: box = {RB channel bytes, TW, TH, TB pixels, 1 node}.  With estride 2 the
@@ -899,7 +899,7 @@ lpdt_status tc_pix(const lpdt_conv_desc &d, int mode, const int8_t *A, const flo
     const int pitchA = mode == 0 ? pt.in : pt.err;
     p.merged = (pitchA == 16 && estride == 1) ? 1 : 0;
     if (p.merged) p.RBa = 16;
-    pick_tile(p.Hm, p.Wm, p.merged ? 16 : 128, &p.TB, &p.TH, &p.TW);
+    pick_tile(d.B, p.Hm, p.Wm, p.merged ? 16 : 128, &p.TB, &p.TH, &p.TW);
     if (p.TW * estride > 256 || p.TH * estride > 256) return LPDT_ERR_UNSUPPORTED;
     p.tilesB = (int)ceil_div(d.B, p.TB); p.tilesH = (int)ceil_div(p.Hm, p.TH); p.tilesW = (int)ceil_div(p.Wm, p.TW);
     // how the result leaves (see PixParams): rows of a multiple of 16 bytes through bulk stores (fp32 only, one class),
@@ -1048,7 +1048,7 @@ lpdt_status tc_wgrad(const lpdt_conv_desc &d, const int8_t *E, const float *sE, 
     p.BNc = pick_bn(d.Cout, p.RBe, 0);
     p.halo = (p.merged && d.S <= 8 && d.R * p.BNc <= 512 && d.R <= 16) ? 1 : 0;
     if (p.halo) { p.TW = 8; p.TH = 16; p.TB = 1; p.PW = 8 + d.S - 1; p.PH = 16 + d.R - 1; p.halo_bytes = (int)align_up((size_t)p.PW * p.PH * 16 + 256, 1024); }
-    else pick_tile(Ho, Wo, p.merged ? 16 : 128, &p.TB, &p.TH, &p.TW);
+    else pick_tile(d.B, Ho, Wo, p.merged ? 16 : 128, &p.TB, &p.TH, &p.TW);
     if (p.TW * d.stride > 256 || p.TH * d.stride > 256) return LPDT_ERR_UNSUPPORTED;
     p.tilesB = (int)ceil_div(d.B, p.TB); p.tilesH = (int)ceil_div(Ho, p.TH); p.tilesW = (int)ceil_div(Wo, p.TW);
     p.kblocks = p.tilesB * p.tilesH * p.tilesW;

@@ -302,6 +302,16 @@ def test_qconv_strided(case):
     assert np.array_equal(dA.cpu().numpy(), ref)
 
 
+# maps of odd sizes with few images: every split of the 128 pixels of a tile, boxes that reach past the map on two axes
+@pytest.mark.parametrize("case", [(2, 5, 27, 27, 32, 48, 3, 3, 1, 1), (1, 3, 25, 13, 48, 32, 3, 3, 2, 1), (2, 12, 7, 7, 64, 80, 3, 3, 1, 1),
+                                  (1, 5, 39, 11, 16, 16, 5, 5, 1, 2), (1, 2, 33, 28, 20, 36, 3, 3, 1, 1), (1, 3, 1, 29, 16, 130, 1, 3, 1, 1),
+                                  (1, 1, 131, 3, 64, 32, 3, 3, 1, 1), (3, 1, 6, 130, 32, 16, 1, 1, 2, 0)])
+def test_qconv_odd_maps(case):
+    test_qconv_all_three(case)
+    test_qconv_fwd_affine(case)
+    test_qconv_bwd_affine(case)
+
+
 @pytest.mark.parametrize("rows,cin,skew", [(300 * 1024, 3, 0), (300 * 1024 + 1, 3, 1), (100 * 1024 - 3, 33, 0), (100 * 1024 + 1, 33, 3),
                                            (303104, 5, 0), (303103, 5, 0), (303103, 1, 2), (7, 17, 1)])
 def test_padded_copies_of_many_rows(rows, cin, skew):
