@@ -6,9 +6,11 @@
 One step = one pass of the whole hot path (quantize, int8 contractions forward /
 backward-data / backward-weight, Range-EvoNorm forward/backward, SGD half-step,
 top-k compression and gossip mix) over one batch for every simulated node.
-Prints ONE JSON line.  The headline workload is the largest single-GPU
+Prints ONE JSON line on stdout, short enough (under 2400 characters) for logs that
+keep the end of the output only.  The headline workload is the largest single-GPU
 configuration: the ResNet-20-shaped network on 40 simulated nodes x batch 32 with
-top-1 % compressed gossip.  At one GPU the line also carries, under "extra":
+top-1 % compressed gossip.  The rest goes to stderr, as one JSON line as well: the
+whole roofline record of the dominant kernel and, at one GPU, under "extra":
 
   workloads     every step workload (single conv layer, ResNet-20 x 16 nodes, VGG-11 x 8
                 nodes, ResNet-20 x 40 nodes with top-1 %): ms per step, images/s, end to end
@@ -506,6 +508,30 @@ def membound_block(peaks, iters=10):
             "554 MB parameter arrays (16 nodes x 8.65 M)", "cases": rows}
 
 
+def rounded(v):
+    """Numbers of a result with six significant digits."""
+    if isinstance(v, float):
+        return float(f"{v:.6g}")
+    if isinstance(v, dict):
+        return {k: rounded(x) for k, x in v.items()}
+    return [rounded(x) for x in v] if isinstance(v, (list, tuple)) else v
+
+
+ROOFLINE_KEYS = ("kernel", "bound", "achieved", "peak", "unit", "frac", "launches_per_step", "ms_per_step_in_kernel")
+
+
+def report(out):
+    """(stdout line, stderr line) of a result: the second holds what the first leaves out."""
+    line = {k: v for k, v in out.items() if k != "extra"}
+    if line.get("roofline"):
+        line["roofline"] = {k: line["roofline"][k] for k in ROOFLINE_KEYS if k in line["roofline"]}
+    if line.get("clocks"):
+        line["clocks"] = {k: v for k, v in line["clocks"].items() if k != "window"}
+    # value and ms_per_step as measured: readers recompute one from the other
+    line = {k: v if k in ("value", "ms_per_step") else rounded(v) for k, v in line.items()}
+    return json.dumps(line), json.dumps(rounded({k: out[k] for k in ("roofline", "clocks", "extra") if k in out}))
+
+
 def run_ours(args):
     import torch
     world, rank, local = dist_setup(args.gpus)
@@ -578,7 +604,9 @@ def run_ours(args):
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
         out["cpu_baseline"] = cpu_baseline(args.workload, nodes=args.cpu_nodes)
     if rank == 0:
-        print(json.dumps(out))
+        line, details = report(out)
+        print(details, file=sys.stderr, flush=True)
+        print(line, flush=True)
     if world > 1:
         import torch.distributed as dist
         dist.destroy_process_group()

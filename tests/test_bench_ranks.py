@@ -58,3 +58,27 @@ def test_reference_arm_runs_on_rank_zero_only():
     r = subprocess.run([sys.executable, os.path.join(ROOT, "bench.py"), "--impl", "reference", "--gpus", "2", "--steps", "1",
                         "--warmup", "0"], env=env, cwd=ROOT, capture_output=True, text=True, timeout=120)
     assert r.returncode == 0 and r.stdout.strip() == ""
+
+
+def test_the_printed_line_is_short_and_loses_nothing():
+    sys.path.insert(0, ROOT)
+    import bench
+    num = 123456.78901234567
+    out = {"metric": bench.METRIC, "value": num, "unit": bench.UNIT, "n_gpus": 8, "steps": 20, "warmup": 5, "ms_per_step": num,
+           "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "int8", "data": "synthetic",
+           "config": {"workload": bench.HEADLINE, "description": max(bench.WORKLOAD_DESC.values(), key=len), "nodes": 40,
+                      "batch_per_node": 32, "params_per_node": 9231114, "parallelism": "1 GPU, nodes batched", "launch": "x" * 105,
+                      "l2": "y" * 85},
+           "int8_tops": num, "macs_per_step": 10 ** 12,
+           "clocks": {"sm_mhz": 1965, "sm_max_mhz": 1965, "reasons": ["sw_power_cap"], "samples": 40, "window": "z" * 100},
+           "e2e": {"value": num, "unit": bench.UNIT, "h2d_bytes_per_step": 10 ** 9, "d2h_bytes_per_step": 160}, "gpu_launches": 99999,
+           "roofline": dict({k: num for k in bench.ROOFLINE_KEYS}, timing="t" * 200, kernels_by_time=[{"kernel": "k" * 40}] * 6),
+           "step": {k: num for k in ("algorithmic_bytes", "gbs", "frac_of_hbm", "launches_per_step", "sum_of_isolated_ms")},
+           "extra": {"breakdown": [{"call": "c" * 80}] * 300},
+           "cpu_baseline": {"value": num, "unit": bench.UNIT, "cores": 128, "kind": "oracle", "sample": "s" * 80}}
+    line, details = bench.report(out)
+    assert len(line) < 2400 and "\n" not in line
+    got, rest = json.loads(line), json.loads(details)
+    assert set(got) == set(out) - {"extra"} and got["value"] == num == got["ms_per_step"]
+    assert rest["extra"] == out["extra"] and rest["roofline"]["timing"] == "t" * 200 and rest["clocks"]["window"] == "z" * 100
+    assert got["clocks"]["reasons"] == ["sw_power_cap"] and got["e2e"]["h2d_bytes_per_step"] == 10 ** 9
