@@ -891,21 +891,12 @@ extern "C" lpdt_status lpdt_qconv_bwd_data_affine(const lpdt_conv_desc *d, const
 static size_t affine_wg_raw_bytes(const lpdt_conv_desc *d) {
     return align_up((size_t)d->nodes * d->Cout * d->R * d->S * d->Cin * sizeof(int32_t), 256);
 }
-// (colE and colA: part of the size that callers are asked for; not written)
-static size_t affine_colE_bytes(const lpdt_conv_desc *d) {
-    const int Ho = conv_out(d->H, d->pad, d->R, d->stride), Wo = conv_out(d->W, d->pad, d->S, d->stride);
-    return align_up((size_t)d->nodes * Ho * Wo * d->Cout * sizeof(int32_t), 256);
-}
-static size_t affine_colA_bytes(const lpdt_conv_desc *d) {
-    return align_up((size_t)d->nodes * d->H * d->W * d->Cin * sizeof(int32_t), 256);
-}
 static size_t affine_tab_bytes(const lpdt_conv_desc *d, int C) {
     return align_up((size_t)d->nodes * d->R * d->S * C * sizeof(int32_t), 256);
 }
 
 static size_t affine_bwd_weight_own(const lpdt_conv_desc *d) {
-    return affine_wg_raw_bytes(d) + affine_colE_bytes(d) + affine_colA_bytes(d) + affine_tab_bytes(d, d->Cout) +
-           affine_tab_bytes(d, d->Cin);
+    return affine_wg_raw_bytes(d) + affine_tab_bytes(d, d->Cout) + affine_tab_bytes(d, d->Cin);
 }
 
 extern "C" size_t lpdt_qconv_bwd_weight_affine_workspace_size(const lpdt_conv_desc *d) {
@@ -929,9 +920,7 @@ extern "C" lpdt_status lpdt_qconv_bwd_weight_affine(const lpdt_conv_desc *d, con
     cudaStream_t st = as_stream(stream);
     const int Ho = conv_out(d->H, d->pad, d->R, d->stride), Wo = conv_out(d->W, d->pad, d->S, d->stride);
     int32_t *raw = (int32_t *)ws;
-    int32_t *colE = (int32_t *)((char *)ws + affine_wg_raw_bytes(d));
-    int32_t *colA = (int32_t *)((char *)colE + affine_colE_bytes(d));
-    int32_t *tabE = (int32_t *)((char *)colA + affine_colA_bytes(d));
+    int32_t *tabE = (int32_t *)((char *)ws + affine_wg_raw_bytes(d));
     int32_t *tabA = (int32_t *)((char *)tabE + affine_tab_bytes(d, d->Cout));
     void *inner = (char *)tabA + affine_tab_bytes(d, d->Cin);
     s = bwd_weight_impl(d, reinterpret_cast<const int8_t *>(E), nullptr, reinterpret_cast<const int8_t *>(A), nullptr,

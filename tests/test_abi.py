@@ -51,3 +51,13 @@ def test_recorded_calls_are_checked():
     for bad in ([77, 0], [-1, 0], [sgd, 1, 0, 0, 0, 0, 0], empty[:-1], [api.CALL_WAIT, 0, 0], [api.CALL_WAIT, 0, 1, 1],
                 [api.CALL_WAIT, 0, 0, 0]):
         assert api.lpdt_run_calls(code(*bad), [0])[0] == 1, bad
+
+
+def test_zero_point_backward_weight_asks_for_what_it_writes():
+    """Raw sums and the two tables of tap sums, besides the contraction's own workspace: nothing that grows with the image."""
+    from paper_2111_09389_b200 import api
+    up = lambda n: (n + 255) // 256 * 256
+    for nodes, H, cin, cout, R in ((1, 8, 64, 32, 3), (3, 56, 64, 32, 3), (2, 20, 48, 80, 1), (2, 9, 7, 10, 3)):
+        d = api.conv_desc(nodes, 4, H, H, cin, cout, R, R, 1, R // 2)
+        own = up(4 * nodes * R * R * cin * cout) + up(4 * nodes * R * R * cout) + up(4 * nodes * R * R * cin)
+        assert api.lpdt_qconv_bwd_weight_affine_workspace_size(d) == own + api.lpdt_qconv_workspace_size(d, 2)
