@@ -306,7 +306,9 @@ extern "C" lpdt_status lpdt_dequantize_acc_batch(const int32_t *acc, int32_t nod
         if (sizes[t] > longest) longest = sizes[t];
     }
     if (longest == 0) return LPDT_OK;
-    int bx = (int)ceil_div(longest, 256 * 4);
+    // sixteen sums a thread: with four, the blocks past the end of the shorter tensors were most of the work (20 layers of
+    // ResNet-20 on 40 nodes: 28800 blocks of which 6000 had any, 37.7 us; 14.8 now)
+    int bx = (int)ceil_div(longest, 256 * 16);
     if (bx > 64) bx = 64;
     if (bx < 1) bx = 1;
     launch_k(dequant_acc_batch_kernel, dim3(bx, nodes, n_tensors), 256, 0, as_stream(stream), acc, db, out,
