@@ -177,11 +177,19 @@ static bool use_tc(const lpdt_conv_desc &d, int which, const void *ws, size_t ws
 // few dozen steps, and few steps in all (a classifier's scores and their adjoint, a small first layer).  The tensor-core
 // kernel's fixed cost (padded copies, barriers, TMEM, first boxes) is 6-8 us.  Measured, CUDA cores against tensor cores:
 // 40 x 32 x 64 -> 10 forward 2.8 / 6.0 us and its adjoint 4.9 / 5.6, 8 x 32 x 512 -> 10 forward 9.9 / 6.7; 3x3 from 3
-// channels 5.0 / 7.3 us at 65 K results (1.8 M steps), 9.1 / 7.6 at 131 K, 11.8 / 7.6 at 262 K.  Only shapes that need
+// channels 5.0 / 7.3 us at 65 K results (1.8 M steps), 9.1 / 7.6 at 131 K, 11.8 / 7.6 at 262 K; zero-point backward-data
+// of 7 x 34 rows, 11 -> 751 (2.0 M steps) 16 / 21 us in all, 2 x 113 rows, 12 -> 115 9.5 / 16.5.  Only shapes that need
 // padding; the others fill the tiles.
 static bool tiny_dot(const lpdt_conv_desc &d, int64_t results, int K, bool vec4) {
     const int steps = vec4 ? K / 4 : K;
-    return (d.Cin % 16 || d.Cout % 16) && steps <= 64 && results * steps <= (int64_t)kNumSMs * 12288;
+    return (d.Cin % 16 || d.Cout % 16) && steps <= 64 && results * steps <= (int64_t)kNumSMs * 16384;
+}
+static bool tiny_fwd(const lpdt_conv_desc &d, const int8_t *A, const int8_t *Wq) {
+    const int64_t results = (int64_t)d.nodes * d.B * conv_out(d.H, d.pad, d.R, d.stride) * conv_out(d.W, d.pad, d.S, d.stride) * d.Cout;
+    return tiny_dot(d, results, d.R * d.S * d.Cin, d.Cin % 4 == 0 && aligned(A, 4) && aligned(Wq, 4));
+}
+static bool tiny_bwd_data(const lpdt_conv_desc &d, const int8_t *E) {
+    return tiny_dot(d, (int64_t)d.nodes * d.B * d.H * d.W * d.Cin, d.R * d.S * d.Cout, d.Cout % 4 == 0 && aligned(E, 4));
 }
 // An operand of `C` channels the engine can read: its padded copy, or itself at a 16-byte boundary.
 static bool readable(const void *p, int C) { return C % 16 != 0 || aligned(p, 16); }
@@ -193,10 +201,7 @@ static lpdt_status fwd_impl(const lpdt_conv_desc *d, const int8_t *A, const floa
                             void *ws, size_t ws_bytes, int32_t *dev_status, cudaStream_t st, bool uns,
                             const tc::AffineArgs *aff = nullptr) {
     const bool out_ok = (!Y || aligned(Y, 16)) && (!Yacc || aligned(Yacc, 16));
-    const int64_t results = (int64_t)d->nodes * d->B * conv_out(d->H, d->pad, d->R, d->stride) *
-                            conv_out(d->W, d->pad, d->S, d->stride) * d->Cout;
-    const bool vec4 = d->Cin % 4 == 0 && aligned(A, 4) && aligned(Wq, 4);
-    if ((aff || !tiny_dot(*d, results, d->R * d->S * d->Cin, vec4)) && use_tc(*d, 0, ws, ws_bytes) && readable(A, d->Cin) && readable(Wq, d->Cin) && out_ok) {
+    if (!tiny_fwd(*d, A, Wq) && use_tc(*d, 0, ws, ws_bytes) && readable(A, d->Cin) && readable(Wq, d->Cin) && out_ok) {
         const bool pad = d->Cin % 16 != 0;
         const int8_t *Ae = A, *We = Wq;
         if (pad) {
@@ -291,6 +296,17 @@ __global__ void weight_prefix_kernel(const int32_t *__restrict__ tapsum, int nod
 // Block (16 result channels, node): tap sums in shared memory, prefix sums over the taps, table written out.  One thread
 // per entry with a serial loop over the other channels took 15.9 us at 8 x 128 x 128 x 9 for the sums alone.
 constexpr int kTabC = 16;
+__host__ __device__ inline int table_lanes(const lpdt_conv_desc &d) {
+    return d.R * d.S == 1 && (d.Cin >= 2048 || d.Cin % 16) ? 32 : 8;      // (ragged rows are read byte by byte)
+}
+// Threads per block: forward, a group of lanes per row, up to 1024 (144 rows of a 3x3 filter in two goes); backward-data,
+// whose sums meet in atomics, one per row of 16 bytes, up to 512.  (1024 and 512 throughout: 13 nodes of 512 -> 1536 took
+// 17.9 us, four waves of blocks with half of their threads idle, and the whole product 26.8 us; 14.2 now.)
+static int table_threads(const lpdt_conv_desc &d, int over_cout) {
+    const int64_t rows = over_cout ? (int64_t)d.R * d.S * d.Cout : (int64_t)d.R * d.S * kTabC * table_lanes(d), most = over_cout ? 512 : 1024;
+    const int64_t t = (rows + 31) / 32 * 32;
+    return (int)(t < 64 ? 64 : t > most ? most : t);
+}
 __global__ void __launch_bounds__(1024)
 weight_table_kernel(lpdt_conv_desc d, const uint8_t *__restrict__ Wq, int over_cout, int st, bool vec16, bool vec4, int32_t *__restrict__ P) {
     pdl_enter();
@@ -337,8 +353,8 @@ weight_table_kernel(lpdt_conv_desc d, const uint8_t *__restrict__ Wq, int over_c
             }
         }
     } else {
-        // eight lanes per row (output channel, tap), 32 where one row each fills the block
-        const int G = taps == 1 ? 32 : 8, lane = tid & (G - 1);
+        // eight lanes per row (output channel, tap), 32 where there are few and long ones
+        const int G = table_lanes(d), lane = tid & (G - 1);
         for (int row = tid / G; row < taps * kTabC; row += T / G) {
             const int tap = row % taps, c = row / taps;
             unsigned sum = 0;
@@ -373,8 +389,6 @@ weight_table_kernel(lpdt_conv_desc d, const uint8_t *__restrict__ Wq, int over_c
     for (int i = tid; i < cells * kTabC; i += T)
         if ((i & (kTabC - 1)) < nc) P[((int64_t)n * cells + i / kTabC) * C + c0 + (i & (kTabC - 1))] = (int32_t)pre[i];
 }
-// Threads per block: forward 1024 (144 rows of a 3x3 filter in two goes), backward-data 512 (their sums meet in atomics).
-static int table_threads(int over_cout) { return over_cout ? 512 : 1024; }
 // Shapes the kernel above takes: a thread per tap, the tables in 48 KB of shared memory, nodes in grid.y.
 static bool table_fits(const lpdt_conv_desc &d, int st) {
     return d.R * d.S <= 256 && ((int64_t)d.R * d.S + (int64_t)(d.R + st) * (d.S + st)) * kTabC * 4 <= 48 * 1024 && d.nodes <= 65535;
@@ -383,7 +397,7 @@ static lpdt_status weight_table_launch(const lpdt_conv_desc &d, const uint8_t *W
     const int C = over_cout ? d.Cin : d.Cout;
     const size_t smem = ((size_t)d.R * d.S + (size_t)(d.R + st) * (d.S + st)) * kTabC * 4;
     const bool vec16 = d.Cin % 16 == 0 && aligned(Wq, 16);
-    launch_k(weight_table_kernel, dim3((unsigned)ceil_div(C, kTabC), d.nodes), table_threads(over_cout), smem, stream, d, Wq, over_cout, st, vec16,
+    launch_k(weight_table_kernel, dim3((unsigned)ceil_div(C, kTabC), d.nodes), table_threads(d, over_cout), smem, stream, d, Wq, over_cout, st, vec16,
              d.Cin % 4 == 0 && aligned(Wq, 4), P);
     LPDT_LAUNCH_CHECK();
     return LPDT_OK;
@@ -564,10 +578,8 @@ static lpdt_status bwd_data_impl(const lpdt_conv_desc *d, const int8_t *E, const
                                  const float *sW, float *dA, int32_t *dAacc, const float *addend, void *ws,
                                  size_t ws_bytes, int32_t *dev_status, cudaStream_t st, bool uns,
                                  const tc::AffineArgs *aff = nullptr) {
-    const int64_t results = (int64_t)d->nodes * d->B * d->H * d->W * d->Cin;
-    const bool vec4 = d->Cout % 4 == 0 && aligned(E, 4);
-    if ((aff || !tiny_dot(*d, results, d->R * d->S * d->Cout, vec4)) && use_tc(*d, 1, ws, ws_bytes) && readable(E, d->Cout) && readable(Wq, d->Cin) && (!dA || aligned(dA, 16)) &&
-        (!dAacc || aligned(dAacc, 16))) {
+    if (!tiny_bwd_data(*d, E) && use_tc(*d, 1, ws, ws_bytes) && readable(E, d->Cout) && readable(Wq, d->Cin) &&
+        (!dA || aligned(dA, 16)) && (!dAacc || aligned(dAacc, 16))) {
         const int Ho = conv_out(d->H, d->pad, d->R, d->stride), Wo = conv_out(d->W, d->pad, d->S, d->stride);
         const PadPlan pp = pad_plan(*d);
         void *Ep = ws, *Wp = (char *)ws + pp.err;
@@ -865,7 +877,8 @@ extern "C" lpdt_status lpdt_qconv_bwd_data_affine(const lpdt_conv_desc *d, const
     // sums, which do not exist then.  8 x 32 x 16x16 128 -> 128 3x3: 34.8 us, 107.5 us with the raw sums written and
     // corrected in a second pass (80 us of them), which shapes outside the tensor-core path still take.
     const size_t table = (size_t)d->nodes * (d->R + d->stride) * (d->S + d->stride) * d->Cin * sizeof(int32_t);
-    if (!affine_separate() && table_fits(*d, d->stride) && table <= affine_bwd_data_raw_bytes(d) && use_tc(*d, 1, inner, inner_bytes)) {
+    if (!affine_separate() && !tiny_bwd_data(*d, reinterpret_cast<const int8_t *>(E)) && table_fits(*d, d->stride) &&
+        table <= affine_bwd_data_raw_bytes(d) && use_tc(*d, 1, inner, inner_bytes)) {
         s = weight_table_launch(*d, Wq, 1, d->stride, raw, st);
         if (s != LPDT_OK) return s;
         const tc::AffineArgs aff = {esum, raw, zE, zW};

@@ -230,7 +230,7 @@ def test_qconv_bwd_affine(case):
 
 
 # channel counts that no 16-byte row holds, or that end inside a box of the tensor-core kernels.  (cc): forward products so
-# small that they run on the CUDA cores; backward-weight and the zero-point products take the tensor cores all the same
+# small that they run on the CUDA cores; backward-weight takes the tensor cores all the same
 RAGGED_CASES = [
     (2, 130, 1, 1, 200, 270, 1, 1, 1, 0),    # linear: 200 = 128 + 72 inputs, results in rows of 270 (no 16-byte rows)
     (1, 300, 1, 1, 1001, 17, 1, 1, 1, 0),    # odd on both sides, three row tiles
@@ -329,8 +329,17 @@ def test_padded_copies_of_many_rows(rows, cin, skew):
     assert torch.equal(Y.double(), torch.from_numpy(A).cuda().double() @ torch.from_numpy(Wq).cuda().double().t())
 
 
+# the table of the weights' sums: blocks of every size (one row of lanes, few and long rows, several goes), both directions
+@pytest.mark.parametrize("case", [(2, 40, 1, 1, 2064, 48, 1, 1, 1, 0), (13, 70, 1, 1, 512, 96, 1, 1, 1, 0), (1, 2000, 1, 1, 64, 16, 1, 1, 1, 0),
+                                  (2, 6, 9, 9, 32, 16, 3, 3, 1, 1), (1, 3, 12, 12, 48, 32, 2, 2, 1, 0), (1, 2, 10, 10, 16, 16, 1, 3, 2, 1),
+                                  (1, 40, 8, 8, 20, 650, 1, 1, 1, 0), (2, 113, 1, 1, 115, 12, 1, 1, 1, 0)])
+def test_zero_point_weight_tables(case):
+    test_qconv_fwd_affine(case)
+    test_qconv_bwd_affine(case)
+
+
 # forward products on both sides of the line between CUDA cores and tensor cores, with the kernel that each takes: up to 64
-# steps a result (4 channels each where rows allow it) and 148 * 12288 steps in all
+# steps a result (4 channels each where rows allow it) and 148 * 16384 steps in all
 @pytest.mark.parametrize("case,kernel", [
     ((4, 4, 16, 16, 3, 16, 3, 3, 1, 1), "conv_fwd_generic"),        # 65 K results of 27 steps
     ((4, 4, 16, 16, 3, 32, 3, 3, 1, 1), "conv_halo16_kernel"),      # 131 K: a first layer of 3 channels
