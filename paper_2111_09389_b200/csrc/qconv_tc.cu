@@ -703,49 +703,36 @@ conv_wgrad_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
                 }
                 valid = valid && (ci < p.Cin);
                 const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + t * p.BNc;
-                const int cols = p.Cout - n0 < p.BNc ? p.Cout - n0 : p.BNc;
-                const int full = cols & ~15;
-                const long long cell = (long long)n0 * cstride + (long long)tap * p.Cin + ci;
-                int32_t *acc = p.acc_out + (long long)node * p.Cout * cstride + cell;
-                float *dst = p.dW + (long long)node * p.dw_stride + cell;
-                int c = 0;
-                if (p.splits > 1) {
-                    for (; c < full; c += 16, acc += 16 * cstride) {
-                        uint32_t v[16];
-                        tmem_ld_32x16(t_row + c, v);
-                        tmem_ld_wait();
-                        if (!valid) continue;
+                for (int c = 0; c < p.BNc && n0 + c < p.Cout; c += 16) {
+                    uint32_t v[16];
+                    tmem_ld_32x16(t_row + c, v);
+                    tmem_ld_wait();
+                    if (!valid) continue;
+                    const long long o = ((long long)(n0 + c) * p.taps + tap) * p.Cin + ci;
+                    int32_t *acc = p.acc_out + (long long)node * p.Cout * cstride + o;
+                    const int nk = p.Cout - n0 - c;
+                    if (nk < 16) {                               // the N group reaches past the last channel
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) {
+                            if (k >= nk) continue;
+                            if (p.splits > 1) { if ((int)v[k] != 0) atomicAdd(acc + k * cstride, (int)v[k]); continue; }
+                            if (p.acc_out) acc[k * cstride] = (int)v[k];
+                            if (p.dW) p.dW[(long long)node * p.dw_stride + o + k * cstride] = __fmul_rn(__int2float_rn((int)v[k]), sc);
+                        }
+                    } else if (p.splits > 1) {
 #pragma unroll
                         for (int k = 0; k < 16; ++k)
                             if ((int)v[k] != 0) atomicAdd(acc + k * cstride, (int)v[k]);
-                    }
-                } else {
-                    for (; c < full; c += 16, acc += 16 * cstride, dst += 16 * cstride) {
-                        uint32_t v[16];
-                        tmem_ld_32x16(t_row + c, v);
-                        tmem_ld_wait();
-                        if (!valid) continue;
+                    } else {
                         if (p.acc_out) {
 #pragma unroll
                             for (int k = 0; k < 16; ++k) acc[k * cstride] = (int)v[k];
                         }
                         if (p.dW) {
+                            float *dst = p.dW + (long long)node * p.dw_stride + o;
 #pragma unroll
                             for (int k = 0; k < 16; ++k) dst[k * cstride] = __fmul_rn(__int2float_rn((int)v[k]), sc);
                         }
-                    }
-                }
-                if (full < cols) {                               // the N group ends inside 16 channels
-                    uint32_t v[16];
-                    tmem_ld_32x16(t_row + full, v);
-                    tmem_ld_wait();
-                    const int nk = valid ? cols - full : 0;
-#pragma unroll
-                    for (int k = 0; k < 16; ++k) {
-                        if (k >= nk) continue;
-                        if (p.splits > 1) { if ((int)v[k] != 0) atomicAdd(acc + k * cstride, (int)v[k]); continue; }
-                        if (p.acc_out) acc[k * cstride] = (int)v[k];
-                        if (p.dW) dst[k * cstride] = __fmul_rn(__int2float_rn((int)v[k]), sc);
                     }
                 }
             }
@@ -1059,7 +1046,10 @@ lpdt_status tc_wgrad(const lpdt_conv_desc &d, const int8_t *E, const float *sE, 
     // give the SMs work, than a split of a loop of a few blocks whose partial sums meet in atomics: the narrowest that
     // leave one tile per SM at most.  (Up to 64 output tiles of the wide groups; from 128 tiles on the split wins.
     // 2 nodes x 815 rows, 128 -> 304: groups of 192 8.1 us, of 16 4.6 us; 8 x 256 rows, 704 -> 160: 160 6.1, 64 4.6 us.)
-    const bool short_k = !p.halo && p.kblocks <= 16 && (long long)d.nodes * all_tiles * ceil_div(d.Cout, p.BNc) <= 64;
+    // Not where a block of pixels takes many boxes (eight taps of 16 channels): a CTA fetches about one in 130 ns (6 images of
+    // 14x14, 16 -> 176 3x3: 14.7 us, split 9.7).
+    const bool short_k = !p.halo && p.kblocks * (1 + (p.total_units < G ? p.total_units : G)) <= 64 && p.kblocks <= 16 &&
+                         (long long)d.nodes * all_tiles * ceil_div(d.Cout, p.BNc) <= 64;
     if (short_k) {
         for (int bn = 16; bn <= 128 && bn <= p.BNc; bn *= 2)
             if ((long long)d.nodes * all_tiles * ceil_div(d.Cout, bn) <= kNumSMs) { p.BNc = p.RBe = bn; break; }
