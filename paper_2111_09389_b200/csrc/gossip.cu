@@ -1,9 +1,10 @@
 // Gossip step of CHOCO-SGD (Algorithm 3) for all simulated nodes at once:
 // exact top-k selection of x_half - x_hat per (node, segment) by radix select
 // on the magnitude bits, then one fused streaming pass that updates the public
-// copies and mixes.  The mix pass is HBM-bound: per parameter and node it reads
-// x_half and x_hat and writes x_hat and x (16 bytes); the neighbours' updated
-// x_hat values are exchanged through shared memory, never re-read from HBM.
+// copies and mixes.  Per parameter and node that pass reads x_half and x_hat and
+// writes x, and x_hat where it changed (12 bytes and few more with top-k, 16 where
+// everything is sent); the neighbours' updated x_hat values are exchanged through
+// shared memory, never re-read from HBM.
 #include "common.cuh"
 
 namespace lpdt {
@@ -203,7 +204,6 @@ __device__ void select_whole_segment(const float *__restrict__ xh, const float *
 struct BigList {
     int32_t n;
     int32_t id[kMaxSeg];               // segment index
-    int32_t chunk_base[kMaxSeg + 1];   // prefix sums of the chunk counts
     int64_t cand_base[kMaxSeg + 1];    // prefix sums of the candidate capacities
 };
 constexpr int kTopBins = 4096;
@@ -222,9 +222,14 @@ __device__ void pick_bucket(const uint32_t *hist, int nbins, long long need, int
                             long long *need_out, long long *eq_out) {
     __shared__ long long wtot[32];
     __shared__ long long res[3];
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5, nwarps = blockDim.x >> 5, per = nbins / blockDim.x;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5, nwarps = blockDim.x >> 5, per = nbins / blockDim.x;   // <= 16
+    // the thread's bins stay in registers: walked in memory, they were up to 15 dependent reads of L2
+    uint32_t bins[16];
     long long mine = 0;
-    for (int b = 0; b < per; ++b) mine += __ldcg(hist + t * per + b);
+#pragma unroll
+    for (int b = 0; b < 16; ++b) bins[b] = b < per ? __ldcg(hist + t * per + b) : 0u;
+#pragma unroll
+    for (int b = 0; b < 16; ++b) mine += bins[b];
     // suffix sums over the 256 slices: inside the warp by shuffles, across warps through shared memory
     long long incl = mine;
 #pragma unroll
@@ -239,13 +244,13 @@ __device__ void pick_bucket(const uint32_t *hist, int nbins, long long need, int
     for (int w = warp + 1; w < nwarps; ++w) above += wtot[w];
     if (above < need && need <= above + mine) {
         long long n = need - above;
-        int b = t * per + per - 1;
-        for (; b > t * per; --b) {
-            const long long hb = __ldcg(hist + b);
-            if (hb >= n) break;
-            n -= hb;
+        bool found = false;
+#pragma unroll
+        for (int b = 15; b >= 0; --b) {
+            if (b >= per || found) continue;
+            if (bins[b] >= n || b == 0) { found = true; res[0] = t * per + b; res[1] = n; res[2] = bins[b]; }
+            else n -= bins[b];
         }
-        res[0] = b; res[1] = n; res[2] = __ldcg(hist + b);
     }
     __syncthreads();
     *bucket = (int)res[0]; *need_out = res[1]; *eq_out = res[2];
@@ -417,14 +422,13 @@ big_collect_kernel(const float *__restrict__ x_half, const float *__restrict__ x
 // number in *count: one pass of the CTA over the list, 16 loads of a thread in flight, one reservation per warp and
 // round (a reservation per key put 29 K atomics on one shared-memory word: 8.65 M normal values, top 1 %, took 163 us
 // for the whole selection, 57 us now).
-template <typename Take, typename What>
-__device__ void gather(const Cand *__restrict__ list, int64_t n, int cap, uint32_t *dst, unsigned int *count, Take take, What what) {
+template <int kU, typename Take, typename What>
+__device__ void gather_by(const Cand *__restrict__ list, int64_t n, int cap, uint32_t *dst, unsigned int *count, Take take, What what) {
     const unsigned long long *l64 = reinterpret_cast<const unsigned long long *>(list);
     const int lane = threadIdx.x & 31;
     __syncthreads();
     if (threadIdx.x == 0) *count = 0;
     __syncthreads();
-    constexpr int kU = 16;
     for (int64_t base = 0; base < n; base += kU * (int64_t)blockDim.x) {
         unsigned long long c[kU];
 #pragma unroll
@@ -450,6 +454,12 @@ __device__ void gather(const Cand *__restrict__ list, int64_t n, int cap, uint32
             if ((hits >> u) & 1u) { if (at < (unsigned)cap) dst[at] = what(c[u]); ++at; }
     }
     __syncthreads();
+}
+
+template <typename Take, typename What>
+__device__ void gather(const Cand *__restrict__ list, int64_t n, int cap, uint32_t *dst, unsigned int *count, Take take, What what) {
+    if (n > 4 * (int64_t)blockDim.x) gather_by<16>(list, n, cap, dst, count, take, what);
+    else gather_by<2>(list, n, cap, dst, count, take, what);           // sixteen mostly empty rounds took longer than the list
 }
 
 // Threshold and tie cut of a long segment from its candidate list (one CTA).  The list holds every key of the
@@ -966,7 +976,7 @@ static lpdt_status gossip_impl(int32_t nodes, int64_t d, const float *x_half, fl
     SelectOut *sel = (SelectOut *)ws;
     int32_t *tab = (int32_t *)((char *)ws + select_bytes(nodes, n_segments));
     BigList big;
-    big.n = 0; big.chunk_base[0] = 0; big.cand_base[0] = 0;
+    big.n = 0; big.cand_base[0] = 0;
     int64_t most_chunks = 0, longest = 0;
     double most_kept = 0.0;                     // largest share of a long segment that is kept
     for (int s = 0; s < n_segments; ++s) {
@@ -975,7 +985,6 @@ static lpdt_status gossip_impl(int32_t nodes, int64_t d, const float *x_half, fl
         if (len > 0xFFFFFFFFll) return LPDT_ERR_UNSUPPORTED;      // candidate positions are 32-bit
         const int64_t nc = ceil_div(len, (int64_t)kChunk);
         big.id[big.n] = s;
-        big.chunk_base[big.n + 1] = big.chunk_base[big.n] + (int32_t)nc;
         big.cand_base[big.n + 1] = big.cand_base[big.n] + cand_capacity(len);
         if (nc > most_chunks) most_chunks = nc;
         if (len > longest) longest = len;
