@@ -646,13 +646,14 @@ select_and_rows_kernel(const float *__restrict__ x_half, const float *__restrict
 // the updated state where it changed, parks the public copies in shared memory, and after one barrier mixes its nodes
 // with their neighbours' copies; x_half stays in registers between the two halves.  Two parking buffers alternate, so a
 // tile costs one barrier.  The mixing rows, and the thresholds while the segment stays the same, are read once per CTA.
-// HBM-bound: x_half, x_hat read, x written, 12 B per parameter and node.  (The form before, a thread per parameter
-// looping over the nodes, kept 128 registers and four CTAs of 128 threads per SM, decided the segment and read the
-// thresholds again for every parameter and node and read x_half twice: 16 x 8.65 M, top 1 %, 461 us; this one 413 us.)
+// Bytes per parameter and node: x_half, x_hat read, x written, 12 with top-k; 16 for dense segments and Deep-Squeeze, which
+// rewrite the state everywhere.  16 x 8.65 M, top 1 %: 413 us, 4.0 TB/s or 62 % of the copy rate; what keeps it from the
+// rest is 48 streams, read and written, of which a tile takes 1 KB each.  (A thread per two parameters looping over the nodes,
+// the form below, keeps 128 registers and four CTAs of 128 threads per SM, decides the segment and reads the thresholds
+// again for every parameter and node and reads x_half twice: 461 us.)
 // ds: Deep-Squeeze form (supplementary Algorithm 2): the state array is the error buffer, the message is the
 // compressed x_half + state, the buffer keeps what was not sent and the mix runs over the messages themselves.
 // q8: the message is the 8-bit code times the step of its (node, segment).
-__host__ __device__ constexpr int mix_el(int npw) { return npw == 1 ? 8 : 4; }           // parameters per lane and node
 struct MixRule { uint32_t thr; uint32_t dense; int64_t cut; float scale, inv; };
 __device__ __forceinline__ MixRule mix_rule(const SelectOut *sel, const float *msg_scale, const float *msg_inv, int64_t at, bool q8) {
     const SelectOut so = sel[at];
@@ -661,14 +662,14 @@ __device__ __forceinline__ MixRule mix_rule(const SelectOut *sel, const float *m
     r.scale = q8 ? msg_scale[at] : 1.f; r.inv = q8 ? msg_inv[at] : 1.f;
     return r;
 }
-template <int V, int NPW>
-__global__ void __launch_bounds__(NPW == 1 ? 512 : 640, 2)
+template <int V, int NPW, int EL, int THREADS>
+__global__ void __launch_bounds__(THREADS, 2)
 gossip_mix_kernel(int nodes, int64_t d, const float *x_half, float *x_hat, float *x_out, float gamma, SegTable seg,
                   const SelectOut *__restrict__ sel, const int32_t *__restrict__ tab, const float *__restrict__ msg_scale,
                   const float *__restrict__ msg_inv, bool q8, bool ds) {
     pdl_enter();
     extern __shared__ __align__(16) float sm[];
-    constexpr int EL = mix_el(NPW), U = EL / V, TILE = 32 * EL;
+    constexpr int U = EL / V, TILE = 32 * EL;
     const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int32_t *s_cnt = reinterpret_cast<int32_t *>(sm);            // [nodes]
     int32_t *s_idx = s_cnt + nodes;                              // [nodes][nodes]
@@ -782,6 +783,106 @@ gossip_mix_kernel(int nodes, int64_t d, const float *x_half, float *x_hat, float
                 }
                 VecIO<V>::st(x_out + (int64_t)i * d + e, o);
             }
+        }
+    }
+}
+
+// The same for fp32 messages with a thread per two parameters that loops over the nodes: a CTA owns 2 * blockDim.x parameters,
+// streams x_half and the state of every node, parks the public copies in shared memory (each read back by the thread that
+// wrote it: no barrier) and reads x_half again for the mix.  With rows of 8-byte accesses (the networks' parameter counts),
+// 6 to 24 nodes and arrays beyond L2 it stays ahead of the kernel above: 8 x 3.75 M, top 1 %, 110 us against 123;
+// 16 x 1.9 M 118 / 123; 24 x 1.25 M 129 / 137; the whole call on 8 x 1.08 M 76.2 / 78.8, on 12 x 1.08 M 97.8 / 106.  (2 x 15 M
+// 212 / 156, 32 x 0.94 M 147 / 144, 16-byte rows, 16 x 1.9 M, 125 / 105; the whole call on 16 x 270410 58.8 / 56.9.)
+__global__ void __launch_bounds__(256)
+gossip_mix_columns_kernel(int nodes, int64_t d, const float *__restrict__ x_half, float *__restrict__ x_hat,
+                          float *__restrict__ x_out, float gamma, SegTable seg, const SelectOut *__restrict__ sel,
+                          const int32_t *__restrict__ tab) {
+    pdl_enter();
+    constexpr int V = 2;
+    extern __shared__ __align__(16) float sm[];
+    const int TE = blockDim.x;
+    int32_t *s_cnt = reinterpret_cast<int32_t *>(sm);            // [nodes]
+    int32_t *s_idx = s_cnt + nodes;                              // [nodes][nodes]
+    float *s_val = reinterpret_cast<float *>(s_idx + nodes * nodes);
+    const int tab_words = nodes + 2 * nodes * nodes;
+    float *s_hat = sm + ((tab_words + 3) & ~3);                  // [nodes][TE][V], 16-byte aligned
+    for (int i = threadIdx.x; i < tab_words; i += TE) s_cnt[i] = tab[i];
+    __syncthreads();       // the only block-wide wait: the parked copies below are read back by the thread that wrote them
+    const int64_t e0 = ((int64_t)blockIdx.x * TE + threadIdx.x) * V;
+    const bool live = e0 < d;                                    // d % V == 0: a thread is all in or all out
+    int s0 = 0;
+    bool one_seg = true;
+    if (live) {   // segment of the first parameter (segments tile [0,d))
+        int a = 0, b = seg.n_seg;
+        while (b - a > 1) { int m = (a + b) >> 1; if (seg.off[m] <= e0) a = m; else b = m; }
+        s0 = a;
+        one_seg = seg.off[s0 + 1] >= e0 + V;
+    }
+    constexpr int kU = 4;                                        // nodes per batch of independent loads (as measured)
+    for (int ib = 0; ib < nodes; ib += kU) {
+        float xh[kU][V], xq[kU][V];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            if (live && ib + u < nodes) {
+                VecIO<V>::ld(x_half + (int64_t)(ib + u) * d + e0, xh[u]);
+                VecIO<V>::ld(x_hat + (int64_t)(ib + u) * d + e0, xq[u]);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const int i = ib + u;
+            if (i >= nodes) break;
+            float hn[V];
+#pragma unroll
+            for (int k = 0; k < V; ++k) hn[k] = 0.f;
+            if (live) {
+                SelectOut so = sel[(int64_t)i * seg.n_seg + s0];
+                bool changed = false;      // the public copy changes only where an entry is sent (top-k: 1 in 100)
+#pragma unroll
+                for (int k = 0; k < V; ++k) {
+                    if (!one_seg && k > 0) {
+                        int sk = s0;
+                        while (seg.off[sk + 1] <= e0 + k) ++sk;
+                        so = sel[(int64_t)i * seg.n_seg + sk];
+                    }
+                    const float delta = __fsub_rn(xh[u][k], xq[u][k]);
+                    const uint32_t key = __float_as_uint(delta) & 0x7fffffffu;
+                    const bool keep = so.dense || key > so.thr || (key == so.thr && e0 + k < so.cut);
+                    changed |= keep;
+                    hn[k] = keep ? __fadd_rn(xq[u][k], delta) : xq[u][k];      // public copy + message, what the neighbours mix
+                }
+                if (changed) VecIO<V>::st(x_hat + (int64_t)i * d + e0, hn);      // unchanged values are not rewritten
+            }
+            VecIO<V>::st(s_hat + ((size_t)i * TE + threadIdx.x) * V, hn);
+        }
+    }
+    if (!live) return;
+    for (int ib = 0; ib < nodes; ib += kU) {
+        float xh[kU][V];
+#pragma unroll
+        for (int u = 0; u < kU; ++u)
+            if (ib + u < nodes) VecIO<V>::ld(x_half + (int64_t)(ib + u) * d + e0, xh[u]);
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const int i = ib + u;
+            if (i >= nodes) break;
+            float hi_[V], acc[V], o[V];
+            VecIO<V>::ld(s_hat + ((size_t)i * TE + threadIdx.x) * V, hi_);
+#pragma unroll
+            for (int k = 0; k < V; ++k) acc[k] = 0.f;
+            const int c = s_cnt[i];
+            for (int m = 0; m < c; ++m) {                        // neighbours in ascending j
+                const int j = s_idx[i * nodes + m];
+                const float w = s_val[i * nodes + m];
+                float hj[V];
+                VecIO<V>::ld(s_hat + ((size_t)j * TE + threadIdx.x) * V, hj);
+#pragma unroll
+                for (int k = 0; k < V; ++k)
+                    acc[k] = __fadd_rn(acc[k], __fmul_rn(w, __fsub_rn(hj[k], hi_[k])));      // sum_j W_ij (xhat_j - xhat_i)
+            }
+#pragma unroll
+            for (int k = 0; k < V; ++k) o[k] = __fadd_rn(xh[u][k], __fmul_rn(gamma, acc[k]));
+            VecIO<V>::st(x_out + (int64_t)i * d + e0, o);
         }
     }
 }
@@ -1051,30 +1152,41 @@ static lpdt_status gossip_impl(int32_t nodes, int64_t d, const float *x_half, fl
     const bool v4 = d % 4 == 0 && aligned(x_half, 16) && aligned(x_hat, 16) && aligned(x_out, 16);
     const bool v2 = !v4 && d % 2 == 0 && aligned(x_half, 8) && aligned(x_hat, 8) && aligned(x_out, 8);
     const int vi = v4 ? 2 : v2 ? 1 : 0;
-    // nodes per warp: one up to 16 nodes (CTAs of 512 threads); beyond, as few, at least two, as keep a CTA within 20 warps
-    const int npw = nodes <= 16 ? 1 : nodes <= 40 ? 2 : (int)ceil_div(nodes, 20), warps = (int)ceil_div(nodes, npw), tile = 32 * mix_el(npw);
     const size_t tab_words = ((size_t)nodes + 2 * (size_t)nodes * nodes + 3) & ~(size_t)3;
+    // Nodes per warp (NPW) and parameters per lane and node (EL): one node and 8 up to 16 nodes (CTAs of 512 threads); two
+    // and 8 up to 20 (CTAs of 320: 20 x 1.5 M, top 1 %, 111 us, 129 with tiles of 4); beyond, as few nodes as keep a CTA
+    // within 20 warps, and 4.
+    const int cfg = nodes <= 16 ? 0 : nodes <= 20 ? 1 : nodes <= 40 ? 2 : nodes <= 60 ? 3 : 4;
+    static const int npws[5] = {1, 2, 2, 3, 4}, els[5] = {8, 8, 4, 4, 4}, threads[5] = {512, 320, 640, 640, 640};
+    const int npw = npws[cfg], warps = (int)ceil_div(nodes, npw), tile = 32 * els[cfg];
     const size_t smem = tab_words * sizeof(int32_t) + 2 * (size_t)nodes * tile * sizeof(float);
-    using MixFn = void (*)(int, int64_t, const float *, float *, float *, float, SegTable, const SelectOut *,
-                           const int32_t *, const float *, const float *, bool, bool);
-    static const MixFn fns[3][4] = {
-        {gossip_mix_kernel<1, 1>, gossip_mix_kernel<1, 2>, gossip_mix_kernel<1, 3>, gossip_mix_kernel<1, 4>},
-        {gossip_mix_kernel<2, 1>, gossip_mix_kernel<2, 2>, gossip_mix_kernel<2, 3>, gossip_mix_kernel<2, 4>},
-        {gossip_mix_kernel<4, 1>, gossip_mix_kernel<4, 2>, gossip_mix_kernel<4, 3>, gossip_mix_kernel<4, 4>}};
-    const MixFn fn = fns[vi][npw - 1];
-    static PerDeviceOnce attr_set[3][4];
-    int dev;
-    if (attr_set[vi][npw - 1].pending(&dev)) {
-        LPDT_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024));
-        attr_set[vi][npw - 1].mark(dev);
-    }
     // as many CTAs as are resident together: two of the largest by their registers
-    int64_t per_sm = (npw == 1 ? 1024 : 1280) / (32 * warps);
+    int64_t per_sm = 2 * threads[cfg] / (32 * warps);
     if (per_sm > 24) per_sm = 24;
     if (per_sm * (int64_t)(smem + 1024) > 224 * 1024) per_sm = (int64_t)(224 * 1024) / (int64_t)(smem + 1024);
     if (per_sm < 1) per_sm = 1;
     int64_t blocks = ceil_div(d, tile);
     if (blocks > per_sm * kNumSMs) blocks = per_sm * kNumSMs;
+    if (v2 && nodes * d >= (int64_t)1 << 23 && !q8 && !ds && nodes >= 6 && nodes <= 24 && cfg != 1) {
+        const int TE = 128;                                      // 1 KB of shared memory per node
+        launch_k(gossip_mix_columns_kernel, (unsigned)ceil_div(d, (int64_t)TE * 2), TE,
+                 tab_words * sizeof(int32_t) + (size_t)nodes * TE * 2 * sizeof(float), st, nodes, d, x_half, x_hat, x_out, gamma, seg, sel, tab);
+        LPDT_LAUNCH_CHECK();
+        return LPDT_OK;
+    }
+    using MixFn = void (*)(int, int64_t, const float *, float *, float *, float, SegTable, const SelectOut *,
+                           const int32_t *, const float *, const float *, bool, bool);
+#define LPDT_MIX_ROW(V) {gossip_mix_kernel<V, 1, 8, 512>, gossip_mix_kernel<V, 2, 8, 320>, gossip_mix_kernel<V, 2, 4, 640>, \
+                         gossip_mix_kernel<V, 3, 4, 640>, gossip_mix_kernel<V, 4, 4, 640>}
+    static const MixFn fns[3][5] = {LPDT_MIX_ROW(1), LPDT_MIX_ROW(2), LPDT_MIX_ROW(4)};
+#undef LPDT_MIX_ROW
+    const MixFn fn = fns[vi][cfg];
+    static PerDeviceOnce attr_set[3][5];
+    int dev;
+    if (attr_set[vi][cfg].pending(&dev)) {
+        LPDT_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024));
+        attr_set[vi][cfg].mark(dev);
+    }
     launch_k(fn, (unsigned)blocks, 32 * warps, smem, st, nodes, d, x_half, x_hat, x_out, gamma, seg, sel, tab,
              q8 ? msg_scale : nullptr, msg_inv, q8, ds);
     LPDT_LAUNCH_CHECK();

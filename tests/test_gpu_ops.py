@@ -886,6 +886,20 @@ def test_gossip_node_counts_and_kept_shares(nodes, d, keep):
     close(xo, x_ref)
 
 
+# parameter counts of 8-byte rows: the form of the mix for 6 to 24 nodes from the parameters on that give the other form more
+# than one tile per CTA, and the nodes and sizes beside it; a pair of parameters that two segments share
+@pytest.mark.parametrize("nodes,d", [(5, 220002), (6, 190002), (8, 40002), (8, 160002), (16, 33002), (16, 80002), (17, 2050), (20, 80002), (21, 60002),
+                                     (24, 2006), (24, 60002), (25, 60002)])
+def test_gossip_with_rows_of_eight_bytes(nodes, d):
+    test_gossip_node_counts_and_kept_shares(nodes, d, 0.1)
+    if d > 50000:
+        return
+    segs = [(0, d - 77, d // 50), (d - 77, d, 7)]
+    test_gossip_mix_q8(nodes, d, segs)
+    for bits in (32, 8):
+        test_deepsqueeze_mix(nodes, d, segs, bits)
+
+
 def test_gossip_topk_with_massive_ties_and_alias():
     # magnitudes from a 4-value set: the tie cut decides almost every pick
     nodes, d, k = 6, 9000, 1234
