@@ -1,5 +1,5 @@
 // Pixel kernel on pairs of SMs: forward and backward-data contractions large enough that every SM has several 128 x 256
-// tiles with long K loops.  Two CTAs of a cluster work on two pixel tiles of one node and the same 256 channels; the
+// tiles with long K loops (signed codes).  Two CTAs of a cluster work on two pixel tiles of one node and the same 256 channels; the
 // leader issues one tcgen05.mma.cta_group::2 of M = 256 for both, each CTA holds its own 128 pixels and half of the
 // channels' weights in shared memory, and its 128 rows of the accumulator in its own tensor memory.
 //
@@ -22,7 +22,7 @@ namespace tc {
 constexpr int kPairThreads = 320, kPairStages = 6, kPairUnit = 16384, kPairBN = 256, kPairRaster = 8;
 
 struct PairParams {
-    int mode, uns;
+    int mode;
     int nodes, B, Hout, Wout, R, S, pad;
     int Nc, cpt, taps;                        // result channels, 128-byte boxes of summed channels per tap
     int w_rows_per_node;
@@ -149,7 +149,7 @@ conv_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
         }
     } else if (warp == 1) {
         if (rank == 0) {
-            const uint32_t idesc = idesc_i8(256, kPairBN, 0, p.mode == 0 ? 0 : 1, p.uns);
+            const uint32_t idesc = idesc_i8(256, kPairBN, 0, p.mode == 0 ? 0 : 1, 0);
             const uint64_t a_tpl = smem_desc(0, 16, 1024, 2), b_tpl = p.mode == 0 ? a_tpl : smem_desc(0, kPairUnit, 1024, 2);
             const uint32_t b_step = p.mode == 0 ? 2 : 256;                  // 32 K bytes of a row, or 32 rows of 128 bytes
             int st = 0; uint32_t ph = 0, tcount = 0;
@@ -255,7 +255,7 @@ conv_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
     }
 }
 
-// LPDT_PIX_PAIR=0: one SM per tile for every shape (A/B timing, parity tests)
+// LPDT_PIX_PAIR=0: one SM per tile for every shape (A/B timing)
 static bool pair_enabled() {
     static int on = -1;
     if (on < 0) { const char *e = getenv("LPDT_PIX_PAIR"); on = (e && e[0] == '0') ? 0 : 1; }
@@ -264,9 +264,9 @@ static bool pair_enabled() {
 
 lpdt_status tc_pix_pair(const lpdt_conv_desc &d, int mode, const PixTile &t, int cpt, const CUtensorMap &mA, const CUtensorMap &mY,
                         const int8_t *Wq, int pitch_w, const float *s1, const float *s2, const float *bias, int64_t bias_stride,
-                        int32_t *dev_status, cudaStream_t st, bool uns, const float *addend) {
+                        int32_t *dev_status, cudaStream_t st, const float *addend) {
     PairParams p = {};
-    p.mode = mode; p.uns = uns ? 1 : 0; p.nodes = d.nodes; p.B = d.B;
+    p.mode = mode; p.nodes = d.nodes; p.B = d.B;
     p.Hout = mode == 0 ? conv_out(d.H, d.pad, d.R, 1) : d.H; p.Wout = mode == 0 ? conv_out(d.W, d.pad, d.S, 1) : d.W;
     p.R = d.R; p.S = d.S; p.pad = d.pad; p.taps = d.R * d.S; p.cpt = cpt;
     p.Nc = mode == 0 ? d.Cout : d.Cin; p.w_rows_per_node = d.Cout;

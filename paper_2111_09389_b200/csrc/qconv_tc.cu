@@ -981,16 +981,17 @@ lpdt_status tc_pix(const lpdt_conv_desc &d, int mode, const int8_t *A, const flo
         if (!make_map(&mY, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, Y, 5, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B))
             return LPDT_ERR_CUDA;
     }
-    // Pairs of SMs (256-channel tiles, half the weights per SM) for long K loops where, in pick_bn's measure, a wave of
+    // Pairs of SMs (256-channel tiles, half the weights per SM; not for unsigned operands, whose zero-point terms its
+    // epilogue does not have) for long K loops where, in pick_bn's measure, a wave of
     // them costs less: they read 128 + 128 operand rows per step for 256 channels.
-    if (p.tma_out && !aff && d.stride == 1 && p.RBa == 128 && !p.merged && (mode == 0 || p.RBn == 128) && p.Nc >= 256 &&
+    if (p.tma_out && !uns && d.stride == 1 && p.RBa == 128 && !p.merged && (mode == 0 || p.RBn == 128) && p.Nc >= 256 &&
         p.cls_iters[0] * U >= 8) {
         const long long mt = (long long)p.tilesB * p.tilesH * p.tilesW;
         const long long one = ceil_div(p.nodes * mt * p.tilesN, kNumSMs) * (128 + p.BN);
         const long long pair = ceil_div(p.nodes * ((mt + 1) / 2) * ceil_div(p.Nc, 256), kNumSMs / 2) * 256;
         if (pair < one) {
             const PixTile t = {p.TB, p.TH, p.TW, p.tilesB, p.tilesH, p.tilesW};
-            lpdt_status r = tc_pix_pair(d, mode, t, p.cpt, mA, mY, Wq, pt.w, s1, s2, bias, bias_stride, dev_status, st, uns, addend);
+            lpdt_status r = tc_pix_pair(d, mode, t, p.cpt, mA, mY, Wq, pt.w, s1, s2, bias, bias_stride, dev_status, st, addend);
             if (r != LPDT_ERR_UNSUPPORTED) return r;
         }
     }

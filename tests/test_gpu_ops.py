@@ -362,8 +362,9 @@ def test_qconv_forward_takes_the_sooner_cores(case, kernel):
 
 
 # long K loops and enough 256-channel tiles for the kernel on pairs of SMs: an odd number of pixel tiles (the last pair is
-# half empty), part-zero boxes on the summed side, a part-empty last channel tile; a convolution with a halo
-PAIR_CASES = [(12, 300, 1, 1, 1300, 1284, 1, 1, 1, 0), (2, 33, 12, 12, 128, 512, 3, 3, 1, 1)]
+# half empty), part-zero boxes on the summed side, a part-empty last channel tile; a convolution with a halo; a filter in
+# both directions, whose boxes of weights end inside the next node's rows
+PAIR_CASES = [(12, 300, 1, 1, 1300, 1284, 1, 1, 1, 0), (2, 33, 12, 12, 128, 512, 3, 3, 1, 1), (3, 23, 8, 16, 368, 488, 3, 3, 1, 1)]
 
 
 @pytest.mark.parametrize("case", PAIR_CASES)
