@@ -24,22 +24,24 @@ __global__ void __launch_bounds__(256) pad_channels_kernel(const PadJob j0, cons
     const PadJob j = blockIdx.y ? j1 : j0;
     const int C = j.C, pieces = (C + 15) / 16, Cp = pieces * 16;
     const int64_t total = j.rows * pieces, bytes = j.rows * C, nth = (int64_t)gridDim.x * blockDim.x;
-    const int64_t whole = ((uintptr_t)j.src & 3) == 0 ? bytes & ~(int64_t)3 : 0;     // bytes that lie in whole words of the tensor
+    const bool words = ((uintptr_t)j.src & 3) == 0;
     for (int64_t o0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; o0 < total; o0 += PIECES * nth) {
         uint32_t w[PIECES][5];
         int64_t row[PIECES];
         int c0[PIECES], n[PIECES];
+        bool fits[PIECES];                                           // the piece's last word lies inside the tensor
 #pragma unroll
         for (int u = 0; u < PIECES; ++u) {
             const int64_t o = o0 + u * nth;
             row[u] = total <= 0x7fffffff ? (int64_t)((uint32_t)o / (uint32_t)pieces) : o / pieces;
             c0[u] = (int)(o - row[u] * pieces) * 16;
             n[u] = o < total ? (C - c0[u] < 16 ? C - c0[u] : 16) : 0;
-            const int64_t off = row[u] * C + c0[u], first = off & ~(int64_t)3;
-            const int need = n[u] > 0 ? ((int)(off & 3) + n[u] + 3) / 4 : 0;
+            const int64_t off = row[u] * C + c0[u];
+            fits[u] = words && ((off + n[u] + 3) & ~(int64_t)3) <= bytes;
+            const uint32_t *p = reinterpret_cast<const uint32_t *>(j.src + (off & ~(int64_t)3));
+            const int need = n[u] > 0 && fits[u] ? ((int)(off & 3) + n[u] + 3) / 4 : 0;
 #pragma unroll
-            for (int k = 0; k < 5; ++k)
-                w[u][k] = k < need && first + 4 * k < whole ? __ldg(reinterpret_cast<const uint32_t *>(j.src + first) + k) : 0u;
+            for (int k = 0; k < 5; ++k) w[u][k] = k < need ? __ldg(p + k) : 0u;
         }
 #pragma unroll
         for (int u = 0; u < PIECES; ++u) {
@@ -53,7 +55,7 @@ __global__ void __launch_bounds__(256) pad_channels_kernel(const PadJob j0, cons
                 const int left = n[u] - 4 * k;                       // bytes of this word that exist
                 r[k] = left >= 4 ? x : left <= 0 ? 0u : x & ((1u << (8 * left)) - 1u);
             }
-            if (off + n[u] > whole) {                                // in the tensor's last, partial word, or not aligned
+            if (!fits[u]) {
                 union { int8_t b[16]; uint32_t w[4]; } t;
 #pragma unroll
                 for (int k = 0; k < 16; ++k) t.b[k] = k < n[u] ? j.src[off + k] : (int8_t)0;
@@ -137,7 +139,8 @@ static lpdt_status pad_launch(PadJob a, PadJob b, cudaStream_t st) {
     // forward) 18.2 us with four, 20.6 with one; 40 nodes 34.6 and 38.9; a thread with one costs small calls less (1 x 32 x
     // 8x8 x 3, backward-weight: 10.7 us, 12.4 with four)
     const int64_t most = na > nb ? na : nb;
-    const bool many = most >= (int64_t)kNumSMs * 2048;
+    // (rows of several pieces have four or five words each in flight as it is)
+    const bool many = most >= (int64_t)kNumSMs * 2048 && (na > nb ? a.C : b.C) < 16;
     launch_k(many ? pad_channels_kernel<4> : pad_channels_kernel<1>, dim3(grid_for(many ? ceil_div(most, 4) : most), b.rows ? 2 : 1), 256, 0,
              st, a, b);
     LPDT_LAUNCH_CHECK();
