@@ -109,6 +109,26 @@ static inline cudaError_t launch_k_cluster(void (*kernel)(KArgs...), dim3 grid, 
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<Args &&>(args)...);
 }
 
+// ---- Two fp32 values in a register pair.  Each operation rounds both halves as its scalar form does, in one issue slot.
+// The assembler joins a mul.rn.f32x2 and the add.rn.f32x2 that takes its result into one rounding, whatever it is told about
+// contraction.  A product that feeds a sum is therefore a multiply-add of -0 that the assembler cannot see through
+// (opaque_minus_zero2; a * b + -0 rounds as a * b does, zeros included).
+typedef unsigned long long F2;
+__device__ __forceinline__ F2 pack2(float a, float b) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(F2 v, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) { F2 r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
+__device__ __forceinline__ F2 add2(F2 a, F2 b) { F2 r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) { F2 r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ F2 mul2(F2 a, F2 b, F2 minus_zero) { return fma2(a, b, minus_zero); }
+__device__ __forceinline__ F2 opaque_minus_zero2(int non_negative) {      // any value that is only known at run time
+    const float z = __uint_as_float(0x80000000u | ((unsigned)non_negative >> 31));
+    return pack2(z, z);
+}
+
 // double atomicAdd is native on sm_60+
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll

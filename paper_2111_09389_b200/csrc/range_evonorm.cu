@@ -63,6 +63,13 @@ __device__ __forceinline__ float hsig(float u) {
     return fminf(fmaxf(h, 0.f), 1.f);
 }
 
+__device__ __forceinline__ F2 hsig2(F2 u) {      // of two values (saturation clamps to [0, 1] and takes NaN to 0, as above)
+    const F2 y = pack2(0x1.555556p-3f, 0x1.555556p-3f), a = add2(u, pack2(3.f, 3.f)), q = mul2(a, y);
+    float h0, h1;
+    unpack2(fma2(fma2(pack2(-6.f, -6.f), q, a), y, q), h0, h1);
+    return pack2(__saturatef(h0), __saturatef(h1));
+}
+
 // Reduce per-thread extrema to per-group extrema.  s_mn/s_mx hold one entry per
 // thread; members of group g are the threads whose column lies in the group.
 template <int V>
@@ -454,8 +461,10 @@ __device__ __forceinline__ void ren_bwd_sample(unsigned char *smem_raw, int HW, 
                                                int64_t pstride, const float *__restrict__ gmin,
                                                const float *__restrict__ gmax, const int32_t *__restrict__ argmin,
                                                const int32_t *__restrict__ argmax, double *__restrict__ acc,
-                                               int64_t sample, int node, float *dxs, float &dmax) {
+                                               int64_t sample, int node, float *dxs, float &dmax, int R = 1, int rank = 0, int ppc = 0) {
+    namespace cg = cooperative_groups;
     const int T = blockDim.x, t = threadIdx.x;
+    const int p_lo = rank * ppc, p_end = R > 1 && p_lo + ppc < HW ? p_lo + ppc : HW;      // this CTA's pixels
     // When the column count divides the warp, lanes that share a column are folded with shuffles and
     // every warp keeps its own partial sums (no atomics, fixed order); otherwise one shared set of
     // fp64 accumulators takes atomic adds.
@@ -472,11 +481,11 @@ __device__ __forceinline__ void ren_bwd_sample(unsigned char *smem_raw, int HW, 
     const int c0 = col * V, grp = c0 / cpg;
     const float *xs = x + sample * (int64_t)HW * C;
     const float *dys = dy + sample * (int64_t)HW * C;
-    const int iters = (HW - 1) / rstep + 1;          // same trip count for every thread (rows are predicated)
+    const int iters = (p_end - p_lo - 1) / rstep + 1;          // same trip count for every thread (rows are predicated)
     auto request = [&](int j) {                      // row j of this thread -> slot j % DEPTH; one group per row, even when empty
         if (DEPTH > 0) {
-            const int p = row0 + j * rstep;
-            if (j < iters && p < HW) {
+            const int p = p_lo + row0 + j * rstep;
+            if (j < iters && p < p_end) {
                 float4 *slot = ring + (size_t)(j % (DEPTH > 0 ? DEPTH : 1)) * kPerSlot * T + t;
                 if (!XHOLD) cp_async16(slot, xs + (int64_t)p * C + c0);
                 cp_async16(slot + (kPerSlot - 1) * T, dys + (int64_t)p * C + c0);
@@ -512,30 +521,62 @@ __device__ __forceinline__ void ren_bwd_sample(unsigned char *smem_raw, int HW, 
 #pragma unroll
     for (int k = 0; k < V; ++k) { fb[k] = 0.0; fg[k] = 0.0; fv[k] = 0.0; }
     __syncthreads();   // s_ch zeroed
+    const F2 nz = opaque_minus_zero2(HW);
     auto term = [&](int p, const float (&xv)[V], const float (&dv_)[V]) {
         float o[V];
+        if constexpr (V == 4) {      // pairs: 58 instructions per element as scalars, and the issue slots are what bounds the kernel
+            const F2 inv2 = pack2(invD, invD);
+            float m4 = 0.f;
 #pragma unroll
-        for (int k = 0; k < V; ++k) {
-            float u = __fmul_rn(vc[k], xv[k]);
-            float hs = hsig(u);
-            float hp = (u > -3.f && u < 3.f) ? sixth : 0.f;
-            float m = __fmul_rn(xv[k], hs);
-            float tt = __fmul_rn(dv_[k], gc[k]);
-            S += (double)__fmul_rn(tt, m);
-            o[k] = __fmul_rn(__fmul_rn(tt, __fadd_rn(hs, __fmul_rn(u, hp))), invD);
-            const int idx = p * C + c0 + k;
-            if (idx != g_amx && idx != g_amn) dmax = fmaxf(dmax, fabsf(o[k]));
-            fb[k] += (double)dv_[k];
-            fg[k] += (double)__fmul_rn(dv_[k], __fmul_rn(m, invD));
-            fv[k] += (double)__fmul_rn(__fmul_rn(__fmul_rn(tt, __fmul_rn(xv[k], xv[k])), hp), invD);
+            for (int k = 0; k < V; k += 2) {
+                const F2 x = pack2(xv[k], xv[k + 1]), d = pack2(dv_[k], dv_[k + 1]);
+                const F2 u = mul2(pack2(vc[k], vc[k + 1]), x, nz), hs = hsig2(u);
+                float a, b;
+                unpack2(u, a, b);
+                const F2 hp = pack2(fabsf(a) < 3.f ? sixth : 0.f, fabsf(b) < 3.f ? sixth : 0.f);
+                const F2 m = mul2(x, hs), tt = mul2(d, pack2(gc[k], gc[k + 1]));
+                unpack2(mul2(tt, m), a, b);
+                S += (double)a; S += (double)b;
+                fb[k] += (double)dv_[k]; fb[k + 1] += (double)dv_[k + 1];
+                unpack2(mul2(d, mul2(m, inv2)), a, b);
+                fg[k] += (double)a; fg[k + 1] += (double)b;
+                unpack2(mul2(mul2(mul2(tt, mul2(x, x)), hp), inv2), a, b);
+                fv[k] += (double)a; fv[k + 1] += (double)b;
+                unpack2(mul2(mul2(tt, add2(hs, mul2(u, hp, nz))), inv2), o[k], o[k + 1]);
+                m4 = fmaxf(m4, fmaxf(fabsf(o[k]), fabsf(o[k + 1])));
+            }
+            const int idx = p * C + c0;
+            if ((unsigned)(g_amx - idx) < (unsigned)V || (unsigned)(g_amn - idx) < (unsigned)V) {
+                m4 = 0.f;
+#pragma unroll
+                for (int k = 0; k < V; ++k)
+                    if (idx + k != g_amx && idx + k != g_amn) m4 = fmaxf(m4, fabsf(o[k]));
+            }
+            dmax = fmaxf(dmax, m4);
+        } else {
+#pragma unroll
+            for (int k = 0; k < V; ++k) {
+                float u = __fmul_rn(vc[k], xv[k]);
+                float hs = hsig(u);
+                float hp = (u > -3.f && u < 3.f) ? sixth : 0.f;
+                float m = __fmul_rn(xv[k], hs);
+                float tt = __fmul_rn(dv_[k], gc[k]);
+                S += (double)__fmul_rn(tt, m);
+                o[k] = __fmul_rn(__fmul_rn(tt, __fadd_rn(hs, __fmul_rn(u, hp))), invD);
+                const int idx = p * C + c0 + k;
+                if (idx != g_amx && idx != g_amn) dmax = fmaxf(dmax, fabsf(o[k]));
+                fb[k] += (double)dv_[k];
+                fg[k] += (double)__fmul_rn(dv_[k], __fmul_rn(m, invD));
+                fv[k] += (double)__fmul_rn(__fmul_rn(__fmul_rn(tt, __fmul_rn(xv[k], xv[k])), hp), invD);
+            }
         }
         VecLoad<V>::st(dxs + (int64_t)p * C + c0, o);
     };
     if (DEPTH > 0) {
         for (int j = 0; j < iters; ++j) {
             cp_async_wait<(DEPTH > 0 ? DEPTH - 1 : 0)>();                // the oldest pending group, row j, has landed
-            const int p = row0 + j * rstep;
-            if (p < HW) {
+            const int p = p_lo + row0 + j * rstep;
+            if (p < p_end) {
                 const float4 *slot = ring + (size_t)(j % (DEPTH > 0 ? DEPTH : 1)) * kPerSlot * T + t;
                 const float4 a = XHOLD ? *reinterpret_cast<const float4 *>(dxs + (size_t)p * C + c0) : slot[0];
                 const float4 b = slot[(kPerSlot - 1) * T];
@@ -548,8 +589,8 @@ __device__ __forceinline__ void ren_bwd_sample(unsigned char *smem_raw, int HW, 
     }
     // DEPTH = 0, two rows per trip: four independent 16-byte loads in flight per thread
     for (int i = 0; DEPTH == 0 && i < iters; i += 2) {
-        const int p0 = row0 + i * rstep, p1 = p0 + rstep;
-        const bool ok0 = p0 < HW, ok1 = (i + 1 < iters) && (p1 < HW);
+        const int p0 = p_lo + row0 + i * rstep, p1 = p0 + rstep;
+        const bool ok0 = p0 < p_end, ok1 = (i + 1 < iters) && (p1 < p_end);
         float xa[V], da[V], xb[V], db[V];
         if (ok0) { VecLoad<V>::ld(xs + (int64_t)p0 * C + c0, xa); VecLoad<V>::ld(dys + (int64_t)p0 * C + c0, da); }
         if (ok1) { VecLoad<V>::ld(xs + (int64_t)p1 * C + c0, xb); VecLoad<V>::ld(dys + (int64_t)p1 * C + c0, db); }
@@ -587,28 +628,54 @@ __device__ __forceinline__ void ren_bwd_sample(unsigned char *smem_raw, int HW, 
             if (lane == 0) g_S[g] = a;
         }
     }
-    for (int i = t; i < 3 * C; i += T) {      // warp sets in order; summed over the batch by the finalize kernel
-        double a = s_ch[i];
-        for (int w = 1; w < nsets; ++w) a += s_ch[(size_t)w * 3 * C + i];
-        acc[sample * 3 * C + i] = a;
+    if (R == 1) {
+        for (int i = t; i < 3 * C; i += T) {      // warp sets in order; summed over the batch by the finalize kernel
+            double a = s_ch[i];
+            for (int w = 1; w < nsets; ++w) a += s_ch[(size_t)w * 3 * C + i];
+            acc[sample * 3 * C + i] = a;
+        }
+        __syncthreads();
+    } else {          // the sample's CTAs meet: sums in rank order, the group sums by all of them, the channel sums by the first
+        cg::cluster_group cluster = cg::this_cluster();
+        cluster.sync();
+        double S_all = 0.0;
+        if (t < groups)
+            for (int r = 0; r < R; ++r) S_all += *cluster.map_shared_rank(g_S + t, r);
+        for (int i = rank * T + t; i < 3 * C; i += R * T) {
+            double a = 0.0;
+            for (int r = 0; r < R; ++r) {
+                const double *other = cluster.map_shared_rank(s_ch, r);
+                for (int w = 0; w < nsets; ++w) a += other[(size_t)w * 3 * C + i];
+            }
+            acc[sample * 3 * C + i] = a;
+        }
+        cluster.sync();                           // nobody reads another's shared memory after this
+        if (t < groups) g_S[t] = S_all;
     }
-    __syncthreads();
     // The group sum only enters dx at the two extremum positions: one thread per group
     // applies the correction to the local term already stored there (same operation order
     // as a fused evaluation: local term first, then -coef at argmax, +coef at argmin).
     if (t < groups) {
         const int64_t sgg = sample * groups + t;
         const int amx = argmax[sgg], amn = argmin[sgg];
+        const bool has_mx = R == 1 || (amx >= p_lo * C && amx < p_end * C), has_mn = R == 1 || (amn >= p_lo * C && amn < p_end * C);
         if (amx != amn) {
             const float rng_g = __fsub_rn(gmax[sgg], gmin[sgg]);
             const float invDg = __fdiv_rn(1.f, __fadd_rn(__fmul_rn(Cst, rng_g), eps));
             float coef = __fmul_rn(Cst, (float)g_S[t]);
             coef = __fmul_rn(coef, invDg);
             coef = __fmul_rn(coef, invDg);
-            const float va = __fsub_rn(dxs[amx], coef), vb = __fadd_rn(dxs[amn], coef);
-            dxs[amx] = va; dxs[amn] = vb;
-            dmax = fmaxf(dmax, fmaxf(fabsf(va), fabsf(vb)));
-        } else {
+            if (has_mx) {
+                const float va = __fsub_rn(dxs[amx], coef);
+                dxs[amx] = va;
+                dmax = fmaxf(dmax, fabsf(va));
+            }
+            if (has_mn) {
+                const float vb = __fadd_rn(dxs[amn], coef);
+                dxs[amn] = vb;
+                dmax = fmaxf(dmax, fabsf(vb));
+            }
+        } else if (has_mx) {
             dmax = fmaxf(dmax, fabsf(dxs[amx]));
         }
     }
@@ -624,14 +691,14 @@ ren_bwd_kernel(int HW, int C, int groups, float eps, float Cst,
                const float *__restrict__ gmin, const float *__restrict__ gmax,
                const int32_t *__restrict__ argmin, const int32_t *__restrict__ argmax,
                float *__restrict__ dx, double *__restrict__ acc /*[nodes][B][3][C] per-sample partial sums*/,
-               float *__restrict__ amax_out) {
+               float *__restrict__ amax_out, int R /*CTAs per sample (cluster size)*/, int ppc /*pixels per CTA*/) {
     pdl_enter();
     extern __shared__ unsigned char smem_raw[];
-    const int64_t sample = blockIdx.x;
+    const int64_t sample = blockIdx.x / R;
     const int node = (int)(sample / B);
     float dmax = 0.f;
     ren_bwd_sample<V, DEPTH>(smem_raw, HW, C, groups, eps, Cst, dy, x, v, gamma, pstride, gmin, gmax, argmin, argmax, acc,
-                             sample, node, dx + sample * (int64_t)HW * C, dmax);
+                             sample, node, dx + sample * (int64_t)HW * C, dmax, R, (int)(blockIdx.x % R), ppc);
     if (amax_out) block_amax_to(dmax, amax_out + node);
 }
 
@@ -829,8 +896,10 @@ extern "C" lpdt_status lpdt_range_evonorm_bwd(int32_t nodes, int32_t B, int32_t 
     // 0.058 -> 0.053 ms; 256 KB samples lose 5 %).  LPDT_REN_BWD_THREADS=128|256 overrides (A/B timing).
     static int tforce = -1;
     if (tforce < 0) { const char *e = getenv("LPDT_REN_BWD_THREADS"); tforce = e ? atoi(e) : 0; }
+    // Not with fewer than three samples for two SMs, where there is nothing to overlap with and half the threads take longer
+    // (99 samples of 32x32x16 12.3 us with 128 threads, 10.0 with 256; 222 15.5 and 14.3; 300 19.3 and 19.1).
     const bool v4 = aligned(x, 16) && aligned(dy, 16) && aligned(dx, 16) && C % 4 == 0 && (C / groups) % 4 == 0;
-    int cap = ((int64_t)H * W * C * 4 <= 64 * 1024 && C / (v4 ? 4 : 1) <= 32) ? 128 : 256;
+    int cap = ((int64_t)H * W * C * 4 <= 64 * 1024 && C / (v4 ? 4 : 1) <= 32 && 2 * (int64_t)nodes * B > 3 * kNumSMs) ? 128 : 256;
     if (tforce == 128 || tforce == 256) cap = tforce;
     if (!plan(C, groups, aligned(x, 16) && aligned(dy, 16) && aligned(dx, 16), &pl, cap)) return LPDT_ERR_UNSUPPORTED;
     const int cv = C / pl.V;
@@ -848,9 +917,22 @@ extern "C" lpdt_status lpdt_range_evonorm_bwd(int32_t nodes, int32_t B, int32_t 
     cudaStream_t st = as_stream(stream);
     double *acc = (double *)ws;
     const float Cst = ren_const(C / groups);
-    dim3 grid((unsigned)((int64_t)nodes * B));
+    // CTAs per sample (a cluster): with few samples, as many as give every SM one CTA at most, up to four, while a thread keeps
+    // four rows.  20 samples: 32x32x16 9.8 -> 7.4 us, 32x32x64 24 -> 11.7, 16x16x128 14.5 -> 9.6; beyond one CTA per SM the
+    // meeting costs more than the split saves (99 samples of 32x32x16 in two 11.0 us, whole 10.2), and so it does for wide
+    // samples of few rows (20 of 4x4x512 in two 11.2 us, whole 9.9).
+    // LPDT_REN_BWD_CLUSTER=1|2|4 overrides (parity tests).
+    static int rforce = -1;
+    if (rforce < 0) { const char *e = getenv("LPDT_REN_BWD_CLUSTER"); rforce = e ? atoi(e) : 0; }
+    const int rstep = pl.threads / cv, rows = (int)ceil_div((int64_t)H * W, rstep);
+    const int64_t samples = (int64_t)nodes * B;
+    int R = 1;
+    while (pl.V == 4 && R < 4 && groups <= pl.threads && 2 * R <= rows && (rforce ? 2 * R <= rforce : samples * 2 * R <= kNumSMs && rows >= 8 * R && cv <= 64)) R *= 2;
+    int ppc = (int)ceil_div(rows, R) * rstep;
+    while (R > 1 && (int64_t)(R - 1) * ppc >= (int64_t)H * W) { R /= 2; ppc = (int)ceil_div(rows, R) * rstep; }    // no CTA without pixels
+    dim3 grid((unsigned)((int64_t)nodes * B * R));
     using Fn = void (*)(int, int, int, float, float, const float *, const float *, const float *, const float *, int64_t, int,
-                        const float *, const float *, const int32_t *, const int32_t *, float *, double *, float *);
+                        const float *, const float *, const int32_t *, const int32_t *, float *, double *, float *, int, int);
     static const Fn fns[2][3] = {{ren_bwd_kernel<1, 256, 0>, ren_bwd_kernel<1, 512, 0>, ren_bwd_kernel<1, 256, 0>},
                                  {ren_bwd_kernel<4, 256, 8>, ren_bwd_kernel<4, 512, 4>, ren_bwd_kernel<4, 256, 6>}};
     static PerDeviceOnce attr;
@@ -864,8 +946,8 @@ extern "C" lpdt_status lpdt_range_evonorm_bwd(int32_t nodes, int32_t B, int32_t 
         }
         attr.mark(dev);
     }
-    launch_k(fns[pl.V == 4 ? 1 : 0][pl.threads > 256 ? 1 : depth == 6 ? 2 : 0], grid, pl.threads, smem, st, H * W, C, groups, eps, Cst, dy, x,
-             v, gamma, pstride, B, gmin, gmax, argmin, argmax, dx, acc, amax_out);
+    launch_k_cluster(fns[pl.V == 4 ? 1 : 0][pl.threads > 256 ? 1 : depth == 6 ? 2 : 0], grid, pl.threads, smem, st, R, H * W, C, groups, eps,
+                     Cst, dy, x, v, gamma, pstride, B, gmin, gmax, argmin, argmax, dx, acc, amax_out, R, ppc);
     LPDT_LAUNCH_CHECK();
     if (deferred) return LPDT_OK;
     launch_k(ren_bwd_finalize, (nodes * 3 * C + 7) / 8, 256, 0, st, acc, nodes, B, C, dv, dgamma, dbeta, gstride);

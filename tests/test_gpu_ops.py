@@ -1286,6 +1286,20 @@ def test_range_evonorm_cases_on_every_cluster_size(cluster):
     assert r.returncode == 0, r.stdout[-3000:] + r.stderr[-2000:]
 
 
+@pytest.mark.parametrize("cluster", ["2", "4"])
+def test_range_evonorm_backward_cases_on_every_cluster_size(cluster):
+    """The same for the backward kernel, which splits the samples of small batches over 2 or 4 CTAs."""
+    import os, subprocess, sys
+    if os.environ.get("LPDT_CHILD") == "1":
+        pytest.skip("already inside a child run")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    child_env = dict(os.environ, LPDT_CHILD="1", LPDT_REN_BWD_CLUSTER=cluster)
+    r = subprocess.run([sys.executable, "-m", "pytest", os.path.join(root, "tests", "test_gpu_ops.py"), "-m", "gpu",
+                        "-q", "-x", "-k", "test_range_evonorm_fwd or test_fused_ranges"], env=child_env,
+                       cwd=root, capture_output=True, text=True, timeout=900)
+    assert r.returncode == 0, r.stdout[-3000:] + r.stderr[-2000:]
+
+
 @pytest.mark.parametrize("env", [{"LPDT_FORCE_HALO": "1"}, {"LPDT_DISABLE_HALO": "1"}, {"LPDT_DISABLE_TC": "1"},
                                  {"LPDT_AFFINE_SEPARATE": "1"}, {"LPDT_PIX_DIRECT_STORE": "1", "LPDT_DISABLE_HALO": "1"},
                                  {"LPDT_PIX_TWO": "0", "LPDT_DISABLE_HALO": "1"}])
