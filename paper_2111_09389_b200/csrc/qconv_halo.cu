@@ -416,8 +416,6 @@ lpdt_status tc_pix_halo(const lpdt_conv_desc &d, int mode, const int8_t *A, cons
         if (!make_map_u8(&mW, Wq, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_NONE)) return LPDT_ERR_CUDA;
     }
     size_t smem = 1024 + (size_t)p.wres_bytes + (size_t)p.stages * p.halo_bytes + kZeroBytes + out_bytes;
-    const size_t smem_floor = (size_t)(228 * 1024) / (per_sm + 1);     // keeps the (per_sm + 1)-th CTA out
-    if (smem < smem_floor) smem = smem_floor;
     static PerDeviceOnce attr;
     int dev;
     if (attr.pending(&dev)) {
@@ -427,6 +425,7 @@ lpdt_status tc_pix_halo(const lpdt_conv_desc &d, int mode, const int8_t *A, cons
     const long long tiles = (long long)p.nodes * p.B * p.tilesH * p.tilesW;
     if (tiles > 0x7fffffff) return LPDT_ERR_UNSUPPORTED;
     const int grid = (int)(tiles < (long long)kNumSMs * per_sm ? tiles : (long long)kNumSMs * per_sm);
+    smem = spread_smem(smem, grid, per_sm, true);                      // keeps the (per_sm + 1)-th CTA out, and few tiles apart
     g_last_kernel = "lpdt::tc::conv_halo16_kernel";
     launch_k(conv_halo16_kernel, grid, kHaloThreads, smem, st, mA, mW, mY, p);
     LPDT_LAUNCH_CHECK();

@@ -1109,7 +1109,7 @@ lpdt_status tc_wgrad(const lpdt_conv_desc &d, const int8_t *E, const float *sE, 
     else if (!act_map(&mX, A, d.nodes, d.B, d.H, d.W, d.Cin, pt.in, p.RBx, p.TB, p.TH, p.TW, d.stride)) return LPDT_ERR_CUDA;
     if (!act_map(&mE, E, d.nodes, d.B, Ho, Wo, d.Cout, pt.err, p.RBe, p.TB, p.TH, p.TW)) return LPDT_ERR_CUDA;
     size_t smem = 1024 + (size_t)p.stages * stage_bytes;
-    if (smem < (size_t)(228 * 1024) / (per_sm + 1)) smem = (size_t)(228 * 1024) / (per_sm + 1);
+    smem = spread_smem(smem, (int64_t)p.splits * p.mgroups * p.ngroups * d.nodes, per_sm, true);
     if (smem > 227 * 1024) return LPDT_ERR_UNSUPPORTED;
     static PerDeviceOnce attr;
     int dev;

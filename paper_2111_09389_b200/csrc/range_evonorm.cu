@@ -826,6 +826,10 @@ static int ren_cluster_size(int64_t samples, int HW, int C, int rstep) {
     return R;
 }
 
+// CTAs to spread (spread_smem).  The CTAs of a cluster of 4 sit in one group of SMs, whose size is no multiple of four: room
+// for a ninth more (108 samples of 64 KB in clusters of 4: 7.4 us, 9.3 with three CTAs per SM; 99 samples 7.4 and 6.4).
+static int64_t spread_grid(int64_t samples, int R) { return R > 2 ? ceil_div(samples * R * 10, 9) : samples * R; }
+
 static float ren_const(int cpg) { return (float)(1.0 / sqrt(2.0 * log((double)cpg))); }
 
 }  // namespace lpdt
@@ -860,6 +864,15 @@ extern "C" lpdt_status lpdt_range_evonorm_fwd(int32_t nodes, int32_t B, int32_t 
                         int, float *, float *, float *, int32_t *, int32_t *, float *, const float *, int, int);
     static const Fn fns[2][2] = {{ren_fwd_kernel<1, false>, ren_fwd_kernel<1, true>},
                                  {ren_fwd_kernel<4, false>, ren_fwd_kernel<4, true>}};
+    if (pl.threads <= 256 && R <= 4) {      // (clusters of 8 need the room of their group of SMs: 50 samples of 64 KB 6.8 us, 9.7 spread)
+        static PerDeviceOnce attr;
+        int dev;
+        if (attr.pending(&dev)) {
+            for (int i = 0; i < 4; ++i) LPDT_CUDA(cudaFuncSetAttribute(fns[i / 2][i % 2], cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024));
+            attr.mark(dev);
+        }
+        smem = spread_smem(smem, spread_grid((int64_t)nodes * B, R), 1024 / pl.threads);
+    }
     launch_k_cluster(fns[pl.V == 4 ? 1 : 0][res ? 1 : 0], grid, pl.threads, smem, as_stream(stream), R, H * W, C, groups, eps,
                      Cst, x, v, gamma, beta, pstride, B, y, gmin, gmax, argmin, argmax, amax_out, res, R, ppc);
     LPDT_LAUNCH_CHECK();
@@ -939,13 +952,14 @@ extern "C" lpdt_status lpdt_range_evonorm_bwd(int32_t nodes, int32_t B, int32_t 
     int dev;
     if (attr.pending(&dev)) {
         for (int i = 0; i < 3; ++i) {
-            LPDT_CUDA(cudaFuncSetAttribute(fns[1][i], cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));
+            LPDT_CUDA(cudaFuncSetAttribute(fns[1][i], cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024));
             // the rings of three (six) resident CTAs need nearly all of the SM's shared memory
             LPDT_CUDA(cudaFuncSetAttribute(fns[1][i], cudaFuncAttributePreferredSharedMemoryCarveout,
                                            (int)cudaSharedmemCarveoutMaxShared));
         }
         attr.mark(dev);
     }
+    if (pl.V == 4) smem = spread_smem(smem, spread_grid((int64_t)nodes * B, R), pl.threads <= 128 ? 6 : pl.threads <= 256 ? 3 : 1);
     launch_k_cluster(fns[pl.V == 4 ? 1 : 0][pl.threads > 256 ? 1 : depth == 6 ? 2 : 0], grid, pl.threads, smem, st, R, H * W, C, groups, eps,
                      Cst, dy, x, v, gamma, pstride, B, gmin, gmax, argmin, argmax, dx, acc, amax_out, R, ppc);
     LPDT_LAUNCH_CHECK();
