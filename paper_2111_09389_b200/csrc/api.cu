@@ -6,10 +6,37 @@ extern "C" const char *lpdt_version(void) { return "lpdt 0.1 (sm_100a)"; }
 extern "C" const char *lpdt_last_kernel(void) { return lpdt::g_last_kernel; }
 extern "C" uint64_t lpdt_launch_count(void) { return lpdt::g_launch_count; }
 
+namespace lpdt {
+
+// ResNet-20 on 40 nodes (sums of 0.2 to 2.9 MB beside the main stream): 2895 us a step, 2938 with kernels for those as well.
+constexpr size_t kZeroByCopyEngine = 64u << 10;
+
+__global__ void __launch_bounds__(256) zero_kernel(uint32_t *__restrict__ p, int n, int head /*words before a 16-byte boundary*/) {
+    pdl_enter();
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
+    uint4 *p4 = reinterpret_cast<uint4 *>(p + head);
+    const int n4 = (n - head) / 4;
+    for (int i = t; i < n4; i += nth) p4[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (t < head) p[t] = 0u;
+    if (t < n - head - 4 * n4) p[head + 4 * n4 + t] = 0u;
+}
+
+cudaError_t zero_async(void *p, size_t bytes, cudaStream_t st) {
+    if (bytes == 0) return cudaSuccess;
+    if (bytes >= kZeroByCopyEngine || bytes % 4 || !aligned(p, 4)) return cudaMemsetAsync(p, 0, bytes, st);
+    const int n = (int)(bytes / 4);
+    int head = (int)((16 - (uintptr_t)p % 16) % 16 / 4);
+    if (head > n) head = n;
+    const int64_t blocks = ceil_div(n, 1024);
+    return launch_k(zero_kernel, (unsigned)(blocks < kNumSMs * 8 ? blocks : kNumSMs * 8), 256, 0, st, (uint32_t *)p, n, head);
+}
+
+}  // namespace lpdt
+
 extern "C" lpdt_status lpdt_fill_zero(void *p, size_t bytes, void *stream) {
     if (bytes == 0) return LPDT_OK;
     LPDT_CHECK_ARG(p != nullptr);
-    LPDT_CUDA(cudaMemsetAsync(p, 0, bytes, lpdt::as_stream(stream)));
+    LPDT_CUDA(lpdt::zero_async(p, bytes, lpdt::as_stream(stream)));
     return LPDT_OK;
 }
 

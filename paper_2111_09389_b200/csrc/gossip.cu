@@ -1107,11 +1107,11 @@ static lpdt_status gossip_impl(int32_t nodes, int64_t d, const float *x_half, fl
         amax_bits = (unsigned int *)((char *)ws + lpdt_gossip_mix_workspace_size(nodes, d, n_segments) - 2 * q8_bytes(nodes, n_segments));
         msg_inv = (float *)((char *)amax_bits + q8_bytes(nodes, n_segments));
         if (nodes > 65535) return LPDT_ERR_UNSUPPORTED;
-        LPDT_CUDA(cudaMemsetAsync(amax_bits, 0, (size_t)nodes * n_segments * sizeof(unsigned int), st));
+        LPDT_CUDA(zero_async(amax_bits, (size_t)nodes * n_segments * sizeof(unsigned int), st));
     }
     if (big.n > 0) {
         if (most_chunks > 0x7fffffff || nodes > 65535) return LPDT_ERR_UNSUPPORTED;
-        LPDT_CUDA(cudaMemsetAsync(ctl, 0, (size_t)nodes * big.n * sizeof(BigCtl), st));
+        LPDT_CUDA(zero_async(ctl, (size_t)nodes * big.n * sizeof(BigCtl), st));
         // elements per CTA of the collect pass: every CTA clears and flushes a 4096-bin histogram, so chunks are as
         // long as still leaves several CTAs per SM (16 K ... 64 K elements)
         int chunk = kChunk;

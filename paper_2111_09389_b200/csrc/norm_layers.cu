@@ -768,7 +768,7 @@ extern "C" lpdt_status lpdt_range_bn_fwd(int32_t nodes, int32_t B, int32_t H, in
     if (!norm_plan(C, C, aligned(x, 16) && aligned(y, 16), &pl)) return LPDT_ERR_UNSUPPORTED;
     cudaStream_t st = as_stream(stream);
     RbnStat *stat = (RbnStat *)ws;
-    LPDT_CUDA(cudaMemsetAsync(stat, 0, (size_t)nodes * C * sizeof(RbnStat), st));
+    LPDT_CUDA(zero_async(stat, (size_t)nodes * C * sizeof(RbnStat), st));
     const int rstep = pl.threads / (C / pl.V);
     const dim3 grid((unsigned)ceil_div(P, (int64_t)rstep * kRbnIters), nodes);
     const size_t smem = (size_t)3 * pl.V * pl.threads * sizeof(double);
@@ -799,7 +799,7 @@ extern "C" lpdt_status lpdt_range_bn_bwd(int32_t nodes, int32_t B, int32_t H, in
     if (!norm_plan(C, C, aligned(x, 16) && aligned(dy, 16) && aligned(dx, 16), &pl)) return LPDT_ERR_UNSUPPORTED;
     cudaStream_t st = as_stream(stream);
     RbnStat *stat = (RbnStat *)ws;
-    LPDT_CUDA(cudaMemsetAsync(stat, 0, (size_t)nodes * C * sizeof(RbnStat), st));
+    LPDT_CUDA(zero_async(stat, (size_t)nodes * C * sizeof(RbnStat), st));
     const int rstep = pl.threads / (C / pl.V);
     const dim3 grid((unsigned)ceil_div(P, (int64_t)rstep * kRbnIters), nodes);
     const size_t smem = (size_t)2 * pl.V * pl.threads * sizeof(double);

@@ -943,7 +943,7 @@ extern "C" lpdt_status lpdt_qconv_bwd_weight_affine(const lpdt_conv_desc *d, con
                         nullptr, 0, raw, inner, ws_bytes - (size_t)((char *)inner - (char *)ws), dev_status, st, true);
     if (s != LPDT_OK) return s;
     // both operands' tap sums; samples are shared out until about two waves of blocks exist
-    LPDT_CUDA(cudaMemsetAsync(tabE, 0, affine_tab_bytes(d, d->Cout) + affine_tab_bytes(d, d->Cin), st));
+    LPDT_CUDA(zero_async(tabE, affine_tab_bytes(d, d->Cout) + affine_tab_bytes(d, d->Cin), st));
     const int sw = d->S < 24 ? d->S : 24, cw = 512;                  // 48 KB of shared memory at most
     const int64_t schunks = ceil_div(d->S, sw);
     TapSumSide sideE = {E, tabE, Ho, Wo, d->Cout, cw, (int)ceil_div(d->Cout, cw), 0};

@@ -267,7 +267,7 @@ lpdt_status generic_bwd_weight(const lpdt_conv_desc &d, const int8_t *E, const f
     const int64_t per_node = (int64_t)d.Cout * d.R * d.S * d.Cin;
     if (d.nodes > 65535) return LPDT_ERR_UNSUPPORTED;        // nodes ride in grid.y
     int32_t *acc = dWacc ? dWacc : (int32_t *)ws;
-    LPDT_CUDA(cudaMemsetAsync(acc, 0, (size_t)d.nodes * per_node * sizeof(int32_t), st));
+    LPDT_CUDA(zero_async(acc, (size_t)d.nodes * per_node * sizeof(int32_t), st));
     const int64_t npix = (int64_t)d.B * Ho * Wo;
     if (npix > 0) {                      // an empty batch leaves the zeroed sums: the gradient of no samples
         int chunk = 4;

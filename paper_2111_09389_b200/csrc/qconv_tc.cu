@@ -1121,7 +1121,7 @@ lpdt_status tc_wgrad(const lpdt_conv_desc &d, const int8_t *E, const float *sE, 
     const int64_t per_node = (int64_t)d.Cout * p.taps * d.Cin;
     if (p.splits > 1) {
         if (!p.acc_out) return LPDT_ERR_WORKSPACE;
-        LPDT_CUDA(cudaMemsetAsync(p.acc_out, 0, (size_t)d.nodes * per_node * sizeof(int32_t), st));
+        LPDT_CUDA(zero_async(p.acc_out, (size_t)d.nodes * per_node * sizeof(int32_t), st));
     }
     g_last_kernel = "lpdt::tc::conv_wgrad_kernel";
     launch_k(conv_wgrad_kernel, dim3(p.splits, p.mgroups * p.ngroups, d.nodes), kThreads, smem, st, mX, mE, p);

@@ -230,7 +230,7 @@ extern "C" lpdt_status lpdt_quantize(const float *x, int32_t nodes, int64_t n, i
     if (!ws || ws_bytes < lpdt_quantize_workspace_size(nodes)) return LPDT_ERR_WORKSPACE;
     cudaStream_t st = as_stream(stream);
     uint32_t *w = (uint32_t *)ws;
-    LPDT_CUDA(cudaMemsetAsync(w, 0, (size_t)nodes * 2 * sizeof(uint32_t), st));
+    LPDT_CUDA(zero_async(w, (size_t)nodes * 2 * sizeof(uint32_t), st));
     const bool vec = aligned(x, 16) && (x_node_stride % 4 == 0) && (n % 4 == 0) && aligned(q, 4);
     dim3 grid(blocks_for(vec ? n / 4 : n, nodes), nodes), block(256);
     const uint2 key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
@@ -465,7 +465,7 @@ extern "C" lpdt_status lpdt_quantize_batch(const float *params, int32_t nodes, i
     if (longest == 0) return LPDT_OK;
     cudaStream_t st = as_stream(stream);
     uint32_t *w = (uint32_t *)ws;
-    LPDT_CUDA(cudaMemsetAsync(w, 0, (size_t)nodes * n_tensors * sizeof(uint32_t), st));
+    LPDT_CUDA(zero_async(w, (size_t)nodes * n_tensors * sizeof(uint32_t), st));
     int bx = (int)ceil_div(longest, 256 * 16);
     if (bx > 64) bx = 64;
     if (bx < 1) bx = 1;

@@ -103,6 +103,18 @@ def test_quantize_batch_matches_per_tensor_calls():
     assert sh[1, 2] == 1.0
 
 
+@pytest.mark.parametrize("words", [1, 2, 3, 4, 5, 1023, 1024, 16383, 16384, 16385])
+@pytest.mark.parametrize("first", [0, 1, 2, 3])
+def test_fill_zero_at_every_alignment(words, first):
+    t = torch.full((words + 8,), 7, dtype=torch.int32, device="cuda")
+    api.lpdt_fill_zero(t[first:first + words])
+    assert not t[first:first + words].any() and (t[:first] == 7).all() and (t[first + words:] == 7).all()
+    b = t.view(torch.uint8)                       # not whole words
+    b.fill_(3)
+    api.lpdt_fill_zero(b[first:first + 4 * words - 1])
+    assert not b[first:first + 4 * words - 1].any() and (b[:first] == 3).all() and (b[first + 4 * words - 1:] == 3).all()
+
+
 def test_quantize_argument_errors():
     x = torch.zeros(8, device="cuda")
     q = torch.zeros(8, dtype=torch.int8, device="cuda")
