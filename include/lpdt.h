@@ -218,6 +218,9 @@ lpdt_status lpdt_qconv_bwd_weight(const lpdt_conv_desc *d, const int8_t *E, cons
                                   const int8_t *A, const float *sA,
                                   float *dW, int64_t dw_node_stride, int32_t *dWacc,
                                   void *ws, size_t ws_bytes, int32_t *dev_status, void *stream);
+/* 1 when lpdt_qconv_bwd_weight of the shape writes dW in its one launch; 0 when it adds int32 sums in memory first, which
+ * lpdt_dequantize_acc_batch converts for many layers at once when they are asked for through dWacc. */
+int32_t lpdt_qconv_bwd_weight_direct(const lpdt_conv_desc *d);
 
 /* Dequantize the raw int32 sums of up to 64 tensors in one launch (all weight gradients of a network, each
  * left by lpdt_qconv_bwd_weight through dWacc as a contiguous [nodes][sizes[t]] block at acc + acc_offsets[t]):

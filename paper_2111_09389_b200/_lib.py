@@ -46,6 +46,7 @@ SIGNATURES = {
                                             _vp, _vp]),
     "lpdt_qconv_bwd_data": (_i32, [C.POINTER(ConvDesc), _vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _sz, _vp, _vp]),
     "lpdt_qconv_bwd_weight": (_i32, [C.POINTER(ConvDesc), _vp, _vp, _vp, _vp, _vp, _i64, _vp, _vp, _sz, _vp, _vp]),
+    "lpdt_qconv_bwd_weight_direct": (_i32, [C.POINTER(ConvDesc)]),
     "lpdt_range_evonorm_fwd": (_i32, [_i32] * 6 + [_f32] + [_vp] * 4 + [_i64] + [_vp] * 7 + [_vp]),
     "lpdt_range_evonorm_q8_ctl_size": (_sz, [_i32]),
     "lpdt_range_evonorm_fwd_q8_fits": (_i32, [_i32] * 5),

@@ -254,6 +254,10 @@ def lpdt_qconv_bwd_weight(desc, E, sE, A, sA, dW=None, dw_node_stride=0, dWacc=N
                                                                 _stream()))
 
 
+def lpdt_qconv_bwd_weight_direct(desc):
+    return lib().lpdt_qconv_bwd_weight_direct(C.byref(desc))
+
+
 def lpdt_range_evonorm_fwd(nodes, B, H, W, Cc, groups, eps, x, v, gamma, beta, param_node_stride, y,
                            gmin, gmax, argmin, argmax, amax_out=None, res=None):
     _check("lpdt_range_evonorm_fwd", lib().lpdt_range_evonorm_fwd(

@@ -646,6 +646,11 @@ extern "C" lpdt_status lpdt_qconv_bwd_weight(const lpdt_conv_desc *d, const int8
     return bwd_weight_impl(d, E, sE, A, sA, dW, dw_node_stride, dWacc, ws, ws_bytes, dev_status, as_stream(stream), false);
 }
 
+extern "C" int32_t lpdt_qconv_bwd_weight_direct(const lpdt_conv_desc *d) {
+    if (check_desc(d) != LPDT_OK || d->nodes == 0 || d->B == 0 || d->Cin % 16 || d->Cout % 16 || d->stride > 2) return 0;
+    return tc::wgrad_direct(*d, pitches(*d)) ? 1 : 0;
+}
+
 // ---- backward products on affine (zero-point) operands -----------------------------------------
 // With e' = qe - zE, w' = qw - zW, a' = qa - zA and the sums running over the taps that exist,
 //   sum e'w' = sum qe*qw - zW * sum qe - zE * sum qw + (terms) * zE*zW          (backward-data)

@@ -43,6 +43,8 @@ lpdt_status tc_pix_halo(const lpdt_conv_desc &d, int mode, const int8_t *A, cons
 lpdt_status tc_wgrad(const lpdt_conv_desc &d, const int8_t *E, const float *sE, const int8_t *A,
                      const float *sA, int32_t *acc_user, int32_t *acc_ws, float *dW, int64_t dw_stride,
                      int32_t *dev_status, cudaStream_t st, bool uns, Pitches pt);
+// Whether that is one launch that writes dW itself (no split of the pixel loop, no sums in memory).
+bool wgrad_direct(const lpdt_conv_desc &d, Pitches pt);
 // The same on pairs of SMs (signed codes, stride 1, 128-byte operand rows, 256-channel tiles, fp32 result in rows of 16 bytes): the
 // tiling and the operand-A and result maps of tc_pix.  UNSUPPORTED where the one-SM kernel is the better one.
 struct PixTile { int TB, TH, TW, tilesB, tilesH, tilesW; };

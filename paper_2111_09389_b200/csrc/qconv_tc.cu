@@ -1022,11 +1022,10 @@ lpdt_status tc_pix(const lpdt_conv_desc &d, int mode, const int8_t *A, const flo
 
 // acc_user: the caller's raw-sum array or null; acc_ws: scratch of the same shape [nodes][Cout][taps][Cin]; dW: fp32 result or null.  With one split the kernel writes both outputs
 // itself; with several it accumulates into zeroed int32 storage and a conversion launch follows.
-lpdt_status tc_wgrad(const lpdt_conv_desc &d, const int8_t *E, const float *sE, const int8_t *A,
-                     const float *sA, int32_t *acc_user, int32_t *acc_ws, float *dW, int64_t dw_stride,
-                     int32_t *dev_status, cudaStream_t st, bool uns, Pitches pt) {
+// Tiling, stages, CTAs per SM and split of the pixel loop.
+static lpdt_status wgrad_plan(const lpdt_conv_desc &d, Pitches pt, WgParams &p, int &per_sm, int &stage_bytes) {
     const int Ho = conv_out(d.H, d.pad, d.R, d.stride), Wo = conv_out(d.W, d.pad, d.S, d.stride);
-    WgParams p = {};
+    p = WgParams{};
     p.nodes = d.nodes; p.B = d.B; p.Ho = Ho; p.Wo = Wo; p.Cin = d.Cin; p.Cout = d.Cout;
     p.R = d.R; p.S = d.S; p.pad = d.pad; p.taps = d.R * d.S; p.stride = d.stride;
     p.RBx = row_bytes_for(d.Cin, kWgRowCost); p.RBe = row_bytes_for(d.Cout, kWgRowCost);
@@ -1076,12 +1075,12 @@ lpdt_status tc_wgrad(const lpdt_conv_desc &d, const int8_t *E, const float *sE, 
     p.mtiles = mt;
     p.mgroups = (int)ceil_div(all_tiles, mt);
     if (p.halo) { p.mtiles = d.R; p.mgroups = 1; }
-    const int stage_bytes = (p.halo ? p.halo_bytes : p.mtiles * 16384) + 128 * p.BNc;
+    stage_bytes = (p.halo ? p.halo_bytes : p.mtiles * 16384) + 128 * p.BNc;
     p.tmem_cols = pow2_at_least(p.mtiles * p.BNc);
     if (p.tmem_cols > 512) return LPDT_ERR_UNSUPPORTED;
     // CTAs per SM: as many (up to four) as leave each at least four stages and fit TMEM; the shared-memory
     // request keeps any further CTA off the SM, so a TMEM allocation never waits
-    int per_sm = 4;
+    per_sm = 4;
     for (;; --per_sm) {
         p.stages = ((224 * 1024) / per_sm - 2048 - 1024) / stage_bytes;
         if (p.stages > 8) p.stages = 8;
@@ -1096,6 +1095,23 @@ lpdt_status tc_wgrad(const lpdt_conv_desc &d, const int8_t *E, const float *sE, 
     if (splits < 1) splits = 1;
     p.kb_per_split = (int)ceil_div(p.kblocks, splits);
     p.splits = (int)ceil_div(p.kblocks, p.kb_per_split);
+    return LPDT_OK;
+}
+
+bool wgrad_direct(const lpdt_conv_desc &d, Pitches pt) {
+    WgParams p;
+    int per_sm, stage_bytes;
+    return wgrad_plan(d, pt, p, per_sm, stage_bytes) == LPDT_OK && p.splits == 1;
+}
+
+lpdt_status tc_wgrad(const lpdt_conv_desc &d, const int8_t *E, const float *sE, const int8_t *A,
+                     const float *sA, int32_t *acc_user, int32_t *acc_ws, float *dW, int64_t dw_stride,
+                     int32_t *dev_status, cudaStream_t st, bool uns, Pitches pt) {
+    const int Ho = conv_out(d.H, d.pad, d.R, d.stride), Wo = conv_out(d.W, d.pad, d.S, d.stride);
+    WgParams p;
+    int per_sm, stage_bytes;
+    const lpdt_status planned = wgrad_plan(d, pt, p, per_sm, stage_bytes);
+    if (planned != LPDT_OK) return planned;
     p.dW = dW; p.dw_stride = dw_stride; p.s1 = sE; p.s2 = sA;
     p.acc_out = p.splits == 1 ? acc_user : (acc_user ? acc_user : acc_ws);
     p.dev_status = dev_status; p.uns = uns ? 1 : 0;

@@ -106,6 +106,8 @@ class TrainStep:
                          E=torch.empty(N, B, Ho, Wo, op["cout"], **i8), sE=torch.empty(N, **f32),
                          dx=torch.empty(N, B, H, W, op["cin"], **f32),
                          wn=op["cout"] * R * S * op["cin"], wi=wi)
+                # whether the layer's weight gradient is complete after one launch, or adds int32 sums first
+                b["direct"] = bool(api.lpdt_qconv_bwd_weight_direct(desc))
                 b["gacc"] = self.g_acc[self.g_acc_off[wi]:self.g_acc_off[wi] + N * b["wn"]].view(N, b["wn"])
                 if quantize_wgrad:
                     b.update(gq=torch.empty(N, b["wn"], **i8), gs=torch.empty(N, **f32),
@@ -160,6 +162,11 @@ class TrainStep:
         if self.node_groups > 1:
             bounds = [N * g // self.node_groups for g in range(self.node_groups + 1)]
             self.groups = [self._node_view(bounds[g], bounds[g + 1], ws_bytes, dev) for g in range(self.node_groups)]
+            for layer in zip(self.buf, *(g.buf for g in self.groups)):      # one answer for all nodes of a layer
+                if "direct" in layer[0]:
+                    direct = all(b["direct"] for b in layer[1:])
+                    for b in layer:
+                        b["direct"] = direct
 
     def _node_view(self, n0, n1, ws_bytes, dev):
         """A TrainStep over nodes [n0, n1) that shares this one's storage: every per-node tensor is a slice,
@@ -181,6 +188,8 @@ class TrainStep:
             for k, v in b.items():
                 if k == "desc":
                     cb[k] = api.conv_desc(n1 - n0, v.B, v.H, v.W, v.Cin, v.Cout, v.R, v.S, v.stride, v.pad)
+                elif k == "direct":
+                    cb[k] = bool(api.lpdt_qconv_bwd_weight_direct(cb["desc"]))
                 elif k == "ws_ren":
                     per = v.numel() // N
                     cb[k] = v[n0 * per:n1 * per]
@@ -422,6 +431,9 @@ class TrainStep:
                                                   dw_node_stride=b["wn"], ws=self.ws_side, dev_status=self.dev_status)
                         api.lpdt_quantize(b["gw"], N, b["wn"], b["wn"], b["gq"], b["gs"], self.ws_side)
                         api.lpdt_dequantize(b["gq"], N, b["wn"], b["gs"], self._g(op["w_off"]), d)
+                    elif b["direct"]:
+                        api.lpdt_qconv_bwd_weight(b["desc"], b["E"], b["sE"], b["qA"], b["sA"], dW=self._g(op["w_off"]),
+                                                  dw_node_stride=d, ws=self.ws_side, dev_status=self.dev_status)
                     else:
                         # raw sums now, one conversion launch for all layers after the last of them
                         api.lpdt_qconv_bwd_weight(b["desc"], b["E"], b["sE"], b["qA"], b["sA"], dWacc=b["gacc"],
@@ -487,14 +499,14 @@ class TrainStep:
 
     def _finish_gradients(self):
         """After every group's backward pass, all nodes at once on the side stream: all norm layers'
-        parameter-gradient sums in one launch, all layers' int32 weight-gradient sums to fp32 in another."""
+        parameter-gradient sums in one launch, the int32 weight-gradient sums that are left to fp32 in another."""
         N, d = self.N, self.d
         pending_ren = [(op, b) for op, b in zip(self.ops, self.buf) if op["op"] == "ren"]
         api.wait_stream(self.side, torch.cuda.current_stream())
         with torch.cuda.stream(self.side):
             self._ren_param_sums(pending_ren)
             if not self.quantize_wgrad:
-                convs = [(op, b) for op, b in zip(self.ops, self.buf) if op["op"] in ("conv", "linear")]
+                convs = [(op, b) for op, b in zip(self.ops, self.buf) if op["op"] in ("conv", "linear") and not b["direct"]]
                 for lo in range(0, len(convs), 64):
                     part = convs[lo:lo + 64]
                     api.lpdt_dequantize_acc_batch(self.g_acc, N, [self.g_acc_off[b["wi"]] for _, b in part],

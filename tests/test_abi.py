@@ -61,3 +61,12 @@ def test_zero_point_backward_weight_asks_for_what_it_writes():
         d = api.conv_desc(nodes, 4, H, H, cin, cout, R, R, 1, R // 2)
         own = up(4 * nodes * R * R * cin * cout) + up(4 * nodes * R * R * cout) + up(4 * nodes * R * R * cin)
         assert api.lpdt_qconv_bwd_weight_affine_workspace_size(d) == own + api.lpdt_qconv_workspace_size(d, 2)
+
+
+def test_which_weight_gradients_take_one_launch():
+    """Many output tiles and a short pixel loop: no sums in memory.  Few tiles, padded channels, no work: sums, or nothing."""
+    from paper_2111_09389_b200 import api
+    direct = lambda *d: api.lpdt_qconv_bwd_weight_direct(api.conv_desc(*d))
+    assert direct(8, 32, 2, 2, 512, 512) == 1 and direct(8, 32, 8, 8, 256, 256) == 1
+    assert direct(16, 32, 32, 32, 16, 16) == 0
+    assert direct(8, 32, 32, 32, 3, 64) == 0 and direct(0, 32, 2, 2, 512, 512) == 0 and direct(8, 0, 2, 2, 512, 512) == 0
