@@ -197,6 +197,12 @@ def call_bytes(name, a, kw):
         return n * (12 if kw.get("res") is not None else 8)
     if name == "lpdt_range_evonorm_bwd":
         return a[0] * a[1] * a[2] * a[3] * a[4] * 12
+    if name == "lpdt_range_evonorm_pool_fwd":   # x read, a quarter of the results and their positions written
+        n = a[0] * a[1] * a[2] * a[3] * a[4]
+        return n * 4 + n // 4 * 5
+    if name == "lpdt_range_evonorm_pool_bwd":   # x, pooled gradient and positions read, dx written
+        n = a[0] * a[1] * a[2] * a[3] * a[4]
+        return n * 8 + n // 4 * 5
     if name == "lpdt_range_evonorm_fwd_q8":     # x read, codes written (+ fp32 y when kept, + shortcut read)
         n = a[0] * a[1] * a[2] * a[3] * a[4]
         return n * (5 + (4 if a[12] is not None else 0) + (4 if kw.get("res") is not None else 0))
@@ -344,6 +350,7 @@ def source_hash(kernel):
 # lpdt_last_kernel)
 KERNEL_OF = {"lpdt_range_evonorm_fwd": "lpdt::ren_fwd_kernel", "lpdt_range_evonorm_bwd": "lpdt::ren_bwd_kernel",
              "lpdt_range_evonorm_fwd_q8": "lpdt::ren_fwd_q8_kernel", "lpdt_range_evonorm_bwd_q8": "lpdt::ren_bwd_q8_kernel",
+             "lpdt_range_evonorm_pool_fwd": "lpdt::ren_fwd_kernel", "lpdt_range_evonorm_pool_bwd": "lpdt::ren_pool_bwd_kernel",
              "lpdt_quantize_with_range": "lpdt::quantize_kernel", "lpdt_quantize": "lpdt::range_kernel + lpdt::quantize_kernel",
              "lpdt_gossip_mix": "lpdt::big_sample_kernel + big_collect_kernel + select_and_rows_kernel + gossip_mix_kernel",
              "lpdt_sgd_gossip_mix": "lpdt::sgd_dense_mix_kernel", "lpdt_residual_add": "lpdt::residual_add_v4_kernel",

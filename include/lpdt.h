@@ -337,6 +337,25 @@ lpdt_status lpdt_range_evonorm_bwd_params_batch(int32_t nodes, int32_t B, int32_
                                                 const void *const *ws, const int64_t *grad_offsets,
                                                 float *grads, int64_t grad_node_stride, void *stream);
 
+/* Range-EvoNorm and the 2x2 max-pooling behind it (H and W even) in one launch each way.  lpdt_range_evonorm_pool_fwd writes
+ * what lpdt_range_evonorm_fwd followed by lpdt_maxpool2x2 writes: the pooled y [nodes][B][H/2][W/2][C], the positions idx of the
+ * maxima (int8, shape of y) and the statistics; amax_out (nullable, caller-zeroed) takes max|pooled y| per node.
+ * lpdt_range_evonorm_pool_bwd takes the pooled gradient dy and idx and writes what lpdt_maxpool2x2_bwd followed by
+ * lpdt_range_evonorm_bwd (parameter gradients left as partial sums in ws, for lpdt_range_evonorm_bwd_params) writes.
+ * Errors: INVALID_ARG, WORKSPACE, CUDA; UNSUPPORTED (serve with the two calls): H or W odd, C or C/groups no multiple of 4,
+ * more than 1024 channels, fp32 tensors not 16-byte aligned, idx not 4-byte aligned. */
+lpdt_status lpdt_range_evonorm_pool_fwd(int32_t nodes, int32_t B, int32_t H, int32_t W, int32_t C, int32_t groups,
+                                        float eps, const float *x, const float *v, const float *gamma,
+                                        const float *beta, int64_t param_node_stride, float *y, int8_t *idx,
+                                        float *gmin, float *gmax, int32_t *argmin, int32_t *argmax,
+                                        float *amax_out, void *stream);
+lpdt_status lpdt_range_evonorm_pool_bwd(int32_t nodes, int32_t B, int32_t H, int32_t W, int32_t C, int32_t groups,
+                                        float eps, const float *dy, const int8_t *idx, const float *x,
+                                        const float *v, const float *gamma, int64_t param_node_stride,
+                                        const float *gmin, const float *gmax, const int32_t *argmin,
+                                        const int32_t *argmax, float *dx, float *amax_out, void *ws,
+                                        size_t ws_bytes, void *stream);
+
 /* Range-EvoNorm with the requantize step inside (Section 3, "Low Precision Training": activations and layer
  * gradients travel between layers as 8-bit tensors).  lpdt_range_evonorm_fwd_q8 computes y as
  * lpdt_range_evonorm_fwd does and ALSO writes y's symmetric 8-bit codes q (int8, shape of y) and per-node scale

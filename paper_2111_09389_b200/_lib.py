@@ -56,6 +56,8 @@ SIGNATURES = {
                                   [_i64, _vp, _vp, _sz, _vp, _sz, _vp, _vp]),
     "lpdt_range_evonorm_bwd_workspace_size": (_sz, [_i32, _i32, _i32]),
     "lpdt_range_evonorm_bwd": (_i32, [_i32] * 6 + [_f32] + [_vp] * 4 + [_i64] + [_vp] * 8 + [_i64, _vp, _vp, _sz, _vp]),
+    "lpdt_range_evonorm_pool_fwd": (_i32, [_i32] * 6 + [_f32] + [_vp] * 4 + [_i64] + [_vp] * 7 + [_vp]),
+    "lpdt_range_evonorm_pool_bwd": (_i32, [_i32] * 6 + [_f32] + [_vp] * 5 + [_i64] + [_vp] * 7 + [_sz, _vp]),
     "lpdt_evonorm_s0_fwd": (_i32, [_i32] * 6 + [_f32] + [_vp] * 4 + [_i64] + [_vp] * 4),
     "lpdt_evonorm_s0_bwd_workspace_size": (_sz, [_i32, _i32, _i32]),
     "lpdt_evonorm_s0_bwd": (_i32, [_i32] * 6 + [_f32] + [_vp] * 4 + [_i64] + [_vp] * 6 + [_i64, _vp, _sz, _vp]),

@@ -16,7 +16,7 @@ from ._lib import lib as _load
 
 
 # Entry points that enqueue kernels (wrapped for the optional call log and per-call timing).
-LAUNCHING = {"lpdt_quantize", "lpdt_quantize_with_range", "lpdt_quantize_static", "lpdt_quantize_batch", "lpdt_dequantize", "lpdt_qconv_fwd", "lpdt_qconv_fwd_affine", "lpdt_qconv_bwd_data_affine", "lpdt_qconv_bwd_weight_affine", "lpdt_qconv_bwd_data", "lpdt_qconv_bwd_weight", "lpdt_range_evonorm_fwd", "lpdt_range_evonorm_bwd", "lpdt_range_evonorm_fwd_q8", "lpdt_range_evonorm_bwd_q8", "lpdt_range_evonorm_bwd_params", "lpdt_range_evonorm_bwd_params_batch", "lpdt_dequantize_acc_batch", "lpdt_gossip_mix", "lpdt_gossip_mix_q8", "lpdt_deepsqueeze_mix", "lpdt_pushsum_debias", "lpdt_sgd_gossip_mix", "lpdt_evonorm_s0_fwd", "lpdt_evonorm_s0_bwd", "lpdt_range_bn_fwd", "lpdt_range_bn_bwd", "lpdt_sgd_update", "lpdt_residual_add", "lpdt_residual_add_bwd", "lpdt_avgpool", "lpdt_avgpool_bwd", "lpdt_maxpool2x2", "lpdt_maxpool2x2_bwd", "lpdt_softmax_ce", "lpdt_colsum", "lpdt_selftest_bounded_wait"}
+LAUNCHING = {"lpdt_quantize", "lpdt_quantize_with_range", "lpdt_quantize_static", "lpdt_quantize_batch", "lpdt_dequantize", "lpdt_qconv_fwd", "lpdt_qconv_fwd_affine", "lpdt_qconv_bwd_data_affine", "lpdt_qconv_bwd_weight_affine", "lpdt_qconv_bwd_data", "lpdt_qconv_bwd_weight", "lpdt_range_evonorm_fwd", "lpdt_range_evonorm_bwd", "lpdt_range_evonorm_fwd_q8", "lpdt_range_evonorm_bwd_q8", "lpdt_range_evonorm_pool_fwd", "lpdt_range_evonorm_pool_bwd", "lpdt_range_evonorm_bwd_params", "lpdt_range_evonorm_bwd_params_batch", "lpdt_dequantize_acc_batch", "lpdt_gossip_mix", "lpdt_gossip_mix_q8", "lpdt_deepsqueeze_mix", "lpdt_pushsum_debias", "lpdt_sgd_gossip_mix", "lpdt_evonorm_s0_fwd", "lpdt_evonorm_s0_bwd", "lpdt_range_bn_fwd", "lpdt_range_bn_bwd", "lpdt_sgd_update", "lpdt_residual_add", "lpdt_residual_add_bwd", "lpdt_avgpool", "lpdt_avgpool_bwd", "lpdt_maxpool2x2", "lpdt_maxpool2x2_bwd", "lpdt_softmax_ce", "lpdt_colsum", "lpdt_selftest_bounded_wait"}
 # A thread that records (see Calls) gets a library whose launching entry points note their arguments as they run.
 class _Recording(threading.local):
     calls = None
@@ -263,6 +263,22 @@ def lpdt_range_evonorm_fwd(nodes, B, H, W, Cc, groups, eps, x, v, gamma, beta, p
     _check("lpdt_range_evonorm_fwd", lib().lpdt_range_evonorm_fwd(
         nodes, B, H, W, Cc, groups, eps, _ptr(x), _ptr(v), _ptr(gamma), _ptr(beta), param_node_stride,
         _ptr(y), _ptr(gmin), _ptr(gmax), _ptr(argmin), _ptr(argmax), _ptr(amax_out), _ptr(res), _stream()))
+
+
+def lpdt_range_evonorm_pool_fwd(nodes, B, H, W, Cc, groups, eps, x, v, gamma, beta, param_node_stride, y, idx, gmin, gmax,
+                                argmin, argmax, amax_out=None):
+    """The layer and the 2x2 max-pooling behind it; y, idx pooled."""
+    _check("lpdt_range_evonorm_pool_fwd", lib().lpdt_range_evonorm_pool_fwd(
+        nodes, B, H, W, Cc, groups, eps, _ptr(x), _ptr(v), _ptr(gamma), _ptr(beta), param_node_stride, _ptr(y), _ptr(idx),
+        _ptr(gmin), _ptr(gmax), _ptr(argmin), _ptr(argmax), _ptr(amax_out), _stream()))
+
+
+def lpdt_range_evonorm_pool_bwd(nodes, B, H, W, Cc, groups, eps, dy, idx, x, v, gamma, param_node_stride, gmin, gmax, argmin,
+                                argmax, dx, ws, amax_out=None):
+    p, nb = _ws(ws)
+    _check("lpdt_range_evonorm_pool_bwd", lib().lpdt_range_evonorm_pool_bwd(
+        nodes, B, H, W, Cc, groups, eps, _ptr(dy), _ptr(idx), _ptr(x), _ptr(v), _ptr(gamma), param_node_stride, _ptr(gmin),
+        _ptr(gmax), _ptr(argmin), _ptr(argmax), _ptr(dx), _ptr(amax_out), p, nb, _stream()))
 
 
 def lpdt_range_evonorm_q8_ctl_size(nodes):

@@ -42,7 +42,8 @@ static const Entry kEntries[] = {
     LPDT_ENTRY(lpdt_fill_zero), LPDT_ENTRY(lpdt_quantize), LPDT_ENTRY(lpdt_quantize_with_range), LPDT_ENTRY(lpdt_quantize_batch),
     LPDT_ENTRY(lpdt_dequantize), LPDT_ENTRY(lpdt_qconv_fwd), LPDT_ENTRY(lpdt_qconv_bwd_data), LPDT_ENTRY(lpdt_qconv_bwd_weight),
     LPDT_ENTRY(lpdt_range_evonorm_fwd), LPDT_ENTRY(lpdt_range_evonorm_bwd), LPDT_ENTRY(lpdt_range_evonorm_fwd_q8),
-    LPDT_ENTRY(lpdt_range_evonorm_bwd_q8), LPDT_ENTRY(lpdt_range_evonorm_bwd_params_batch), LPDT_ENTRY(lpdt_dequantize_acc_batch),
+    LPDT_ENTRY(lpdt_range_evonorm_bwd_q8), LPDT_ENTRY(lpdt_range_evonorm_pool_fwd),
+    LPDT_ENTRY(lpdt_range_evonorm_pool_bwd), LPDT_ENTRY(lpdt_range_evonorm_bwd_params_batch), LPDT_ENTRY(lpdt_dequantize_acc_batch),
     LPDT_ENTRY(lpdt_gossip_mix), LPDT_ENTRY(lpdt_gossip_mix_q8), LPDT_ENTRY(lpdt_sgd_gossip_mix), LPDT_ENTRY(lpdt_sgd_update),
     LPDT_ENTRY(lpdt_residual_add), LPDT_ENTRY(lpdt_residual_add_bwd), LPDT_ENTRY(lpdt_avgpool), LPDT_ENTRY(lpdt_avgpool_bwd),
     LPDT_ENTRY(lpdt_maxpool2x2), LPDT_ENTRY(lpdt_maxpool2x2_bwd), LPDT_ENTRY(lpdt_softmax_ce), LPDT_ENTRY(lpdt_colsum)};

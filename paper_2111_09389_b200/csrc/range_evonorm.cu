@@ -94,14 +94,18 @@ __device__ void reduce_groups(Ext mn, Ext mx, Ext *s_mn, Ext *s_mx, Ext *g_mn, E
     __syncthreads();
 }
 
-template <int V, bool RES>
+// POOL (V = 4): y is the 2 x 2 max-pooled result and idx the position of the maximum in its window (0 to 3 in row order, the
+// first of equals), and amax_out takes max|pooled|: the full result, which only the pooling reads, stays off memory (8 B less
+// per element than layer and pooling apart).
+template <int V, bool RES, bool POOL = false>
 __global__ void __launch_bounds__(512, 2)
 ren_fwd_kernel(int HW, int C, int groups, float eps, float Cst,
                const float *__restrict__ x, const float *__restrict__ v,
                const float *__restrict__ gamma, const float *__restrict__ beta, int64_t pstride,
                int B, float *__restrict__ y, float *__restrict__ gmin, float *__restrict__ gmax,
                int32_t *__restrict__ argmin, int32_t *__restrict__ argmax, float *__restrict__ amax_out,
-               const float *__restrict__ res, int R /*CTAs per sample (cluster size)*/, int ppc /*pixels per CTA*/) {
+               const float *__restrict__ res, int R /*CTAs per sample (cluster size)*/, int ppc /*pixels per CTA*/,
+               int W /*POOL: pixels per row*/, char4 *__restrict__ idx) {
     namespace cg = cooperative_groups;
     pdl_enter();
     extern __shared__ unsigned char smem_raw[];
@@ -184,6 +188,41 @@ ren_fwd_kernel(int HW, int C, int groups, float eps, float Cst,
         vc[k] = v[(int64_t)node * pstride + c0 + k];
         gc[k] = gamma[(int64_t)node * pstride + c0 + k];
         bc[k] = beta[(int64_t)node * pstride + c0 + k];
+    }
+    if constexpr (POOL) {
+        const int Wo = W / 2, n = HW / 4, share = (n + R - 1) / R;           // windows of this CTA, wherever its first pass was
+        const int end = (rank + 1) * share < n ? (rank + 1) * share : n;
+        const F2 nz = opaque_minus_zero2(HW), inv2 = pack2(invD, invD);
+        const F2 v01 = pack2(vc[0], vc[1]), v23 = pack2(vc[2], vc[3]), g01 = pack2(gc[0], gc[1]), g23 = pack2(gc[2], gc[3]);
+        const F2 b01 = pack2(bc[0], bc[1]), b23 = pack2(bc[2], bc[3]);
+        auto norm = [&](F2 x, F2 v2, F2 g2, F2 b2, float &a, float &b) {
+            unpack2(add2(mul2(mul2(g2, mul2(x, hsig2(mul2(v2, x, nz)))), inv2, nz), b2), a, b);
+        };
+        for (int q = rank * share + row0; q < end; q += rstep) {
+            const float *w0 = xs + (int64_t)(q / Wo * 2 * W + q % Wo * 2) * C + c0;
+            float4 xv[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) xv[k] = *reinterpret_cast<const float4 *>(w0 + ((k >> 1) * W + (k & 1)) * (int64_t)C);
+            float best[4];
+            int at[4] = {0, 0, 0, 0};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                float yv[4];
+                norm(pack2(xv[k].x, xv[k].y), v01, g01, b01, yv[0], yv[1]);
+                norm(pack2(xv[k].z, xv[k].w), v23, g23, b23, yv[2], yv[3]);
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (k == 0 || yv[j] > best[j]) { best[j] = yv[j]; at[j] = k; }
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) ymax = fmaxf(ymax, fabsf(best[j]));
+            const int64_t o = sample * (int64_t)n * C + (int64_t)q * C + c0;
+            *reinterpret_cast<float4 *>(y + o) = make_float4(best[0], best[1], best[2], best[3]);
+            idx[o / 4] = make_char4((signed char)at[0], (signed char)at[1], (signed char)at[2], (signed char)at[3]);
+        }
+        if (amax_out) block_amax_to(ymax, amax_out + node);
+        if (R > 1) cg::this_cluster().barrier_wait();
+        return;
     }
     const float *rs = RES ? res + sample * (int64_t)HW * C : nullptr;
     auto emit = [&](int pp, const float (&xv)[V], const float (&rv)[V]) {
@@ -454,14 +493,17 @@ ren_fwd_q8_kernel(int HW, int C, int groups, float eps, float Cst,
 // statistics and parameters are read.  DEPTH = 0: rows are loaded into registers, two per trip.
 // XHOLD (with DEPTH > 0): the sample's x has been requested into `dxs` (shared memory) as the oldest pending
 // copy group; only dy goes through the ring, and dx overwrites x in place.
-template <int V, int DEPTH, bool XHOLD = false>
+// POOL (V = 4, DEPTH = 0): dy and pool_idx are those of the 2 x 2 pooling behind the layer; a thread walks windows.  All but one
+// of a window's gradients are zero, so only that one's terms are evaluated (all, where a value is not finite).
+template <int V, int DEPTH, bool XHOLD = false, bool POOL = false>
 __device__ __forceinline__ void ren_bwd_sample(unsigned char *smem_raw, int HW, int C, int groups, float eps, float Cst,
                                                const float *__restrict__ dy, const float *__restrict__ x,
                                                const float *__restrict__ v, const float *__restrict__ gamma,
                                                int64_t pstride, const float *__restrict__ gmin,
                                                const float *__restrict__ gmax, const int32_t *__restrict__ argmin,
                                                const int32_t *__restrict__ argmax, double *__restrict__ acc,
-                                               int64_t sample, int node, float *dxs, float &dmax, int R = 1, int rank = 0, int ppc = 0) {
+                                               int64_t sample, int node, float *dxs, float &dmax, int R = 1, int rank = 0, int ppc = 0,
+                                               int W = 0, const char4 *__restrict__ pool_idx = nullptr) {
     namespace cg = cooperative_groups;
     const int T = blockDim.x, t = threadIdx.x;
     const int p_lo = rank * ppc, p_end = R > 1 && p_lo + ppc < HW ? p_lo + ppc : HW;      // this CTA's pixels
@@ -587,8 +629,84 @@ __device__ __forceinline__ void ren_bwd_sample(unsigned char *smem_raw, int HW, 
         }
         cp_async_wait<0>();
     }
+    if constexpr (POOL) {
+        const int Wo = W / 2, n = HW / 4, share = (n + R - 1) / R, end = (rank + 1) * share < n ? (rank + 1) * share : n;
+        const float *dps = dy + sample * (int64_t)n * C;
+        const char4 *ids = pool_idx + sample * (int64_t)n * C / 4;
+        const F2 inv2 = pack2(invD, invD), zero2 = 0;
+        auto load = [&](int q, float4 (&x)[4], float4 &g, char4 &id) {
+            const float *w0 = xs + (int64_t)(q / Wo * 2 * W + q % Wo * 2) * C + c0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) x[k] = *reinterpret_cast<const float4 *>(w0 + ((k >> 1) * W + (k & 1)) * (int64_t)C);
+            g = *reinterpret_cast<const float4 *>(dps + (int64_t)q * C + c0);
+            id = ids[((int64_t)q * C + c0) / 4];
+        };
+        for (int q = rank * share + row0; q < end; q += rstep) {
+            float4 x4[4], g4;
+            char4 id4;
+            load(q, x4, g4, id4);
+            const int p0 = q / Wo * 2 * W + q % Wo * 2;
+            const float g[4] = {g4.x, g4.y, g4.z, g4.w};
+            const int id[4] = {id4.x, id4.y, id4.z, id4.w};
+            // x * 0 is 0 unless a value is infinite or not a number
+            F2 probe = zero2;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) probe = fma2(pack2(x4[k].x, x4[k].y), zero2, fma2(pack2(x4[k].z, x4[k].w), zero2, probe));
+            float pa, pb;
+            unpack2(probe, pa, pb);
+            if (!(pa == 0.f && pb == 0.f)) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const float xk[4] = {x4[k].x, x4[k].y, x4[k].z, x4[k].w};
+                    const float dk[4] = {id[0] == k ? g[0] : 0.f, id[1] == k ? g[1] : 0.f, id[2] == k ? g[2] : 0.f, id[3] == k ? g[3] : 0.f};
+                    term(p0 + (k >> 1) * W + (k & 1), reinterpret_cast<const float (&)[V]>(xk), reinterpret_cast<const float (&)[V]>(dk));
+                }
+                continue;
+            }
+            float o[4], m4 = 0.f;
+#pragma unroll
+            for (int k = 0; k < 4; k += 2) {
+                const float xa = k ? (id[2] & 1 ? (id[2] & 2 ? x4[3].z : x4[1].z) : (id[2] & 2 ? x4[2].z : x4[0].z))
+                                   : (id[0] & 1 ? (id[0] & 2 ? x4[3].x : x4[1].x) : (id[0] & 2 ? x4[2].x : x4[0].x));
+                const float xb = k ? (id[3] & 1 ? (id[3] & 2 ? x4[3].w : x4[1].w) : (id[3] & 2 ? x4[2].w : x4[0].w))
+                                   : (id[1] & 1 ? (id[1] & 2 ? x4[3].y : x4[1].y) : (id[1] & 2 ? x4[2].y : x4[0].y));
+                const F2 x = pack2(xa, xb), d = pack2(g[k], g[k + 1]);
+                const F2 u = mul2(pack2(vc[k], vc[k + 1]), x, nz), hs = hsig2(u);
+                float a, b;
+                unpack2(u, a, b);
+                const F2 hp = pack2(fabsf(a) < 3.f ? sixth : 0.f, fabsf(b) < 3.f ? sixth : 0.f);
+                const F2 m = mul2(x, hs), tt = mul2(d, pack2(gc[k], gc[k + 1]));
+                unpack2(mul2(tt, m), a, b);
+                S += (double)a; S += (double)b;
+                fb[k] += (double)g[k]; fb[k + 1] += (double)g[k + 1];
+                unpack2(mul2(d, mul2(m, inv2)), a, b);
+                fg[k] += (double)a; fg[k + 1] += (double)b;
+                unpack2(mul2(mul2(mul2(tt, mul2(x, x)), hp), inv2), a, b);
+                fv[k] += (double)a; fv[k + 1] += (double)b;
+                unpack2(mul2(mul2(tt, add2(hs, mul2(u, hp, nz))), inv2), o[k], o[k + 1]);
+                m4 = fmaxf(m4, fmaxf(fabsf(o[k]), fabsf(o[k + 1])));
+            }
+            bool extremum = false;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int at = (p0 + (k >> 1) * W + (k & 1)) * C + c0;
+                *reinterpret_cast<float4 *>(dxs + at) = make_float4(id[0] == k ? o[0] : 0.f, id[1] == k ? o[1] : 0.f,
+                                                                    id[2] == k ? o[2] : 0.f, id[3] == k ? o[3] : 0.f);
+                extremum |= (unsigned)(g_amx - at) < 4u || (unsigned)(g_amn - at) < 4u;
+            }
+            if (extremum) {
+                m4 = 0.f;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int at = (p0 + (id[j] >> 1) * W + (id[j] & 1)) * C + c0 + j;
+                    if (at != g_amx && at != g_amn) m4 = fmaxf(m4, fabsf(o[j]));
+                }
+            }
+            dmax = fmaxf(dmax, m4);
+        }
+    }
     // DEPTH = 0, two rows per trip: four independent 16-byte loads in flight per thread
-    for (int i = 0; DEPTH == 0 && i < iters; i += 2) {
+    for (int i = 0; !POOL && DEPTH == 0 && i < iters; i += 2) {
         const int p0 = p_lo + row0 + i * rstep, p1 = p0 + rstep;
         const bool ok0 = p0 < p_end, ok1 = (i + 1 < iters) && (p1 < p_end);
         float xa[V], da[V], xb[V], db[V];
@@ -658,7 +776,12 @@ __device__ __forceinline__ void ren_bwd_sample(unsigned char *smem_raw, int HW, 
     if (t < groups) {
         const int64_t sgg = sample * groups + t;
         const int amx = argmax[sgg], amn = argmin[sgg];
-        const bool has_mx = R == 1 || (amx >= p_lo * C && amx < p_end * C), has_mn = R == 1 || (amn >= p_lo * C && amn < p_end * C);
+        bool has_mx = R == 1 || (amx >= p_lo * C && amx < p_end * C), has_mn = R == 1 || (amn >= p_lo * C && amn < p_end * C);
+        if (POOL && R > 1) {          // whose window
+            const int share = (HW / 4 + R - 1) / R, Wo = W / 2, a = amx / C, b = amn / C;
+            has_mx = (a / W / 2 * Wo + a % W / 2) / share == rank;
+            has_mn = (b / W / 2 * Wo + b % W / 2) / share == rank;
+        }
         if (amx != amn) {
             const float rng_g = __fsub_rn(gmax[sgg], gmin[sgg]);
             const float invDg = __fdiv_rn(1.f, __fadd_rn(__fmul_rn(Cst, rng_g), eps));
@@ -699,6 +822,23 @@ ren_bwd_kernel(int HW, int C, int groups, float eps, float Cst,
     float dmax = 0.f;
     ren_bwd_sample<V, DEPTH>(smem_raw, HW, C, groups, eps, Cst, dy, x, v, gamma, pstride, gmin, gmax, argmin, argmax, acc,
                              sample, node, dx + sample * (int64_t)HW * C, dmax, R, (int)(blockIdx.x % R), ppc);
+    if (amax_out) block_amax_to(dmax, amax_out + node);
+}
+
+// Backward of the layer and the 2 x 2 max-pooling behind it.
+__global__ void __launch_bounds__(256, 2)
+ren_pool_bwd_kernel(int HW, int C, int groups, float eps, float Cst, const float *__restrict__ dy, const float *__restrict__ x,
+                    const float *__restrict__ v, const float *__restrict__ gamma, int64_t pstride, int B,
+                    const float *__restrict__ gmin, const float *__restrict__ gmax, const int32_t *__restrict__ argmin,
+                    const int32_t *__restrict__ argmax, float *__restrict__ dx, double *__restrict__ acc,
+                    float *__restrict__ amax_out, int R, int W, const char4 *__restrict__ idx) {
+    pdl_enter();
+    extern __shared__ unsigned char smem_raw[];
+    const int64_t sample = blockIdx.x / R;
+    const int node = (int)(sample / B);
+    float dmax = 0.f;
+    ren_bwd_sample<4, 0, false, true>(smem_raw, HW, C, groups, eps, Cst, dy, x, v, gamma, pstride, gmin, gmax, argmin, argmax, acc,
+                                      sample, node, dx + sample * (int64_t)HW * C, dmax, R, (int)(blockIdx.x % R), HW, W, idx);
     if (amax_out) block_amax_to(dmax, amax_out + node);
 }
 
@@ -842,11 +982,9 @@ static float ren_const(int cpg) { return (float)(1.0 / sqrt(2.0 * log((double)cp
 
 using namespace lpdt;
 
-extern "C" lpdt_status lpdt_range_evonorm_fwd(int32_t nodes, int32_t B, int32_t H, int32_t W, int32_t C,
-                                              int32_t groups, float eps, const float *x, const float *v,
-                                              const float *gamma, const float *beta, int64_t pstride,
-                                              float *y, float *gmin, float *gmax, int32_t *argmin,
-                                              int32_t *argmax, float *amax_out, const float *res, void *stream) {
+static lpdt_status ren_fwd(int32_t nodes, int32_t B, int32_t H, int32_t W, int32_t C, int32_t groups, float eps, const float *x,
+                           const float *v, const float *gamma, const float *beta, int64_t pstride, float *y, float *gmin, float *gmax,
+                           int32_t *argmin, int32_t *argmax, float *amax_out, const float *res, int8_t *idx, void *stream) {
     LPDT_CHECK_ARG(nodes >= 0 && B >= 0 && H > 0 && W > 0 && C > 0 && groups > 0);
     LPDT_CHECK_ARG(C % groups == 0 && C / groups >= 2);
     if (nodes == 0 || B == 0) return LPDT_OK;
@@ -858,6 +996,7 @@ extern "C" lpdt_status lpdt_range_evonorm_fwd(int32_t nodes, int32_t B, int32_t 
     if (tforce < 0) { const char *e = getenv("LPDT_REN_FWD_THREADS"); tforce = e ? atoi(e) : 0; }
     if (!plan(C, groups, aligned(x, 16) && aligned(y, 16) && (!res || aligned(res, 16)), &pl, tforce == 128 ? 128 : 256))
         return LPDT_ERR_UNSUPPORTED;
+    if (idx && (pl.V != 4 || H % 2 || W % 2 || !aligned(idx, 4))) return LPDT_ERR_UNSUPPORTED;
     size_t smem = (size_t)(2 * pl.threads + 4 * groups) * sizeof(Ext);
     if (smem > 48 * 1024) return LPDT_ERR_UNSUPPORTED;
     const float Cst = ren_const(C / groups);
@@ -867,22 +1006,39 @@ extern "C" lpdt_status lpdt_range_evonorm_fwd(int32_t nodes, int32_t B, int32_t 
     if ((int64_t)nodes * B * R > 0x7fffffff) return LPDT_ERR_UNSUPPORTED;
     dim3 grid((unsigned)((int64_t)nodes * B * R));
     using Fn = void (*)(int, int, int, float, float, const float *, const float *, const float *, const float *, int64_t,
-                        int, float *, float *, float *, int32_t *, int32_t *, float *, const float *, int, int);
-    static const Fn fns[2][2] = {{ren_fwd_kernel<1, false>, ren_fwd_kernel<1, true>},
-                                 {ren_fwd_kernel<4, false>, ren_fwd_kernel<4, true>}};
+                        int, float *, float *, float *, int32_t *, int32_t *, float *, const float *, int, int, int, char4 *);
+    static const Fn fns[5] = {ren_fwd_kernel<1, false>, ren_fwd_kernel<1, true>, ren_fwd_kernel<4, false>, ren_fwd_kernel<4, true>,
+                              ren_fwd_kernel<4, false, true>};
     if (pl.threads <= 256 && R <= 4) {      // (clusters of 8 need the room of their group of SMs: 50 samples of 64 KB 6.8 us, 9.7 spread)
         static PerDeviceOnce attr;
         int dev;
         if (attr.pending(&dev)) {
-            for (int i = 0; i < 4; ++i) LPDT_CUDA(cudaFuncSetAttribute(fns[i / 2][i % 2], cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024));
+            for (int i = 0; i < 5; ++i) LPDT_CUDA(cudaFuncSetAttribute(fns[i], cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024));
             attr.mark(dev);
         }
         smem = spread_smem(smem, spread_grid((int64_t)nodes * B, R), 1024 / pl.threads);
     }
-    launch_k_cluster(fns[pl.V == 4 ? 1 : 0][res ? 1 : 0], grid, pl.threads, smem, as_stream(stream), R, H * W, C, groups, eps,
-                     Cst, x, v, gamma, beta, pstride, B, y, gmin, gmax, argmin, argmax, amax_out, res, R, ppc);
+    launch_k_cluster(fns[idx ? 4 : (pl.V == 4 ? 2 : 0) + (res ? 1 : 0)], grid, pl.threads, smem, as_stream(stream), R, H * W, C, groups, eps,
+                     Cst, x, v, gamma, beta, pstride, B, y, gmin, gmax, argmin, argmax, amax_out, res, R, ppc, W,
+                     reinterpret_cast<char4 *>(idx));
     LPDT_LAUNCH_CHECK();
     return LPDT_OK;
+}
+
+extern "C" lpdt_status lpdt_range_evonorm_fwd(int32_t nodes, int32_t B, int32_t H, int32_t W, int32_t C,
+                                              int32_t groups, float eps, const float *x, const float *v,
+                                              const float *gamma, const float *beta, int64_t pstride,
+                                              float *y, float *gmin, float *gmax, int32_t *argmin,
+                                              int32_t *argmax, float *amax_out, const float *res, void *stream) {
+    return ren_fwd(nodes, B, H, W, C, groups, eps, x, v, gamma, beta, pstride, y, gmin, gmax, argmin, argmax, amax_out, res, nullptr, stream);
+}
+
+extern "C" lpdt_status lpdt_range_evonorm_pool_fwd(int32_t nodes, int32_t B, int32_t H, int32_t W, int32_t C, int32_t groups,
+                                                   float eps, const float *x, const float *v, const float *gamma,
+                                                   const float *beta, int64_t pstride, float *y, int8_t *idx, float *gmin,
+                                                   float *gmax, int32_t *argmin, int32_t *argmax, float *amax_out, void *stream) {
+    LPDT_CHECK_ARG(nodes == 0 || B == 0 || idx);
+    return ren_fwd(nodes, B, H, W, C, groups, eps, x, v, gamma, beta, pstride, y, gmin, gmax, argmin, argmax, amax_out, nullptr, idx, stream);
 }
 
 extern "C" size_t lpdt_range_evonorm_bwd_workspace_size(int32_t nodes, int32_t B, int32_t C) {
@@ -971,6 +1127,43 @@ extern "C" lpdt_status lpdt_range_evonorm_bwd(int32_t nodes, int32_t B, int32_t 
     LPDT_LAUNCH_CHECK();
     if (deferred) return LPDT_OK;
     launch_k(ren_bwd_finalize, nodes * ((3 * C + 31) / 32), 256, 0, st, acc, nodes, B, C, dv, dgamma, dbeta, gstride);
+    LPDT_LAUNCH_CHECK();
+    return LPDT_OK;
+}
+
+extern "C" lpdt_status lpdt_range_evonorm_pool_bwd(int32_t nodes, int32_t B, int32_t H, int32_t W, int32_t C, int32_t groups,
+                                                   float eps, const float *dy, const int8_t *idx, const float *x, const float *v,
+                                                   const float *gamma, int64_t pstride, const float *gmin, const float *gmax,
+                                                   const int32_t *argmin, const int32_t *argmax, float *dx, float *amax_out,
+                                                   void *ws, size_t ws_bytes, void *stream) {
+    LPDT_CHECK_ARG(nodes >= 0 && B >= 0 && H > 0 && W > 0 && C > 0 && groups > 0);
+    LPDT_CHECK_ARG(C % groups == 0 && C / groups >= 2);
+    if (nodes == 0 || B == 0) return LPDT_OK;
+    LPDT_CHECK_ARG(dy && idx && x && v && gamma && gmin && gmax && argmin && argmax && dx);
+    LPDT_CHECK_ARG(pstride >= C || nodes == 1);
+    if ((int64_t)H * W * C > 0x7fffffff || H % 2 || W % 2 || !aligned(idx, 4)) return LPDT_ERR_UNSUPPORTED;
+    if (!ws || ws_bytes < lpdt_range_evonorm_bwd_workspace_size(nodes, B, C) || !aligned(ws, 8)) return LPDT_ERR_WORKSPACE;
+    RenPlan pl;
+    if (!plan(C, groups, aligned(x, 16) && aligned(dy, 16) && aligned(dx, 16), &pl) || pl.V != 4 || pl.threads > 256) return LPDT_ERR_UNSUPPORTED;
+    const int cv = C / 4, nsets = (cv <= 32 && 32 % cv == 0) ? pl.threads / 32 : 1;
+    size_t smem = (size_t)(nsets * 3 * C + pl.threads + groups) * sizeof(double);
+    if (smem > 48 * 1024 || groups > pl.threads) return LPDT_ERR_UNSUPPORTED;
+    // CTAs per sample: up to four, while every thread keeps two windows and the grid stays within one wave (two CTAs per SM)
+    const int64_t samples = (int64_t)nodes * B, rows = ceil_div((int64_t)(H / 2) * (W / 2), pl.threads / cv);
+    int R = 1;
+    while (R < 4 && rows >= 4 * R && samples * 2 * R <= 2 * kNumSMs) R *= 2;
+    while (R > 1 && (R - 1) * ceil_div((int64_t)(H / 2) * (W / 2), R) >= (int64_t)(H / 2) * (W / 2)) R /= 2;
+    if (samples * R > 0x7fffffff) return LPDT_ERR_UNSUPPORTED;
+    static PerDeviceOnce attr;
+    int dev;
+    if (attr.pending(&dev)) {
+        LPDT_CUDA(cudaFuncSetAttribute(ren_pool_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024));
+        attr.mark(dev);
+    }
+    smem = spread_smem(smem, spread_grid(samples, R), 512 / pl.threads);
+    launch_k_cluster(ren_pool_bwd_kernel, dim3((unsigned)(samples * R)), pl.threads, smem, as_stream(stream), R, H * W, C, groups, eps,
+                     ren_const(C / groups), dy, x, v, gamma, pstride, B, gmin, gmax, argmin, argmax, dx, (double *)ws, amax_out, R, W,
+                     reinterpret_cast<const char4 *>(idx));
     LPDT_LAUNCH_CHECK();
     return LPDT_OK;
 }

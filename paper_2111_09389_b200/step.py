@@ -128,6 +128,9 @@ class TrainStep:
                 b["q8_fwd"] = self.fuse_requantize and bool(api.lpdt_range_evonorm_fwd_q8_fits(B, H, W, Cc, G))
                 b["q8_bwd"] = (self.fuse_requantize and not grad_rounding and
                                bool(api.lpdt_range_evonorm_bwd_q8_fits(B, H, W, Cc, G)))
+                # 2x2 max-pooling right behind: one launch for both, in either direction
+                nxt = ops[len(self.buf) + 1] if len(self.buf) + 1 < len(ops) else {"op": ""}
+                b["pool"] = bool(nxt["op"] == "maxpool" and Cc % 4 == 0 and Cc // G % 4 == 0 and Cc <= 1024 and H % 2 == 0 and W % 2 == 0)
                 b["ctl"] = torch.zeros(api.lpdt_range_evonorm_q8_ctl_size(N), dtype=torch.uint8, device=dev)
             elif k == "add":
                 Ho, Wo = (op["H"] + op["stride"] - 1) // op["stride"], (op["W"] + op["stride"] - 1) // op["stride"]
@@ -317,6 +320,14 @@ class TrainStep:
         self.out = self.buf[-1]["out"]
         return self.out
 
+    def _pooled(self, li):
+        """Whether the max-pooling li runs in the launch of the norm layer in front of it."""
+        return li > 0 and self.buf[li - 1].get("pool", False)
+
+    def _bwd_q8(self, li):
+        """Whether the backward pass of the norm layer li writes the codes of the convolution in front of it itself."""
+        return self.buf[li]["q8_bwd"] and li > 0 and self.ops[li - 1]["op"] == "conv"
+
     def _forward_layers(self):
         N, B, d = self.N, self.B, self.d
         cur = self.x
@@ -363,6 +374,13 @@ class TrainStep:
                                                   b["ctl"], res=res, dev_status=self.dev_status)
                     cb["pre_quantized"] = True
                     cur, cur_range = b["out"], None
+                elif b["pool"]:
+                    mb = self.buf[li + 1]
+                    api.lpdt_range_evonorm_pool_fwd(N, B, op["H"], op["W"], Cc, op["groups"], self.eps, cur,
+                                                    self._p(op["p_off"]), self._p(op["p_off"] + Cc),
+                                                    self._p(op["p_off"] + 2 * Cc), d, mb["out"], mb["idx"], b["gmin"], b["gmax"],
+                                                    b["amin"], b["amax"], amax_out=self.ranges[li + 1])
+                    cur, cur_range = mb["out"], self.ranges[li + 1]
                 else:
                     api.lpdt_range_evonorm_fwd(N, B, op["H"], op["W"], Cc, op["groups"], self.eps, cur,
                                                self._p(op["p_off"]), self._p(op["p_off"] + Cc),
@@ -379,7 +397,7 @@ class TrainStep:
                 api.lpdt_residual_add(N, B, op["H"], op["W"], op["Ca"], op["C"], op["stride"], op["ch_off"],
                                       cur, a, b["out"], amax_out=self.ranges[li])
                 cur, cur_range = b["out"], self.ranges[li]
-            elif k == "maxpool":
+            elif k == "maxpool" and not self._pooled(li):
                 api.lpdt_maxpool2x2(N, B, op["H"], op["W"], op["C"], cur, b["out"], b["idx"])
                 cur = b["out"]        # max-pooling keeps max|x| only for non-negative maxima: range recomputed
                 cur_range = None
@@ -462,7 +480,7 @@ class TrainStep:
                                        bias=self._p(cop["b_off"]) if cop["op"] == "linear" else None,
                                        bias_node_stride=d, ws=self.ws, dev_status=self.dev_status)
                 # dx only; the parameter-gradient sums stay as partial sums and are reduced on the side stream
-                if b["q8_bwd"] and li > 0 and self.ops[li - 1]["op"] == "conv":
+                if self._bwd_q8(li):
                     # dx goes nowhere but into that convolution's quantizer: its codes are written here
                     cb = self.buf[li - 1]
                     api.lpdt_range_evonorm_bwd_q8(N, B, op["H"], op["W"], Cc, op["groups"], self.eps, g, b["x"],
@@ -471,6 +489,12 @@ class TrainStep:
                                                   d, b["ws_ren"], b["ctl"], dev_status=self.dev_status)
                     cb["E_ready"] = True
                     g, g_range = None, None
+                elif b["pool"]:
+                    api.lpdt_range_evonorm_pool_bwd(N, B, op["H"], op["W"], Cc, op["groups"], self.eps, g, self.buf[li + 1]["idx"],
+                                                    b["x"], self._p(op["p_off"]), self._p(op["p_off"] + Cc), d, b["gmin"],
+                                                    b["gmax"], b["amin"], b["amax"], b["dx"], b["ws_ren"],
+                                                    amax_out=self.ranges[L + li])
+                    g, g_range = b["dx"], self.ranges[L + li]
                 else:
                     api.lpdt_range_evonorm_bwd(N, B, op["H"], op["W"], Cc, op["groups"], self.eps, g, b["x"],
                                                self._p(op["p_off"]), self._p(op["p_off"] + Cc), d, b["gmin"],
@@ -487,6 +511,8 @@ class TrainStep:
                     api.lpdt_residual_add_bwd(N, B, aop["H"], aop["W"], aop["Ca"], aop["C"], aop["stride"],
                                               aop["ch_off"], dy_sc, g, b["dx"])
                     g, g_range = b["dx"], None
+            elif k == "maxpool" and self._pooled(li) and not self._bwd_q8(li - 1):
+                g_range = None                      # in the launch of the layer in front
             elif k == "maxpool":
                 api.lpdt_maxpool2x2_bwd(N, B, op["H"], op["W"], op["C"], g, b["idx"], b["dx"])
                 g, g_range = b["dx"], None
@@ -788,12 +814,13 @@ class _Reads:
 
 # The code that a walk over the layers executes, as it is here (TrainStep._own_walk compares).
 _METHOD_NAMES = frozenset(("_run", "_prepare", "_each_group", "forward", "_forward_layers", "backward", "_backward_layers",
-                           "_finish_gradients", "_ren_param_sums", "update", "_p", "_g"))
+                           "_finish_gradients", "_ren_param_sums", "update", "_p", "_g", "_pooled", "_bwd_q8"))
 _API = vars(api)
 _methods_of, _bindings_of = operator.attrgetter(*_METHOD_NAMES), operator.itemgetter(
     "wait_stream", "lpdt_fill_zero", "lpdt_quantize", "lpdt_quantize_with_range", "lpdt_quantize_batch", "lpdt_dequantize",
     "lpdt_qconv_fwd", "lpdt_qconv_bwd_data", "lpdt_qconv_bwd_weight", "lpdt_range_evonorm_fwd", "lpdt_range_evonorm_bwd",
-    "lpdt_range_evonorm_fwd_q8", "lpdt_range_evonorm_bwd_q8", "lpdt_range_evonorm_bwd_params_batch", "lpdt_dequantize_acc_batch",
+    "lpdt_range_evonorm_fwd_q8", "lpdt_range_evonorm_bwd_q8", "lpdt_range_evonorm_pool_fwd", "lpdt_range_evonorm_pool_bwd",
+    "lpdt_range_evonorm_bwd_params_batch", "lpdt_dequantize_acc_batch",
     "lpdt_gossip_mix", "lpdt_gossip_mix_q8", "lpdt_sgd_gossip_mix", "lpdt_sgd_update", "lpdt_residual_add",
     "lpdt_residual_add_bwd", "lpdt_avgpool", "lpdt_avgpool_bwd", "lpdt_maxpool2x2", "lpdt_maxpool2x2_bwd", "lpdt_softmax_ce",
     "lpdt_colsum")

@@ -754,6 +754,49 @@ def _ren_q8_check(case, ties, with_res, keep_y):
     assert not ctl.any() and int(status.item()) == 0
 
 
+@pytest.mark.parametrize("case", [(2, 3, 8, 8, 16, 2), (1, 2, 2, 2, 64, 8), (2, 2, 4, 6, 12, 3), (1, 5, 32, 32, 64, 8),
+                                  (2, 3, 16, 16, 128, 16), (1, 2, 4, 4, 512, 64), (1, 3, 6, 10, 160, 20), (5, 120, 8, 8, 32, 4)])
+@pytest.mark.parametrize("special", ["", "ties", "infinite"])
+def test_range_evonorm_and_max_pooling_in_one_launch(case, special):
+    """Equal to the layer and the pooling as two calls: everything to the bit, sums in double up to their order."""
+    nodes, B, H, W, C, groups = case
+    x, P, dy = _ren_inputs(case, seed=31, ties=special == "ties")
+    if special == "infinite":
+        x[0, 0, 0, 1, 0] = np.inf
+        x[-1, -1, 1, 1, -1] = np.nan
+    xd, Pd, stride = dev(x), dev(P), P.shape[1]
+    f = lambda *s: torch.full(s, 7.0, device="cuda")
+    i = lambda *s: torch.full(s, -5, dtype=torch.int32, device="cuda")
+    stats = lambda: (f(nodes, B, groups), f(nodes, B, groups), i(nodes, B, groups), i(nodes, B, groups))
+    half = (nodes, B, H // 2, W // 2, C)
+    same = lambda a, b: np.testing.assert_array_equal(a.cpu().numpy(), b.cpu().numpy())          # (NaN equals NaN, 0 equals -0)
+    y, st, pooled, idx = f(*x.shape), stats(), f(*half), torch.full(half, 9, dtype=torch.int8, device="cuda")
+    api.lpdt_range_evonorm_fwd(nodes, B, H, W, C, groups, 1e-5, xd, Pd, Pd[:, C:], Pd[:, 2 * C:], stride, y, *st)
+    api.lpdt_maxpool2x2(nodes, B, H, W, C, y, pooled, idx)
+    st2, pooled2, idx2, amax = stats(), f(*half), torch.full(half, 9, dtype=torch.int8, device="cuda"), torch.zeros(nodes, device="cuda")
+    api.lpdt_range_evonorm_pool_fwd(nodes, B, H, W, C, groups, 1e-5, xd, Pd, Pd[:, C:], Pd[:, 2 * C:], stride, pooled2, idx2, *st2,
+                                    amax_out=amax)
+    for a, b in zip((pooled, idx, *st), (pooled2, idx2, *st2)):
+        same(a, b)
+    same(amax, pooled.abs().reshape(nodes, -1).nan_to_num(0.0, posinf=float("inf")).amax(1))
+    if special == "infinite" and any(int(t.max()) == 2 ** 31 - 1 for t in st[2:]):
+        return                                   # a group of NaN alone has no extremum to go back to
+    g = dev(np.random.default_rng(3).standard_normal(half).astype(np.float32))
+    full, dx, dx2, r, r2 = f(*x.shape), f(*x.shape), f(*x.shape), torch.zeros(nodes, device="cuda"), torch.zeros(nodes, device="cuda")
+    n = api.lpdt_range_evonorm_bwd_workspace_size(nodes, B, C)
+    acc, acc2 = torch.zeros(n, dtype=torch.uint8, device="cuda"), torch.zeros(n, dtype=torch.uint8, device="cuda")
+    api.lpdt_maxpool2x2_bwd(nodes, B, H, W, C, g, idx, full)
+    api.lpdt_range_evonorm_bwd(nodes, B, H, W, C, groups, 1e-5, full, xd, Pd, Pd[:, C:], stride, *st, dx, None, None, None, stride, acc,
+                               amax_out=r)
+    api.lpdt_range_evonorm_pool_bwd(nodes, B, H, W, C, groups, 1e-5, g, idx, xd, Pd, Pd[:, C:], stride, *st, dx2, acc2, amax_out=r2)
+    # dx at the extrema holds the group sum, whose rounding may go the other way when its terms are added in another order
+    np.testing.assert_allclose(dx2.cpu().numpy(), dx.cpu().numpy(), rtol=1.2e-7, atol=0)
+    assert int((dx2 != dx).logical_and(~dx.isnan()).sum()) <= 2 * nodes * B * groups
+    np.testing.assert_allclose(r2.cpu().numpy(), r.cpu().numpy(), rtol=1.2e-7, atol=0)
+    a, b = (t[:nodes * B * 3 * C * 8].view(torch.float64).cpu().numpy() for t in (acc, acc2))
+    np.testing.assert_allclose(b, a, rtol=0, atol=1e-15 * H * W * np.nanmax(np.abs(np.where(np.isinf(a), 0, a))))      # H W / 4 terms
+
+
 @pytest.mark.parametrize("case", REN_Q8_CASES)
 @pytest.mark.parametrize("ties", [False, True])
 def test_range_evonorm_q8(case, ties):
