@@ -379,6 +379,255 @@ evonorm_bwd_cl_kernel(int HW, int C, int groups, float eps, const float *__restr
     if (R > 1) cluster.barrier_wait();
 }
 
+// ---- EvoNorm-S0 with the second read from L2 ---------------------------------------------------------------
+// A cluster of R CTAs owns a sample, small enough a part of the device that the samples in flight (one per cluster) stay well
+// inside the L2: the second pass reads them there, and nothing is held in between, so that three or four CTAs of an SM copy, meet
+// and write beside one another.  For widths whose channel columns divide a warp (the sums fold by shuffles).  Against the kernels
+// that hold the sample: 8 x 64 x 32x32x64 forward 81.9 -> 63.5 us (66 % of the HBM copy rate), backward 154.6 -> 126 (49 %:
+// its two passes issue the logistic twice); 16 x 32 x 32x32x16 32.8 -> 22.5 and 64 -> 48; 4 x 16 x 56x56x64 backward 314 -> 73.
+// The logistic function of two values, as sigmoidf_acc has it.
+__device__ __forceinline__ F2 sigmoid2(F2 u) {
+    float a, b;
+    unpack2(mul2(u, pack2(-1.44269504f, -1.44269504f)), a, b);
+    asm("ex2.approx.f32 %0, %0;" : "+f"(a));
+    asm("ex2.approx.f32 %0, %0;" : "+f"(b));
+    unpack2(add2(pack2(a, b), pack2(1.f, 1.f)), a, b);
+    asm("rcp.approx.f32 %0, %0;" : "+f"(a));
+    asm("rcp.approx.f32 %0, %0;" : "+f"(b));
+    return pack2(a, b);
+}
+template <int kU, class F> __device__ __forceinline__ void walk_rows(int p, int p_end, int rstep, const float *__restrict__ x, int C, F f) {
+    for (; p + (kU - 1) * rstep < p_end; p += kU * rstep) {
+        float4 v[kU];
+#pragma unroll
+        for (int j = 0; j < kU; ++j) v[j] = *reinterpret_cast<const float4 *>(x + (int64_t)(p + j * rstep) * C);
+#pragma unroll
+        for (int j = 0; j < kU; ++j) f(p + j * rstep, v[j]);
+    }
+    for (; p < p_end; p += rstep) f(p, *reinterpret_cast<const float4 *>(x + (int64_t)p * C));
+}
+template <int kU, class F> __device__ __forceinline__ void walk_rows2(int p, int p_end, int rstep, const float *__restrict__ x,
+                                                                      const float *__restrict__ y, int C, F f) {
+    for (; p + (kU - 1) * rstep < p_end; p += kU * rstep) {
+        float4 v[kU], w[kU];
+#pragma unroll
+        for (int j = 0; j < kU; ++j) {
+            v[j] = *reinterpret_cast<const float4 *>(x + (int64_t)(p + j * rstep) * C);
+            w[j] = *reinterpret_cast<const float4 *>(y + (int64_t)(p + j * rstep) * C);
+        }
+#pragma unroll
+        for (int j = 0; j < kU; ++j) f(p + j * rstep, v[j], w[j]);
+    }
+    for (; p < p_end; p += rstep) f(p, *reinterpret_cast<const float4 *>(x + (int64_t)p * C), *reinterpret_cast<const float4 *>(y + (int64_t)p * C));
+}
+
+__global__ void __launch_bounds__(256, 4)
+evonorm_fwd_l2_kernel(int HW, int C, int groups, float eps, const float *__restrict__ x, const float *__restrict__ v,
+                      const float *__restrict__ gamma, const float *__restrict__ beta, int64_t pstride, int B,
+                      float *__restrict__ y, float *__restrict__ gmean, float *__restrict__ gvar, int R, int ppc) {
+    namespace cg = cooperative_groups;
+    pdl_enter();
+    extern __shared__ double sm_d[];
+    const int T = blockDim.x, t = threadIdx.x, lane = t & 31, warp = t >> 5, nw = T >> 5;
+    double *s_sum = sm_d, *s_sq = sm_d + T, *part = sm_d + 2 * T;       // part: this CTA's [sum | sum of squares][groups]
+    double *g_inv = part + 2 * groups;
+    const int CV = C / 4, cpg = C / groups, col = t % CV, row0 = t / CV, rstep = T / CV, c0 = col * 4, grp = c0 / cpg;
+    const int rank = (int)(blockIdx.x % R), p_lo = rank * ppc, p_end = p_lo + ppc < HW ? p_lo + ppc : HW;
+    const int64_t sample = blockIdx.x / R;
+    const int node = (int)(sample / B);
+    const float *xs = x + sample * (int64_t)HW * C + c0;
+    double sum = 0.0, sq = 0.0;
+    walk_rows<8>(p_lo + row0, p_end, rstep, xs, C, [&](int, float4 a) {
+        const double d0 = a.x, d1 = a.y, d2 = a.z, d3 = a.w;
+        sum += d0; sq += d0 * d0; sum += d1; sq += d1 * d1; sum += d2; sq += d2 * d2; sum += d3; sq += d3 * d3;
+    });
+    s_sum[t] = sum; s_sq[t] = sq;
+    __syncthreads();
+    const int cols = cpg / 4, members = cols * rstep;
+    for (int g = warp; g < groups; g += nw) {
+        double a = 0.0, b = 0.0;
+        for (int m = lane; m < members; m += 32) {
+            const int th = (m / cols) * CV + g * cols + (m % cols);
+            a += s_sum[th]; b += s_sq[th];
+        }
+        a = warp_sum(a); b = warp_sum(b);
+        if (lane == 0) { part[g] = a; part[groups + g] = b; }
+    }
+    float vc[4], gc[4], bc[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        vc[k] = v[(int64_t)node * pstride + c0 + k];
+        gc[k] = gamma[(int64_t)node * pstride + c0 + k];
+        bc[k] = beta[(int64_t)node * pstride + c0 + k];
+    }
+    cg::cluster_group cluster = cg::this_cluster();
+    if (R > 1) cluster.sync(); else __syncthreads();
+    for (int g = t; g < groups; g += T) {
+        double a = 0.0, b = 0.0;
+        for (int r = 0; r < R; ++r) {
+            const double *pr = R > 1 ? cluster.map_shared_rank(part, r) : part;
+            a += pr[g]; b += pr[groups + g];
+        }
+        const double cnt = (double)HW * cpg, mu = a / cnt;
+        double var = b / cnt - mu * mu;
+        if (var < 0.0) var = 0.0;
+        g_inv[g] = 1.0 / sqrt(var + (double)eps);
+        if (rank == 0) { gmean[sample * groups + g] = (float)mu; gvar[sample * groups + g] = (float)var; }
+    }
+    __syncthreads();
+    if (R > 1) cluster.barrier_arrive();          // done reading the others' shared memory; waited for before exit
+    const float invD = (float)g_inv[grp];
+    float *ys = y + sample * (int64_t)HW * C + c0;
+    const F2 v01 = pack2(vc[0], vc[1]), v23 = pack2(vc[2], vc[3]), b01 = pack2(bc[0], bc[1]), b23 = pack2(bc[2], bc[3]);
+    const F2 g01 = pack2(gc[0] * invD, gc[1] * invD), g23 = pack2(gc[2] * invD, gc[3] * invD);
+    walk_rows<4>(p_lo + row0, p_end, rstep, xs, C, [&](int p, float4 a) {
+        const F2 x01 = pack2(a.x, a.y), x23 = pack2(a.z, a.w);
+        float yv[4];
+        unpack2(fma2(g01, mul2(x01, sigmoid2(mul2(v01, x01))), b01), yv[0], yv[1]);
+        unpack2(fma2(g23, mul2(x23, sigmoid2(mul2(v23, x23))), b23), yv[2], yv[3]);
+        NVec<4>::st(ys + (int64_t)p * C, yv);
+    });
+    if (R > 1) cluster.barrier_wait();
+}
+
+__global__ void __launch_bounds__(256, 3)
+evonorm_bwd_l2_kernel(int HW, int C, int groups, float eps, const float *__restrict__ dy, const float *__restrict__ x,
+                      const float *__restrict__ v, const float *__restrict__ gamma, int64_t pstride, int B,
+                      const float *__restrict__ gmean, const float *__restrict__ gvar, float *__restrict__ dx,
+                      double *__restrict__ acc, int R, int ppc) {
+    namespace cg = cooperative_groups;
+    pdl_enter();
+    extern __shared__ double sm_d[];
+    const int T = blockDim.x, t = threadIdx.x, lane = t & 31, warp = t >> 5, nw = T >> 5;
+    // [this CTA's group sums][group sums][channel sums: of the CTA, of every warp][the threads' parts of group sums]
+    double *part_S = sm_d, *g_S = part_S + groups, *part_ch = g_S + groups, *s_ch = part_ch + 3 * C, *s_S = s_ch + (size_t)nw * 3 * C;
+    const int CV = C / 4, cpg = C / groups, col = t % CV, row0 = t / CV, rstep = T / CV, c0 = col * 4, grp = c0 / cpg;
+    const int rank = (int)(blockIdx.x % R), p_lo = rank * ppc, p_end = p_lo + ppc < HW ? p_lo + ppc : HW;
+    const int64_t sample = blockIdx.x / R;
+    const int node = (int)(sample / B);
+    const int64_t at0 = sample * (int64_t)HW * C + c0;
+    const double mu = (double)gmean[sample * groups + grp];
+    const double Dd = sqrt((double)gvar[sample * groups + grp] + (double)eps);
+    const float invD = (float)(1.0 / Dd);
+    float vc[4], gc[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        vc[k] = v[(int64_t)node * pstride + c0 + k];
+        gc[k] = gamma[(int64_t)node * pstride + c0 + k];
+    }
+    // Partial sums of eight rows stay in fp32; every combination of them is done in double.  The factors that a channel's terms
+    // share (gamma, 1/D) follow the sums, and the group's sum is made of its channels'.
+    const F2 v01 = pack2(vc[0], vc[1]), v23 = pack2(vc[2], vc[3]), one = pack2(1.f, 1.f), minus = pack2(-1.f, -1.f);
+    double S = 0.0, sv[4] = {}, sg[4] = {}, sb[4] = {};
+    F2 fv01 = 0, fv23 = 0, fg01 = 0, fg23 = 0, fb01 = 0, fb23 = 0;
+    int n = 0;
+    auto flush2 = [&](F2 &f, double &a, double &b) {
+        float lo, hi;
+        unpack2(f, lo, hi);
+        a += (double)lo; b += (double)hi;
+        f = 0;
+    };
+    auto flush = [&]() {
+        flush2(fv01, sv[0], sv[1]); flush2(fv23, sv[2], sv[3]);
+        flush2(fg01, sg[0], sg[1]); flush2(fg23, sg[2], sg[3]);
+        flush2(fb01, sb[0], sb[1]); flush2(fb23, sb[2], sb[3]);
+    };
+    auto add_pair = [&](F2 xx, F2 d, F2 vv, F2 &fv, F2 &fg, F2 &fb) {
+        const F2 sig = sigmoid2(mul2(vv, xx)), q = mul2(d, mul2(xx, sig));
+        fb = add2(fb, d);
+        fg = add2(fg, q);                                                    // dy x sig
+        fv = fma2(q, mul2(xx, fma2(sig, minus, one)), fv);                   // dy x sig x (1 - sig)
+    };
+    walk_rows2<4>(p_lo + row0, p_end, rstep, x + at0, dy + at0, C, [&](int, float4 a, float4 b) {
+        add_pair(pack2(a.x, a.y), pack2(b.x, b.y), v01, fv01, fg01, fb01);
+        add_pair(pack2(a.z, a.w), pack2(b.z, b.w), v23, fv23, fg23, fb23);
+        if ((++n & 7) == 0) flush();
+    });
+    flush();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        S += (double)gc[k] * sg[k];
+        sv[k] *= (double)gc[k] * (double)invD;
+        sg[k] *= (double)invD;
+    }
+    s_S[t] = S;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        double a = sv[k], b = sg[k], c = sb[k];
+        for (int o = 16; o >= CV; o >>= 1) {
+            a += __shfl_xor_sync(0xffffffffu, a, o);
+            b += __shfl_xor_sync(0xffffffffu, b, o);
+            c += __shfl_xor_sync(0xffffffffu, c, o);
+        }
+        if (lane < CV) {
+            double *mine = s_ch + (size_t)warp * 3 * C + c0 + k;
+            mine[0] = a; mine[C] = b; mine[2 * C] = c;
+        }
+    }
+    __syncthreads();
+    const int cols = cpg / 4, members = cols * rstep;
+    for (int g = warp; g < groups; g += nw) {
+        double a = 0.0;
+        for (int m = lane; m < members; m += 32) a += s_S[(m / cols) * CV + g * cols + (m % cols)];
+        a = warp_sum(a);
+        if (lane == 0) part_S[g] = a;
+    }
+    for (int i = t; i < 3 * C; i += T) {
+        double a = s_ch[i];
+        for (int w = 1; w < nw; ++w) a += s_ch[(size_t)w * 3 * C + i];
+        part_ch[i] = a;
+    }
+    cg::cluster_group cluster = cg::this_cluster();
+    if (R > 1) cluster.sync(); else __syncthreads();
+    for (int g = t; g < groups; g += T) {
+        double a = 0.0;
+        for (int r = 0; r < R; ++r) a += (R > 1 ? cluster.map_shared_rank(part_S, r) : part_S)[g];
+        g_S[g] = a;
+    }
+    for (int i = rank * T + t; i < 3 * C; i += R * T) {
+        double a = 0.0;
+        for (int r = 0; r < R; ++r) a += (R > 1 ? cluster.map_shared_rank(part_ch, r) : part_ch)[i];
+        acc[sample * 3 * C + i] = a;
+    }
+    __syncthreads();
+    if (R > 1) cluster.barrier_arrive();
+    const double cnt = (double)HW * cpg;
+    const float coef = (float)(g_S[grp] / (cnt * Dd * Dd * Dd));
+    const float muf = (float)mu;
+    const F2 g01 = pack2(gc[0] * invD, gc[1] * invD), g23 = pack2(gc[2] * invD, gc[3] * invD), minus_coef = pack2(-coef, -coef), minus_mu = pack2(-muf, -muf);
+    auto out_pair = [&](F2 xx, F2 d, F2 vv, F2 gg) {
+        const F2 u = mul2(vv, xx), sig = sigmoid2(u);
+        const F2 slope = mul2(sig, fma2(u, fma2(sig, minus, one), one));     // sig (1 + u (1 - sig))
+        return fma2(mul2(d, gg), slope, mul2(minus_coef, add2(xx, minus_mu)));
+    };
+    walk_rows2<4>(p_lo + row0, p_end, rstep, x + at0, dy + at0, C, [&](int p, float4 a, float4 b) {
+        float o[4];
+        unpack2(out_pair(pack2(a.x, a.y), pack2(b.x, b.y), v01, g01), o[0], o[1]);
+        unpack2(out_pair(pack2(a.z, a.w), pack2(b.z, b.w), v23, g23), o[2], o[3]);
+        NVec<4>::st(dx + at0 + (int64_t)p * C, o);
+    });
+    if (R > 1) cluster.barrier_wait();
+}
+
+// CTAs per sample of these kernels (0: widths that they do not take): the samples in flight (`per_sm` CTAs on every SM, `bytes` a
+// sample) within 60 MB of the 126 MB of L2 - with 40 MB, 8 x 64 x 32x32x64 backward runs in clusters of 8, which the device has
+// trouble placing (150 us, in fours 126) - and two CTAs for every SM, while a thread keeps four rows.
+static int evonorm_l2_cluster(int64_t samples, int HW, int CV, int threads, double bytes, int per_sm, int *ppc_out) {
+    if (CV > 32 || 32 % CV || threads % 32) return 0;
+    const int rstep = threads / CV, rows = (int)ceil_div(HW, rstep);
+    const int64_t slots = (int64_t)kNumSMs * per_sm;
+    int R = 1;
+    while (R < 8 && rows >= 8 * R) {
+        const int64_t in_flight = samples < slots / R ? samples : slots / R;
+        if (in_flight * bytes <= 60.0 * 1024 * 1024 && samples * R >= 2 * (int64_t)kNumSMs) break;
+        R *= 2;
+    }
+    int ppc = (int)ceil_div(rows, R) * rstep;
+    while (R > 1 && (int64_t)(R - 1) * ppc >= HW) { R /= 2; ppc = (int)ceil_div(rows, R) * rstep; }       // no CTA without pixels
+    *ppc_out = ppc;
+    return R;
+}
+
 // Cluster size and pixels per CTA for the kernels above: the smallest power of two (up to 8, and so that every
 // CTA keeps a thread row) whose share of `bytes_per_pixel` fits `target` bytes; 0 when even 8 CTAs would need
 // more than `limit`.
@@ -397,24 +646,15 @@ static int evonorm_cluster(int HW, int rstep, size_t bytes_per_pixel, size_t tar
     }
 }
 
-// out[node][which][c] = sum over the node's samples of acc[node*B + b][which][c], rounded once.
-// One warp per output; lanes stride the samples and combine in a fixed shuffle tree.
-__global__ void norm_param_finalize(const double *__restrict__ acc, int nodes, int B, int C, int nwhich,
-                                    float *__restrict__ o0, float *__restrict__ o1, float *__restrict__ o2,
-                                    int64_t gstride) {
+// out[node][which][c] = sum over the node's samples of acc[node*B + b][which][c], rounded once.  Blocks of a node: ceil(nwhich C / 32).
+__global__ void __launch_bounds__(256)
+norm_param_finalize(const double *__restrict__ acc, int nodes, int B, int C, int nwhich,
+                    float *__restrict__ o0, float *__restrict__ o1, float *__restrict__ o2,
+                    int64_t gstride) {
     pdl_enter();
-    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (i >= nodes * nwhich * C) return;
-    const int node = i / (nwhich * C), j = i % (nwhich * C), which = j / C, c = j % C;
-    const double *a = acc + (int64_t)node * B * nwhich * C + j;
-    double s = 0.0;
-    for (int b = lane; b < B; b += 32) s += a[(int64_t)b * nwhich * C];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) {
-        float *dst = which == 0 ? o0 : which == 1 ? o1 : o2;
-        dst[(int64_t)node * gstride + c] = (float)s;
-    }
+    const int n = nwhich * C, per = (n + 31) / 32, node = blockIdx.x / per, j = blockIdx.x % per * 32 + (threadIdx.x & 31);
+    const double s = sum_over_samples(acc + (int64_t)node * B * n + j, B, n, j < n);
+    if (threadIdx.x < 32 && j < n) (j < C ? o0 : j < 2 * C ? o1 : o2)[(int64_t)node * gstride + j % C] = (float)s;
 }
 
 // ------------------------------------------------------------------ range batch-norm
@@ -672,6 +912,13 @@ extern "C" lpdt_status lpdt_evonorm_s0_fwd(int32_t nodes, int32_t B, int32_t H, 
     if (pl.V == 4 && !two_pass) {
         const int rstep = pl.threads / (C / 4);
         int ppc = 0;
+        const int Rl = evonorm_l2_cluster((int64_t)nodes * B, H * W, C / 4, pl.threads, (double)H * W * C * 4, 4, &ppc);
+        if (Rl > 0 && (int64_t)nodes * B * Rl <= 0x7fffffff) {
+            launch_k_cluster(evonorm_fwd_l2_kernel, dim3((unsigned)((int64_t)nodes * B * Rl)), pl.threads, (size_t)(2 * pl.threads + 3 * groups) * sizeof(double),
+                             as_stream(stream), Rl, H * W, C, groups, eps, x, v, gamma, beta, pstride, B, y, gmean, gvar, Rl, ppc);
+            LPDT_LAUNCH_CHECK();
+            return LPDT_OK;
+        }
         // shares of up to 64 KB: measured best (clusters of 8 lose to cluster scheduling, 128 KB shares to occupancy)
         const int R = evonorm_cluster(H * W, rstep, (size_t)C * 4, 64 * 1024, 160 * 1024, &ppc);
         const size_t scratch = align_up((size_t)(2 * pl.threads + 4 * groups) * sizeof(double), 16);
@@ -723,7 +970,14 @@ extern "C" lpdt_status lpdt_evonorm_s0_bwd(int32_t nodes, int32_t B, int32_t H, 
     if (pl.V == 4 && !two_pass) {
         const int rstep = pl.threads / (C / 4);
         int ppc = 0;
-        const int R = evonorm_cluster(H * W, rstep, (size_t)C * 8, 64 * 1024, 160 * 1024, &ppc);
+        const int Rl = evonorm_l2_cluster((int64_t)nodes * B, H * W, C / 4, pl.threads, (double)H * W * C * 8, 3, &ppc);
+        if (Rl > 0 && (int64_t)nodes * B * Rl <= 0x7fffffff) {
+            launch_k_cluster(evonorm_bwd_l2_kernel, dim3((unsigned)((int64_t)nodes * B * Rl)), pl.threads,
+                             (size_t)(2 * groups + 3 * C + pl.threads / 32 * 3 * C + pl.threads) * sizeof(double), st, Rl, H * W, C, groups, eps,
+                             dy, x, v, gamma, pstride, B, gmean, gvar, dx, acc, Rl, ppc);
+            done = true;
+        }
+        const int R = done ? 0 : evonorm_cluster(H * W, rstep, (size_t)C * 8, 64 * 1024, 160 * 1024, &ppc);
         const size_t scratch = align_up((size_t)(pl.threads + 2 * groups + 12 * pl.threads + 3 * C) * sizeof(double), 16);
         if (R > 0 && scratch <= 48 * 1024 && (int64_t)nodes * B * R <= 0x7fffffff) {
             static PerDeviceOnce attr;
@@ -743,7 +997,7 @@ extern "C" lpdt_status lpdt_evonorm_s0_bwd(int32_t nodes, int32_t B, int32_t H, 
         else launch_k(evonorm_bwd_kernel<1>, grid, pl.threads, smem, st, H * W, C, groups, eps, dy, x, v, gamma, pstride, B, gmean, gvar, dx, acc);
     }
     LPDT_LAUNCH_CHECK();
-    launch_k(norm_param_finalize, (nodes * 3 * C + 7) / 8, 256, 0, st, acc, nodes, B, C, 3, dv, dgamma, dbeta, gstride);
+    launch_k(norm_param_finalize, nodes * ((3 * C + 31) / 32), 256, 0, st, acc, nodes, B, C, 3, dv, dgamma, dbeta, gstride);
     LPDT_LAUNCH_CHECK();
     return LPDT_OK;
 }

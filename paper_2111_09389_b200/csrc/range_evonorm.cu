@@ -878,35 +878,14 @@ ren_bwd_q8_kernel(int HW, int C, int groups, float eps, float Cst,
     node_meet_and_quantize(dmax, hold, n_el, nodes, B, node, sample, ctl, q, scale, amax_out, dev_status);
 }
 
-// Sum the per-sample partials of a node and round once.  A block takes 32 neighbouring outputs (a row of 256 bytes per sample) and
-// its eight warps every eighth sample, four rows in flight; the warps' sums meet in order, so the result is deterministic.  (A
-// warp per output, lanes striding the samples, read 32 bytes for every 8: 26 us for ResNet-20's layers on 40 nodes, 7 now.)
-__device__ __forceinline__ double ren_sum_samples(const double *__restrict__ a, int B, int row, bool valid) {
-    __shared__ double s_part[8][32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    double s = 0.0;
-    for (int b = warp; b < B; b += 32) {
-        double v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = valid && b + 8 * u < B ? a[(int64_t)(b + 8 * u) * row] : 0.0;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) s += v[u];
-    }
-    s_part[warp][lane] = s;
-    __syncthreads();
-    s = 0.0;
-    if (warp == 0)
-        for (int w = 0; w < 8; ++w) s += s_part[w][lane];
-    return s;
-}
-// Blocks of one node: ceil(3 C / 32).
+// Sum the per-sample partials of a node and round once.  Blocks of one node: ceil(3 C / 32).
 __global__ void __launch_bounds__(256)
 ren_bwd_finalize(const double *__restrict__ acc, int nodes, int B, int C,
                  float *__restrict__ dv, float *__restrict__ dgamma,
                  float *__restrict__ dbeta, int64_t gstride) {
     pdl_enter();
     const int per = (3 * C + 31) / 32, node = blockIdx.x / per, j = blockIdx.x % per * 32 + (threadIdx.x & 31);
-    const double s = ren_sum_samples(acc + (int64_t)node * B * 3 * C + j, B, 3 * C, j < 3 * C);
+    const double s = sum_over_samples(acc + (int64_t)node * B * 3 * C + j, B, 3 * C, j < 3 * C);
     if (threadIdx.x < 32 && j < 3 * C) (j < C ? dv : j < 2 * C ? dgamma : dbeta)[(int64_t)node * gstride + j % C] = (float)s;
 }
 
@@ -925,7 +904,7 @@ __global__ void __launch_bounds__(256) ren_bwd_finalize_batch(RenBatch rb, int n
     while ((int)blockIdx.x >= rb.start[l + 1]) ++l;         // at most 64 layers: a short scan, uniform per block
     const int C = rb.C[l], i = blockIdx.x - rb.start[l];
     const int per = (3 * C + 31) / 32, node = i / per, j = i % per * 32 + (threadIdx.x & 31);
-    const double s = ren_sum_samples(rb.acc[l] + (int64_t)node * B * 3 * C + j, B, 3 * C, j < 3 * C);
+    const double s = sum_over_samples(rb.acc[l] + (int64_t)node * B * 3 * C + j, B, 3 * C, j < 3 * C);
     // the layer's three parameter vectors sit back to back in the gradient row: v, gamma, beta
     if (threadIdx.x < 32 && j < 3 * C) grads[(int64_t)node * gstride + rb.off[l] + j] = (float)s;
 }
