@@ -161,8 +161,8 @@ __device__ __forceinline__ double warp_sum(double v) {
 }
 
 // Block-wide max of non-negative values, then one atomicMax on the float's bit pattern
-// (non-negative floats order like unsigned integers).  Every thread of the block must call.
-__device__ __forceinline__ void block_amax_to(float v, float *dst) {
+// (non-negative floats order like unsigned integers), or a store of it.  Every thread of the block must call.
+__device__ __forceinline__ void block_amax_to(float v, float *dst, bool store = false) {
     __shared__ float s_blk_amax[32];
     v = warp_max(v);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -172,7 +172,10 @@ __device__ __forceinline__ void block_amax_to(float v, float *dst) {
         const int nw = (blockDim.x + 31) >> 5;
         v = lane < nw ? s_blk_amax[lane] : 0.f;
         v = warp_max(v);
-        if (lane == 0) atomicMax(reinterpret_cast<unsigned int *>(dst), __float_as_uint(v));
+        if (lane == 0) {
+            if (store) *dst = v;
+            else atomicMax(reinterpret_cast<unsigned int *>(dst), __float_as_uint(v));
+        }
     }
 }
 
