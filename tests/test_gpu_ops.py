@@ -115,6 +115,27 @@ def test_fill_zero_at_every_alignment(words, first):
     assert not b[first:first + 4 * words - 1].any() and (b[:first] == 3).all() and (b[first + 4 * words - 1:] == 3).all()
 
 
+@pytest.mark.parametrize("n", [1, 4095, 4096, 4097, 8193])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_quantize_with_a_workspace_that_holds_anything(n, mode):
+    """Short tensors store their range, longer ones gather it in words that the call clears."""
+    rng = np.random.default_rng(n)
+    x = rng.standard_normal((3, n)).astype(np.float32)
+    q = torch.empty(3, n, dtype=torch.uint8 if mode else torch.int8, device="cuda")
+    s, z = torch.empty(3, device="cuda"), torch.zeros(3, dtype=torch.int32, device="cuda")
+    ws = ws_bytes(api.lpdt_quantize_workspace_size(3)).fill_(255)
+    api.lpdt_quantize(dev(x), 3, n, n, q, s, ws, mode=mode, zero_point=z if mode else None)
+    ref = oracle.quantize_affine_u8(x) if mode else oracle.quantize_sym_s8(x)
+    assert np.array_equal(q.cpu().numpy(), ref[0]) and np.array_equal(s.cpu().numpy(), ref[1])
+    if mode:
+        assert np.array_equal(z.cpu().numpy(), ref[2])
+    else:
+        q2, s2 = torch.empty_like(q), torch.empty(1, 3, device="cuda")
+        ws = ws_bytes(api.lpdt_quantize_batch_workspace_size(3, 1)).fill_(255)
+        api.lpdt_quantize_batch(dev(x), 3, n, [0], [n], [0], q2, s2, ws)
+        assert torch.equal(q2, q) and torch.equal(s2[0], s)
+
+
 def test_quantize_argument_errors():
     x = torch.zeros(8, device="cuda")
     q = torch.zeros(8, dtype=torch.int8, device="cuda")
@@ -1217,6 +1238,18 @@ def test_glue_ops():
     cs = torch.zeros(3, 14, device="cuda")
     api.lpdt_colsum(3, 32, 10, dev(z), cs[:, 4:], 14)
     close(cs[:, 4:], oracle.colsum(z), 1e-6, 1e-7)
+
+
+@pytest.mark.parametrize("K", [1, 2, 4, 5, 16, 17, 32, 33])
+@pytest.mark.parametrize("B", [1, 31, 33, 300])
+def test_softmax_ce_widths(K, B):
+    rng = np.random.default_rng(K + B)
+    z = (3 * rng.standard_normal((2, B, K))).astype(np.float32)
+    lab = rng.integers(0, K, (2, B)).astype(np.int32)
+    loss_ref, dz_ref = oracle.softmax_ce(z, lab)
+    loss, dz = torch.empty(2, device="cuda"), torch.full((2, B, K), 9.0, device="cuda")
+    api.lpdt_softmax_ce(2, B, K, dev(z), dev(lab), loss, dz)
+    close(loss, loss_ref); close(dz, dz_ref)
 
 
 def test_softmax_ce_label_out_of_range_is_guarded():
