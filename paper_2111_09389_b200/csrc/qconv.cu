@@ -246,12 +246,17 @@ namespace lpdt {
 
 // out[row] = sum of the `len` unsigned bytes of row `row`.  A group of G lanes (a power of two up to
 // 32, chosen by the launcher from the row length) shares a row: 16-byte loads when the rows allow.
-__global__ void row_sum_u8_kernel(const uint8_t *__restrict__ src, int64_t rows, int len, int G, bool vec16,
-                                  int32_t *__restrict__ out) {
-    pdl_enter();
+// `block` of `blocks` blocks that share the rows.
+struct RowSums { const uint8_t *src; int32_t *out; int64_t rows; int len, G; bool vec16; };
+__device__ __forceinline__ void row_sums(const RowSums &rs, unsigned block, unsigned blocks) {
+    const int G = rs.G, len = rs.len;
+    const int64_t rows = rs.rows;
+    const uint8_t *__restrict__ src = rs.src;
+    int32_t *__restrict__ out = rs.out;
+    const bool vec16 = rs.vec16;
     const int lane_in_group = threadIdx.x & (G - 1);
-    const int64_t groups_total = ((int64_t)gridDim.x * blockDim.x) / G;
-    for (int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;; row += groups_total) {
+    const int64_t groups_total = ((int64_t)blocks * blockDim.x) / G;
+    for (int64_t row = ((int64_t)block * blockDim.x + threadIdx.x) / G;; row += groups_total) {
         if (row - (int)((threadIdx.x & 31) / G) >= rows) break;      // warp-uniform: the warp's first row is past the end
         const bool valid = row < rows;                               // lanes past the end still take part in the shuffles
         const uint8_t *a = src + (valid ? row : 0) * len;
@@ -270,6 +275,10 @@ __global__ void row_sum_u8_kernel(const uint8_t *__restrict__ src, int64_t rows,
         for (int o = G >> 1; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
         if (valid && lane_in_group == 0) out[row] = (int32_t)sum;
     }
+}
+__global__ void row_sum_u8_kernel(RowSums rs) {
+    pdl_enter();
+    row_sums(rs, blockIdx.x, gridDim.x);
 }
 
 // P[n][r][s][co] for 0 <= r <= R, 0 <= s <= S: sum of tapsum[n][co][r'][s'] over r' < r, s' < s.  The output
@@ -310,13 +319,22 @@ static int table_threads(const lpdt_conv_desc &d, int over_cout) {
     const int64_t t = (rows + 31) / 32 * 32;
     return (int)(t < 64 ? 64 : t > most ? most : t);
 }
+// The activations' (or errors') row sums, which the contraction's epilogue reads beside the table, ride in the same launch:
+// the blocks behind the `tables` first ones.  The few table blocks, a serial chain each, run beside them
+// (8 x 32 x 16x16 128 -> 128 3x3: forward 30.3 us with two launches, 28.6 with one; backward-data 35.9 and 33.1).
 __global__ void __launch_bounds__(1024)
-weight_table_kernel(lpdt_conv_desc d, const uint8_t *__restrict__ Wq, int over_cout, int st, bool vec16, bool vec4, int32_t *__restrict__ P) {
+weight_table_kernel(lpdt_conv_desc d, const uint8_t *__restrict__ Wq, int over_cout, int st, bool vec16, bool vec4, int32_t *__restrict__ P,
+                    unsigned tables, RowSums rs) {
     pdl_enter();
+    if (blockIdx.x >= tables) {
+        row_sums(rs, blockIdx.x - tables, gridDim.x - tables);
+        return;
+    }
     extern __shared__ unsigned s_tab[];
     const int taps = d.R * d.S, C = over_cout ? d.Cin : d.Cout, PS = d.S + st, cells = (d.R + st) * PS;
     unsigned *t = s_tab, *pre = s_tab + taps * kTabC;             // [taps][16], [cells][16]
-    const int n = blockIdx.y, c0 = blockIdx.x * kTabC, nc = C - c0 < kTabC ? C - c0 : kTabC, tid = threadIdx.x, T = blockDim.x;
+    const unsigned chunks = (C + kTabC - 1) / kTabC;
+    const int n = blockIdx.x / chunks, c0 = (blockIdx.x - n * chunks) * kTabC, nc = C - c0 < kTabC ? C - c0 : kTabC, tid = threadIdx.x, T = blockDim.x;
     const uint8_t *w = Wq + (int64_t)n * d.Cout * taps * d.Cin;
     for (int i = tid; i < taps * kTabC; i += T) t[i] = 0;
     __syncthreads();
@@ -392,16 +410,38 @@ weight_table_kernel(lpdt_conv_desc d, const uint8_t *__restrict__ Wq, int over_c
     for (int i = tid; i < cells * kTabC; i += T)
         if ((i & (kTabC - 1)) < nc) P[((int64_t)n * cells + i / kTabC) * C + c0 + (i & (kTabC - 1))] = (int32_t)pre[i];
 }
-// Shapes the kernel above takes: a thread per tap, the tables in 48 KB of shared memory, nodes in grid.y.
+// Shapes the kernel above takes: a thread per tap, the tables in 48 KB of shared memory, blocks of all nodes and row sums in one grid.
 static bool table_fits(const lpdt_conv_desc &d, int st) {
-    return d.R * d.S <= 256 && ((int64_t)d.R * d.S + (int64_t)(d.R + st) * (d.S + st)) * kTabC * 4 <= 48 * 1024 && d.nodes <= 65535;
+    return d.R * d.S <= 256 && ((int64_t)d.R * d.S + (int64_t)(d.R + st) * (d.S + st)) * kTabC * 4 <= 48 * 1024 && d.nodes <= 65535 &&
+           (int64_t)d.nodes * (d.Cin > d.Cout ? d.Cin : d.Cout) <= (int64_t)1 << 30;
 }
-static lpdt_status weight_table_launch(const lpdt_conv_desc &d, const uint8_t *Wq, int over_cout, int st, int32_t *P, cudaStream_t stream) {
-    const int C = over_cout ? d.Cin : d.Cout;
+// rows of `len` bytes -> out[row]; lanes per row grow with the row length
+static RowSums row_sums_of(const uint8_t *src, int64_t rows, int len, int32_t *out) {
+    const bool vec16 = len % 16 == 0 && aligned(src, 16);
+    const int units = vec16 ? len / 16 : len;
+    int G = 1;
+    while (G < 32 && G * 4 <= units) G <<= 1;             // at least four loads per lane
+    return {src, out, rows, len, G, vec16};
+}
+static unsigned row_sum_blocks(const RowSums &rs, int threads) {
+    int64_t blocks = ceil_div(rs.rows * rs.G, threads);
+    const int64_t cap = (int64_t)kNumSMs * 32 * 256 / threads;
+    if (blocks > cap) blocks = cap;
+    return (unsigned)(blocks < 1 ? 1 : blocks);
+}
+static lpdt_status row_sum_launch(const RowSums &rs, cudaStream_t st) {
+    launch_k(row_sum_u8_kernel, row_sum_blocks(rs, 256), 256, 0, st, rs);
+    LPDT_LAUNCH_CHECK();
+    return LPDT_OK;
+}
+static lpdt_status weight_table_launch(const lpdt_conv_desc &d, const uint8_t *Wq, int over_cout, int st, int32_t *P, const RowSums &rs,
+                                       cudaStream_t stream) {
+    const int C = over_cout ? d.Cin : d.Cout, T = table_threads(d, over_cout);
     const size_t smem = ((size_t)d.R * d.S + (size_t)(d.R + st) * (d.S + st)) * kTabC * 4;
     const bool vec16 = d.Cin % 16 == 0 && aligned(Wq, 16);
-    launch_k(weight_table_kernel, dim3((unsigned)ceil_div(C, kTabC), d.nodes), table_threads(d, over_cout), smem, stream, d, Wq, over_cout, st, vec16,
-             d.Cin % 4 == 0 && aligned(Wq, 4), P);
+    const unsigned tables = (unsigned)(ceil_div(C, kTabC) * d.nodes);
+    launch_k(weight_table_kernel, tables + row_sum_blocks(rs, T), T, smem, stream, d, Wq, over_cout, st, vec16,
+             d.Cin % 4 == 0 && aligned(Wq, 4), P, tables, rs);
     LPDT_LAUNCH_CHECK();
     return LPDT_OK;
 }
@@ -476,21 +516,6 @@ __global__ void affine_fix_kernel(lpdt_conv_desc d, int Ho, int Wo, const int32_
     }
 }
 
-// rows of `len` bytes -> out[row]; lanes per row grow with the row length
-static lpdt_status row_sum_launch(const uint8_t *src, int64_t rows, int len, int32_t *out, cudaStream_t st) {
-    const bool vec16 = len % 16 == 0 && aligned(src, 16);
-    const int units = vec16 ? len / 16 : len;
-    int G = 1;
-    while (G < 32 && G * 4 <= units) G <<= 1;             // at least four loads per lane
-    int64_t blocks = ceil_div(rows * G, 256);
-    const int64_t cap = (int64_t)kNumSMs * 32;
-    if (blocks > cap) blocks = cap;
-    if (blocks < 1) blocks = 1;
-    launch_k(row_sum_u8_kernel, (unsigned)blocks, 256, 0, st, src, rows, len, G, vec16, out);
-    LPDT_LAUNCH_CHECK();
-    return LPDT_OK;
-}
-
 }  // namespace lpdt
 
 // LPDT_AFFINE_SEPARATE=1 keeps the separate correction passes of forward and backward-data on every shape.
@@ -539,15 +564,15 @@ extern "C" lpdt_status lpdt_qconv_fwd_affine(const lpdt_conv_desc *d, const uint
     int32_t *P = (int32_t *)((char *)asum + affine_asum_bytes(d));
     void *inner = (char *)P + affine_prefix_bytes(d);
     const int64_t pixels = (int64_t)d->nodes * d->B * d->H * d->W;
-    s = row_sum_launch(A, pixels, d->Cin, asum, st);
-    if (s != LPDT_OK) return s;
+    const RowSums sums = row_sums_of(A, pixels, d->Cin, asum);
     const int rows = d->nodes * d->Cout;
     int32_t *tapsum = (int32_t *)((char *)P + align_up((size_t)rows * (d->R + 1) * (d->S + 1) * sizeof(int32_t), 256));
     if (table_fits(*d, 1)) {
-        s = weight_table_launch(*d, Wq, 0, 1, P, st);
+        s = weight_table_launch(*d, Wq, 0, 1, P, sums, st);
         if (s != LPDT_OK) return s;
     } else {
-        s = row_sum_launch(Wq, (int64_t)rows * d->R * d->S, d->Cin, tapsum, st);
+        s = row_sum_launch(sums, st);
+        if (s == LPDT_OK) s = row_sum_launch(row_sums_of(Wq, (int64_t)rows * d->R * d->S, d->Cin, tapsum), st);
         if (s != LPDT_OK) return s;
         launch_k(weight_prefix_kernel, (rows + 127) / 128, 128, 0, st, tapsum, d->nodes, d->Cout, d->R, d->S, P);
         LPDT_LAUNCH_CHECK();
@@ -612,10 +637,10 @@ extern "C" lpdt_status lpdt_qconv_bwd_data(const lpdt_conv_desc *d, const int8_t
 }
 
 // Backward-weight contraction on raw codes.  Workspace: [int32 sums (used unless the caller gave dWacc) |
-// padded input | padded layer gradient].
+// padded input | padded layer gradient].  `more_clear` as in tc_wgrad.
 static lpdt_status bwd_weight_impl(const lpdt_conv_desc *d, const int8_t *E, const float *sE, const int8_t *A,
                                    const float *sA, float *dW, int64_t dw_node_stride, int32_t *dWacc, void *ws,
-                                   size_t ws_bytes, int32_t *dev_status, cudaStream_t st, bool uns) {
+                                   size_t ws_bytes, int32_t *dev_status, cudaStream_t st, bool uns, size_t *more_clear = nullptr) {
     const size_t acc_bytes = align_up((size_t)d->nodes * d->Cout * d->R * d->S * d->Cin * sizeof(int32_t), 256);
     int32_t *acc_ws = (int32_t *)ws;
     if (use_tc(*d, 2, ws, ws_bytes) && d->B > 0 && readable(E, d->Cout) && readable(A, d->Cin)) {
@@ -626,7 +651,7 @@ static lpdt_status bwd_weight_impl(const lpdt_conv_desc *d, const int8_t *E, con
                                    pad_job(E, Ep, pp.err ? (int64_t)d->nodes * d->B * Ho * Wo : 0, d->Cout), st);
         if (s != LPDT_OK) return s;
         lpdt_status r = tc::tc_wgrad(*d, pp.err ? (int8_t *)Ep : E, sE, pp.in ? (int8_t *)Ap : A, sA, dWacc, acc_ws, dW,
-                                     dw_node_stride, dev_status, st, uns, pitches(*d));
+                                     dw_node_stride, dev_status, st, uns, pitches(*d), more_clear);
         if (r != LPDT_ERR_UNSUPPORTED) return r;
     }
     return generic_bwd_weight(*d, E, sE, A, sA, dW, dw_node_stride, dWacc, acc_ws, st, uns);
@@ -730,6 +755,8 @@ __global__ void affine_fix_bwd_data_kernel(lpdt_conv_desc d, int Ho, int Wo, con
 // to every filter column that reaches it in shared memory, and the result to every filter row that reaches the row,
 // with integer atomics into zeroed tables.  (Batch sums in memory and one serial loop over the positions per tap and
 // channel took 141 us at 8 x 32 x 16x16 x 128.)
+// (Column sums meet in shared memory with a warp's words on neighbouring banks: stride-4 words, 64-bit divisions of the
+// item number and two divisions per entry of the result took 15 us there instead of 9, with the launches around it.)
 struct TapSumSide { const uint8_t *src; int32_t *tab; int rows, cols, C, cw, chunks; long long items; };
 constexpr int kTapThreads = 512;
 template <int V>
@@ -742,10 +769,14 @@ tap_sum_kernel(lpdt_conv_desc d, int Ho, int Wo, TapSumSide sideE, TapSumSide si
         const bool in = item >= sideE.items;
         const TapSumSide sd = in ? sideA : sideE;
         long long q = in ? item - sideE.items : item;
-        const int share = (int)(q % bshares); q /= bshares;
-        const int row = (int)(q % sd.rows); q /= sd.rows;
-        const int s0 = (int)(q % schunks) * sw; q /= schunks;
-        const int c0 = (int)(q % sd.chunks) * sd.cw, n = (int)(q / sd.chunks);
+        const bool narrow = q <= 0x7fffffff;                  // (a 64-bit division is some hundred instructions in a chain)
+        auto take = [&](int by) {
+            const long long w = narrow ? (long long)((unsigned)q / (unsigned)by) : q / by;
+            const int rest = (int)(q - w * by);
+            q = w;
+            return rest;
+        };
+        const int share = take(bshares), row = take(sd.rows), s0 = take(schunks) * sw, c0 = take(sd.chunks) * sd.cw, n = (int)q;
         const int cw = sd.cw, nc = sd.C - c0 < cw ? sd.C - c0 : cw, ns = d.S - s0 < sw ? d.S - s0 : sw;
         for (int i = tid; i < ns * cw; i += kTapThreads) s_acc[i] = 0;
         __syncthreads();
@@ -781,23 +812,24 @@ tap_sum_kernel(lpdt_conv_desc d, int Ho, int Wo, TapSumSide sideE, TapSumSide si
             for (int k = 0; k < ns; ++k) {
                 const int s = s0 + k;
                 bool ok;                                      // filter column s reaches this image column
-                if (in) { const int t = col + d.pad - s; ok = t >= 0 && t % d.stride == 0 && t / d.stride < Wo; }
+                if (in) { const int t = col + d.pad - s; ok = t >= 0 && (d.stride == 1 || t % d.stride == 0) && t < Wo * d.stride; }
                 else { const int iw = col * d.stride + s - d.pad; ok = iw >= 0 && iw < d.W; }
                 if (!ok) continue;
 #pragma unroll
-                for (int v = 0; v < V; ++v) atomicAdd(s_acc + k * cw + wd * V + v, sum[v]);
+                for (int v = 0; v < V; ++v) atomicAdd(s_acc + k * cw + v * (cw / V) + wd, sum[v]);      // a warp's words on all banks
             }
         }
         __syncthreads();
-        for (int r = 0; r < d.R; ++r) {
-            bool ok;
-            if (in) { const int t = row + d.pad - r; ok = t >= 0 && t % d.stride == 0 && t / d.stride < Ho; }
-            else { const int ih = row * d.stride + r - d.pad; ok = ih >= 0 && ih < d.H; }
-            if (!ok) continue;
-            int32_t *t = sd.tab + (((int64_t)n * d.R + r) * d.S + s0) * sd.C + c0;
-            for (int i = tid; i < ns * nc; i += kTapThreads) {
-                const unsigned v = s_acc[i / nc * cw + i % nc];
-                if (v) atomicAdd(t + (int64_t)(i / nc) * sd.C + i % nc, (int)v);
+        for (int i = tid; i < ns * nc; i += kTapThreads) {
+            const int k = i / nc, c = i - k * nc;
+            const unsigned v = s_acc[k * cw + c % V * (cw / V) + c / V];
+            if (!v) continue;
+            int32_t *t = sd.tab + ((int64_t)n * d.R * d.S + s0 + k) * sd.C + c0 + c;
+            for (int r = 0; r < d.R; ++r, t += (int64_t)d.S * sd.C) {
+                bool ok;
+                if (in) { const int u = row + d.pad - r; ok = u >= 0 && (d.stride == 1 || u % d.stride == 0) && u < Ho * d.stride; }
+                else { const int ih = row * d.stride + r - d.pad; ok = ih >= 0 && ih < d.H; }
+                if (ok) atomicAdd(t, (int)v);
             }
         }
         __syncthreads();
@@ -814,29 +846,51 @@ __device__ inline int taps_inside(int No, int len, int r, int pad, int st) {
     return hi >= lo ? hi - lo + 1 : 0;
 }
 
-// Block (output channel, node), threads over the entries (r, s, ci) of its filter.
+// A group of G lanes per row (output channel, tap) of a node's filter, V input channels per lane and step: the row's
+// tables and counts once per row.  Bound by the sums' traffic: a thread per entry, each
+// with its own divisions and counts, took 14.7 us at 8 x 128 x 128 x 9, 6.4 now (9.4 MB), and the whole backward-weight
+// call 49.2 us, 34.9 with faster tap sums and one clear for sums and tables.
+template <int V>
 __global__ void __launch_bounds__(256)
-affine_fix_bwd_weight_kernel(lpdt_conv_desc d, int Ho, int Wo, const int32_t *__restrict__ raw,
+affine_fix_bwd_weight_kernel(lpdt_conv_desc d, int Ho, int Wo, int G, const int32_t *__restrict__ raw,
                              const int32_t *__restrict__ tabE, const int32_t *__restrict__ tabA,
                              const int32_t *__restrict__ zE, const int32_t *__restrict__ zA,
                              const float *__restrict__ sE, const float *__restrict__ sA,
                              float *__restrict__ dW, int64_t dw_stride, int32_t *__restrict__ dWacc) {
     pdl_enter();
-    const int taps = d.R * d.S, n = blockIdx.y, co = blockIdx.x;
-    const int64_t per_co = (int64_t)taps * d.Cin;
+    const int taps = d.R * d.S, n = blockIdx.y, lane = threadIdx.x & (G - 1);
+    const int64_t rows = (int64_t)d.Cout * taps;
     const unsigned ze = (unsigned)zE[n], za = (unsigned)zA[n];
     const float sc = dW ? __fmul_rn(sE[n], sA[n]) : 0.f;
-    const int64_t o0 = ((int64_t)n * d.Cout + co) * per_co;
-    const int32_t *ta = tabA + (int64_t)n * per_co;           // entry (tap, ci): the filter's own layout
-#pragma unroll 4
-    for (int64_t i = threadIdx.x; i < per_co; i += blockDim.x) {
-        const int tap = per_co <= 0x7fffffff ? (int)((uint32_t)i / (uint32_t)d.Cin) : (int)(i / d.Cin), r = tap / d.S, s = tap % d.S;
+    for (int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G; row < rows; row += (int64_t)gridDim.x * blockDim.x / G) {
+        const int co = rows <= 0x7fffffff ? (int)((uint32_t)row / (uint32_t)taps) : (int)(row / taps), tap = (int)(row - (int64_t)co * taps);
+        const int r = tap / d.S, s = tap - r * d.S;
         const unsigned cnt = (unsigned)d.B * (unsigned)taps_inside(Ho, d.H, r, d.pad, d.stride) *
                              (unsigned)taps_inside(Wo, d.W, s, d.pad, d.stride);
         const unsigned te = (unsigned)__ldg(tabE + ((int64_t)n * taps + tap) * d.Cout + co);
-        const int acc = (int)((unsigned)raw[o0 + i] - za * te - ze * (unsigned)__ldg(ta + i) + cnt * ze * za);
-        if (dWacc) dWacc[o0 + i] = acc;
-        if (dW) dW[(int64_t)n * dw_stride + co * per_co + i] = __fmul_rn(__int2float_rn(acc), sc);
+        const unsigned fixed = cnt * ze * za - za * te;
+        const int64_t o0 = (int64_t)n * rows * d.Cin + row * d.Cin;
+        const int32_t *ta = tabA + ((int64_t)n * taps + tap) * d.Cin;
+        float *dw = dW ? dW + (int64_t)n * dw_stride + row * d.Cin : nullptr;
+#pragma unroll 2
+        for (int i = lane * V; i < d.Cin; i += G * V) {
+            int rv[V], tv[V], acc[V];
+            if constexpr (V == 4) {
+                const int4 t = *reinterpret_cast<const int4 *>(raw + o0 + i), u = __ldg(reinterpret_cast<const int4 *>(ta + i));
+                rv[0] = t.x; rv[1] = t.y; rv[2] = t.z; rv[3] = t.w;
+                tv[0] = u.x; tv[1] = u.y; tv[2] = u.z; tv[3] = u.w;
+            } else { rv[0] = raw[o0 + i]; tv[0] = __ldg(ta + i); }
+#pragma unroll
+            for (int k = 0; k < V; ++k) acc[k] = (int)((unsigned)rv[k] + fixed - ze * (unsigned)tv[k]);
+            if constexpr (V == 4) {
+                if (dWacc) *reinterpret_cast<int4 *>(dWacc + o0 + i) = make_int4(acc[0], acc[1], acc[2], acc[3]);
+                if (dw) *reinterpret_cast<float4 *>(dw + i) = make_float4(__fmul_rn(__int2float_rn(acc[0]), sc), __fmul_rn(__int2float_rn(acc[1]), sc),
+                                                                          __fmul_rn(__int2float_rn(acc[2]), sc), __fmul_rn(__int2float_rn(acc[3]), sc));
+            } else {
+                if (dWacc) dWacc[o0 + i] = acc[0];
+                if (dw) dw[i] = __fmul_rn(__int2float_rn(acc[0]), sc);
+            }
+        }
     }
 }
 
@@ -879,20 +933,22 @@ extern "C" lpdt_status lpdt_qconv_bwd_data_affine(const lpdt_conv_desc *d, const
     int32_t *wsum = (int32_t *)((char *)esum + affine_esum_bytes(d));
     void *inner = (char *)wsum + affine_wsum_bytes(d);
     const size_t inner_bytes = ws_bytes - (size_t)((char *)inner - (char *)ws);
-    s = row_sum_launch(E, (int64_t)d->nodes * d->B * Ho * Wo, d->Cout, esum, st);
-    if (s != LPDT_OK) return s;
+    const RowSums sums = row_sums_of(E, (int64_t)d->nodes * d->B * Ho * Wo, d->Cout, esum);
     // Zero-point terms in the contraction's epilogue, as in the forward product; the table takes the place of the raw
     // sums, which do not exist then.  8 x 32 x 16x16 128 -> 128 3x3: 34.8 us, 107.5 us with the raw sums written and
     // corrected in a second pass (80 us of them), which shapes outside the tensor-core path still take.
     const size_t table = (size_t)d->nodes * (d->R + d->stride) * (d->S + d->stride) * d->Cin * sizeof(int32_t);
     if (!affine_separate() && !tiny_bwd_data(*d, reinterpret_cast<const int8_t *>(E)) && table_fits(*d, d->stride) &&
         table <= affine_bwd_data_raw_bytes(d) && use_tc(*d, 1, inner, inner_bytes)) {
-        s = weight_table_launch(*d, Wq, 1, d->stride, raw, st);
+        s = weight_table_launch(*d, Wq, 1, d->stride, raw, sums, st);
         if (s != LPDT_OK) return s;
         const tc::AffineArgs aff = {esum, raw, zE, zW};
         s = bwd_data_impl(d, reinterpret_cast<const int8_t *>(E), sE, reinterpret_cast<const int8_t *>(Wq), sW, dA, dAacc,
                           nullptr, inner, inner_bytes, dev_status, st, true, &aff);
         if (s != LPDT_ERR_UNSUPPORTED) return s;
+    } else {
+        s = row_sum_launch(sums, st);
+        if (s != LPDT_OK) return s;
     }
     s = bwd_data_impl(d, reinterpret_cast<const int8_t *>(E), nullptr, reinterpret_cast<const int8_t *>(Wq), nullptr,
                       nullptr, raw, nullptr, inner, inner_bytes, dev_status, st, true);
@@ -944,11 +1000,12 @@ extern "C" lpdt_status lpdt_qconv_bwd_weight_affine(const lpdt_conv_desc *d, con
     int32_t *tabE = (int32_t *)((char *)ws + affine_wg_raw_bytes(d));
     int32_t *tabA = (int32_t *)((char *)tabE + affine_tab_bytes(d, d->Cout));
     void *inner = (char *)tabA + affine_tab_bytes(d, d->Cin);
+    size_t tabs = affine_tab_bytes(d, d->Cout) + affine_tab_bytes(d, d->Cin);      // cleared with the sums where these are
     s = bwd_weight_impl(d, reinterpret_cast<const int8_t *>(E), nullptr, reinterpret_cast<const int8_t *>(A), nullptr,
-                        nullptr, 0, raw, inner, ws_bytes - (size_t)((char *)inner - (char *)ws), dev_status, st, true);
+                        nullptr, 0, raw, inner, ws_bytes - (size_t)((char *)inner - (char *)ws), dev_status, st, true, &tabs);
     if (s != LPDT_OK) return s;
     // both operands' tap sums; samples are shared out until about two waves of blocks exist
-    LPDT_CUDA(zero_async(tabE, affine_tab_bytes(d, d->Cout) + affine_tab_bytes(d, d->Cin), st));
+    if (tabs) LPDT_CUDA(zero_async(tabE, tabs, st));
     const int sw = d->S < 24 ? d->S : 24, cw = 512;                  // 48 KB of shared memory at most
     const int64_t schunks = ceil_div(d->S, sw);
     TapSumSide sideE = {E, tabE, Ho, Wo, d->Cout, cw, (int)ceil_div(d->Cout, cw), 0};
@@ -963,8 +1020,15 @@ extern "C" lpdt_status lpdt_qconv_bwd_weight_affine(const lpdt_conv_desc *d, con
     launch_k(v4 ? tap_sum_kernel<4> : tap_sum_kernel<1>, (unsigned)blocks, kTapThreads, (size_t)sw * cw * 4, st, *d, Ho, Wo, sideE, sideA, sw,
              (int)shares);
     LPDT_LAUNCH_CHECK();
-    launch_k(affine_fix_bwd_weight_kernel, dim3(d->Cout, d->nodes), 256, 0, st, *d, Ho, Wo, raw, tabE, tabA, zE, zA, sE, sA, dW,
-             dw_node_stride, dWacc);
+    // four channels a step where every row of the three arrays begins on 16 bytes
+    const bool f4 = d->Cin % 4 == 0 && (!dWacc || aligned(dWacc, 16)) && (!dW || (aligned(dW, 16) && (d->nodes == 1 || dw_node_stride % 4 == 0)));
+    int G = 1;
+    while (G < 32 && G * (f4 ? 4 : 1) < d->Cin) G <<= 1;
+    int64_t fblocks = ceil_div((int64_t)d->Cout * d->R * d->S * G, 256);
+    const int64_t fcap = ceil_div((int64_t)kNumSMs * 64, d->nodes);
+    if (fblocks > fcap) fblocks = fcap;
+    launch_k(f4 ? affine_fix_bwd_weight_kernel<4> : affine_fix_bwd_weight_kernel<1>, dim3((unsigned)fblocks, d->nodes), 256, 0, st, *d, Ho, Wo, G,
+             raw, tabE, tabA, zE, zA, sE, sA, dW, dw_node_stride, dWacc);
     LPDT_LAUNCH_CHECK();
     return LPDT_OK;
 }

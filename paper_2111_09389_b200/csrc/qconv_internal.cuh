@@ -40,9 +40,11 @@ bool halo_supported(const lpdt_conv_desc &d, int mode);
 lpdt_status tc_pix_halo(const lpdt_conv_desc &d, int mode, const int8_t *A, const float *s1, const int8_t *Wq,
                         const float *s2, const float *bias, int64_t bias_stride, float *Y, int32_t *Yacc,
                         int32_t *dev_status, cudaStream_t st, bool uns = false, const float *addend = nullptr);
+// *more_clear bytes behind acc_user (its size rounded up to 256 bytes) are cleared together with it where it is cleared
+// at all; *more_clear is 0 then.
 lpdt_status tc_wgrad(const lpdt_conv_desc &d, const int8_t *E, const float *sE, const int8_t *A,
                      const float *sA, int32_t *acc_user, int32_t *acc_ws, float *dW, int64_t dw_stride,
-                     int32_t *dev_status, cudaStream_t st, bool uns, Pitches pt);
+                     int32_t *dev_status, cudaStream_t st, bool uns, Pitches pt, size_t *more_clear = nullptr);
 // Whether that is one launch that writes dW itself (no split of the pixel loop, no sums in memory).
 bool wgrad_direct(const lpdt_conv_desc &d, Pitches pt);
 // The same on pairs of SMs (signed codes, stride 1, 128-byte operand rows, 256-channel tiles, fp32 result in rows of 16 bytes): the

@@ -1106,7 +1106,7 @@ bool wgrad_direct(const lpdt_conv_desc &d, Pitches pt) {
 
 lpdt_status tc_wgrad(const lpdt_conv_desc &d, const int8_t *E, const float *sE, const int8_t *A,
                      const float *sA, int32_t *acc_user, int32_t *acc_ws, float *dW, int64_t dw_stride,
-                     int32_t *dev_status, cudaStream_t st, bool uns, Pitches pt) {
+                     int32_t *dev_status, cudaStream_t st, bool uns, Pitches pt, size_t *more_clear) {
     const int Ho = conv_out(d.H, d.pad, d.R, d.stride), Wo = conv_out(d.W, d.pad, d.S, d.stride);
     WgParams p;
     int per_sm, stage_bytes;
@@ -1137,7 +1137,9 @@ lpdt_status tc_wgrad(const lpdt_conv_desc &d, const int8_t *E, const float *sE, 
     const int64_t per_node = (int64_t)d.Cout * p.taps * d.Cin;
     if (p.splits > 1) {
         if (!p.acc_out) return LPDT_ERR_WORKSPACE;
-        LPDT_CUDA(zero_async(p.acc_out, (size_t)d.nodes * per_node * sizeof(int32_t), st));
+        size_t bytes = (size_t)d.nodes * per_node * sizeof(int32_t);
+        if (more_clear && p.acc_out == acc_user) { bytes = align_up(bytes, 256) + *more_clear; *more_clear = 0; }
+        LPDT_CUDA(zero_async(p.acc_out, bytes, st));
     }
     g_last_kernel = "lpdt::tc::conv_wgrad_kernel";
     launch_k(conv_wgrad_kernel, dim3(p.splits, p.mgroups * p.ngroups, d.nodes), kThreads, smem, st, mX, mE, p);

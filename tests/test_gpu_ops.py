@@ -262,6 +262,39 @@ def test_qconv_bwd_affine(case):
     assert not dW[:, wn:].any()
 
 
+@pytest.mark.parametrize("nodes,Cin,Cout,R,stride", [(1, 1, 3, 3, 1), (2, 4, 4, 1, 1), (2, 12, 5, 3, 2), (3, 64, 16, 3, 1),
+                                                     (2, 132, 8, 3, 1), (2, 160, 32, 1, 2)])
+def test_qconv_bwd_weight_affine_destinations(nodes, Cin, Cout, R, stride):
+    """Weight gradients of zero-point operands at every alignment of their destination (four channels a store or one)
+    and node stride: int32 sums exact, fp32 as dequant_acc, nothing written beside them."""
+    B, H, pad = 3, 9, R // 2
+    rng = np.random.default_rng(79)
+    Ho = (H + 2 * pad - R) // stride + 1
+    A = rng.integers(0, 256, (nodes, B, H, H, Cin), dtype=np.uint8)
+    E = rng.integers(0, 256, (nodes, B, Ho, Ho, Cout), dtype=np.uint8)
+    zA, zE = (rng.integers(0, 256, nodes).astype(np.int32) for _ in range(2))
+    sA, sE = (rng.uniform(0.001, 0.1, nodes).astype(np.float32) for _ in range(2))
+    ref, ovf = oracle.qconv_bwd_weight_affine(E, zE, A, zA, R, R, stride, pad)
+    assert ovf == 0
+    wn = Cout * R * R * Cin
+    want = oracle.dequant_acc(ref, sE, sA).reshape(nodes, wn)
+    desc = api.conv_desc(nodes, B, H, H, Cin, Cout, R, R, stride, pad)
+    ws = ws_bytes(api.lpdt_qconv_bwd_weight_affine_workspace_size(desc))
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for offset, more in ((0, 0), (0, 1), (1, 4), (4, 4), (2, 2)):
+        step = wn + more
+        flat = torch.full((offset + nodes * step + 8,), 7.0, device="cuda")
+        accs = torch.full((offset + nodes * wn + 8,), 7, dtype=torch.int32, device="cuda")
+        api.lpdt_qconv_bwd_weight_affine(desc, dev(E), dev(sE), dev(zE), dev(A), dev(sA), dev(zA), dW=flat[offset:],
+                                         dw_node_stride=step, dWacc=accs[offset:], ws=ws, dev_status=status)
+        got = flat[offset:offset + nodes * step].view(nodes, step)
+        assert np.array_equal(got[:, :wn].cpu().numpy(), want)
+        assert np.array_equal(accs[offset:offset + nodes * wn].cpu().numpy(), ref.reshape(-1))
+        assert (got[:, wn:] == 7).all() and (flat[:offset] == 7).all() and (flat[offset + nodes * step:] == 7).all()
+        assert (accs[:offset] == 7).all() and (accs[offset + nodes * wn:] == 7).all()
+    assert int(status.item()) == 0
+
+
 # channel counts that no 16-byte row holds, or that end inside a box of the tensor-core kernels.  (cc): forward products so
 # small that they run on the CUDA cores; backward-weight takes the tensor cores all the same
 RAGGED_CASES = [
