@@ -3,6 +3,7 @@
 // HBM-bound streaming kernels: 16-byte loads, warp-shuffle reduction of the
 // range, one atomic per block; the second pass stores 4 codes per thread.
 #include <atomic>
+#include <type_traits>
 #include "common.cuh"
 
 namespace lpdt {
@@ -19,14 +20,12 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
     }
     return c;
 }
-// (r >> 8) * 2^-24 without the conversion unit: 1 + (r >> 9) * 2^-23 and 1 - b * 2^-24, b the 24th bit, are floats by
-// construction, and their difference has 24 significant bits, so the subtraction is exact.
-__device__ __forceinline__ float u24(uint32_t r) {
-    return __fsub_rn(__uint_as_float(0x3f800000u | (r >> 9)), __uint_as_float(0x3f800000u - ((r >> 8) & 1u)));
-}
+// (r >> 8) * 2^-24 without the conversion unit: the bits of a 24-bit integer m, read as a float, are m * 2^-149 (below 2^23
+// a denormal, from there on the first normal binade, which has the same spacing), and the scaling is exact.
+__device__ __forceinline__ float u24(uint32_t r) { return __fmul_rn(__uint_as_float(r >> 8), 0x1p125f); }
 // Rounding to integers by adding 1.5 * 2^23 (nearest-even, exact for |t| < 2^22): the conversion unit, which rintf,
-// floorf and (int) use, runs at an eighth of the adders' rate (stochastic quantizer, 8 x 4.2 M values: 52.8 -> 50.1 us;
-// Philox's wide multiplies remain).  The low byte of the biased sum is the two's-complement code.
+// floorf and (int) use, runs at an eighth of the adders' rate (stochastic quantizer, 8 x 4.2 M values: 52.8 -> 50.1 us
+// together with the range; without it 47.6, and 41.1 with the shorter u24 and q_sym_sr below and a 32-bit Philox counter).  The low byte of the biased sum is the two's-complement code.
 constexpr float kRoundBias = 12582912.f;
 __device__ __forceinline__ float clamp127(float r) { return fminf(fmaxf(r, -127.f), 127.f); }
 __device__ __forceinline__ uint32_t biased(float r) { return __float_as_uint(__fadd_rn(r, kRoundBias)); }
@@ -36,8 +35,11 @@ __device__ __forceinline__ uint32_t pack_low_bytes(uint32_t a, uint32_t b, uint3
 
 // ws[2*node] = bits of max(0, max x) or of max|x|; ws[2*node+1] = bits of -min(0, min x).
 // Non-negative floats order like their bit patterns, so atomicMax on uint works.
+// (eight blocks an SM, which the grid is made for, leave 32 registers; with 33 it ran in two waves: 8 x 4.2 M values, range
+// and nearest codes 47.4 us, 42.0 with one)
 template <bool AFFINE, bool VEC>
-__global__ void range_kernel(const float *__restrict__ x, int64_t n, int64_t stride,
+__global__ void __launch_bounds__(256, 8)
+range_kernel(const float *__restrict__ x, int64_t n, int64_t stride,
                              uint32_t *__restrict__ ws) {
     pdl_enter();
     const int node = blockIdx.y;
@@ -89,21 +91,26 @@ __global__ void range_kernel(const float *__restrict__ x, int64_t n, int64_t str
 
 // Codes as the low byte of a word; +-127 are integers, so clamping before the rounding gives the same code.
 __device__ __forceinline__ uint32_t q_sym_rne(float x, float inv) { return biased(clamp127(__fmul_rn(x, inv))); }
+// The sum rounded down is floor(t) + bias; beyond 2^22 (a caller's range below max|x|) it may be off by the float's spacing,
+// and the clamp, on the biased sum, decides.
 __device__ __forceinline__ uint32_t q_sym_sr(float x, float inv, float u) {
-    const float t = __fmul_rn(x, inv);
-    // floor(t); beyond 2^22 (a caller's range below max|x|) it may be off by the float's spacing, and the clamp decides
-    float fl = __fsub_rn(__fadd_rn(t, kRoundBias), kRoundBias);
-    fl = fl > t ? __fsub_rn(fl, 1.f) : fl;
-    const float f = __fsub_rn(t, fl);
-    return biased(clamp127(fl + ((u < f) ? 1.f : 0.f)));
+    const float t = __fmul_rn(x, inv), fl = __fadd_rd(t, kRoundBias);
+    const float f = __fsub_rn(t, __fsub_rn(fl, kRoundBias));
+    const float r = u < f ? __fadd_rn(fl, 1.f) : fl;
+    return __float_as_uint(fminf(fmaxf(r, kRoundBias - 127.f), kRoundBias + 127.f));
 }
 __device__ __forceinline__ uint32_t q_affine(float x, float s, float zf) {
     const float r = __fadd_rn(rintf(__fdiv_rn(x, s)), zf);
     return biased(fminf(fmaxf(r, 0.f), 255.f));
 }
 
+// The range pass before this one went upwards, so the last values of every node are the ones that L2 still holds: this
+// pass goes downwards (8 x 4.2 M values, with the range: nearest 53.1 -> 47.4 us, affine 64.4 -> 58.8).  Stochastic codes are
+// bound by Philox's wide multiplies and the rounding's instructions, not by memory: as many registers as it likes, 41.1 us
+// without the range, 47.1 at 32 registers and eight blocks an SM.
 template <int MODE /*0 sym rne, 1 sym stochastic, 2 affine*/, bool VEC>
-__global__ void quantize_kernel(const float *__restrict__ x, int64_t n, int64_t stride,
+__global__ void __launch_bounds__(256, MODE == 1 ? 4 : 8)
+quantize_kernel(const float *__restrict__ x, int64_t n, int64_t stride,
                                 const uint32_t *__restrict__ ws, int8_t *__restrict__ q,
                                 float *__restrict__ scale, int32_t *__restrict__ zero_point,
                                 uint2 key, uint32_t ctr_offset, int wstride) {
@@ -132,15 +139,16 @@ __global__ void quantize_kernel(const float *__restrict__ x, int64_t n, int64_t 
     if (VEC) {
         const float4 *x4 = reinterpret_cast<const float4 *>(xn);
         uint32_t *q4 = reinterpret_cast<uint32_t *>(qn);
+        auto walk = [&](auto wide) {
 #pragma unroll 4
-        for (int64_t i = tid; i < n / 4; i += nth) {
+        for (int64_t i = n / 4 - 1 - tid; i >= 0; i -= nth) {
             const float4 v = __ldg(x4 + i);
             uint32_t a, b, c, d;
             if (MODE == 0) {
                 a = q_sym_rne(v.x, inv); b = q_sym_rne(v.y, inv);
                 c = q_sym_rne(v.z, inv); d = q_sym_rne(v.w, inv);
             } else if (MODE == 1) {
-                uint4 r = philox4x32_10(make_uint4((uint32_t)i, (uint32_t)((uint64_t)i >> 32),
+                uint4 r = philox4x32_10(make_uint4((uint32_t)i, decltype(wide)::value ? (uint32_t)((uint64_t)i >> 32) : 0u,
                                                    (uint32_t)node, ctr_offset), key);
                 a = q_sym_sr(v.x, inv, u24(r.x)); b = q_sym_sr(v.y, inv, u24(r.y));
                 c = q_sym_sr(v.z, inv, u24(r.z)); d = q_sym_sr(v.w, inv, u24(r.w));
@@ -150,6 +158,10 @@ __global__ void quantize_kernel(const float *__restrict__ x, int64_t n, int64_t 
             }
             q4[i] = pack_low_bytes(a, b, c, d);
         }
+        };
+        // (a counter whose upper word is known to be zero saves two of the twenty wide multiplies)
+        if (MODE == 1 && n / 4 > (int64_t)0xffffffff) walk(std::true_type{});
+        else walk(std::false_type{});
     } else {
         for (int64_t i = tid; i < n; i += nth) {
             float v = xn[i];
@@ -392,6 +404,7 @@ __device__ __forceinline__ float4 load4(const float *p, int width) {
 }
 __device__ __forceinline__ float amax4(float4 v) { return fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))); }
 
+// (The codes are written from the last tensor back: 8 x 9.2 M weights 112.7 -> 102.5 us.)
 // grid = (blocks, nodes, tensors); blocks beyond a tensor's length fall through.  Four groups of four values in flight
 // per thread (one value per step: 62 + 81 us for the two passes over 8 x 9.2 M weights, 45 + 60 us now).
 __global__ void __launch_bounds__(256)
@@ -420,7 +433,7 @@ __global__ void __launch_bounds__(256)
 batch_quantize_kernel(const float *__restrict__ params, long long row_stride, QuantBatch qb,
                       const uint32_t *__restrict__ ws, int8_t *__restrict__ q, float *__restrict__ scales) {
     pdl_enter();
-    const int t = blockIdx.z, node = blockIdx.y, nodes = gridDim.y;
+    const int nodes = gridDim.y, t = gridDim.z - 1 - blockIdx.z, node = nodes - 1 - blockIdx.y;      // what the range pass read last first
     const long long n = qb.size[t], n4 = n / 4;
     const float *x = params + (long long)node * row_stride + qb.src_off[t];
     int8_t *dst = q + qb.dst_off[t] + (long long)node * n;

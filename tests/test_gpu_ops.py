@@ -48,6 +48,31 @@ def test_quantize_sym(nodes, n, rounding):
     assert np.array_equal(y.cpu().numpy(), oracle.dequantize(q_ref, s_ref))
 
 
+@pytest.mark.parametrize("n", [4096, 4099])          # words of four codes, single ones
+def test_stochastic_rounding_at_its_edges(n):
+    """Integers, values just below and above them, denormals: the oracle's codes exactly; values beyond a caller's range,
+    infinities and NaN: the clamp's codes."""
+    rng = np.random.default_rng(n)
+    x = rng.uniform(-127, 127, (2, n)).astype(np.float32)
+    x[:, 0] = 127.0
+    x[:, 1:256] = np.arange(-127, 128)
+    x[:, 256:511] = np.nextafter(x[:, 1:256], np.float32(-200))
+    x[:, 511:766] = np.nextafter(x[:, 1:256], np.float32(200))
+    x[:, 766:1024] = np.clip(x[:, 766:1024], -126, 126) * np.float32(1e-30)
+    x[:, 1024:1280] = np.exp2(rng.uniform(-149, -20, (2, 256))).astype(np.float32) * rng.choice([-1, 1], (2, 256))
+    x = np.clip(x, -127, 127).astype(np.float32)
+    q_ref, _ = oracle.quantize_sym_s8(x, 1, seed=5, ctr_offset=1)
+    amax = dev(np.abs(x).max(1).astype(np.float32))
+    beyond = np.array([3e38, -3e38, np.inf, -np.inf, np.nan, 4194303.75, -4194304.5, 8388609, -1.3e7, 200.5, -128.25], np.float32)
+    clamped = np.array([127, -127, 127, -127, -127, 127, -127, 127, -127, 127, -127], np.int8)
+    x[:, 2000:2000 + len(beyond)] = beyond
+    q_ref[:, 2000:2000 + len(beyond)] = clamped
+    q = torch.empty(2, n, dtype=torch.int8, device="cuda")
+    s = torch.empty(2, dtype=torch.float32, device="cuda")
+    api.lpdt_quantize_with_range(dev(x), 2, n, n, amax, q, s, rounding=1, seed=5, ctr_offset=1)
+    assert np.array_equal(q.cpu().numpy(), q_ref)
+
+
 def test_quantize_strided_rows_zero_tensor_and_ties():
     # rows inside a wider flat vector (odd stride -> scalar path), an all-zero node, exact ties
     rng = np.random.default_rng(0)
