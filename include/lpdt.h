@@ -292,7 +292,9 @@ lpdt_status lpdt_qconv_bwd_weight_affine(const lpdt_conv_desc *d, const uint8_t 
  *   dx = (t*(hs + u*hp))*(1/D), then dx[argmax] -= Cst*S/D^2, dx[argmin] += Cst*S/D^2
  *   (skipped when argmax == argmin);  dbeta_c = sum dy;  dgamma_c = sum dy*(m/D);
  *   dv_c = sum t*x*x*hp/D, sums over the node's (b,h,w).
- * argmax/argmin: lowest (h*W+w)*C+c index attaining the extremum.
+ * argmax/argmin: lowest (h*W+w)*C+c index attaining the extremum (NaN is passed over; in a group of nothing
+ *            but NaN and the infinity that no value beats, the group's first element).  Backward skips a
+ *            position outside the sample.
  *
  * x, y, dy, dx : fp32 NHWC;  v, gamma, beta : fp32, node n at p + n*param_node_stride
  * gmin, gmax : fp32 [nodes][B][groups];  argmin, argmax : int32, same shape

@@ -70,6 +70,10 @@ __device__ __forceinline__ F2 hsig2(F2 u) {      // of two values (saturation cl
     return pack2(__saturatef(h0), __saturatef(h1));
 }
 
+// Position to store for a group's extremum.  Where no value beat the infinity that the search began with (a group of NaN, or
+// of NaN and that infinity), it is the group's first element: backward uses the positions as indices.
+__device__ __forceinline__ int ext_position(Ext e, int first) { return e.idx == 0x7fffffff ? first : e.idx; }
+
 // Reduce per-thread extrema to per-group extrema.  s_mn/s_mx hold one entry per
 // thread; members of group g are the threads whose column lies in the group.
 template <int V>
@@ -176,7 +180,8 @@ ren_fwd_kernel(int HW, int C, int groups, float eps, float Cst,
     }
     if (t < groups && rank == 0) {
         int64_t sg = sample * groups + t;
-        gmin[sg] = g_mn[t].v; gmax[sg] = g_mx[t].v; argmin[sg] = g_mn[t].idx; argmax[sg] = g_mx[t].idx;
+        gmin[sg] = g_mn[t].v; gmax[sg] = g_mx[t].v;
+        argmin[sg] = ext_position(g_mn[t], t * cpg); argmax[sg] = ext_position(g_mx[t], t * cpg);
     }
     const float rng = __fsub_rn(g_mx[grp].v, g_mn[grp].v);
     const float D = __fadd_rn(__fmul_rn(Cst, rng), eps);
@@ -445,7 +450,8 @@ ren_fwd_q8_kernel(int HW, int C, int groups, float eps, float Cst,
     reduce_groups<V>(mn, mx, s_mn, s_mx, g_mn, g_mx, CV, cpg, groups);
     if (t < groups) {
         const int64_t sg = sample * groups + t;
-        gmin[sg] = g_mn[t].v; gmax[sg] = g_mx[t].v; argmin[sg] = g_mn[t].idx; argmax[sg] = g_mx[t].idx;
+        gmin[sg] = g_mn[t].v; gmax[sg] = g_mx[t].v;
+        argmin[sg] = ext_position(g_mn[t], t * cpg); argmax[sg] = ext_position(g_mx[t], t * cpg);
     }
     const float rng = __fsub_rn(g_mx[grp].v, g_mn[grp].v);
     const float D = __fadd_rn(__fmul_rn(Cst, rng), eps);
@@ -776,11 +782,15 @@ __device__ __forceinline__ void ren_bwd_sample(unsigned char *smem_raw, int HW, 
     if (t < groups) {
         const int64_t sgg = sample * groups + t;
         const int amx = argmax[sgg], amn = argmin[sgg];
-        bool has_mx = R == 1 || (amx >= p_lo * C && amx < p_end * C), has_mn = R == 1 || (amn >= p_lo * C && amn < p_end * C);
+        // The CTA that wrote the position applies the term; a caller's position outside the sample belongs to none.
+        bool has_mx, has_mn;
         if (POOL && R > 1) {          // whose window
             const int share = (HW / 4 + R - 1) / R, Wo = W / 2, a = amx / C, b = amn / C;
-            has_mx = (a / W / 2 * Wo + a % W / 2) / share == rank;
-            has_mn = (b / W / 2 * Wo + b % W / 2) / share == rank;
+            has_mx = (unsigned)amx < (unsigned)(HW * C) && (a / W / 2 * Wo + a % W / 2) / share == rank;
+            has_mn = (unsigned)amn < (unsigned)(HW * C) && (b / W / 2 * Wo + b % W / 2) / share == rank;
+        } else {
+            has_mx = amx >= p_lo * C && amx < p_end * C;
+            has_mn = amn >= p_lo * C && amn < p_end * C;
         }
         if (amx != amn) {
             const float rng_g = __fsub_rn(gmax[sgg], gmin[sgg]);

@@ -858,8 +858,6 @@ def test_range_evonorm_and_max_pooling_in_one_launch(case, special):
     for a, b in zip((pooled, idx, *st), (pooled2, idx2, *st2)):
         same(a, b)
     same(amax, pooled.abs().reshape(nodes, -1).nan_to_num(0.0, posinf=float("inf")).amax(1))
-    if special == "infinite" and any(int(t.max()) == 2 ** 31 - 1 for t in st[2:]):
-        return                                   # a group of NaN alone has no extremum to go back to
     g = dev(np.random.default_rng(3).standard_normal(half).astype(np.float32))
     full, dx, dx2, r, r2 = f(*x.shape), f(*x.shape), f(*x.shape), torch.zeros(nodes, device="cuda"), torch.zeros(nodes, device="cuda")
     n = api.lpdt_range_evonorm_bwd_workspace_size(nodes, B, C)
@@ -874,6 +872,108 @@ def test_range_evonorm_and_max_pooling_in_one_launch(case, special):
     np.testing.assert_allclose(r2.cpu().numpy(), r.cpu().numpy(), rtol=1.2e-7, atol=0)
     a, b = (t[:nodes * B * 3 * C * 8].view(torch.float64).cpu().numpy() for t in (acc, acc2))
     np.testing.assert_allclose(b, a, rtol=0, atol=1e-15 * H * W * np.nanmax(np.abs(np.where(np.isinf(a), 0, a))))      # H W / 4 terms
+
+
+def _ren_forms(case, xd, Pd, stride):
+    """The forms of the layer that serve a case: name -> (forward, backward).  forward() -> (gmin, gmax, argmin, argmax);
+    backward(statistics) -> (gradient of x or its codes and scales, max|gradient|), with every byte around the gradient checked."""
+    nodes, B, H, W, C, groups = case
+    f = lambda *s: torch.empty(*s, device="cuda")
+    args, par = (nodes, B, H, W, C, groups, 1e-5), (Pd, Pd[:, C:])
+    ws = ws_bytes(api.lpdt_range_evonorm_bwd_workspace_size(nodes, B, C))
+    half = (nodes, B, H // 2, W // 2, C)
+    rng = np.random.default_rng(17)
+    dy, dyp = dev(rng.standard_normal(xd.shape).astype(np.float32)), dev(rng.standard_normal(half).astype(np.float32))
+    idx = torch.empty(half, dtype=torch.int8, device="cuda")
+
+    def stats():
+        return (f(nodes, B, groups), f(nodes, B, groups), *(torch.full((nodes, B, groups), -7, dtype=torch.int32, device="cuda") for _ in "12"))
+
+    def guarded(call, dtype=torch.float32, seal=93):
+        buf = torch.full((xd.numel() + 8192,), seal, dtype=dtype, device="cuda")
+        amax = torch.zeros(nodes, device="cuda")
+        call(buf[4096:-4096].view(xd.shape), amax)
+        assert bool((buf[:4096] == seal).all()) and bool((buf[-4096:] == seal).all())
+        return buf[4096:-4096].view(xd.shape), amax
+
+    def fwd():
+        st = stats()
+        api.lpdt_range_evonorm_fwd(*args, xd, *par, Pd[:, 2 * C:], stride, f(xd.shape), *st)
+        return st
+
+    def bwd(st):
+        return guarded(lambda dx, amax: api.lpdt_range_evonorm_bwd(*args, dy, xd, *par, stride, *st, dx, None, None, None, stride, ws,
+                                                                   amax_out=amax))
+    forms = {"plain": (fwd, bwd)}
+    if C // groups % 4 == 0 and H % 2 == 0 and W % 2 == 0:
+        def fwd_pool():
+            st = stats()
+            api.lpdt_range_evonorm_pool_fwd(*args, xd, *par, Pd[:, 2 * C:], stride, f(half), idx, *st)
+            return st
+
+        def bwd_pool(st):
+            return guarded(lambda dx, amax: api.lpdt_range_evonorm_pool_bwd(*args, dyp, idx, xd, *par, stride, *st, dx, ws, amax_out=amax))
+        forms["pool"] = (fwd_pool, bwd_pool)
+    if api.lpdt_range_evonorm_fwd_q8_fits(B, H, W, C, groups) and api.lpdt_range_evonorm_bwd_q8_fits(B, H, W, C, groups):
+        ctl = torch.zeros(api.lpdt_range_evonorm_q8_ctl_size(nodes), dtype=torch.uint8, device="cuda")
+
+        def fwd_q8():
+            st = stats()
+            api.lpdt_range_evonorm_fwd_q8(*args, xd, *par, Pd[:, 2 * C:], stride, None, *st,
+                                          torch.empty(xd.shape, dtype=torch.int8, device="cuda"), f(nodes), ctl)
+            return st
+
+        def bwd_q8(st):
+            return guarded(lambda q, amax: api.lpdt_range_evonorm_bwd_q8(*args, dy, xd, *par, stride, *st, q, f(nodes), None, None, None,
+                                                                         stride, ws, ctl, amax_out=amax), torch.int8)
+        forms["q8"] = (fwd_q8, bwd_q8)
+    return forms
+
+
+# whole samples and samples split over a cluster (forward, backward or both), 2 to 32 channels per group, vector width 1 and 4
+REN_POSITION_CASES = [(2, 4, 8, 8, 16, 2), (1, 5, 6, 6, 6, 3), (1, 4, 32, 32, 64, 8), (2, 4, 16, 16, 128, 4), (4, 120, 4, 4, 32, 4),
+                      (1, 4, 7, 9, 24, 3)]
+
+
+@pytest.mark.parametrize("case", REN_POSITION_CASES)
+def test_range_evonorm_fwd_positions_of_groups_without_finite_values(case):
+    """Every position that the forward pass stores is one of the sample (the oracle's), also where no value beats the infinity
+    that a search begins with; the backward pass from these statistics writes inside the gradient and agrees with the oracle."""
+    nodes, B, H, W, C, groups = case
+    x, P, _ = _ren_inputs(case, seed=41)
+    last = x.reshape(nodes * B, H * W, groups, C // groups)
+    last[0], last[1], last[2] = np.nan, -np.inf, np.inf
+    last[-1, 1:, -1] = np.nan                   # one group of infinities and NaN
+    last[-1, 0, -1] = -np.inf
+    xd, Pd = dev(x), dev(P)
+    _, mn, mx, amn, amx = oracle.range_evonorm_fwd(x, P[:, :C], P[:, C:2 * C], P[:, 2 * C:], groups, 1e-5, "f32")
+    dy = np.random.default_rng(17).standard_normal(x.shape).astype(np.float32)
+    want = oracle.range_evonorm_bwd(dy, x, P[:, :C], P[:, C:2 * C], mn, mx, amn, amx, groups, 1e-5, "f32")[0]
+    for name, (fwd, bwd) in _ren_forms(case, xd, Pd, P.shape[1]).items():
+        st = fwd()
+        assert np.array_equal(st[2].cpu().numpy(), amn) and np.array_equal(st[3].cpu().numpy(), amx), name
+        dx, amax = bwd(st)
+        if name == "plain":
+            got = dx.cpu().numpy()
+            assert np.array_equal(np.isnan(got), np.isnan(want))
+            close(got[~np.isnan(want)], want[~np.isnan(want)], 1e-6, 1e-7)
+
+
+@pytest.mark.parametrize("case", REN_POSITION_CASES)
+@pytest.mark.parametrize("low,high", [(-1, -1), (-1, 2 ** 31 - 1), (2 ** 31 - 1, -2 ** 31), ("end", 2 ** 31 - 1), ("end", "end")])
+def test_range_evonorm_fwd_then_backward_skips_positions_outside_the_sample(case, low, high):
+    """A caller's position outside the sample takes no correction: the gradient is that of equal positions (whose corrections
+    cancel), and nothing around it is touched."""
+    nodes, B, H, W, C, groups = case
+    x, P, _ = _ren_inputs(case, seed=43)
+    low, high = (H * W * C if v == "end" else v for v in (low, high))
+    for name, (fwd, bwd) in _ren_forms(case, dev(x), dev(P), P.shape[1]).items():
+        st = fwd()
+        st[2].fill_(0), st[3].fill_(0)
+        want, amax_want = bwd(st)
+        st[2].fill_(low), st[3].fill_(high)
+        dx, amax = bwd(st)
+        assert torch.equal(dx, want) and torch.equal(amax, amax_want), name
 
 
 @pytest.mark.parametrize("case", REN_Q8_CASES)
