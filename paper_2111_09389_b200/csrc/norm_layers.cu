@@ -383,8 +383,8 @@ evonorm_bwd_cl_kernel(int HW, int C, int groups, float eps, const float *__restr
 // A cluster of R CTAs owns a sample, small enough a part of the device that the samples in flight (one per cluster) stay well
 // inside the L2: the second pass reads them there, and nothing is held in between, so that three or four CTAs of an SM copy, meet
 // and write beside one another.  For widths whose channel columns divide a warp (the sums fold by shuffles).  Against the kernels
-// that hold the sample: 8 x 64 x 32x32x64 forward 81.9 -> 63.5 us (66 % of the HBM copy rate), backward 154.6 -> 126 (49 %:
-// its two passes issue the logistic twice); 16 x 32 x 32x32x16 32.8 -> 22.5 and 64 -> 48; 4 x 16 x 56x56x64 backward 314 -> 73.
+// that hold the sample: 8 x 64 x 32x32x64 forward 81.9 -> 63.5 us (66 % of the HBM copy rate); backward, calls back to back:
+// 8 x 64 x 32x32x64 150.5 -> 111.7 us, 16 x 32 x 32x32x16 56.3 -> 31.3, 4 x 16 x 56x56x64 (which none of them held) 307.6 -> 57.6.
 // The logistic function of two values, as sigmoidf_acc has it.
 __device__ __forceinline__ F2 sigmoid2(F2 u) {
     float a, b;
@@ -515,35 +515,26 @@ evonorm_bwd_l2_kernel(int HW, int C, int groups, float eps, const float *__restr
         vc[k] = v[(int64_t)node * pstride + c0 + k];
         gc[k] = gamma[(int64_t)node * pstride + c0 + k];
     }
-    // Partial sums of eight rows stay in fp32; every combination of them is done in double.  The factors that a channel's terms
-    // share (gamma, 1/D) follow the sums, and the group's sum is made of its channels'.
+    // Every term is added in double: runs of eight in fp32 doubled the error of dbeta (2.5e-8 -> 6e-8) for no more speed where
+    // the chip is full (8 x 64 x 32x32x64 117.9 us, 111.7 so; 16 samples of 56x56x64 21.5 and 23.9).  The factors that a channel's terms share (gamma, 1/D) follow the sums,
+    // and the group's sum is made of its channels'.
     const F2 v01 = pack2(vc[0], vc[1]), v23 = pack2(vc[2], vc[3]), one = pack2(1.f, 1.f), minus = pack2(-1.f, -1.f);
     double S = 0.0, sv[4] = {}, sg[4] = {}, sb[4] = {};
-    F2 fv01 = 0, fv23 = 0, fg01 = 0, fg23 = 0, fb01 = 0, fb23 = 0;
-    int n = 0;
-    auto flush2 = [&](F2 &f, double &a, double &b) {
+    auto add = [](F2 terms, double *sum) {
         float lo, hi;
-        unpack2(f, lo, hi);
-        a += (double)lo; b += (double)hi;
-        f = 0;
+        unpack2(terms, lo, hi);
+        sum[0] += (double)lo; sum[1] += (double)hi;
     };
-    auto flush = [&]() {
-        flush2(fv01, sv[0], sv[1]); flush2(fv23, sv[2], sv[3]);
-        flush2(fg01, sg[0], sg[1]); flush2(fg23, sg[2], sg[3]);
-        flush2(fb01, sb[0], sb[1]); flush2(fb23, sb[2], sb[3]);
-    };
-    auto add_pair = [&](F2 xx, F2 d, F2 vv, F2 &fv, F2 &fg, F2 &fb) {
+    auto add_pair = [&](F2 xx, F2 d, F2 vv, int k) {
         const F2 sig = sigmoid2(mul2(vv, xx)), q = mul2(d, mul2(xx, sig));
-        fb = add2(fb, d);
-        fg = add2(fg, q);                                                    // dy x sig
-        fv = fma2(q, mul2(xx, fma2(sig, minus, one)), fv);                   // dy x sig x (1 - sig)
+        add(d, sb + k);
+        add(q, sg + k);                                                      // dy x sig
+        add(mul2(q, mul2(xx, fma2(sig, minus, one))), sv + k);               // dy x sig x (1 - sig)
     };
     walk_rows2<4>(p_lo + row0, p_end, rstep, x + at0, dy + at0, C, [&](int, float4 a, float4 b) {
-        add_pair(pack2(a.x, a.y), pack2(b.x, b.y), v01, fv01, fg01, fb01);
-        add_pair(pack2(a.z, a.w), pack2(b.z, b.w), v23, fv23, fg23, fb23);
-        if ((++n & 7) == 0) flush();
+        add_pair(pack2(a.x, a.y), pack2(b.x, b.y), v01, 0);
+        add_pair(pack2(a.z, a.w), pack2(b.z, b.w), v23, 2);
     });
-    flush();
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         S += (double)gc[k] * sg[k];
@@ -597,7 +588,7 @@ evonorm_bwd_l2_kernel(int HW, int C, int groups, float eps, const float *__restr
     const F2 g01 = pack2(gc[0] * invD, gc[1] * invD), g23 = pack2(gc[2] * invD, gc[3] * invD), minus_coef = pack2(-coef, -coef), minus_mu = pack2(-muf, -muf);
     auto out_pair = [&](F2 xx, F2 d, F2 vv, F2 gg) {
         const F2 u = mul2(vv, xx), sig = sigmoid2(u);
-        const F2 slope = mul2(sig, fma2(u, fma2(sig, minus, one), one));     // sig (1 + u (1 - sig))
+        const F2 slope = fma2(mul2(u, sig), fma2(sig, minus, one), sig);     // sig + u sig (1 - sig)
         return fma2(mul2(d, gg), slope, mul2(minus_coef, add2(xx, minus_mu)));
     };
     walk_rows2<4>(p_lo + row0, p_end, rstep, x + at0, dy + at0, C, [&](int p, float4 a, float4 b) {

@@ -79,6 +79,35 @@ def test_evonorm_s0_fwd_bwd(case, groups):
     assert not Gh[:, 3 * C:].any()
 
 
+@pytest.mark.parametrize("case", [(1, 3, 56, 56, 64), (2, 2, 96, 96, 16), (2, 5, 32, 32, 64), (1, 4, 33, 31, 128), (3, 2, 7, 9, 4)])
+def test_evonorm_s0_gradient_sums_lose_nothing(case):
+    """With v = 0, gamma = 1 and x and dy on grids every term of a parameter gradient is exact in fp32, with no bit to spare for
+    sums of them; in double these are exact too, and what remains is the rounding of 1/D and of the result, half an ulp (2^-24)
+    each."""
+    nodes, B, H, W, C = case
+    groups, eps = C // 4, 1e-5
+    rng = np.random.default_rng(C + H)
+    x = rng.integers(-32, 33, (nodes, B, H, W, C)).astype(np.float32) / 16
+    f = lambda *s: torch.empty(*s, dtype=torch.float32, device="cuda")
+    v, one = torch.zeros(nodes, C, device="cuda"), torch.ones(nodes, C, device="cuda")
+    xd, y, dx, gmean, gvar = dev(x), f(*x.shape), f(*x.shape), f(nodes, B, groups), f(nodes, B, groups)
+    api.lpdt_evonorm_s0_fwd(nodes, B, H, W, C, groups, eps, xd, v, one, v, C, y, gmean, gvar)
+    D = np.sqrt(gvar.cpu().numpy().astype(np.float64) + np.float64(np.float32(eps))).repeat(4, -1)      # [nodes][B][C]
+    ws = ws_bytes(api.lpdt_evonorm_s0_bwd_workspace_size(nodes, B, C))
+    for power, bits in ((0, 24), (1, 19), (2, 14)):        # of x in the terms, and of dy: 5 bits less for each x
+        dy = rng.integers(-2 ** (bits - 1), 2 ** (bits - 1), x.shape).astype(np.float32) * np.float32(2.0 ** (2 - bits))
+        out = f(3, nodes, C)
+        api.lpdt_evonorm_s0_bwd(nodes, B, H, W, C, groups, eps, dev(dy), xd, v, one, C, gmean, gvar, dx, out[2], out[1], out[0], C, ws)
+        parts = (dy.astype(np.float64) * (x.astype(np.float64) / 2) ** power).sum((2, 3))               # sigmoid(0) = 1/2
+        if power:
+            parts /= D
+        want = parts.sum(1)
+        # (1/D is rounded once per sample: that half ulp is of the samples' parts)
+        bar = 1.001 * 2.0 ** -24 * (np.abs(want) + (np.abs(parts).sum(1) if power else 0))
+        err = np.abs(out[power].cpu().numpy() - want)
+        assert (err <= bar).all(), (power, (err / np.maximum(bar, 1e-30)).max())
+
+
 RBN_CASES = [(4, 8, 16, 16, 16), (2, 3, 32, 32, 16), (2, 2, 8, 8, 64), (1, 3, 5, 7, 6), (1, 2, 1, 1, 12),
              (2, 32, 8, 8, 64), (1, 2, 2, 2, 512), (3, 40, 9, 7, 24)]
 
