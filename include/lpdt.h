@@ -343,7 +343,8 @@ lpdt_status lpdt_range_evonorm_bwd_params_batch(int32_t nodes, int32_t B, int32_
  * what lpdt_range_evonorm_fwd followed by lpdt_maxpool2x2 writes: the pooled y [nodes][B][H/2][W/2][C], the positions idx of the
  * maxima (int8, shape of y) and the statistics; amax_out (nullable, caller-zeroed) takes max|pooled y| per node.
  * lpdt_range_evonorm_pool_bwd takes the pooled gradient dy and idx and writes what lpdt_maxpool2x2_bwd followed by
- * lpdt_range_evonorm_bwd (parameter gradients left as partial sums in ws, for lpdt_range_evonorm_bwd_params) writes.
+ * lpdt_range_evonorm_bwd (parameter gradients left as partial sums in ws, for lpdt_range_evonorm_bwd_params) writes, NaN and
+ * infinities included; the zeros of dx are all positive, and sums run in another order.
  * Errors: INVALID_ARG, WORKSPACE, CUDA; UNSUPPORTED (serve with the two calls): H or W odd, C or C/groups no multiple of 4,
  * more than 1024 channels, fp32 tensors not 16-byte aligned, idx not 4-byte aligned. */
 lpdt_status lpdt_range_evonorm_pool_fwd(int32_t nodes, int32_t B, int32_t H, int32_t W, int32_t C, int32_t groups,

@@ -500,7 +500,7 @@ ren_fwd_q8_kernel(int HW, int C, int groups, float eps, float Cst,
 // XHOLD (with DEPTH > 0): the sample's x has been requested into `dxs` (shared memory) as the oldest pending
 // copy group; only dy goes through the ring, and dx overwrites x in place.
 // POOL (V = 4, DEPTH = 0): dy and pool_idx are those of the 2 x 2 pooling behind the layer; a thread walks windows.  All but one
-// of a window's gradients are zero, so only that one's terms are evaluated (all, where a value is not finite).
+// of a window's gradients are zero, so only that one's terms are evaluated (all, where a product in them might not be finite).
 template <int V, int DEPTH, bool XHOLD = false, bool POOL = false>
 __device__ __forceinline__ void ren_bwd_sample(unsigned char *smem_raw, int HW, int C, int groups, float eps, float Cst,
                                                const float *__restrict__ dy, const float *__restrict__ x,
@@ -639,7 +639,15 @@ __device__ __forceinline__ void ren_bwd_sample(unsigned char *smem_raw, int HW, 
         const int Wo = W / 2, n = HW / 4, share = (n + R - 1) / R, end = (rank + 1) * share < n ? (rank + 1) * share : n;
         const float *dps = dy + sample * (int64_t)n * C;
         const char4 *ids = pool_idx + sample * (int64_t)n * C / 4;
-        const F2 inv2 = pack2(invD, invD), zero2 = 0;
+        const F2 inv2 = pack2(invD, invD);
+        // A zero gradient's terms are zero while gamma, v x, x x and x / D are finite: for x below plain, as a square (NaN: never)
+        float top = fmaxf(fabsf(invD), 2e20f), none = __fmul_rn(invD, 0.f);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            top = fmaxf(top, fabsf(vc[k]));
+            none = __fadd_rn(none, __fadd_rn(__fmul_rn(vc[k], 0.f), __fmul_rn(gc[k], 0.f)));
+        }
+        const float plain = __fdiv_rn(2e38f, top), plain2 = __fadd_rn(__fmul_rn(plain, plain), none);
         auto load = [&](int q, float4 (&x)[4], float4 &g, char4 &id) {
             const float *w0 = xs + (int64_t)(q / Wo * 2 * W + q % Wo * 2) * C + c0;
 #pragma unroll
@@ -654,13 +662,15 @@ __device__ __forceinline__ void ren_bwd_sample(unsigned char *smem_raw, int HW, 
             const int p0 = q / Wo * 2 * W + q % Wo * 2;
             const float g[4] = {g4.x, g4.y, g4.z, g4.w};
             const int id[4] = {id4.x, id4.y, id4.z, id4.w};
-            // x * 0 is 0 unless a value is infinite or not a number
-            F2 probe = zero2;
+            F2 squares = 0;
 #pragma unroll
-            for (int k = 0; k < 4; ++k) probe = fma2(pack2(x4[k].x, x4[k].y), zero2, fma2(pack2(x4[k].z, x4[k].w), zero2, probe));
-            float pa, pb;
-            unpack2(probe, pa, pb);
-            if (!(pa == 0.f && pb == 0.f)) {
+            for (int k = 0; k < 4; ++k) {
+                const F2 x01 = pack2(x4[k].x, x4[k].y), x23 = pack2(x4[k].z, x4[k].w);
+                squares = fma2(x01, x01, fma2(x23, x23, squares));
+            }
+            float sa, sb;
+            unpack2(squares, sa, sb);
+            if (!(sa < plain2 && sb < plain2)) {
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     const float xk[4] = {x4[k].x, x4[k].y, x4[k].z, x4[k].w};

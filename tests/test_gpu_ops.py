@@ -835,7 +835,7 @@ def _ren_q8_check(case, ties, with_res, keep_y):
 
 @pytest.mark.parametrize("case", [(2, 3, 8, 8, 16, 2), (1, 2, 2, 2, 64, 8), (2, 2, 4, 6, 12, 3), (1, 5, 32, 32, 64, 8),
                                   (2, 3, 16, 16, 128, 16), (1, 2, 4, 4, 512, 64), (1, 3, 6, 10, 160, 20), (5, 120, 8, 8, 32, 4)])
-@pytest.mark.parametrize("special", ["", "ties", "infinite"])
+@pytest.mark.parametrize("special", ["", "ties", "infinite", "large", "v", "gamma", "constant"])
 def test_range_evonorm_and_max_pooling_in_one_launch(case, special):
     """Equal to the layer and the pooling as two calls: everything to the bit, sums in double up to their order."""
     nodes, B, H, W, C, groups = case
@@ -843,6 +843,16 @@ def test_range_evonorm_and_max_pooling_in_one_launch(case, special):
     if special == "infinite":
         x[0, 0, 0, 1, 0] = np.inf
         x[-1, -1, 1, 1, -1] = np.nan
+    # products of finite values that are not finite, in the terms of positions that the pooling did not choose
+    if special == "large":
+        x[0, 0, 0, 1, 0] = x[-1, -1, 1, 0, -1] = -1e30
+    if special == "v":
+        P[0, 0], P[-1, C - 1] = 3e38, -np.inf
+    if special == "gamma":
+        P[0, C], P[-1, 2 * C - 1] = np.inf, np.nan
+    if special == "constant":
+        x[0, 0], x[-1, -1] = 1.5, -1.5
+    eps = 0.0 if special == "constant" else 1e-5
     xd, Pd, stride = dev(x), dev(P), P.shape[1]
     f = lambda *s: torch.full(s, 7.0, device="cuda")
     i = lambda *s: torch.full(s, -5, dtype=torch.int32, device="cuda")
@@ -850,10 +860,10 @@ def test_range_evonorm_and_max_pooling_in_one_launch(case, special):
     half = (nodes, B, H // 2, W // 2, C)
     same = lambda a, b: np.testing.assert_array_equal(a.cpu().numpy(), b.cpu().numpy())          # (NaN equals NaN, 0 equals -0)
     y, st, pooled, idx = f(*x.shape), stats(), f(*half), torch.full(half, 9, dtype=torch.int8, device="cuda")
-    api.lpdt_range_evonorm_fwd(nodes, B, H, W, C, groups, 1e-5, xd, Pd, Pd[:, C:], Pd[:, 2 * C:], stride, y, *st)
+    api.lpdt_range_evonorm_fwd(nodes, B, H, W, C, groups, eps, xd, Pd, Pd[:, C:], Pd[:, 2 * C:], stride, y, *st)
     api.lpdt_maxpool2x2(nodes, B, H, W, C, y, pooled, idx)
     st2, pooled2, idx2, amax = stats(), f(*half), torch.full(half, 9, dtype=torch.int8, device="cuda"), torch.zeros(nodes, device="cuda")
-    api.lpdt_range_evonorm_pool_fwd(nodes, B, H, W, C, groups, 1e-5, xd, Pd, Pd[:, C:], Pd[:, 2 * C:], stride, pooled2, idx2, *st2,
+    api.lpdt_range_evonorm_pool_fwd(nodes, B, H, W, C, groups, eps, xd, Pd, Pd[:, C:], Pd[:, 2 * C:], stride, pooled2, idx2, *st2,
                                     amax_out=amax)
     for a, b in zip((pooled, idx, *st), (pooled2, idx2, *st2)):
         same(a, b)
@@ -863,9 +873,9 @@ def test_range_evonorm_and_max_pooling_in_one_launch(case, special):
     n = api.lpdt_range_evonorm_bwd_workspace_size(nodes, B, C)
     acc, acc2 = torch.zeros(n, dtype=torch.uint8, device="cuda"), torch.zeros(n, dtype=torch.uint8, device="cuda")
     api.lpdt_maxpool2x2_bwd(nodes, B, H, W, C, g, idx, full)
-    api.lpdt_range_evonorm_bwd(nodes, B, H, W, C, groups, 1e-5, full, xd, Pd, Pd[:, C:], stride, *st, dx, None, None, None, stride, acc,
+    api.lpdt_range_evonorm_bwd(nodes, B, H, W, C, groups, eps, full, xd, Pd, Pd[:, C:], stride, *st, dx, None, None, None, stride, acc,
                                amax_out=r)
-    api.lpdt_range_evonorm_pool_bwd(nodes, B, H, W, C, groups, 1e-5, g, idx, xd, Pd, Pd[:, C:], stride, *st, dx2, acc2, amax_out=r2)
+    api.lpdt_range_evonorm_pool_bwd(nodes, B, H, W, C, groups, eps, g, idx, xd, Pd, Pd[:, C:], stride, *st, dx2, acc2, amax_out=r2)
     # dx at the extrema holds the group sum, whose rounding may go the other way when its terms are added in another order
     np.testing.assert_allclose(dx2.cpu().numpy(), dx.cpu().numpy(), rtol=1.2e-7, atol=0)
     assert int((dx2 != dx).logical_and(~dx.isnan()).sum()) <= 2 * nodes * B * groups
