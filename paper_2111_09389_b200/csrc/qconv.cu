@@ -672,8 +672,8 @@ extern "C" lpdt_status lpdt_qconv_bwd_weight(const lpdt_conv_desc *d, const int8
 }
 
 extern "C" int32_t lpdt_qconv_bwd_weight_direct(const lpdt_conv_desc *d) {
-    if (check_desc(d) != LPDT_OK || d->nodes == 0 || d->B == 0 || d->Cin % 16 || d->Cout % 16 || d->stride > 2) return 0;
-    return tc::wgrad_direct(*d, pitches(*d)) ? 1 : 0;
+    if (check_desc(d) != LPDT_OK || d->nodes == 0 || d->B == 0 || d->Cin % 16 || d->Cout % 16) return 0;
+    return tc_enabled() && tc::tc_shape(*d) && tc::wgrad_direct(*d, pitches(*d)) ? 1 : 0;      // else the CUDA cores add in memory
 }
 
 // ---- backward products on affine (zero-point) operands -----------------------------------------

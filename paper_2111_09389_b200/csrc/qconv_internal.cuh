@@ -27,6 +27,7 @@ namespace tc {
 // Bytes between the channel rows of the operands in memory (multiples of 16, at least the channel count).
 struct Pitches { int in, err, w; };      // activations (Cin), layer gradients (Cout), weights (Cin)
 bool tc_supported(const lpdt_conv_desc &d);
+bool tc_shape(const lpdt_conv_desc &d);      // the part of it that the shape decides
 // Zero-point correction applied in the epilogue (unsigned operands): per-pixel channel sums of operand A (the input, or
 // backward-data the layer gradient), the table of the weights' channel sums over the filter taps (see PixParams; up to
 // 124 bytes past its end are read), and the per-node zero points of operand A and of the weights.

@@ -801,12 +801,10 @@ static bool pix_two_enabled() {
     return on == 1;
 }
 
-bool tc_supported(const lpdt_conv_desc &d) {
-    if (d.stride != 1 && d.stride != 2) return false;
-    if (d.R * d.S > kMaxTaps || d.R > 100 || d.S > 100 || d.pad > 100) return false;
-    if (!encode_tiled_fn()) return false;
-    return true;
+bool tc_shape(const lpdt_conv_desc &d) {
+    return (d.stride == 1 || d.stride == 2) && d.R * d.S <= kMaxTaps && d.R <= 100 && d.S <= 100 && d.pad <= 100;
 }
+bool tc_supported(const lpdt_conv_desc &d) { return tc_shape(d) && encode_tiled_fn(); }
 
 // LPDT_PIX_DIRECT_STORE=1 keeps the pixel kernel's per-lane global stores (A/B timing and parity tests).
 static bool pix_tma_out_enabled() {

@@ -70,3 +70,10 @@ def test_which_weight_gradients_take_one_launch():
     assert direct(8, 32, 2, 2, 512, 512) == 1 and direct(8, 32, 8, 8, 256, 256) == 1
     assert direct(16, 32, 32, 32, 16, 16) == 0
     assert direct(8, 32, 32, 32, 3, 64) == 0 and direct(0, 32, 2, 2, 512, 512) == 0 and direct(8, 0, 2, 2, 512, 512) == 0
+    assert direct(8, 4, 16, 16, 512, 512, 9, 9, 1, 4) == 0 and direct(8, 32, 4, 4, 512, 512, 1, 1, 3, 0) == 0      # CUDA cores only
+    import os, subprocess, sys
+    out = subprocess.run([sys.executable, "-c", "from paper_2111_09389_b200 import api\n"
+                          "print(api.lpdt_qconv_bwd_weight_direct(api.conv_desc(8, 32, 2, 2, 512, 512)))"],
+                         env=dict(os.environ, LPDT_DISABLE_TC="1"), capture_output=True, text=True, timeout=300,
+                         cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
+    assert out.stdout.split() == ["0"], out.stderr
