@@ -320,9 +320,11 @@ class TrainStep:
         self.out = self.buf[-1]["out"]
         return self.out
 
-    def _pooled(self, li):
-        """Whether the max-pooling li runs in the launch of the norm layer in front of it."""
-        return li > 0 and self.buf[li - 1].get("pool", False)
+    def _pooled(self, li, *tensors):
+        """Whether the norm layer li and the operation behind it are one launch: a max-pooling, and `tensors`, which that
+        launch reads and writes four values at a time, lie where it can."""
+        return self.buf[li].get("pool", False) and not any(
+            t.data_ptr() % (4 * t.element_size()) for t in (*tensors, self.buf[li + 1]["idx"]))
 
     def _bwd_q8(self, li):
         """Whether the backward pass of the norm layer li writes the codes of the convolution in front of it itself."""
@@ -374,7 +376,7 @@ class TrainStep:
                                                   b["ctl"], res=res, dev_status=self.dev_status)
                     cb["pre_quantized"] = True
                     cur, cur_range = b["out"], None
-                elif b["pool"]:
+                elif b["pool"] and self._pooled(li, cur, self.buf[li + 1]["out"]):
                     mb = self.buf[li + 1]
                     api.lpdt_range_evonorm_pool_fwd(N, B, op["H"], op["W"], Cc, op["groups"], self.eps, cur,
                                                     self._p(op["p_off"]), self._p(op["p_off"] + Cc),
@@ -397,7 +399,7 @@ class TrainStep:
                 api.lpdt_residual_add(N, B, op["H"], op["W"], op["Ca"], op["C"], op["stride"], op["ch_off"],
                                       cur, a, b["out"], amax_out=self.ranges[li])
                 cur, cur_range = b["out"], self.ranges[li]
-            elif k == "maxpool" and not self._pooled(li):
+            elif k == "maxpool" and cur is not b["out"]:        # (it is in the launch of the layer in front)
                 api.lpdt_maxpool2x2(N, B, op["H"], op["W"], op["C"], cur, b["out"], b["idx"])
                 cur = b["out"]        # max-pooling keeps max|x| only for non-negative maxima: range recomputed
                 cur_range = None
@@ -423,7 +425,7 @@ class TrainStep:
         g_range = None
         L = len(self.ops)
         sc = []
-        fused_shortcut = False
+        fused_shortcut = fused_pool = False
         ctr = 0
         for li in range(len(self.ops) - 1, -1, -1):
             op, b = self.ops[li], self.buf[li]
@@ -489,7 +491,8 @@ class TrainStep:
                                                   d, b["ws_ren"], b["ctl"], dev_status=self.dev_status)
                     cb["E_ready"] = True
                     g, g_range = None, None
-                elif b["pool"]:
+                elif fused_pool:
+                    fused_pool = False
                     api.lpdt_range_evonorm_pool_bwd(N, B, op["H"], op["W"], Cc, op["groups"], self.eps, g, self.buf[li + 1]["idx"],
                                                     b["x"], self._p(op["p_off"]), self._p(op["p_off"] + Cc), d, b["gmin"],
                                                     b["gmax"], b["amin"], b["amax"], b["dx"], b["ws_ren"],
@@ -511,11 +514,13 @@ class TrainStep:
                     api.lpdt_residual_add_bwd(N, B, aop["H"], aop["W"], aop["Ca"], aop["C"], aop["stride"],
                                               aop["ch_off"], dy_sc, g, b["dx"])
                     g, g_range = b["dx"], None
-            elif k == "maxpool" and self._pooled(li) and not self._bwd_q8(li - 1):
-                g_range = None                      # in the launch of the layer in front
             elif k == "maxpool":
-                api.lpdt_maxpool2x2_bwd(N, B, op["H"], op["W"], op["C"], g, b["idx"], b["dx"])
-                g, g_range = b["dx"], None
+                nb = self.buf[li - 1]
+                fused_pool = nb.get("pool", False) and not self._bwd_q8(li - 1) and self._pooled(li - 1, g, nb["x"], nb["dx"])
+                if not fused_pool:                  # else in the launch of the layer in front
+                    api.lpdt_maxpool2x2_bwd(N, B, op["H"], op["W"], op["C"], g, b["idx"], b["dx"])
+                    g = b["dx"]
+                g_range = None
             elif k == "avgpool":
                 api.lpdt_avgpool_bwd(N, B, op["H"] * op["W"], op["C"], g, b["dx"])
                 g, g_range = b["dx"], None
@@ -727,11 +732,11 @@ class _Reads:
         steps = (step, *self.groups)
         self.device = current.device_index
         self.layers = [list(st.buf) for st in steps]
-        names = [[n for n in self.BUFFERS + (self.WHOLE_STEP if st is step else ()) if n != "labels" or st.labels is not None]
-                 for st in steps]
-        self.getters = [operator.attrgetter(*n) for n in names]
+        self.names = [[n for n in self.BUFFERS + (self.WHOLE_STEP if st is step else ()) if n != "labels" or st.labels is not None]
+                      for st in steps]
+        self.getters = [operator.attrgetter(*n) for n in self.names]
         # (with rounding, groups would draw with seeds of their own, and a replay is given one)
-        self.complete = all(getattr(st, n) is not None for st, ns in zip(steps, names) for n in ns) and not (
+        self.complete = all(getattr(st, n) is not None for st, ns in zip(steps, self.names) for n in ns) and not (
             self.groups and any(st.grad_rounding for st in steps)) and all(g.ops is step.ops for g in self.groups) and all(
             type(v) is list for v in self.lists(step))
         if not self.complete:
@@ -780,9 +785,10 @@ class _Reads:
         return out
 
     def alike(self, tensors, addresses):
-        """Whether the tensors that lie elsewhere than in the last run could take the places of those of the recording."""
-        return all(self.kind(t) == kind and t.stride() == stride for t, a, old, kind, stride in
-                   zip(tensors, addresses, self.addresses, self.kinds, self.strides) if a != old)
+        """Whether the tensors that lie elsewhere than in the last run could take the places of those of the recording (whose
+        calls, with pooling in them, also depend on where four values at a time can be read: see TrainStep._pooled)."""
+        return all(self.kind(t) == kind and t.stride() == stride and not (a ^ old) % vector for t, a, old, kind, stride, vector in
+                   zip(tensors, addresses, self.addresses, self.kinds, self.strides, self.vectors) if a != old)
 
     def bind(self, step, current, calls):
         """Ties a recording to the tensors.  False if it cannot be replayed."""
@@ -791,6 +797,8 @@ class _Reads:
         tensors = self.tensors(step)
         self.addresses = list(map(torch.Tensor.data_ptr, tensors))
         self.kinds, self.strides = list(map(self.kind, tensors)), list(map(torch.Tensor.stride, tensors))
+        whole, pool = [n in ("x", "dy") for ns in self.names for n in ns], any(b.get("pool") for layers in self.layers for b in layers)
+        self.vectors = [4 * t.element_size() if pool and (i >= len(whole) or whole[i]) else 1 for i, t in enumerate(tensors)]
         extents = [t.nbytes if t.is_contiguous() else 0 if t.numel() == 0 else
                    t.element_size() * (1 + sum((n - 1) * s for n, s in zip(t.shape, t.stride()))) for t in tensors]
         calls.bind(self.addresses, extents, step._streams(current))

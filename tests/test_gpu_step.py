@@ -383,3 +383,33 @@ def test_recorded_runs_with_buffers_swapped_and_replaced(kw):
         for t in ("x_half", "x_hat", "x_out", "grads", "params", "out", "loss"):
             assert torch.equal(getattr(a, t), getattr(b, t)), (i, t)
     assert a._calls.code is not None or kw
+
+
+def test_step_on_inputs_off_a_vector_boundary():
+    """A norm layer with pooling behind it at either end of a step: an input and an upstream gradient 4 bytes off a 16-byte
+    boundary take the two calls, with the results of the one launch (group sums in another order: an ulp)."""
+    ren = lambda H, at: dict(op="ren", H=H, W=H, C=16, groups=2, p_off=at)
+    pool = lambda H: dict(op="maxpool", H=H, W=H, C=16)
+    ops = [ren(8, 0), pool(8), dict(op="conv", H=4, W=4, cin=16, cout=16, R=3, S=3, stride=1, pad=1, w_off=48), ren(4, 2352), pool(4)]
+    g = torch.Generator(device="cuda")
+    make = lambda: TrainStep(ops, 2400, 4, 3, (8, 8, 16), has_labels=False, input_grad=True)
+    a, b = make(), make()
+    for st in (a, b):
+        g.manual_seed(3)
+        for t in (st.params, st.x, st.dy):
+            t.copy_(torch.randn(t.shape, generator=g, device="cuda"))
+        st.params[:, :32] = 1.0
+        st.params[:, 2352:2384] = 1.0
+        st.x_hat.copy_(st.params)
+        st.Wmix.copy_(torch.eye(4))
+    for name in ("x", "dy"):
+        t = getattr(b, name)
+        flat = torch.empty(t.numel() + 1, device="cuda")
+        setattr(b, name, flat[1:].view(t.shape).copy_(t))
+    for _ in range(4):                                     # walked, noted and replayed
+        a.run(), b.run()
+        torch.cuda.synchronize()
+        assert torch.equal(a.out, b.out)
+        # sums of terms of about 1, in another order and partly in fp32 pairs: some ulps of the largest
+        assert torch.allclose(a.input_grad_out, b.input_grad_out, rtol=1e-6, atol=1e-6)
+        assert torch.allclose(a.grads, b.grads, rtol=1e-6, atol=1e-6 * float(a.grads.abs().max()))

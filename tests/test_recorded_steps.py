@@ -376,6 +376,54 @@ def test_swapped_and_new_buffers_do_not_walk():
             assert same(st)
 
 
+def off_boundary(t):
+    """A copy of a tensor, four bytes off a 16-byte boundary."""
+    flat = torch.zeros(t.numel() + 4, dtype=t.dtype)
+    at = next(i for i in range(4) if flat[i:].data_ptr() % 16 == 4)
+    return flat[at:at + t.numel()].view(t.shape).copy_(t)
+
+
+def pooled_step(**kw):
+    """A norm layer with pooling behind it at either end of the step."""
+    ren = lambda H, at: dict(op="ren", H=H, W=H, C=16, groups=2, p_off=at)
+    pool = lambda H: dict(op="maxpool", H=H, W=H, C=16)
+    ops = [ren(8, 0), pool(8), dict(op="conv", H=4, W=4, cin=16, cout=16, R=3, S=3, stride=1, pad=1, w_off=48), ren(4, 2352), pool(4)]
+    return TrainStep(ops, 2400, 4, 3, (8, 8, 16), has_labels=False, input_grad=True, device="cpu", **kw)
+
+
+@pytest.mark.parametrize("kw", [{}, dict(node_groups=2)])
+def test_pooling_takes_a_launch_of_its_own_where_four_values_cannot_be_read(kw):
+    """Whatever lies off a 16-byte boundary, in the walk and between recorded runs: that layer and its pooling are two calls."""
+    st = pooled_step(**kw)
+    groups = st.groups or [st]
+
+    def counts():
+        got = [c[0] for c in issued(st.run)]
+        return [got.count("lpdt_range_evonorm_" + n) // len(groups) for n in ("pool_fwd", "pool_bwd")] + [
+            got.count("lpdt_maxpool2x2" + n) // len(groups) for n in ("", "_bwd")]
+    for _ in range(4):
+        same(st)
+    assert same(st) and counts() == [2, 2, 0, 0]
+    for name, want in (("x", [1, 1, 1, 1]), ("dy", [2, 1, 0, 1]), (("out", 2), [1, 1, 1, 1]), (("dx", 0), [2, 1, 0, 1]),
+                       (("out", 4), [1, 2, 1, 0])):
+        who = groups[0]
+        entry, key = (who.__dict__, name) if isinstance(name, str) else (who.buf[name[1]], name[0])
+        old = entry[key]
+        entry[key] = off_boundary(old)
+        for _ in range(3):
+            same(st, name)
+        if not kw:
+            assert counts() == want, name
+        entry[key] = old
+        for _ in range(3):
+            same(st, name)
+        assert counts() == [2, 2, 0, 0]
+    if not kw:
+        replaying(st)
+        st.loss = off_boundary(st.loss)                    # not one of theirs
+        assert same(st)
+
+
 def test_recordings_that_are_never_replayed_become_rare():
     st = make()
     noted = 0
