@@ -77,12 +77,16 @@ class TrainStep:
             self.w_src.append(op["w_off"]); self.w_size.append(wn); self.w_dst.append(qbytes)
             qbytes += (N * wn + 255) // 256 * 256
         self.qW_all = torch.empty(max(qbytes, 256), **i8)
-        # raw int32 weight-gradient sums of every layer, each a contiguous [nodes][size] block (256-byte aligned
-        # starts): converted to fp32 by one batched launch at the end of the backward pass
+        # raw int32 weight-gradient sums of every layer whose gradient takes more than one launch, each a contiguous
+        # [nodes][size] block (256-byte aligned starts): converted to fp32 by one batched launch at the end of the backward pass
+        bounds = [N * g // self.node_groups for g in range(self.node_groups + 1)]
+        descs = [self._conv_desc(op, N) for op in wlist]
+        direct = [all(bool(api.lpdt_qconv_bwd_weight_direct(self._conv_desc(op, hi - lo))) for lo, hi in zip(bounds, bounds[1:]))
+                  for op in wlist]                                     # (one answer for all nodes of a layer)
         self.g_acc_off, n_acc = [], 0
-        for wn in self.w_size:
+        for wn, one in zip(self.w_size, direct):
             self.g_acc_off.append(n_acc)
-            n_acc += (N * wn + 63) // 64 * 64
+            n_acc += 0 if one else (N * wn + 63) // 64 * 64
         self.g_acc = torch.empty(max(n_acc, 64), **i32)
         self.sW_all = torch.empty(max(len(wlist), 1), N, **f32)
         ws_bytes = max(ws_bytes, api.lpdt_quantize_batch_workspace_size(N, min(len(wlist), 64)))
@@ -91,13 +95,10 @@ class TrainStep:
             k = op["op"]
             b = {}
             if k in ("conv", "linear"):
-                if k == "linear":
-                    H = W = 1; R = S = 1; stride = 1; pad = 0
-                else:
-                    H, W, R, S, stride, pad = op["H"], op["W"], op["R"], op["S"], op["stride"], op["pad"]
-                desc = api.conv_desc(N, B, H, W, op["cin"], op["cout"], R, S, stride, pad)
-                Ho = (H + 2 * pad - R) // stride + 1
-                Wo = (W + 2 * pad - S) // stride + 1
+                desc = descs[wi]
+                H, W, R, S = desc.H, desc.W, desc.R, desc.S
+                Ho = (H + 2 * desc.pad - R) // desc.stride + 1
+                Wo = (W + 2 * desc.pad - S) // desc.stride + 1
                 b.update(desc=desc, in_shape=(H, W, op["cin"]),
                          qA=torch.empty(N, B, H, W, op["cin"], **i8), sA=torch.empty(N, **f32),
                          qW=self.qW_all[self.w_dst[wi]:self.w_dst[wi] + N * self.w_size[wi]].view(N, op["cout"], R, S, op["cin"]),
@@ -107,8 +108,9 @@ class TrainStep:
                          dx=torch.empty(N, B, H, W, op["cin"], **f32),
                          wn=op["cout"] * R * S * op["cin"], wi=wi)
                 # whether the layer's weight gradient is complete after one launch, or adds int32 sums first
-                b["direct"] = bool(api.lpdt_qconv_bwd_weight_direct(desc))
-                b["gacc"] = self.g_acc[self.g_acc_off[wi]:self.g_acc_off[wi] + N * b["wn"]].view(N, b["wn"])
+                b["direct"] = direct[wi]
+                if not direct[wi]:
+                    b["gacc"] = self.g_acc[self.g_acc_off[wi]:self.g_acc_off[wi] + N * b["wn"]].view(N, b["wn"])
                 if quantize_wgrad:
                     b.update(gq=torch.empty(N, b["wn"], **i8), gs=torch.empty(N, **f32),
                              gw=torch.empty(N, b["wn"], **f32))
@@ -118,7 +120,7 @@ class TrainStep:
                 shape = (Ho, Wo, op["cout"])
             elif k == "ren":
                 H, W, Cc, G = op["H"], op["W"], op["C"], op["groups"]
-                b.update(out=torch.empty(N, B, H, W, Cc, **f32), dx=torch.empty(N, B, H, W, Cc, **f32),
+                b.update(dx=torch.empty(N, B, H, W, Cc, **f32),
                          gmin=torch.empty(N, B, G, **f32), gmax=torch.empty(N, B, G, **f32),
                          amin=torch.empty(N, B, G, **i32), amax=torch.empty(N, B, G, **i32))
                 # per-sample partial sums of the parameter gradients: a buffer per layer, because their reduction
@@ -131,6 +133,8 @@ class TrainStep:
                 # 2x2 max-pooling right behind: one launch for both, in either direction
                 nxt = ops[len(self.buf) + 1] if len(self.buf) + 1 < len(ops) else {"op": ""}
                 b["pool"] = bool(nxt["op"] == "maxpool" and Cc % 4 == 0 and Cc // G % 4 == 0 and Cc <= 1024 and H % 2 == 0 and W % 2 == 0)
+                if not b["pool"]:
+                    b["out"] = torch.empty(N, B, H, W, Cc, **f32)       # (else see _full_size)
                 b["ctl"] = torch.zeros(api.lpdt_range_evonorm_q8_ctl_size(N), dtype=torch.uint8, device=dev)
             elif k == "add":
                 Ho, Wo = (op["H"] + op["stride"] - 1) // op["stride"], (op["W"] + op["stride"] - 1) // op["stride"]
@@ -140,8 +144,9 @@ class TrainStep:
             elif k == "maxpool":
                 H, W, Cc = op["H"], op["W"], op["C"]
                 b.update(out=torch.empty(N, B, H // 2, W // 2, Cc, **f32),
-                         idx=torch.empty(N, B, H // 2, W // 2, Cc, **i8),
-                         dx=torch.empty(N, B, H, W, Cc, **f32))
+                         idx=torch.empty(N, B, H // 2, W // 2, Cc, **i8))
+                if not (self.buf and self.buf[-1].get("pool", False)):
+                    b["dx"] = torch.empty(N, B, H, W, Cc, **f32)
                 shape = (H // 2, W // 2, Cc)
             elif k == "avgpool":
                 b.update(out=torch.empty(N, B, 1, 1, op["C"], **f32),
@@ -163,13 +168,12 @@ class TrainStep:
         self.side = torch.cuda.Stream(device=dev)
         self.groups = []
         if self.node_groups > 1:
-            bounds = [N * g // self.node_groups for g in range(self.node_groups + 1)]
             self.groups = [self._node_view(bounds[g], bounds[g + 1], ws_bytes, dev) for g in range(self.node_groups)]
-            for layer in zip(self.buf, *(g.buf for g in self.groups)):      # one answer for all nodes of a layer
-                if "direct" in layer[0]:
-                    direct = all(b["direct"] for b in layer[1:])
-                    for b in layer:
-                        b["direct"] = direct
+
+    def _conv_desc(self, op, nodes):
+        if op["op"] == "linear":
+            return api.conv_desc(nodes, self.B, 1, 1, op["cin"], op["cout"], 1, 1, 1, 0)
+        return api.conv_desc(nodes, self.B, op["H"], op["W"], op["cin"], op["cout"], op["R"], op["S"], op["stride"], op["pad"])
 
     def _node_view(self, n0, n1, ws_bytes, dev):
         """A TrainStep over nodes [n0, n1) that shares this one's storage: every per-node tensor is a slice,
@@ -191,8 +195,6 @@ class TrainStep:
             for k, v in b.items():
                 if k == "desc":
                     cb[k] = api.conv_desc(n1 - n0, v.B, v.H, v.W, v.Cin, v.Cout, v.R, v.S, v.stride, v.pad)
-                elif k == "direct":
-                    cb[k] = bool(api.lpdt_qconv_bwd_weight_direct(cb["desc"]))
                 elif k == "ws_ren":
                     per = v.numel() // N
                     cb[k] = v[n0 * per:n1 * per]
@@ -326,6 +328,14 @@ class TrainStep:
         return self.buf[li].get("pool", False) and not any(
             t.data_ptr() % (4 * t.element_size()) for t in (*tensors, self.buf[li + 1]["idx"]))
 
+    def _full_size(self, li, name):
+        """The result of a norm layer before the pooling, or the gradient behind it.  One launch for both leaves neither in
+        memory: where that is the rule, they are made when two calls need them first."""
+        op, b = self.ops[li], self.buf[li]
+        if name not in b:
+            b[name] = torch.empty(self.N, self.B, op["H"], op["W"], op["C"], dtype=torch.float32, device=self.params.device)
+        return b[name]
+
     def _bwd_q8(self, li):
         """Whether the backward pass of the norm layer li writes the codes of the convolution in front of it itself."""
         return self.buf[li]["q8_bwd"] and li > 0 and self.ops[li - 1]["op"] == "conv"
@@ -386,7 +396,7 @@ class TrainStep:
                 else:
                     api.lpdt_range_evonorm_fwd(N, B, op["H"], op["W"], Cc, op["groups"], self.eps, cur,
                                                self._p(op["p_off"]), self._p(op["p_off"] + Cc),
-                                               self._p(op["p_off"] + 2 * Cc), d, b["out"], b["gmin"], b["gmax"],
+                                               self._p(op["p_off"] + 2 * Cc), d, self._full_size(li, "out"), b["gmin"], b["gmax"],
                                                b["amin"], b["amax"], amax_out=self.ranges[li], res=res)
                     cur, cur_range = b["out"], self.ranges[li]
                 b["fused_add"] = fuse
@@ -518,7 +528,7 @@ class TrainStep:
                 nb = self.buf[li - 1]
                 fused_pool = nb.get("pool", False) and not self._bwd_q8(li - 1) and self._pooled(li - 1, g, nb["x"], nb["dx"])
                 if not fused_pool:                  # else in the launch of the layer in front
-                    api.lpdt_maxpool2x2_bwd(N, B, op["H"], op["W"], op["C"], g, b["idx"], b["dx"])
+                    api.lpdt_maxpool2x2_bwd(N, B, op["H"], op["W"], op["C"], g, b["idx"], self._full_size(li, "dx"))
                     g = b["dx"]
                 g_range = None
             elif k == "avgpool":
@@ -822,7 +832,7 @@ class _Reads:
 
 # The code that a walk over the layers executes, as it is here (TrainStep._own_walk compares).
 _METHOD_NAMES = frozenset(("_run", "_prepare", "_each_group", "forward", "_forward_layers", "backward", "_backward_layers",
-                           "_finish_gradients", "_ren_param_sums", "update", "_p", "_g", "_pooled", "_bwd_q8"))
+                           "_finish_gradients", "_ren_param_sums", "update", "_p", "_g", "_pooled", "_full_size", "_bwd_q8"))
 _API = vars(api)
 _methods_of, _bindings_of = operator.attrgetter(*_METHOD_NAMES), operator.itemgetter(
     "wait_stream", "lpdt_fill_zero", "lpdt_quantize", "lpdt_quantize_with_range", "lpdt_quantize_batch", "lpdt_dequantize",

@@ -404,6 +404,8 @@ def test_pooling_takes_a_launch_of_its_own_where_four_values_cannot_be_read(kw):
     for _ in range(4):
         same(st)
     assert same(st) and counts() == [2, 2, 0, 0]
+    for who in (st, *st.groups):                           # nothing is kept that the one launch does not write
+        assert [("out" in b, "dx" in b) for b in who.buf] == [(False, True), (True, False), (True, True), (False, True), (True, False)]
     for name, want in (("x", [1, 1, 1, 1]), ("dy", [2, 1, 0, 1]), (("out", 2), [1, 1, 1, 1]), (("dx", 0), [2, 1, 0, 1]),
                        (("out", 4), [1, 2, 1, 0])):
         who = groups[0]
@@ -422,6 +424,20 @@ def test_pooling_takes_a_launch_of_its_own_where_four_values_cannot_be_read(kw):
         replaying(st)
         st.loss = off_boundary(st.loss)                    # not one of theirs
         assert same(st)
+
+
+@pytest.mark.parametrize("kw", [{}, dict(node_groups=2)])
+def test_no_sums_are_kept_for_weight_gradients_of_one_launch(kw):
+    conv = lambda c, at: dict(op="conv", H=2, W=2, cin=c, cout=c, R=3, S=3, stride=1, pad=1, w_off=at)
+    size = lambda c: 9 * c * c
+    ops = [conv(256, 0), conv(256, size(256))]
+    st = TrainStep(ops, 2 * size(256), 8, 4, (2, 2, 256), has_labels=False, device="cpu", **kw)
+    assert all(b["direct"] and "gacc" not in b for who in (st, *st.groups) for b in who.buf) and st.g_acc.numel() == 64
+    calls = [c for c in issued(st.run) if c[0].startswith(("lpdt_qconv_bwd_weight", "lpdt_dequantize_acc"))]
+    assert len(calls) == 2 * max(len(st.groups), 1)
+    few = TrainStep([conv(16, 0), conv(32, size(16))], size(16) + size(32), 8, 4, (2, 2, 16), has_labels=False, device="cpu", **kw)
+    sums = [b for b in few.buf if not b["direct"]]
+    assert few.g_acc.numel() == max(64, sum(8 * b["wn"] for b in sums)) and all(b["gacc"].shape == (8, b["wn"]) for b in sums)
 
 
 def test_recordings_that_are_never_replayed_become_rare():
