@@ -31,12 +31,22 @@ cudaError_t zero_async(void *p, size_t bytes, cudaStream_t st) {
     return launch_k(zero_kernel, (unsigned)(blocks < kNumSMs * 8 ? blocks : kNumSMs * 8), 256, 0, st, (uint32_t *)p, n, head);
 }
 
+// Whether the byte at p is memory of the current device.
+static bool on_device(const void *p) {
+    cudaPointerAttributes a;
+    int dev;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) { (void)cudaGetLastError(); return false; }
+    return a.type == cudaMemoryTypeDevice && cudaGetDevice(&dev) == cudaSuccess && a.device == dev;
+}
+
 }  // namespace lpdt
 
+// (Anything but memory of this device, first byte and last, is for the runtime's fill to take or to refuse: a kernel would fault.)
 extern "C" lpdt_status lpdt_fill_zero(void *p, size_t bytes, void *stream) {
     if (bytes == 0) return LPDT_OK;
     LPDT_CHECK_ARG(p != nullptr);
-    LPDT_CUDA(lpdt::zero_async(p, bytes, lpdt::as_stream(stream)));
+    const bool ours = lpdt::on_device(p) && lpdt::on_device((const char *)p + bytes - 1);
+    LPDT_CUDA(ours ? lpdt::zero_async(p, bytes, lpdt::as_stream(stream)) : cudaMemsetAsync(p, 0, bytes, lpdt::as_stream(stream)));
     return LPDT_OK;
 }
 

@@ -140,6 +140,18 @@ def test_fill_zero_at_every_alignment(words, first):
     assert not b[first:first + 4 * words - 1].any() and (b[:first] == 3).all() and (b[first + 4 * words - 1:] == 3).all()
 
 
+def test_fill_zero_leaves_other_memory_to_the_runtime():
+    """A kernel fills memory of the device; what lies elsewhere (here pinned host memory) goes to the runtime's fill, which
+    checks it."""
+    stream = torch.cuda.current_stream().cuda_stream
+    for t, kernels in ((torch.ones(64, device="cuda"), 1), (torch.ones(64).pin_memory(), 0)):
+        before = api.lpdt_launch_count()
+        assert api.lib().lpdt_fill_zero(t.data_ptr(), 256, stream) == 0
+        assert api.lpdt_launch_count() - before == kernels
+        torch.cuda.synchronize()
+        assert not t.any()
+
+
 @pytest.mark.parametrize("n", [1, 4095, 4096, 4097, 8193])
 @pytest.mark.parametrize("mode", [0, 1])
 def test_quantize_with_a_workspace_that_holds_anything(n, mode):
