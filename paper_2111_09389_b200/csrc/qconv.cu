@@ -439,8 +439,15 @@ static lpdt_status weight_table_launch(const lpdt_conv_desc &d, const uint8_t *W
     const int C = over_cout ? d.Cin : d.Cout, T = table_threads(d, over_cout);
     const size_t smem = ((size_t)d.R * d.S + (size_t)(d.R + st) * (d.S + st)) * kTabC * 4;
     const bool vec16 = d.Cin % 16 == 0 && aligned(Wq, 16);
-    const unsigned tables = (unsigned)(ceil_div(C, kTabC) * d.nodes);
-    launch_k(weight_table_kernel, tables + row_sum_blocks(rs, T), T, smem, stream, d, Wq, over_cout, st, vec16,
+    const unsigned tables = (unsigned)(ceil_div(C, kTabC) * d.nodes), blocks = tables + row_sum_blocks(rs, T);
+    static PerDeviceOnce attr;
+    int dev;
+    if (attr.pending(&dev)) {
+        LPDT_CUDA(cudaFuncSetAttribute(weight_table_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024));
+        attr.mark(dev);
+    }
+    // (2 x 50 x 6x6, 502 -> 42 backward-data behind itself: 30.4 us with the blocks on the first SMs to be free, 27.1 spread)
+    launch_k(weight_table_kernel, blocks, T, spread_smem(smem, blocks, 2048 / T), stream, d, Wq, over_cout, st, vec16,
              d.Cin % 4 == 0 && aligned(Wq, 4), P, tables, rs);
     LPDT_LAUNCH_CHECK();
     return LPDT_OK;
@@ -806,8 +813,13 @@ tap_sum_kernel(lpdt_conv_desc d, int Ho, int Wo, TapSumSide sideE, TapSumSide si
                 sum[0] = e & 0xffffu; sum[1] = o & 0xffffu; sum[2] = e >> 16; sum[3] = o >> 16;
             } else {
                 sum[0] = 0;
-#pragma unroll 8
-                for (int b = lo; b < hi; ++b) sum[0] += p[b * image];
+                for (int b = lo; b < hi; b += 16) {
+                    unsigned w[16];
+#pragma unroll
+                    for (int u = 0; u < 16; ++u) w[u] = b + u < hi ? __ldg(p + (b + u) * image) : 0u;
+#pragma unroll
+                    for (int u = 0; u < 16; ++u) sum[0] += w[u];
+                }
             }
             for (int k = 0; k < ns; ++k) {
                 const int s = s0 + k;
@@ -1017,8 +1029,20 @@ extern "C" lpdt_status lpdt_qconv_bwd_weight_affine(const lpdt_conv_desc *d, con
     sideE.items *= shares; sideA.items *= shares;
     const int64_t blocks = sideE.items + sideA.items < (int64_t)kNumSMs * 64 ? sideE.items + sideA.items : (int64_t)kNumSMs * 64;
     const bool v4 = d->Cin % 4 == 0 && d->Cout % 4 == 0 && aligned(E, 4) && aligned(A, 4);
-    launch_k(v4 ? tap_sum_kernel<4> : tap_sum_kernel<1>, (unsigned)blocks, kTapThreads, (size_t)sw * cw * 4, st, *d, Ho, Wo, sideE, sideA, sw,
-             (int)shares);
+    static PerDeviceOnce attr;
+    int dev;
+    if (attr.pending(&dev)) {
+        for (auto fn : {tap_sum_kernel<4>, tap_sum_kernel<1>})
+            LPDT_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024));
+        attr.mark(dev);
+    }
+    // Two blocks fit an SM.  Where one operand's blocks have more than twice the other's bytes and are no more than the SMs, each
+    // gets one of its own (whole product, 2 x 239 x 21x21, 34 -> 334, 1x1 of stride 2: 84.2 us, 64.4 so; 6 x 38 x 18x18,
+    // 249 -> 15, 3x3 of stride 2: 83.8, 68.8).
+    const int64_t e_bytes = (int64_t)Wo * (d->Cout < cw ? d->Cout : cw), a_bytes = (int64_t)d->W * (d->Cin < cw ? d->Cin : cw);
+    const bool apart = (e_bytes > 2 * a_bytes && sideE.items <= kNumSMs) || (a_bytes > 2 * e_bytes && sideA.items <= kNumSMs);
+    launch_k(v4 ? tap_sum_kernel<4> : tap_sum_kernel<1>, (unsigned)blocks, kTapThreads, spread_smem((size_t)sw * cw * 4, apart ? 1 : blocks, 2), st,
+             *d, Ho, Wo, sideE, sideA, sw, (int)shares);
     LPDT_LAUNCH_CHECK();
     // four channels a step where every row of the three arrays begins on 16 bytes
     const bool f4 = d->Cin % 4 == 0 && (!dWacc || aligned(dWacc, 16)) && (!dW || (aligned(dW, 16) && (d->nodes == 1 || dw_node_stride % 4 == 0)));
