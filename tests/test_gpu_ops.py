@@ -1432,6 +1432,13 @@ def test_softmax_ce_widths(K, B):
     close(loss, loss_ref); close(dz, dz_ref)
 
 
+# both sides of the lines between a group of lanes and a thread per sample, groups of every size with ragged last turns
+@pytest.mark.parametrize("K,B", [(2, 257), (3, 520), (5, 128), (8, 129), (8, 129 * 4), (9, 65), (16, 128), (16, 129), (16, 305), (20, 96),
+                                 (24, 129), (32, 160), (32, 161), (32, 304)])
+def test_softmax_ce_on_lanes_and_threads(K, B):
+    test_softmax_ce_widths(K, B)
+
+
 def test_softmax_ce_label_out_of_range_is_guarded():
     """A label outside [0, K) is never used as an index: the sample adds nothing to the loss, its gradient has
     no one-hot term, the status word reports the bad argument, and the other samples are untouched."""
