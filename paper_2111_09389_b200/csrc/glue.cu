@@ -119,6 +119,7 @@ __global__ void residual_add_bwd_kernel(int64_t NB, int H, int W, int Ca, int C,
     }
 }
 
+template <bool MANY /*pixels: sixteen or more*/>
 __global__ void avgpool_kernel(int64_t NB, int HW, int C, const float *__restrict__ x, float *__restrict__ y) {
     pdl_enter();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -128,7 +129,7 @@ __global__ void avgpool_kernel(int64_t NB, int HW, int C, const float *__restric
     double s = 0.0;
     const float *px = x + nb * HW * C + c;
     int p = 0;
-    for (; p + 16 <= HW; p += 16) {
+    for (; MANY && p + 16 <= HW; p += 16) {
         float v[16];
 #pragma unroll
         for (int u = 0; u < 16; ++u) v[u] = __ldg(px + (int64_t)(p + u) * C);
@@ -381,7 +382,10 @@ extern "C" lpdt_status lpdt_avgpool(int32_t nodes, int32_t B, int32_t HW, int32_
     if (nodes == 0 || B == 0) return LPDT_OK;
     LPDT_CHECK_ARG(x && y);
     int64_t n = (int64_t)nodes * B * C;
-    launch_k(avgpool_kernel, (unsigned)ceil_div(n, 64), 64, 0, as_stream(stream), (int64_t)nodes * B, HW, C, x, y);
+    // Small blocks spread few outputs of many pixels over the SMs; for others their launches are the time (14 x 256 x 317 outputs
+    // of one pixel 19.0 us in blocks of 64, 5.6 of 256; 9 x 154 x 14 of 191 pixels 9.2 and 10.9).
+    const int threads = HW >= 16 && n <= (int64_t)kNumSMs * 24 * 64 ? 64 : 256;
+    launch_k(HW >= 16 ? avgpool_kernel<true> : avgpool_kernel<false>, (unsigned)ceil_div(n, threads), threads, 0, as_stream(stream), (int64_t)nodes * B, HW, C, x, y);
     LPDT_LAUNCH_CHECK();
     return LPDT_OK;
 }
