@@ -1143,7 +1143,12 @@ extern "C" lpdt_status lpdt_range_evonorm_pool_bwd(int32_t nodes, int32_t B, int
     if ((int64_t)H * W * C > 0x7fffffff || H % 2 || W % 2 || !aligned(idx, 4)) return LPDT_ERR_UNSUPPORTED;
     if (!ws || ws_bytes < lpdt_range_evonorm_bwd_workspace_size(nodes, B, C) || !aligned(ws, 8)) return LPDT_ERR_WORKSPACE;
     RenPlan pl;
-    if (!plan(C, groups, aligned(x, 16) && aligned(dy, 16) && aligned(dx, 16), &pl) || pl.V != 4 || pl.threads > 256) return LPDT_ERR_UNSUPPORTED;
+    // 256 threads, which also clear and add a sample's sums; beyond one wave of those (two CTAs per SM) no more than windows and
+    // columns ask for (2x2x32: of 256 all but eight idled, 40 x 30 samples 19.7 us, 7.0 with 32; 4 x 2 of 2x2x64 4.2 and 6.2)
+    const bool v4 = aligned(x, 16) && aligned(dy, 16) && aligned(dx, 16);
+    int cap = (int64_t)nodes * B > 2 * kNumSMs ? 32 : 256;
+    while (cap < 256 && (cap < (int64_t)(H / 2) * (W / 2) * (C / 4) || !plan(C, groups, v4, &pl, cap))) cap *= 2;
+    if (!plan(C, groups, v4, &pl, cap) || pl.V != 4 || pl.threads > 256) return LPDT_ERR_UNSUPPORTED;
     const int cv = C / 4, nsets = (cv <= 32 && 32 % cv == 0) ? pl.threads / 32 : 1;
     size_t smem = (size_t)(nsets * 3 * C + pl.threads + groups) * sizeof(double);
     if (smem > 48 * 1024 || groups > pl.threads) return LPDT_ERR_UNSUPPORTED;

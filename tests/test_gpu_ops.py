@@ -846,7 +846,9 @@ def _ren_q8_check(case, ties, with_res, keep_y):
 
 
 @pytest.mark.parametrize("case", [(2, 3, 8, 8, 16, 2), (1, 2, 2, 2, 64, 8), (2, 2, 4, 6, 12, 3), (1, 5, 32, 32, 64, 8),
-                                  (2, 3, 16, 16, 128, 16), (1, 2, 4, 4, 512, 64), (1, 3, 6, 10, 160, 20), (5, 120, 8, 8, 32, 4)])
+                                  (2, 3, 16, 16, 128, 16), (1, 2, 4, 4, 512, 64), (1, 3, 6, 10, 160, 20), (5, 120, 8, 8, 32, 4),
+                                  # more samples than fit with 256 threads each: 32, 64, 96 and 128 threads
+                                  (3, 120, 2, 2, 16, 2), (3, 120, 4, 4, 64, 8), (2, 160, 2, 6, 96, 12), (2, 160, 2, 2, 512, 64)])
 @pytest.mark.parametrize("special", ["", "ties", "infinite", "large", "v", "gamma", "constant"])
 def test_range_evonorm_and_max_pooling_in_one_launch(case, special):
     """Equal to the layer and the pooling as two calls: everything to the bit, sums in double up to their order."""
