@@ -192,6 +192,27 @@ __device__ __forceinline__ void nl_cp_async_commit_wait() {
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
+// The logistic function of two values, as sigmoidf_acc has it.
+__device__ __forceinline__ F2 sigmoid2(F2 u) {
+    float a, b;
+    unpack2(mul2(u, pack2(-1.44269504f, -1.44269504f)), a, b);
+    asm("ex2.approx.f32 %0, %0;" : "+f"(a));
+    asm("ex2.approx.f32 %0, %0;" : "+f"(b));
+    unpack2(add2(pack2(a, b), pack2(1.f, 1.f)), a, b);
+    asm("rcp.approx.f32 %0, %0;" : "+f"(a));
+    asm("rcp.approx.f32 %0, %0;" : "+f"(b));
+    return pack2(a, b);
+}
+// y of four channels: (gamma / D) (x sigmoid(v x)) + beta, `g` the first factor.
+__device__ __forceinline__ void evonorm_y(float4 a, const F2 (&v)[2], const F2 (&g)[2], const F2 (&b)[2], float (&y)[4]) {
+    const F2 x01 = pack2(a.x, a.y), x23 = pack2(a.z, a.w);
+    unpack2(fma2(g[0], mul2(x01, sigmoid2(mul2(v[0], x01))), b[0]), y[0], y[1]);
+    unpack2(fma2(g[1], mul2(x23, sigmoid2(mul2(v[1], x23))), b[1]), y[2], y[3]);
+}
+
+// PAIRS: y as the kernel with the second read from L2 has it, for the widths that both take.  (For others, held in larger shares,
+// it is the slower form: 2 x 3 samples of 34x34x256 10.3 us, 11.2 in pairs.)
+template <bool PAIRS>
 __global__ void __launch_bounds__(256, 2)
 evonorm_fwd_cl_kernel(int HW, int C, int groups, float eps, const float *__restrict__ x, const float *__restrict__ v,
                       const float *__restrict__ gamma, const float *__restrict__ beta, int64_t pstride, int B,
@@ -257,12 +278,16 @@ evonorm_fwd_cl_kernel(int HW, int C, int groups, float eps, const float *__restr
     __syncthreads();
     if (R > 1) cluster.barrier_arrive();          // done reading the others' shared memory; waited for before exit
     const float invD = (float)g_inv[grp];
+    const F2 v2[2] = {pack2(vc[0], vc[1]), pack2(vc[2], vc[3])}, b2[2] = {pack2(bc[0], bc[1]), pack2(bc[2], bc[3])};
+    const F2 g2[2] = {pack2(gc[0] * invD, gc[1] * invD), pack2(gc[2] * invD, gc[3] * invD)};
     for (int p = p_lo + row0; p < p_end; p += rstep) {
         const float4 a = *reinterpret_cast<const float4 *>(hold + (size_t)(p - p_lo) * C + c0);
         const float xv[V] = {a.x, a.y, a.z, a.w};
         float yv[V];
+        if constexpr (PAIRS) evonorm_y(a, v2, g2, b2, yv);
+        else
 #pragma unroll
-        for (int k = 0; k < V; ++k) yv[k] = gc[k] * (xv[k] * sigmoidf_acc(vc[k] * xv[k])) * invD + bc[k];
+            for (int k = 0; k < V; ++k) yv[k] = gc[k] * (xv[k] * sigmoidf_acc(vc[k] * xv[k])) * invD + bc[k];
         NVec<V>::st(ys + (int64_t)p * C + c0, yv);
     }
     if (R > 1) cluster.barrier_wait();
@@ -385,17 +410,6 @@ evonorm_bwd_cl_kernel(int HW, int C, int groups, float eps, const float *__restr
 // and write beside one another.  For widths whose channel columns divide a warp (the sums fold by shuffles).  Against the kernels
 // that hold the sample: 8 x 64 x 32x32x64 forward 81.9 -> 63.5 us (66 % of the HBM copy rate); backward, calls back to back:
 // 8 x 64 x 32x32x64 150.5 -> 111.7 us, 16 x 32 x 32x32x16 56.3 -> 31.3, 4 x 16 x 56x56x64 (which none of them held) 307.6 -> 57.6.
-// The logistic function of two values, as sigmoidf_acc has it.
-__device__ __forceinline__ F2 sigmoid2(F2 u) {
-    float a, b;
-    unpack2(mul2(u, pack2(-1.44269504f, -1.44269504f)), a, b);
-    asm("ex2.approx.f32 %0, %0;" : "+f"(a));
-    asm("ex2.approx.f32 %0, %0;" : "+f"(b));
-    unpack2(add2(pack2(a, b), pack2(1.f, 1.f)), a, b);
-    asm("rcp.approx.f32 %0, %0;" : "+f"(a));
-    asm("rcp.approx.f32 %0, %0;" : "+f"(b));
-    return pack2(a, b);
-}
 template <int kU, class F> __device__ __forceinline__ void walk_rows(int p, int p_end, int rstep, const float *__restrict__ x, int C, F f) {
     for (; p + (kU - 1) * rstep < p_end; p += kU * rstep) {
         float4 v[kU];
@@ -478,13 +492,11 @@ evonorm_fwd_l2_kernel(int HW, int C, int groups, float eps, const float *__restr
     if (R > 1) cluster.barrier_arrive();          // done reading the others' shared memory; waited for before exit
     const float invD = (float)g_inv[grp];
     float *ys = y + sample * (int64_t)HW * C + c0;
-    const F2 v01 = pack2(vc[0], vc[1]), v23 = pack2(vc[2], vc[3]), b01 = pack2(bc[0], bc[1]), b23 = pack2(bc[2], bc[3]);
-    const F2 g01 = pack2(gc[0] * invD, gc[1] * invD), g23 = pack2(gc[2] * invD, gc[3] * invD);
+    const F2 v2[2] = {pack2(vc[0], vc[1]), pack2(vc[2], vc[3])}, b2[2] = {pack2(bc[0], bc[1]), pack2(bc[2], bc[3])};
+    const F2 g2[2] = {pack2(gc[0] * invD, gc[1] * invD), pack2(gc[2] * invD, gc[3] * invD)};
     walk_rows<4>(p_lo + row0, p_end, rstep, xs, C, [&](int p, float4 a) {
-        const F2 x01 = pack2(a.x, a.y), x23 = pack2(a.z, a.w);
         float yv[4];
-        unpack2(fma2(g01, mul2(x01, sigmoid2(mul2(v01, x01))), b01), yv[0], yv[1]);
-        unpack2(fma2(g23, mul2(x23, sigmoid2(mul2(v23, x23))), b23), yv[2], yv[3]);
+        evonorm_y(a, v2, g2, b2, yv);
         NVec<4>::st(ys + (int64_t)p * C, yv);
     });
     if (R > 1) cluster.barrier_wait();
@@ -903,24 +915,32 @@ extern "C" lpdt_status lpdt_evonorm_s0_fwd(int32_t nodes, int32_t B, int32_t H, 
     if (pl.V == 4 && !two_pass) {
         const int rstep = pl.threads / (C / 4);
         int ppc = 0;
-        const int Rl = evonorm_l2_cluster((int64_t)nodes * B, H * W, C / 4, pl.threads, (double)H * W * C * 4, 4, &ppc);
-        if (Rl > 0 && (int64_t)nodes * B * Rl <= 0x7fffffff) {
-            launch_k_cluster(evonorm_fwd_l2_kernel, dim3((unsigned)((int64_t)nodes * B * Rl)), pl.threads, (size_t)(2 * pl.threads + 3 * groups) * sizeof(double),
-                             as_stream(stream), Rl, H * W, C, groups, eps, x, v, gamma, beta, pstride, B, y, gmean, gvar, Rl, ppc);
-            LPDT_LAUNCH_CHECK();
-            return LPDT_OK;
-        }
+        const int64_t samples = (int64_t)nodes * B;
         // shares of up to 64 KB: measured best (clusters of 8 lose to cluster scheduling, 128 KB shares to occupancy)
         const int R = evonorm_cluster(H * W, rstep, (size_t)C * 4, 64 * 1024, 160 * 1024, &ppc);
         const size_t scratch = align_up((size_t)(2 * pl.threads + 4 * groups) * sizeof(double), 16);
+        // Within one wave (two CTAs per SM) the second trip to L2 is time that nothing covers, and the sample is held where the
+        // sums of its groups, a thread each, are short: at most sixteen parts (84 samples of 8x8x128 6.1 us from L2, 4.6 held;
+        // 30 of 26x26x128 10.2 and 7.9; but 8 of 5x5x64, 32 parts, 3.4 and 3.9, 15 of 22x22x32 4.8 and 7.4).
+        const bool held = R > 0 && scratch <= 32 * 1024 && samples * R <= 2 * kNumSMs && C / groups / 4 * rstep <= 16;
+        int ppc_l2 = 0;
+        const int Rl = evonorm_l2_cluster(samples, H * W, C / 4, pl.threads, (double)H * W * C * 4, 4, &ppc_l2);
+        const bool held_l2 = held && Rl > 0;
+        if (Rl > 0 && !held && samples * Rl <= 0x7fffffff) {
+            launch_k_cluster(evonorm_fwd_l2_kernel, dim3((unsigned)(samples * Rl)), pl.threads, (size_t)(2 * pl.threads + 3 * groups) * sizeof(double),
+                             as_stream(stream), Rl, H * W, C, groups, eps, x, v, gamma, beta, pstride, B, y, gmean, gvar, Rl, ppc_l2);
+            LPDT_LAUNCH_CHECK();
+            return LPDT_OK;
+        }
         if (R > 0 && scratch <= 32 * 1024 && (int64_t)nodes * B * R <= 0x7fffffff) {
             static PerDeviceOnce attr;
             int dev;
             if (attr.pending(&dev)) {
-                LPDT_CUDA(cudaFuncSetAttribute(evonorm_fwd_cl_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+                for (auto fn : {evonorm_fwd_cl_kernel<false>, evonorm_fwd_cl_kernel<true>})
+                    LPDT_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
                 attr.mark(dev);
             }
-            launch_k_cluster(evonorm_fwd_cl_kernel, dim3((unsigned)((int64_t)nodes * B * R)), pl.threads,
+            launch_k_cluster(held_l2 ? evonorm_fwd_cl_kernel<true> : evonorm_fwd_cl_kernel<false>, dim3((unsigned)((int64_t)nodes * B * R)), pl.threads,
                              scratch + (size_t)ppc * C * 4, as_stream(stream), R, H * W, C, groups, eps, x, v, gamma, beta,
                              pstride, B, y, gmean, gvar, R, ppc, (unsigned)scratch);
             LPDT_LAUNCH_CHECK();

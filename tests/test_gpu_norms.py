@@ -79,6 +79,13 @@ def test_evonorm_s0_fwd_bwd(case, groups):
     assert not Gh[:, 3 * C:].any()
 
 
+# samples held in shared memory by one to eight CTAs (ragged last share) because the batch is less than a wave, and just beyond one
+@pytest.mark.parametrize("case,groups", [((3, 2, 8, 8, 128), 16), ((1, 2, 33, 31, 128), 16), ((2, 2, 17, 19, 64), 16), ((1, 3, 1, 1, 128), 32),
+                                         ((4, 37, 5, 5, 128), 16), ((3, 99, 3, 3, 128), 16)])
+def test_evonorm_s0_held_samples(case, groups):
+    test_evonorm_s0_fwd_bwd(case, groups)
+
+
 @pytest.mark.parametrize("case", [(1, 3, 56, 56, 64), (2, 2, 96, 96, 16), (2, 5, 32, 32, 64), (1, 4, 33, 31, 128), (3, 2, 7, 9, 4)])
 def test_evonorm_s0_gradient_sums_lose_nothing(case):
     """With v = 0, gamma = 1 and x and dy on grids every term of a parameter gradient is exact in fp32, with no bit to spare for
