@@ -43,8 +43,7 @@ def _inputs(case, seed):
 EVO_CASES = [((4, 8, 16, 16, 16), 4), ((2, 3, 32, 32, 16), 2), ((2, 2, 8, 8, 64), 8), ((1, 3, 5, 7, 6), 3),
              ((1, 2, 4, 4, 12), 1), ((2, 2, 32, 32, 64), 8), ((1, 2, 2, 2, 512), 64), ((1, 1, 1, 1, 8), 2),
              ((1, 2, 9, 9, 24), 3),
-             # samples split over a cluster of 2, 4 or 8 CTAs (ragged last share), and one too large for the
-             # kernels that hold the sample in shared memory
+             # samples split over a cluster of 2, 4 or 8 CTAs (ragged last share)
              ((1, 2, 31, 33, 64), 16), ((2, 2, 40, 40, 64), 8), ((1, 3, 64, 64, 32), 4), ((1, 1, 96, 96, 64), 8),
              ((1, 1, 160, 160, 64), 8)]
 
@@ -77,6 +76,14 @@ def test_evonorm_s0_fwd_bwd(case, groups):
     close(Gh[:, C:2 * C], dg_ref, scale=float(np.abs(dg_ref).max()))
     close(Gh[:, 2 * C:3 * C], db_ref, scale=float(np.abs(db_ref).max()))
     assert not Gh[:, 3 * C:].any()
+
+
+# Widths whose channel columns divide no warp: held by a cluster of 2, 4 or 8 CTAs (ragged last share) in either direction, by
+# none of them in the backward pass, and by none at all.
+@pytest.mark.parametrize("case,groups", [((1, 3, 15, 15, 96), 12), ((2, 2, 33, 31, 48), 6), ((2, 2, 40, 40, 96), 12), ((1, 2, 28, 28, 512), 64),
+                                         ((1, 2, 16, 16, 256), 32), ((1, 1, 64, 64, 48), 4), ((1, 1, 96, 96, 48), 6)])
+def test_evonorm_s0_widths_beyond_a_warp(case, groups):
+    test_evonorm_s0_fwd_bwd(case, groups)
 
 
 # samples held in shared memory by one to eight CTAs (ragged last share) because the batch is less than a wave, and just beyond one
@@ -168,8 +175,8 @@ def test_norm_layer_errors():
 
 
 def test_evonorm_s0_two_pass_kernels():
-    """The kernels that read a sample twice serve shapes the shared-memory kernels do not take; the cases are
-    re-run on them in a child process."""
+    """The kernels of one CTA per sample serve what neither clusters nor shared memory take; the cases are re-run on them in a
+    child process."""
     import os, subprocess, sys
     if os.environ.get("LPDT_CHILD") == "1":
         pytest.skip("already inside a child run")
