@@ -27,7 +27,7 @@
  *     individually rounded fp32 operations (no contraction, no fast math).
  *     Reductions that decide later integer codes (ranges, the Range-EvoNorm
  *     group sum) are exact or accumulated in fp64; the per-channel parameter
- *     gradient sums add fp32 runs of at most 16 terms into fp64 accumulators.
+ *     gradient sums add individually rounded fp32 terms into fp64 accumulators.
  *     Everything is rounded to fp32 once.
  */
 #ifndef LPDT_H
@@ -411,7 +411,9 @@ lpdt_status lpdt_range_evonorm_bwd_q8(int32_t nodes, int32_t B, int32_t H, int32
  *   dbeta_c = sum dy;  dgamma_c = sum dy*m/D;  dv_c = sum t*x*x*sig*(1 - sig)/D   (over b, h, w)
  * Layouts as lpdt_range_evonorm_*: x, y, dy, dx fp32 NHWC; parameters per node at p + n*param_node_stride;
  * gmean, gvar : fp32 [nodes][B][groups], written by the forward, read by the backward.
- * Statistics and parameter-gradient sums are accumulated in double; elementwise work is fp32.
+ * Statistics and parameter-gradient sums are accumulated in double (backward, samples whose share fits shared memory
+ * and whose C/4 divides no 32: a thread's own terms, a few dozen, in fp32 first); elementwise work is fp32, fused
+ * multiply-adds included.
  * Errors: INVALID_ARG, UNSUPPORTED (more than 256 channel vectors), WORKSPACE, CUDA.
  */
 lpdt_status lpdt_evonorm_s0_fwd(int32_t nodes, int32_t B, int32_t H, int32_t W, int32_t C, int32_t groups,

@@ -2,7 +2,8 @@
 // full precision) and range batch-norm (Eq. "rbn"), forward and backward.  Same data layout
 // and thread mapping as the Range-EvoNorm kernels: fp32 NHWC, a thread owns a fixed vector of
 // V channels and walks pixels, so every global access is a coalesced 16-byte load or store.
-// Sums that feed statistics or parameter gradients are accumulated in double.  All four
+// Sums that feed statistics or parameter gradients are accumulated in double (EvoNorm-S0 backward with the sample held in
+// shared memory: a thread's own sums over its share in fp32, everything across threads in double).  All four
 // passes are HBM-bound streaming kernels.
 #include <math.h>
 #include <cooperative_groups.h>

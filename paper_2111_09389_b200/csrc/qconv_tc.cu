@@ -1018,9 +1018,7 @@ lpdt_status tc_pix(const lpdt_conv_desc &d, int mode, const int8_t *A, const flo
     return LPDT_OK;
 }
 
-// acc_user: the caller's raw-sum array or null; acc_ws: scratch of the same shape [nodes][Cout][taps][Cin]; dW: fp32 result or null.  With one split the kernel writes both outputs
-// itself; with several it accumulates into zeroed int32 storage and a conversion launch follows.
-// Tiling, stages, CTAs per SM and split of the pixel loop.
+// Backward-weight: tiling, stages, CTAs per SM and split of the pixel loop.
 static lpdt_status wgrad_plan(const lpdt_conv_desc &d, Pitches pt, WgParams &p, int &per_sm, int &stage_bytes) {
     const int Ho = conv_out(d.H, d.pad, d.R, d.stride), Wo = conv_out(d.W, d.pad, d.S, d.stride);
     p = WgParams{};
@@ -1102,6 +1100,8 @@ bool wgrad_direct(const lpdt_conv_desc &d, Pitches pt) {
     return wgrad_plan(d, pt, p, per_sm, stage_bytes) == LPDT_OK && p.splits == 1;
 }
 
+// acc_user: the caller's raw-sum array or null; acc_ws: scratch of the same shape [nodes][Cout][taps][Cin]; dW: fp32 result or null.  With one split the kernel writes both outputs
+// itself; with several it accumulates into zeroed int32 storage and a conversion launch follows.
 lpdt_status tc_wgrad(const lpdt_conv_desc &d, const int8_t *E, const float *sE, const int8_t *A,
                      const float *sA, int32_t *acc_user, int32_t *acc_ws, float *dW, int64_t dw_stride,
                      int32_t *dev_status, cudaStream_t st, bool uns, Pitches pt, size_t *more_clear) {

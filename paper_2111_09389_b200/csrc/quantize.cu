@@ -371,7 +371,7 @@ extern "C" lpdt_status lpdt_quantize_static(const float *x, int32_t nodes, int64
     uint32_t *words = nullptr;
     lpdt_status s = static_range_words(&words);
     if (s != LPDT_OK) return s;
-    // Same two passes as lpdt_quantize; it zeroes the words it uses before the range pass,
+    // Same two passes as lpdt_quantize; the words it uses are zeroed before the range pass, or stored by it,
     // so whatever the previous call left in the array does not matter.
     return lpdt_quantize(x, nodes, n_per_node, x_node_stride, mode, rounding, seed, ctr_offset, q, scale,
                          zero_point, words, sizeof(uint32_t) * 2 * kStaticMaxNodes, stream);

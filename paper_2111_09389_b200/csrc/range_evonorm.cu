@@ -1,7 +1,6 @@
 // Range-EvoNorm (Eq. "ren") forward and backward.
 //
-// One CTA per (node, sample); the forward kernel can split a sample over a cluster
-// of up to 8 CTAs.  Every thread owns a fixed vector-column of V channels and walks
+// One CTA per (node, sample), or a cluster: up to 8 CTAs forward, up to 4 backward.  Every thread owns a fixed vector-column of V channels and walks
 // the pixels, so global accesses are fully coalesced 16-byte loads and the thread's
 // channel parameters and group live in registers.
 // Forward: pass 1 finds the per-group extrema; a warp-shuffle reduction with a
@@ -9,7 +8,8 @@
 // cluster exchange their group extrema through distributed shared memory; pass 2
 // re-reads the sample and writes the output.  The second read is an L2 hit as long
 // as the samples in flight fit the L2: with large samples the cluster split keeps
-// that footprint small (fewer samples in flight, each finished sooner).  Backward is a single pass: the local term of dx is written while the
+// that footprint small (fewer samples in flight, each finished sooner).  Backward, where the CTAs of a cluster
+// meet once to add their sums, is a single pass: the local term of dx is written while the
 // group sum S and the per-channel gradient sums accumulate, and S is applied
 // afterwards at the two extremum positions of each group.  Both kernels are
 // HBM-bound: forward moves 4 B in + 4 B out per element, backward 8 B in + 4 B out.
@@ -824,7 +824,7 @@ __device__ __forceinline__ void ren_bwd_sample(unsigned char *smem_raw, int HW, 
     }
 }
 
-// One CTA per (node, sample).  MAXT = 256: three CTAs per SM at 80 registers (the thirteen double accumulators
+// R CTAs per (node, sample).  MAXT = 256: three CTAs per SM at 80 registers (the thirteen double accumulators
 // of a thread stay in registers); MAXT = 512 serves the rare plans with more than 256 threads.
 template <int V, int MAXT, int DEPTH>
 __global__ void __launch_bounds__(MAXT, MAXT == 256 ? 3 : 1)
